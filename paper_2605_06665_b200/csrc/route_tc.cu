@@ -40,34 +40,50 @@ struct RouteParams {
   int32_t* status;
 };
 
-// W_r fp32 [n_layers][M*d] -> three bf16 terms per layer [n_layers][3][M*d]; any[4 l + s] != 0 iff term
-// s of layer l has a non-zero element.
+// W_r fp32 [n_layers][n] -> three bf16 terms per layer [n_layers][3][n] (n = M*d); any[4 l + s] != 0 iff
+// term s of layer l has a non-zero element.  A grid row per layer, kSplitVec elements per thread and step.
+// Bound by HBM (4 bytes in, 6 out per weight).  The flags are what needs care: weights that use all of
+// fp32 set them everywhere, and one atomicOr per warp on one address per layer took 1.05 ms for the 12
+// routers of 96 x 768 (9.3 ms for 24 of 192 x 1536); one block-wide vote and at most one atomic per
+// block, skipped when the flag is already seen, takes 16 us (51 us).
+template <int kSplitVec>
 __global__ void __launch_bounds__(256)
 router_split_kernel(const float* __restrict__ W, int64_t n, int n_layers, __nv_bfloat16* __restrict__ out,
                     int32_t* __restrict__ any) {
-  const int64_t total = n * n_layers;
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < total; base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t g = base + threadIdx.x;
+  for (int64_t l = blockIdx.y; l < n_layers; l += gridDim.y) {
+    const float* w_l = W + l * n;
+    __nv_bfloat16* o = out + l * 3 * n;
     int flags = 0;
-    const int64_t l = (g < total ? g : total - 1) / n;
-    if (g < total) {
-      const int64_t i = g - l * n;
-      const float w = W[g];
-      const __nv_bfloat16 h0 = __float2bfloat16_rn(w);
-      const float r1 = w - __bfloat162float(h0);
-      const __nv_bfloat16 h1 = __float2bfloat16_rn(r1);
-      const float r2 = r1 - __bfloat162float(h1);
-      const __nv_bfloat16 h2 = __float2bfloat16_rn(r2);
-      __nv_bfloat16* o = out + l * 3 * n;
-      o[i] = h0;
-      o[n + i] = h1;
-      o[2 * n + i] = h2;
-      if (__bfloat162float(h1) != 0.f) flags |= 2;
-      if (__bfloat162float(h2) != 0.f) flags |= 4;
+    for (int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * kSplitVec; i < n;
+         i += (int64_t)gridDim.x * blockDim.x * kSplitVec) {
+      float w[kSplitVec];
+      if constexpr (kSplitVec == 4) {
+        const float4 v = __ldg(reinterpret_cast<const float4*>(w_l + i));
+        w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+      } else {
+        w[0] = w_l[i];
+      }
+      alignas(8) __nv_bfloat16 h[3][kSplitVec];
+#pragma unroll
+      for (int q = 0; q < kSplitVec; ++q) {
+        h[0][q] = __float2bfloat16_rn(w[q]);
+        const float r1 = w[q] - __bfloat162float(h[0][q]);
+        h[1][q] = __float2bfloat16_rn(r1);
+        h[2][q] = __float2bfloat16_rn(r1 - __bfloat162float(h[1][q]));
+        if (__bfloat162float(h[1][q]) != 0.f) flags |= 2;
+        if (__bfloat162float(h[2][q]) != 0.f) flags |= 4;
+      }
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        if constexpr (kSplitVec == 4) *reinterpret_cast<uint2*>(o + t * n + i) = *reinterpret_cast<const uint2*>(h[t]);
+        else o[t * n + i] = h[t][0];
+      }
     }
-    // a warp may straddle two layers: every lane reports for its own
-    if (flags & 2) atomicOr(&any[4 * l + 1], 1);
-    if (flags & 4) atomicOr(&any[4 * l + 2], 1);
+#pragma unroll
+    for (int t = 1; t < 3; ++t) {
+      const int set = __syncthreads_or(flags & (1 << t));
+      if (threadIdx.x == 0 && set && *static_cast<volatile int32_t*>(&any[4 * l + t]) == 0) atomicOr(&any[4 * l + t], 1);
+    }
   }
 }
 
@@ -580,9 +596,12 @@ static int router_split_launch(unipool_ctx* ctx, const float* W_r, int n_layers,
                                int32_t* flags, cudaStream_t s) {
   const int64_t n = (int64_t)M * ctx->cfg.d_model;
   UP_CUDA(cudaMemsetAsync(flags, 0, (size_t)n_layers * 4 * sizeof(int32_t), s));
-  const int64_t total = n * n_layers;
-  const int blocks = (int)((total + 255) / 256 < 1184 ? (total + 255) / 256 : 1184);
-  router_split_kernel<<<blocks, 256, 0, s>>>(W_r, n, n_layers, out, flags);
+  // n is a multiple of 64 (d is): four weights per thread unless the caller's array is not 16-byte aligned
+  const bool vec = (reinterpret_cast<uintptr_t>(W_r) & 15) == 0;
+  const int64_t blocks = (n + (vec ? 1023 : 255)) / (vec ? 1024 : 256);
+  const dim3 grid((unsigned)(blocks < 1184 ? blocks : 1184), (unsigned)(n_layers < 65535 ? n_layers : 65535));
+  if (vec) router_split_kernel<4><<<grid, 256, 0, s>>>(W_r, n, n_layers, out, flags);
+  else router_split_kernel<1><<<grid, 256, 0, s>>>(W_r, n, n_layers, out, flags);
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;
 }
