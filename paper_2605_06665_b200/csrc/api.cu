@@ -53,14 +53,18 @@ Workspace carve_workspace(const unipool_config& cfg, void* base) {
   };
   const size_t eb = cfg.dtype == UNIPOOL_BF16 ? 2 : 4;
   const int64_t cap = row_capacity_of(cfg);
-  const int64_t blocks = ((int64_t)cfg.max_tokens + kDispatchMinChunkTokens - 1) / kDispatchMinChunkTokens;
+  // most chunks of a permute: 256 tokens each, or smaller ones while that gives up to two per SM
+  const int64_t few = ((int64_t)cfg.max_tokens + kDispatchMinChunkTokens - 1) / kDispatchMinChunkTokens;
+  const int64_t many = ((int64_t)cfg.max_tokens + kDispatchChunkTokens - 1) / kDispatchChunkTokens;
+  const int64_t chunks = few < 2 * kDispatchMaxSms ? few : (many > 2 * kDispatchMaxSms ? many : 2 * kDispatchMaxSms);
+  const int64_t supers = (chunks + kDispatchSuperChunks - 1) / kDispatchSuperChunks;
   w.status = reinterpret_cast<int32_t*>(take(4 * sizeof(int32_t)));
   w.route_counts = reinterpret_cast<int32_t*>(take(UNIPOOL_MAX_EXPERTS * sizeof(int32_t)));
   w.route_sums = reinterpret_cast<double*>(take(UNIPOOL_MAX_EXPERTS * sizeof(double)));
   w.tickets = reinterpret_cast<uint32_t*>(take(8 * sizeof(uint32_t)));
   w.dsigma_acc = reinterpret_cast<double*>(take(2 * sizeof(double)));
   w.split_any = reinterpret_cast<int32_t*>(take((size_t)(cfg.n_layers + 1) * 4 * sizeof(int32_t)));
-  w.block_hist = reinterpret_cast<int32_t*>(take((size_t)blocks * UNIPOOL_MAX_EXPERTS * sizeof(int32_t)));
+  w.block_hist = reinterpret_cast<int32_t*>(take((size_t)supers * 36 * UNIPOOL_MAX_EXPERTS));
   {
     const size_t mp = ((size_t)cfg.pool_size + 63) / 64 * 64;
     const size_t per_token = cfg.dtype == UNIPOOL_BF16 ? mp * 2 : (size_t)cfg.pool_size * sizeof(float);

@@ -50,7 +50,7 @@ struct Workspace {
   double*  route_sums;    // [MAX_EXPERTS]
   uint32_t* tickets;      // [8]   "last block done" counters, self-cleaning
   double*  dsigma_acc;    // [2]   self-cleaning accumulator of route_bwd / calibrate_c
-  int32_t* block_hist;    // [dispatch_blocks, MAX_EXPERTS]
+  int32_t* block_hist;    // permute scratch: per-chunk counts (16 bits) and their sums over 16 chunks, per expert
   float*   dz;            // route_bwd scratch: fp32 [max_tokens, pool_size], or bf16 [max_tokens, ceil64(pool_size)]
   int32_t* split_any;     // [n_layers + 1][4] which bf16 terms of a router's split weights are non-zero
   void*    w_split;       // [n_layers + 1][3, pool_size, d] bf16 terms of the router weights (bf16 mode): one slot
@@ -67,8 +67,10 @@ constexpr int kGuardBytes = 256;
 constexpr unsigned kGuardWord = 0xA5A5A5A5u;
 constexpr int kGuardSite = 200;               // status site of guard band i: kGuardSite + i
 
-constexpr int kDispatchChunkTokens = 256;     // most tokens per block of the permute kernels (eight warps of 32)
-constexpr int kDispatchMinChunkTokens = 64;   // fewest
+constexpr int kDispatchChunkTokens = 256;     // most tokens per block of the placing kernel (eight warps of 32)
+constexpr int kDispatchMinChunkTokens = 16;   // fewest
+constexpr int kDispatchSuperChunks = 16;      // chunks whose counts are summed up together
+constexpr int kDispatchMaxSms = 1024;         // chunks smaller than 256 tokens are used up to two per SM of so many
 
 Workspace carve_workspace(const unipool_config& cfg, void* base);
 
@@ -108,7 +110,7 @@ namespace unipool {
 struct PhaseTimer {
   unipool_ctx* ctx; cudaStream_t s; cudaEvent_t stop = nullptr;
   PhaseTimer(unipool_ctx* c, int phase, int launches, cudaStream_t stream) : ctx(c), s(stream) {
-    if (!ctx->prof.enabled) return;
+    if (ctx == nullptr || !ctx->prof.enabled) return;
     cudaEvent_t start = ctx->prof.get();
     stop = ctx->prof.get();
     if (!start || !stop) { stop = nullptr; return; }
