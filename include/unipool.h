@@ -203,6 +203,31 @@ int unipool_expert_fwd(unipool_ctx* ctx, const void* Xp, const int32_t* offsets,
                        int32_t expert_base, int32_t n_experts, void* GU, void* A, void* Yp,
                        unipool_stream stream);
 
+/* The permute, the expert FFN and its derivatives with the group sizes at hand.  unipool_dispatch_rows also
+ * writes rows [n_experts] int32, the tokens of each group (group e = rows offsets[e] .. offsets[e] + rows[e]
+ * - 1; the rest up to offsets[e+1] is padding).  Given to the other three ([n_layers, n_experts] for
+ * unipool_pool_wgrad_rows), the tensor-core kernels leave the padding out of their products instead of
+ * multiplying its zeros; results and contents of the buffers are those of the calls without `rows`, which
+ * they are when it is NULL.  `rows` must be what the dispatch of the same layer wrote. */
+int unipool_dispatch_rows(unipool_ctx* ctx, const void* x, int32_t T, const int32_t* idx,
+                          int32_t n_experts, int32_t* offsets, int32_t* row_of, int32_t* token_of,
+                          int32_t* tile_expert, int32_t* rows, void* Xp, unipool_stream stream);
+int unipool_expert_fwd_rows(unipool_ctx* ctx, const void* Xp, const int32_t* offsets, const int32_t* rows,
+                            const int32_t* tile_expert, const void* W_gu, const void* W_down,
+                            int32_t expert_base, int32_t n_experts, void* GU, void* A, void* Yp,
+                            unipool_stream stream);
+int unipool_expert_bwd_rows(unipool_ctx* ctx, const void* dy, int32_t T, const int32_t* row_of,
+                            const float* gate, const int32_t* token_of, const int32_t* offsets,
+                            const int32_t* rows, const int32_t* tile_expert, const void* Xp, const void* GU,
+                            const void* A, const void* Yp, const void* W_gu, const void* W_down,
+                            int32_t expert_base, int32_t n_experts, const void* dx_residual, void* dYp,
+                            void* dGU, void* dx, float* dgate, float* dW_gu, float* dW_down, int32_t flags,
+                            unipool_stream stream);
+int unipool_pool_wgrad_rows(unipool_ctx* ctx, int32_t n_layers, int64_t layer_stride_rows,
+                            const int32_t* offsets, const int32_t* rows, const void* Xp, const void* A,
+                            const void* dYp, const void* dGU, int32_t expert_base, int32_t n_experts,
+                            float* dW_gu, float* dW_down, int32_t flags, unipool_stream stream);
+
 /* Gate-weighted combine (Eq. 2): y_t = sum_j gate[t,j] * Yp[row_of[t,j]], summed in
  * fp32 and rounded once; with residual != NULL the output is residual + y (the
  * residual block x_{l+1} = x_l + FFN_l(x_l)).

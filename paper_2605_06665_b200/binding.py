@@ -26,6 +26,7 @@ EXPORTS = (
     "unipool_pool_aux_loss", "unipool_route_bwd", "unipool_calibrate_c",
     "unipool_profile_enable", "unipool_profile_read", "unipool_dispatch_static",
     "unipool_unique_experts", "unipool_router_prepare", "unipool_selftest_wait",
+    "unipool_dispatch_rows", "unipool_expert_fwd_rows", "unipool_expert_bwd_rows", "unipool_pool_wgrad_rows",
 )
 
 PHASES = (
@@ -83,6 +84,15 @@ def lib():
     L.unipool_router_prepare.argtypes = [vp, vp, i32, i32, vp]
     L.unipool_dispatch.restype = ctypes.c_int
     L.unipool_dispatch.argtypes = [vp, vp, i32, vp, i32, vp, vp, vp, vp, vp, vp]
+    L.unipool_dispatch_rows.restype = ctypes.c_int
+    L.unipool_dispatch_rows.argtypes = [vp, vp, i32, vp, i32, vp, vp, vp, vp, vp, vp, vp]
+    L.unipool_expert_fwd_rows.restype = ctypes.c_int
+    L.unipool_expert_fwd_rows.argtypes = [vp, vp, vp, vp, vp, vp, vp, i32, i32, vp, vp, vp, vp]
+    L.unipool_expert_bwd_rows.restype = ctypes.c_int
+    L.unipool_expert_bwd_rows.argtypes = [vp, vp, i32, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, vp, i32, i32,
+                                          vp, vp, vp, vp, vp, vp, vp, i32, vp]
+    L.unipool_pool_wgrad_rows.restype = ctypes.c_int
+    L.unipool_pool_wgrad_rows.argtypes = [vp, i32, i64, vp, vp, vp, vp, vp, vp, i32, i32, vp, vp, i32, vp]
     L.unipool_dispatch_static.restype = ctypes.c_int
     L.unipool_dispatch_static.argtypes = [vp, i32, i32, i32, i32, vp, i32, i64, vp, vp, vp, vp, vp, vp]
     L.unipool_expert_fwd.restype = ctypes.c_int
@@ -190,31 +200,32 @@ class Context:
     def router_prepare(self, W_r, n_layers, n_experts):
         _check(lib().unipool_router_prepare(self.handle, _p(W_r), n_layers, n_experts, _stream()))
 
-    def dispatch(self, x, T, idx, n_experts, offsets, row_of, token_of, tile_expert, Xp):
-        _check(lib().unipool_dispatch(self.handle, _p(x), T, _p(idx), n_experts, _p(offsets), _p(row_of),
-                                      _p(token_of), _p(tile_expert), _p(Xp), _stream()))
+    # (``rows`` [.., n_experts]: the group sizes; NULL makes the _rows calls the plain ones)
+    def dispatch(self, x, T, idx, n_experts, offsets, row_of, token_of, tile_expert, Xp, rows=None):
+        _check(lib().unipool_dispatch_rows(self.handle, _p(x), T, _p(idx), n_experts, _p(offsets), _p(row_of),
+                                           _p(token_of), _p(tile_expert), _p(rows), _p(Xp), _stream()))
 
-    def expert_fwd(self, Xp, offsets, tile_expert, W_gu, W_down, expert_base, n_experts, GU, A, Yp):
-        _check(lib().unipool_expert_fwd(self.handle, _p(Xp), _p(offsets), _p(tile_expert), _p(W_gu),
-                                        _p(W_down), expert_base, n_experts, _p(GU), _p(A), _p(Yp), _stream()))
+    def expert_fwd(self, Xp, offsets, tile_expert, W_gu, W_down, expert_base, n_experts, GU, A, Yp, rows=None):
+        _check(lib().unipool_expert_fwd_rows(self.handle, _p(Xp), _p(offsets), _p(rows), _p(tile_expert), _p(W_gu),
+                                             _p(W_down), expert_base, n_experts, _p(GU), _p(A), _p(Yp), _stream()))
 
     def combine(self, Yp, row_of, gate, T, residual, y):
         _check(lib().unipool_combine(self.handle, _p(Yp), _p(row_of), _p(gate), T, _p(residual), _p(y),
                                      _stream()))
 
     def expert_bwd(self, dy, T, row_of, gate, token_of, offsets, tile_expert, Xp, GU, A, Yp, W_gu, W_down,
-                   expert_base, n_experts, dx_residual, dYp, dGU, dx, dgate, dW_gu, dW_down, flags=0):
-        _check(lib().unipool_expert_bwd(self.handle, _p(dy), T, _p(row_of), _p(gate), _p(token_of),
-                                        _p(offsets), _p(tile_expert), _p(Xp), _p(GU), _p(A), _p(Yp),
-                                        _p(W_gu), _p(W_down), expert_base, n_experts, _p(dx_residual),
-                                        _p(dYp), _p(dGU), _p(dx), _p(dgate), _p(dW_gu), _p(dW_down),
-                                        flags, _stream()))
+                   expert_base, n_experts, dx_residual, dYp, dGU, dx, dgate, dW_gu, dW_down, flags=0, rows=None):
+        _check(lib().unipool_expert_bwd_rows(self.handle, _p(dy), T, _p(row_of), _p(gate), _p(token_of),
+                                             _p(offsets), _p(rows), _p(tile_expert), _p(Xp), _p(GU), _p(A), _p(Yp),
+                                             _p(W_gu), _p(W_down), expert_base, n_experts, _p(dx_residual),
+                                             _p(dYp), _p(dGU), _p(dx), _p(dgate), _p(dW_gu), _p(dW_down),
+                                             flags, _stream()))
 
     def pool_wgrad(self, n_layers, layer_stride_rows, offsets, Xp, A, dYp, dGU, expert_base, n_experts,
-                   dW_gu, dW_down, flags=0):
-        _check(lib().unipool_pool_wgrad(self.handle, n_layers, layer_stride_rows, _p(offsets), _p(Xp), _p(A),
-                                        _p(dYp), _p(dGU), expert_base, n_experts, _p(dW_gu), _p(dW_down),
-                                        flags, _stream()))
+                   dW_gu, dW_down, flags=0, rows=None):
+        _check(lib().unipool_pool_wgrad_rows(self.handle, n_layers, layer_stride_rows, _p(offsets), _p(rows), _p(Xp),
+                                             _p(A), _p(dYp), _p(dGU), expert_base, n_experts, _p(dW_gu), _p(dW_down),
+                                             flags, _stream()))
 
     def pool_aux_loss(self, counts, score_sum, L, n_experts, T, alpha, fbar_prev, loss, dscore_coef, fbar_out):
         _check(lib().unipool_pool_aux_loss(self.handle, _p(counts), _p(score_sum), L, n_experts, T, alpha,

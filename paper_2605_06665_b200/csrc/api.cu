@@ -256,26 +256,40 @@ int unipool_router_prepare(unipool_ctx* ctx, const float* W_r, int32_t n_layers,
   return router_prepare_launch(ctx, W_r, n_layers, n_experts, static_cast<cudaStream_t>(stream));
 }
 
-int unipool_dispatch(unipool_ctx* ctx, const void* x, int32_t T, const int32_t* idx,
-                     int32_t n_experts, int32_t* offsets, int32_t* row_of, int32_t* token_of,
-                     int32_t* tile_expert, void* Xp, unipool_stream stream) {
+int unipool_dispatch_rows(unipool_ctx* ctx, const void* x, int32_t T, const int32_t* idx,
+                          int32_t n_experts, int32_t* offsets, int32_t* row_of, int32_t* token_of,
+                          int32_t* tile_expert, int32_t* rows, void* Xp, unipool_stream stream) {
   CHECK_CTX(ctx); CHECK_T(ctx, T); CHECK_ROUTER_WIDTH(ctx, n_experts);
   CHECK_PTR(x); CHECK_PTR(idx); CHECK_PTR(offsets); CHECK_PTR(row_of); CHECK_PTR(token_of);
   CHECK_PTR(tile_expert); CHECK_PTR(Xp);
-  return dispatch_launch(ctx, x, T, idx, n_experts, offsets, row_of, token_of, tile_expert, Xp,
+  return dispatch_launch(ctx, x, T, idx, n_experts, offsets, row_of, token_of, tile_expert, rows, Xp,
                          static_cast<cudaStream_t>(stream));
+}
+
+int unipool_dispatch(unipool_ctx* ctx, const void* x, int32_t T, const int32_t* idx,
+                     int32_t n_experts, int32_t* offsets, int32_t* row_of, int32_t* token_of,
+                     int32_t* tile_expert, void* Xp, unipool_stream stream) {
+  return unipool_dispatch_rows(ctx, x, T, idx, n_experts, offsets, row_of, token_of, tile_expert, nullptr, Xp, stream);
+}
+
+int unipool_expert_fwd_rows(unipool_ctx* ctx, const void* Xp, const int32_t* offsets, const int32_t* rows,
+                            const int32_t* tile_expert, const void* W_gu, const void* W_down,
+                            int32_t expert_base, int32_t n_experts, void* GU, void* A, void* Yp,
+                            unipool_stream stream) {
+  CHECK_CTX(ctx); CHECK_VIEW(ctx, expert_base, n_experts);
+  CHECK_PTR(Xp); CHECK_PTR(offsets); CHECK_PTR(tile_expert); CHECK_PTR(W_gu); CHECK_PTR(W_down);
+  CHECK_PTR(GU); CHECK_PTR(A); CHECK_PTR(Yp);
+  ExpertFwdArgs a{Xp, offsets, tile_expert, W_gu, W_down, expert_base, n_experts, GU, A, Yp, rows};
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  return use_tensor_cores(ctx) ? expert_fwd_tc(ctx, a, s) : expert_fwd_simt(ctx, a, s);
 }
 
 int unipool_expert_fwd(unipool_ctx* ctx, const void* Xp, const int32_t* offsets,
                        const int32_t* tile_expert, const void* W_gu, const void* W_down,
                        int32_t expert_base, int32_t n_experts, void* GU, void* A, void* Yp,
                        unipool_stream stream) {
-  CHECK_CTX(ctx); CHECK_VIEW(ctx, expert_base, n_experts);
-  CHECK_PTR(Xp); CHECK_PTR(offsets); CHECK_PTR(tile_expert); CHECK_PTR(W_gu); CHECK_PTR(W_down);
-  CHECK_PTR(GU); CHECK_PTR(A); CHECK_PTR(Yp);
-  ExpertFwdArgs a{Xp, offsets, tile_expert, W_gu, W_down, expert_base, n_experts, GU, A, Yp};
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  return use_tensor_cores(ctx) ? expert_fwd_tc(ctx, a, s) : expert_fwd_simt(ctx, a, s);
+  return unipool_expert_fwd_rows(ctx, Xp, offsets, nullptr, tile_expert, W_gu, W_down, expert_base, n_experts, GU, A, Yp,
+                                 stream);
 }
 
 int unipool_combine(unipool_ctx* ctx, const void* Yp, const int32_t* row_of, const float* gate,
@@ -285,8 +299,8 @@ int unipool_combine(unipool_ctx* ctx, const void* Yp, const int32_t* row_of, con
   return combine_launch(ctx, Yp, row_of, gate, T, residual, y, static_cast<cudaStream_t>(stream));
 }
 
-int unipool_expert_bwd(unipool_ctx* ctx, const void* dy, int32_t T, const int32_t* row_of,
-                       const float* gate, const int32_t* token_of, const int32_t* offsets,
+int unipool_expert_bwd_rows(unipool_ctx* ctx, const void* dy, int32_t T, const int32_t* row_of,
+                       const float* gate, const int32_t* token_of, const int32_t* offsets, const int32_t* rows,
                        const int32_t* tile_expert, const void* Xp, const void* GU, const void* A,
                        const void* Yp, const void* W_gu, const void* W_down, int32_t expert_base,
                        int32_t n_experts, const void* dx_residual, void* dYp, void* dGU, void* dx,
@@ -304,14 +318,26 @@ int unipool_expert_bwd(unipool_ctx* ctx, const void* dy, int32_t T, const int32_
   int rc = combine_bwd_launch(ctx, dy, T, row_of, gate, token_of, offsets, n_experts, Yp, dYp, dgate, s);
   if (rc != UNIPOOL_OK) return rc;
   ExpertBwdArgs a{offsets, tile_expert, Xp, GU, A, W_gu, W_down, expert_base, n_experts,
-                  dYp, dGU, ctx->ws.dXp, dW_gu, dW_down, wgrad, (flags & UNIPOOL_WGRAD_OVERWRITE) != 0};
+                  dYp, dGU, ctx->ws.dXp, dW_gu, dW_down, wgrad, (flags & UNIPOOL_WGRAD_OVERWRITE) != 0, rows};
   rc = use_tensor_cores(ctx) ? expert_bwd_tc(ctx, a, s) : expert_bwd_simt(ctx, a, s);
   if (rc != UNIPOOL_OK) return rc;
   return unpermute_sum_launch(ctx, ctx->ws.dXp, row_of, T, dx_residual, dx, s);
 }
 
-int unipool_pool_wgrad(unipool_ctx* ctx, int32_t n_layers, int64_t layer_stride_rows,
-                       const int32_t* offsets, const void* Xp, const void* A, const void* dYp,
+int unipool_expert_bwd(unipool_ctx* ctx, const void* dy, int32_t T, const int32_t* row_of,
+                       const float* gate, const int32_t* token_of, const int32_t* offsets,
+                       const int32_t* tile_expert, const void* Xp, const void* GU, const void* A,
+                       const void* Yp, const void* W_gu, const void* W_down, int32_t expert_base,
+                       int32_t n_experts, const void* dx_residual, void* dYp, void* dGU, void* dx,
+                       float* dgate, float* dW_gu, float* dW_down, int32_t flags,
+                       unipool_stream stream) {
+  return unipool_expert_bwd_rows(ctx, dy, T, row_of, gate, token_of, offsets, nullptr, tile_expert, Xp, GU, A, Yp,
+                                 W_gu, W_down, expert_base, n_experts, dx_residual, dYp, dGU, dx, dgate, dW_gu,
+                                 dW_down, flags, stream);
+}
+
+int unipool_pool_wgrad_rows(unipool_ctx* ctx, int32_t n_layers, int64_t layer_stride_rows,
+                       const int32_t* offsets, const int32_t* rows, const void* Xp, const void* A, const void* dYp,
                        const void* dGU, int32_t expert_base, int32_t n_experts, float* dW_gu,
                        float* dW_down, int32_t flags, unipool_stream stream) {
   CHECK_CTX(ctx); CHECK_VIEW(ctx, expert_base, n_experts);
@@ -327,9 +353,17 @@ int unipool_pool_wgrad(unipool_ctx* ctx, int32_t n_layers, int64_t layer_stride_
   if (dW_down != nullptr) { CHECK_PTR(A); CHECK_PTR(dYp); }
   UP_REQUIRE((flags & ~UNIPOOL_WGRAD_OVERWRITE) == 0, UNIPOOL_ERR_INVALID_ARG, "unknown flags 0x%x", flags);
   PoolWgradArgs a{n_layers, layer_stride_rows, offsets, Xp, A, dYp, dGU, expert_base, n_experts,
-                  dW_gu, dW_down, (flags & UNIPOOL_WGRAD_OVERWRITE) != 0};
+                  dW_gu, dW_down, (flags & UNIPOOL_WGRAD_OVERWRITE) != 0, rows};
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   return use_tensor_cores(ctx) ? pool_wgrad_tc(ctx, a, s) : pool_wgrad_simt(ctx, a, s);
+}
+
+int unipool_pool_wgrad(unipool_ctx* ctx, int32_t n_layers, int64_t layer_stride_rows,
+                       const int32_t* offsets, const void* Xp, const void* A, const void* dYp,
+                       const void* dGU, int32_t expert_base, int32_t n_experts, float* dW_gu,
+                       float* dW_down, int32_t flags, unipool_stream stream) {
+  return unipool_pool_wgrad_rows(ctx, n_layers, layer_stride_rows, offsets, nullptr, Xp, A, dYp, dGU, expert_base,
+                                 n_experts, dW_gu, dW_down, flags, stream);
 }
 
 int unipool_pool_aux_loss(unipool_ctx* ctx, const int32_t* counts, const float* score_sum,

@@ -149,7 +149,7 @@ int route_bwd_launch(unipool_ctx*, const void* x, int T, const float* W_r, float
                      cudaStream_t);
 int dispatch_launch(unipool_ctx*, const void* x, int T, const int32_t* idx, int n_experts,
                     int32_t* offsets, int32_t* row_of, int32_t* token_of, int32_t* tile_expert,
-                    void* Xp, cudaStream_t);
+                    int32_t* rows, void* Xp, cudaStream_t);
 int combine_launch(unipool_ctx*, const void* Yp, const int32_t* row_of, const float* gate, int T,
                    const void* residual, void* y, cudaStream_t);
 int combine_bwd_launch(unipool_ctx*, const void* dy, int T, const int32_t* row_of,
@@ -172,17 +172,20 @@ struct ExpertFwdArgs {
   const void* Xp; const int32_t* offsets; const int32_t* tile_expert;
   const void* W_gu; const void* W_down; int expert_base; int n_experts;
   void* GU; void* A; void* Yp;
+  const int32_t* rows;                   // true group sizes, NULL: the padded ones
 };
 struct ExpertBwdArgs {
   const int32_t* offsets; const int32_t* tile_expert;
   const void* Xp; const void* GU; const void* A; const void* W_gu; const void* W_down;
   int expert_base; int n_experts;
   const void* dYp; void* dGU; void* dXp; float* dW_gu; float* dW_down; bool wgrad; bool overwrite;
+  const int32_t* rows;
 };
 struct PoolWgradArgs {
   int n_layers; int64_t layer_stride_rows; const int32_t* offsets;
   const void* Xp; const void* A; const void* dYp; const void* dGU;
   int expert_base; int n_experts; float* dW_gu; float* dW_down; bool overwrite;
+  const int32_t* rows;                   // [n_layers, n_experts]
 };
 int route_tc_launch(unipool_ctx*, const void* x, int T, const float* W_r, float sigma, const float* bias,
                     int n_experts, int32_t* idx, float* gate, int32_t* counts, float* score_sum,
@@ -202,6 +205,10 @@ int pool_wgrad_simt(unipool_ctx*, const PoolWgradArgs&, cudaStream_t);
 int expert_fwd_tc(unipool_ctx*, const ExpertFwdArgs&, cudaStream_t);
 int expert_bwd_tc(unipool_ctx*, const ExpertBwdArgs&, cudaStream_t);
 int pool_wgrad_tc(unipool_ctx*, const PoolWgradArgs&, cudaStream_t);
+int wm_fwd_gu(unipool_ctx*, const ExpertFwdArgs&, cudaStream_t);
+int wm_fwd_down(unipool_ctx*, const ExpertFwdArgs&, cudaStream_t);
+int wm_dgrad_down(unipool_ctx*, const ExpertBwdArgs&, cudaStream_t);
+int wm_dgrad_gu(unipool_ctx*, const ExpertBwdArgs&, cudaStream_t);
 int tc_module_init(unipool_ctx*);
 void tc_module_destroy(unipool_ctx*);
 

@@ -92,7 +92,7 @@ dispatch_place_kernel(const int32_t* __restrict__ idx, int T, int k, int M, int 
                       int32_t* __restrict__ status, const uint4* __restrict__ x,
                       int row_vecs, int row_capacity, int32_t* __restrict__ offsets,
                       int32_t* __restrict__ row_of, int32_t* __restrict__ token_of,
-                      int32_t* __restrict__ tile_expert, uint4* __restrict__ Xp) {
+                      int32_t* __restrict__ tile_expert, int32_t* __restrict__ group_rows, uint4* __restrict__ Xp) {
   extern __shared__ int sm[];
   int* hist = sm;                                   // [8][M] per-warp histograms, then per-warp next rows
   int* start = hist + kDispatchWarps * M;           // [M + 1] group starts
@@ -246,7 +246,10 @@ dispatch_place_kernel(const int32_t* __restrict__ idx, int T, int k, int M, int 
   }
   // (f) bookkeeping, shared out over the blocks
   if (me == 0)
-    for (int e = threadIdx.x; e <= M; e += blockDim.x) offsets[e] = start[e];
+    for (int e = threadIdx.x; e <= M; e += blockDim.x) {
+      offsets[e] = start[e];
+      if (group_rows != nullptr && e < M) group_rows[e] = total[e];
+    }
   for (int p = me * kDispatchWarps + warp; p < M * UNIPOOL_ROW_ALIGN; p += (int)gridDim.x * kDispatchWarps) {
     const int e = p / UNIPOOL_ROW_ALIGN;                                   // pad row p % 128 of expert e, if it has so many
     const int r = start[e] + total[e] + p % UNIPOOL_ROW_ALIGN;
@@ -420,9 +423,10 @@ combine_bwd_kernel(const uint4* __restrict__ dy, const uint4* __restrict__ Yp,
   }
 }
 
-__global__ void dispatch_empty_kernel(int32_t* offsets, int32_t* token_of, int32_t* tile_expert, int M,
-                                      int row_capacity) {
+__global__ void dispatch_empty_kernel(int32_t* offsets, int32_t* token_of, int32_t* tile_expert, int32_t* group_rows,
+                                      int M, int row_capacity) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (group_rows != nullptr && i < M) group_rows[i] = 0;
   if (i <= M) offsets[i] = 0;
   if (i < row_capacity) token_of[i] = -1;
   if (i < row_capacity / UNIPOOL_ROW_ALIGN) tile_expert[i] = -1;
@@ -448,7 +452,8 @@ constexpr int64_t kSelfCountAssignments = 4096;
 // The two launches of the permute (T > 0).  counts: scratch, 36 bytes per (16 chunks, expert).
 static int permute_launch(unipool_ctx* prof, const void* x, int T, int k, const int32_t* idx, int M, int chunk,
                           int sm_count, void* counts, int32_t* status, int row_vecs, int cap, int32_t* offsets,
-                          int32_t* row_of, int32_t* token_of, int32_t* tile_expert, void* Xp, cudaStream_t s) {
+                          int32_t* row_of, int32_t* token_of, int32_t* tile_expert, int32_t* rows, void* Xp,
+                          cudaStream_t s) {
   const int n_chunks = (T + chunk - 1) / chunk;
   ChunkCounts cc = chunk_counts(counts, n_chunks, M);
   if ((int64_t)T * k <= kSelfCountAssignments) {
@@ -463,7 +468,7 @@ static int permute_launch(unipool_ctx* prof, const void* x, int T, int k, const 
   const int grid = n_chunks > sm_count ? n_chunks : sm_count;
   dispatch_place_kernel<<<grid, kDispatchWarps * 32, place_smem_bytes(M, k, chunk), s>>>(
       idx, T, k, M, chunk, cc, status, static_cast<const uint4*>(x), row_vecs, cap, offsets, row_of, token_of, tile_expert,
-      static_cast<uint4*>(Xp));
+      rows, static_cast<uint4*>(Xp));
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;
 }
@@ -476,17 +481,17 @@ static int row_mover_grid(const unipool_ctx* ctx, int64_t rows) {
 
 int dispatch_launch(unipool_ctx* ctx, const void* x, int T, const int32_t* idx, int M,
                     int32_t* offsets, int32_t* row_of, int32_t* token_of, int32_t* tile_expert,
-                    void* Xp, cudaStream_t s) {
+                    int32_t* rows, void* Xp, cudaStream_t s) {
   const int k = ctx->cfg.top_k, d = ctx->cfg.d_model;
   const int cap = (int)ctx->row_capacity;
   if (T == 0) {
-    dispatch_empty_kernel<<<(cap + 255) / 256, 256, 0, s>>>(offsets, token_of, tile_expert, M, cap);
+    dispatch_empty_kernel<<<(cap + 255) / 256, 256, 0, s>>>(offsets, token_of, tile_expert, rows, M, cap);
     UP_LAUNCH_CHECK();
     return UNIPOOL_OK;
   }
   return permute_launch(ctx, x, T, k, idx, M, dispatch_chunk_tokens(T, ctx->sm_count), ctx->sm_count, ctx->ws.block_hist,
                         ctx->ws.status, (int)((size_t)d * ctx->elem_bytes / 16), cap, offsets, row_of, token_of,
-                        tile_expert, Xp, s);
+                        tile_expert, rows, Xp, s);
 }
 
 template <typename T>
@@ -618,7 +623,7 @@ extern "C" int unipool_dispatch_static(const void* x, int32_t T, int32_t d_model
   int32_t* counts = info->addr + 64;
   const int cap = (int)row_capacity;
   if (T == 0) {
-    dispatch_empty_kernel<<<(cap + 255) / 256, 256, 0, s>>>(offsets, token_of, tile_expert, n_experts, cap);
+    dispatch_empty_kernel<<<(cap + 255) / 256, 256, 0, s>>>(offsets, token_of, tile_expert, nullptr, n_experts, cap);
     UP_LAUNCH_CHECK();
     return UNIPOOL_OK;
   }
@@ -627,5 +632,5 @@ extern "C" int unipool_dispatch_static(const void* x, int32_t T, int32_t d_model
   int sm_count = 0;
   UP_CUDA(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
   return permute_launch(nullptr, x, T, top_k, idx, n_experts, kDispatchChunkTokens, sm_count, counts, status,
-                        (int)((size_t)d_model * eb / 16), cap, offsets, row_of, token_of, tile_expert, Xp, s);
+                        (int)((size_t)d_model * eb / 16), cap, offsets, row_of, token_of, tile_expert, nullptr, Xp, s);
 }

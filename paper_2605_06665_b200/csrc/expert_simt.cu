@@ -173,7 +173,7 @@ static int bwd_impl(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
   }
   if (a.wgrad) {
     PoolWgradArgs w{1, 0, a.offsets, a.Xp, a.A, a.dYp, a.dGU, a.expert_base, a.n_experts, a.dW_gu, a.dW_down,
-                    a.overwrite};
+                    a.overwrite, a.rows};
     return wgrad_impl<TE>(ctx, w, s);
   }
   return UNIPOOL_OK;

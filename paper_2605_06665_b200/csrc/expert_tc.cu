@@ -15,9 +15,11 @@
 //   wgrad_pair_kernel             the weight gradient on CTA pairs (cta_group::2, M = 256)
 //   row_pair_kernel<MODE>         the four row-tile GEMMs on CTA pairs (M = 256, and M = 128 for a
 //                                 group's odd last tile)
+// and, in expert_wm.cu, wm_kernel<MODE>: the four row GEMMs with the weights on the M side.
 #include <cuda.h>
 
 #include "common.cuh"
+#include "tc_maps.cuh"
 #include "tc_ptx.cuh"
 
 namespace unipool {
@@ -41,14 +43,6 @@ static_assert(kSmemTotal <= 227 * 1024, "shared-memory budget");
 constexpr int kChunk = 32;       // output columns one epilogue step moves (a 32 x 32 box per warp)
 constexpr uint32_t kBf16ChunkBytes = 32 * kChunk * 2;      // 2 KiB, 64-byte rows, 64-byte swizzle
 constexpr uint32_t kF32ChunkBytes = 32 * kChunk * 4;       // 4 KiB, 128-byte rows, 128-byte swizzle
-
-enum Mode : int {
-  kFwd1 = 0,    // GU = Xp W_gu^T, A = silu(G)*U        A K-major, B K-major (3-D map), row tiles
-  kFwd2 = 1,    // Yp = A W_down^T                      A K-major, B K-major,           row tiles
-  kDgrad1 = 2,  // dGU = swiglu'(dYp W_down, GU)        A K-major, B MN-major,          row tiles
-  kDgrad2 = 3,  // dXp = dGU W_gu                       A K-major, B MN-major,          row tiles
-  kWgrad = 4,   // dW[e] (+)= P_e^T Q_e                 A MN-major, B MN-major,         ragged K
-};
 
 struct GemmParams {
   const int32_t* offsets;       // row tiles: &offsets[n_experts]; wgrad: [n_layers][n_experts+1]
@@ -170,18 +164,6 @@ __device__ __forceinline__ void report_timeout(const GemmParams& p, volatile int
   }
 }
 
-__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
-  return *reinterpret_cast<uint32_t*>(&v);
-}
-
-// logistic function through one special-function op: sig(a) = 0.5 + 0.5 tanh(a/2)
-__device__ __forceinline__ float sigmoid_fast(float a) {
-  float t;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(t) : "f"(0.5f * a));
-  return fmaf(0.5f, t, 0.5f);
-}
-
 // Staging tiles are 32 rows (one per lane) of kChunk columns in the layout the TMA
 // swizzle modes expect, so that a warp's 16-byte accesses never collide on a bank:
 //   bf16: 64-byte rows, 16-byte piece q of row r sits at piece q ^ ((r >> 1) & 3)
@@ -196,8 +178,8 @@ __device__ __forceinline__ void stage_row_bf16(uint8_t* tile, int r, const float
 #pragma unroll
   for (int q = 0; q < 4; ++q)
     *bf16_piece(tile, r, q) =
-        make_uint4(pack_bf16(v[8 * q + 0], v[8 * q + 1]), pack_bf16(v[8 * q + 2], v[8 * q + 3]),
-                   pack_bf16(v[8 * q + 4], v[8 * q + 5]), pack_bf16(v[8 * q + 6], v[8 * q + 7]));
+        make_uint4(tc::pack_bf16(v[8 * q + 0], v[8 * q + 1]), tc::pack_bf16(v[8 * q + 2], v[8 * q + 3]),
+                   tc::pack_bf16(v[8 * q + 4], v[8 * q + 5]), tc::pack_bf16(v[8 * q + 6], v[8 * q + 7]));
 }
 __device__ __forceinline__ void unstage_row_bf16(uint8_t* tile, int r, float (&v)[32]) {
 #pragma unroll
@@ -262,7 +244,7 @@ __device__ __forceinline__ void epilogue_swiglu(const CUtensorMap* tmC0, const C
     for (int i = 0; i < 32; ++i) {
       g[i] = __uint_as_float(rg[i]);
       u[i] = __uint_as_float(ru[i]);
-      a[i] = g[i] * sigmoid_fast(g[i]) * u[i];
+      a[i] = g[i] * tc::sigmoid_fast(g[i]) * u[i];
     }
     // lanes 0, 1, 2 each own one of the three stores (G, U, A), so the stores are issued and
     // their shared-memory reads awaited side by side
@@ -586,7 +568,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
             const float dA = __uint_as_float(rr[i]);
-            const float sig = sigmoid_fast(g[i]);
+            const float sig = tc::sigmoid_fast(g[i]);
             const float sl = g[i] * sig;
             dg[i] = dA * u[i] * (sig + sl * (1.0f - sig));   // silu'(g) = sig (1 + g (1 - sig))
             du[i] = dA * sl;
@@ -890,7 +872,7 @@ struct TcModule {
   EncodeTiledFn encode;
 };
 
-enum MapKind { kMapOperand, kMapBf16Chunk, kMapF32Chunk };
+}  // namespace
 
 // Tensor map over a dense row-major tensor; dims/box innermost first, strides in elements.
 //   kMapOperand   bf16, 128-byte swizzle (MMA operand tiles)
@@ -916,7 +898,7 @@ int make_tmap(const unipool_ctx* ctx, CUtensorMap* out, MapKind kind, const void
 }
 
 int map_2d(const unipool_ctx* ctx, CUtensorMap* out, const void* base, uint64_t cols, uint64_t rows,
-           uint32_t box_cols, uint32_t box_rows, MapKind kind = kMapOperand) {
+           uint32_t box_cols, uint32_t box_rows, MapKind kind) {
   const uint64_t dims[2] = {cols, rows}, strides[1] = {cols};
   const uint32_t box[2] = {box_cols, box_rows};
   return make_tmap(ctx, out, kind, base, 2, dims, strides, box);
@@ -931,6 +913,8 @@ int map_mn(const unipool_ctx* ctx, CUtensorMap* out, const void* base, uint64_t 
   const uint32_t box[3] = {64, 64, blocks};
   return make_tmap(ctx, out, kMapOperand, base, 3, dims, strides, box);
 }
+
+namespace {
 
 // 32 x 32 epilogue chunk map
 int map_chunk(const unipool_ctx* ctx, CUtensorMap* out, const void* base, uint64_t cols, uint64_t rows,
@@ -1254,7 +1238,7 @@ row_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
 #pragma unroll
           for (int i = 0; i < 32; ++i) {
             const float dA = __uint_as_float(rr[i]);
-            const float sig = sigmoid_fast(g[i]);
+            const float sig = tc::sigmoid_fast(g[i]);
             const float sl = g[i] * sig;
             dg[i] = dA * u[i] * (sig + sl * (1.0f - sig));   // silu'(g) = sig (1 + g (1 - sig))
             du[i] = dA * sl;
@@ -1328,6 +1312,31 @@ int launch(unipool_ctx* ctx, int phase, const CUtensorMap& tmA, const CUtensorMa
 bool rows_on_pairs(const unipool_ctx* ctx, int n_experts) {
   if (ctx->sm_count < 2 || ctx->row_capacity / (2 * BM) + n_experts >= 65535) return false;
   return (int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k >= (int64_t)4 * BM * n_experts;
+}
+
+// Weights or tokens on the M side, by the rows the average expert gets from a full batch (the group sizes
+// themselves are on the device).  Measured per GEMM, interleaved, tokens / weights on M in us (768 x 2048; the
+// figures of 1536 x 4096 are marked *):
+//   rows                85        125       170       341        500         682         1024*       1365
+//   gate/up          126/130   143/145   180/171   271/266    363/363     *1678/1602  1589/1590   213/223
+//   down              70/75     78/82     90/86    132/123    169/169     *760/763    728/724     101/107
+//   dgrad down        91/93    110/104   138/120   201/193    262/246     *1073/971   1013/952    164/164
+//   dgrad gate/up    117/124   132/132   154/142   240/212    308/308     *1494/1474  1413/1392   185/191
+// Below ~128 rows every launch is bound by streaming the weights and the token-major kernels keep more bytes in
+// flight; large groups waste nothing in 256-row pair-tiles.  Down and dgrad gate/up gain while a group is one or
+// two chunks (and need a contraction long enough to hide the epilogue of a wide unit: 384 experts of 768 x 512 lost
+// 10 % on the down projection, 4 % on dgrad gate/up); dgrad down gains longest, its G and U traffic being the
+// same on fewer padded rows; gate/up gains beyond 450 rows only where its contraction is long.
+bool weights_on_m(const unipool_ctx* ctx, int mode, int n_experts) {
+  if (ctx->sm_count < 2 || n_experts > kWmMaxExperts) return false;
+  const int64_t rows = (int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k / n_experts;
+  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff;
+  switch (mode) {
+    case kFwd1: return rows > 150 && rows <= (d >= 1024 ? 1024 : 450);
+    case kFwd2: return rows > 150 && rows <= 450 && f > 1024;
+    case kDgrad1: return rows > 100 && rows <= 1200;
+    default: return rows > 150 && rows <= 450 && 2 * f > 1024;
+  }
 }
 
 // One row-tile GEMM.  tmA / tmB / tmB64: the operand maps of the single-CTA kernel (tmB64: 64 x 64 boxes
@@ -1409,17 +1418,24 @@ void tc_module_destroy(unipool_ctx* ctx) {
   ctx->tmap_cache = nullptr;
 }
 
-int expert_fwd_tc(unipool_ctx* ctx, const ExpertFwdArgs& a, cudaStream_t s) {
-  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff, M = ctx->cfg.pool_size;
-  const uint64_t cap = (uint64_t)ctx->row_capacity;
+// The four row GEMMs with tokens on the M side.
+template <typename Args>
+static GemmParams row_params(const unipool_ctx* ctx, const Args& a) {
   GemmParams p{};
   p.offsets = a.offsets + a.n_experts;
   p.tile_expert = a.tile_expert;
   p.n_experts = a.n_experts;
   p.expert_base = a.expert_base;
-  p.f = f;
+  p.f = ctx->cfg.d_ff;
   p.status = ctx->ws.status;
   p.group_offsets = a.offsets;
+  return p;
+}
+
+static int rows_fwd_gu(unipool_ctx* ctx, const ExpertFwdArgs& a, cudaStream_t s) {
+  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff, M = ctx->cfg.pool_size;
+  const uint64_t cap = (uint64_t)ctx->row_capacity;
+  GemmParams p = row_params(ctx, a);
   const bool plan = rows_on_pairs(ctx, a.n_experts);
   CUtensorMap tmA, tmA64, tmB, tmBp, tmC0, tmC1;
   int rc;
@@ -1438,8 +1454,16 @@ int expert_fwd_tc(unipool_ctx* ctx, const ExpertFwdArgs& a, cudaStream_t s) {
   if ((rc = map_chunk(ctx, &tmC0, a.GU, 2 * f, cap, kMapBf16Chunk)) != UNIPOOL_OK) return rc;
   if ((rc = map_chunk(ctx, &tmC1, a.A, f, cap, kMapBf16Chunk)) != UNIPOOL_OK) return rc;
   p.Ndim = f; p.Kdim = d;
-  if ((rc = launch_rows<kFwd1>(ctx, UNIPOOL_PH_EXPERT_FWD_GU, plan, tmA, tmA64, tmB, tmB, tmBp, tmC0, tmC1, p, s)) != UNIPOOL_OK)
-    return rc;
+  return launch_rows<kFwd1>(ctx, UNIPOOL_PH_EXPERT_FWD_GU, plan, tmA, tmA64, tmB, tmB, tmBp, tmC0, tmC1, p, s);
+}
+
+static int rows_fwd_down(unipool_ctx* ctx, const ExpertFwdArgs& a, cudaStream_t s) {
+  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff, M = ctx->cfg.pool_size;
+  const uint64_t cap = (uint64_t)ctx->row_capacity;
+  GemmParams p = row_params(ctx, a);
+  const bool plan = rows_on_pairs(ctx, a.n_experts);
+  CUtensorMap tmA, tmA64, tmB, tmBp, tmC0, tmC1;
+  int rc;
   // Yp = A W_down^T
   if ((rc = map_2d(ctx, &tmA, a.A, f, cap, 64, BM)) != UNIPOOL_OK) return rc;
   if ((rc = map_2d(ctx, &tmA64, a.A, f, cap, 64, 64)) != UNIPOOL_OK) return rc;
@@ -1451,17 +1475,10 @@ int expert_fwd_tc(unipool_ctx* ctx, const ExpertFwdArgs& a, cudaStream_t s) {
   return launch_rows<kFwd2>(ctx, UNIPOOL_PH_EXPERT_FWD_DOWN, plan, tmA, tmA64, tmB, tmB, tmBp, tmC0, tmC1, p, s);
 }
 
-int expert_bwd_tc(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
+static int rows_dgrad_down(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
   const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff, M = ctx->cfg.pool_size;
   const uint64_t cap = (uint64_t)ctx->row_capacity;
-  GemmParams p{};
-  p.offsets = a.offsets + a.n_experts;
-  p.tile_expert = a.tile_expert;
-  p.n_experts = a.n_experts;
-  p.expert_base = a.expert_base;
-  p.f = f;
-  p.status = ctx->ws.status;
-  p.group_offsets = a.offsets;
+  GemmParams p = row_params(ctx, a);
   const bool plan = rows_on_pairs(ctx, a.n_experts);
   CUtensorMap tmA, tmA64, tmB, tmB64, tmBp, tmC0, tmC1;
   int rc;
@@ -1474,8 +1491,16 @@ int expert_bwd_tc(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
   if ((rc = map_chunk(ctx, &tmC0, a.dGU, 2 * f, cap, kMapBf16Chunk)) != UNIPOOL_OK) return rc;
   if ((rc = map_chunk(ctx, &tmC1, a.GU, 2 * f, cap, kMapBf16Chunk)) != UNIPOOL_OK) return rc;
   p.Ndim = f; p.Kdim = d;
-  rc = launch_rows<kDgrad1>(ctx, UNIPOOL_PH_DGRAD_DOWN, plan, tmA, tmA64, tmB, tmB64, tmBp, tmC0, tmC1, p, s);
-  if (rc != UNIPOOL_OK) return rc;
+  return launch_rows<kDgrad1>(ctx, UNIPOOL_PH_DGRAD_DOWN, plan, tmA, tmA64, tmB, tmB64, tmBp, tmC0, tmC1, p, s);
+}
+
+static int rows_dgrad_gu(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
+  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff, M = ctx->cfg.pool_size;
+  const uint64_t cap = (uint64_t)ctx->row_capacity;
+  GemmParams p = row_params(ctx, a);
+  const bool plan = rows_on_pairs(ctx, a.n_experts);
+  CUtensorMap tmA, tmA64, tmB, tmB64, tmBp, tmC0;
+  int rc;
   // dXp = dGU [W_gate; W_up]
   if ((rc = map_2d(ctx, &tmA, a.dGU, 2 * f, cap, 64, BM)) != UNIPOOL_OK) return rc;
   if ((rc = map_mn(ctx, &tmB, a.W_gu, d, (uint64_t)M * 2 * f, BN / 64)) != UNIPOOL_OK) return rc;
@@ -1484,14 +1509,23 @@ int expert_bwd_tc(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
   if ((rc = map_chunk(ctx, &tmC0, a.dXp, d, cap, kMapBf16Chunk)) != UNIPOOL_OK) return rc;
   p.Ndim = d; p.Kdim = 2 * f; p.overwrite = 1;
   if ((rc = map_2d(ctx, &tmA64, a.dGU, 2 * f, cap, 64, 64)) != UNIPOOL_OK) return rc;
-  rc = launch_rows<kDgrad2>(ctx, UNIPOOL_PH_DGRAD_GU, plan, tmA, tmA64, tmB, tmB64, tmBp, tmC0, tmC0, p, s);
+  return launch_rows<kDgrad2>(ctx, UNIPOOL_PH_DGRAD_GU, plan, tmA, tmA64, tmB, tmB64, tmBp, tmC0, tmC0, p, s);
+}
+
+int expert_fwd_tc(unipool_ctx* ctx, const ExpertFwdArgs& a, cudaStream_t s) {
+  const int rc = weights_on_m(ctx, kFwd1, a.n_experts) ? wm_fwd_gu(ctx, a, s) : rows_fwd_gu(ctx, a, s);
   if (rc != UNIPOOL_OK) return rc;
-  if (a.wgrad) {
-    PoolWgradArgs w{1, 0, a.offsets, a.Xp, a.A, a.dYp, a.dGU, a.expert_base, a.n_experts, a.dW_gu, a.dW_down,
-                    a.overwrite};
-    return wgrad_pair(ctx, w, s);
-  }
-  return UNIPOOL_OK;
+  return weights_on_m(ctx, kFwd2, a.n_experts) ? wm_fwd_down(ctx, a, s) : rows_fwd_down(ctx, a, s);
+}
+
+int expert_bwd_tc(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
+  int rc = weights_on_m(ctx, kDgrad1, a.n_experts) ? wm_dgrad_down(ctx, a, s) : rows_dgrad_down(ctx, a, s);
+  if (rc != UNIPOOL_OK) return rc;
+  rc = weights_on_m(ctx, kDgrad2, a.n_experts) ? wm_dgrad_gu(ctx, a, s) : rows_dgrad_gu(ctx, a, s);
+  if (rc != UNIPOOL_OK || !a.wgrad) return rc;
+  PoolWgradArgs w{1, 0, a.offsets, a.Xp, a.A, a.dYp, a.dGU, a.expert_base, a.n_experts, a.dW_gu, a.dW_down,
+                  a.overwrite, a.rows};
+  return wgrad_pair(ctx, w, s);
 }
 
 int pool_wgrad_tc(unipool_ctx* ctx, const PoolWgradArgs& a, cudaStream_t s) { return wgrad_pair(ctx, a, s); }

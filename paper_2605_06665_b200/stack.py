@@ -76,6 +76,7 @@ class UniPoolStack:
         self.znorm = e(L, T, dtype=f32)
         self.z = e(L, T, self.m, dtype=f32)
         self.offsets = e(L, self.m + 1, dtype=i32)
+        self.rows = e(L, self.m, dtype=i32)                # tokens of each group (the statistics may become global ones)
         self.row_of = e(L, T, k, dtype=i32)
         self.token_of = e(L, cap, dtype=i32)
         self.tile_expert = e(L, cap // B.ROW_ALIGN, dtype=i32)
@@ -141,9 +142,9 @@ class UniPoolStack:
         recompute step of backward)."""
         c, s = self.ctx, self.slot(l)
         c.dispatch(self.x[l], T, self.idx[l], self.m, self.offsets[l], self.row_of[l], self.token_of[l],
-                   self.tile_expert[l], self.Xp[s])
+                   self.tile_expert[l], self.Xp[s], self.rows[l])
         c.expert_fwd(self.Xp[s], self.offsets[l], self.tile_expert[l], self.W_gu, self.W_down,
-                     self.base(l), self.m, self.GU[s], self.A[s], self.Yp[s])
+                     self.base(l), self.m, self.GU[s], self.A[s], self.Yp[s], self.rows[l])
 
     def forward(self, x0=None, T=None):
         T = self.T if T is None else T
@@ -183,7 +184,7 @@ class UniPoolStack:
         c.expert_bwd(dx_next, T, self.row_of[l], self.gate[l], self.token_of[l], self.offsets[l],
                      self.tile_expert[l], self.Xp[a], self.GU[a], self.A[a], self.Yp[a], self.W_gu,
                      self.W_down, self.base(l), self.m, dx_next, self.dYp[s], self.dGU[s], dx_out,
-                     self.dgate, self.dW_gu, self.dW_down, flags)
+                     self.dgate, self.dW_gu, self.dW_down, flags, self.rows[l])
         coef = None
         if with_aux:
             coef = self.coef[l // self.Lg]
@@ -211,12 +212,12 @@ class UniPoolStack:
                 args = (self.Lg, self.cap, self.offsets[l0:], self.Xp[l0:], self.A[l0:], self.dYp[l0:],
                         self.dGU[l0:], g * self.m, self.m)
                 if exchange is None:
-                    self.ctx.pool_wgrad(*args, self.dW_gu, self.dW_down, flags)
+                    self.ctx.pool_wgrad(*args, self.dW_gu, self.dW_down, flags, self.rows[l0:])
                 else:
                     e0, e1 = g * self.m, (g + 1) * self.m
-                    self.ctx.pool_wgrad(*args, None, self.dW_down, flags)
+                    self.ctx.pool_wgrad(*args, None, self.dW_down, flags, self.rows[l0:])
                     exchange.launch([self.dW_down[e0:e1]])
-                    self.ctx.pool_wgrad(*args, self.dW_gu, None, flags)
+                    self.ctx.pool_wgrad(*args, self.dW_gu, None, flags, self.rows[l0:])
                     exchange.launch([self.dW_gu[e0:e1]])
         if exchange is not None:
             if not self.deferred_wgrad:

@@ -76,3 +76,69 @@ def test_dispatch_maps_at_the_edges_of_its_chunking(T, k, M, static):
     for e in range(M):
         exp[r_off[e] // 128:r_off[e + 1] // 128] = e
     assert (te.cpu().numpy() == exp).all()
+
+
+# group sizes (k = 1, so rows = tokens) around the steps of the weights-on-M kernels: 16 and 32 tokens, 192 / 256 /
+# 384 per unit, one and two MMAs, empty groups; the average decides the dispatch, so both layouts run
+@pytest.mark.parametrize("sizes,d,f", [
+    ([0, 1, 15, 16, 17, 31, 33, 191, 192, 193, 255, 256, 257, 383, 384, 385], 128, 1088),
+    ([129, 512, 513, 0, 639, 640, 300], 192, 576),               # partial weight tiles
+    ([768, 769, 1000, 1, 1152, 1153, 900], 1024, 64),            # gate/up beyond 450 rows, one k-block of K = 64
+    ([200] * 40 + [0, 97, 1300], 64, 1216),
+    ([110, 120, 130, 140], 256, 320),                            # dgrad down only
+])
+@pytest.mark.parametrize("with_rows", [True, False])
+def test_expert_ffn_at_the_edges_of_its_units(sizes, d, f, with_rows):
+    """Forward and both dgrads against a float32 restatement with the same bf16 roundings.  The kernels round
+    G, U, A, Y, dGU and dX once each: |error| <= 2^-8 of the largest value plus the inputs' share, 1e-2."""
+    import torch
+    from paper_2605_06665_b200 import binding as B
+    torch.backends.cuda.matmul.allow_tf32 = False
+    M, T = len(sizes), sum(sizes)
+    base, pool = 1, len(sizes) + 2
+    ctx = B.Context(B.make_config(d, f, pool, 1, 1, T, B.BF16, 1e-6, 2.0))
+    cap = ctx.row_capacity
+    g = torch.Generator(device="cuda").manual_seed(5)
+    bf = lambda *s, std=1.0: torch.empty(*s, device="cuda").normal_(0, std, generator=g).bfloat16()
+    i32 = dict(dtype=torch.int32, device="cuda")
+    x, dy = bf(T, d), bf(T, d)
+    Wgu, Wd = bf(pool, 2 * f, d, std=0.05), bf(pool, d, f, std=0.05)
+    idx = torch.repeat_interleave(torch.arange(M), torch.tensor(sizes))[torch.randperm(T)].to(torch.int32).cuda()[:, None]
+    off, row_of, tok, te, rows = (torch.empty(s, **i32) for s in ((M + 1,), (T, 1), (cap,), (cap // 128,), (M,)))
+    nan = lambda *s: torch.full(s, float("nan"), dtype=torch.bfloat16, device="cuda")
+    Xp, GU, A, Yp, dYp, dGU, dx = nan(cap, d), nan(cap, 2 * f), nan(cap, f), nan(cap, d), nan(cap, d), nan(cap, 2 * f), nan(T, d)
+    gate, dgate = torch.rand(T, 1, device="cuda", generator=g) + 0.5, torch.empty(T, 1, device="cuda")
+    ctx.dispatch(x, T, idx.contiguous(), M, off, row_of, tok, te, Xp, rows)
+    assert rows.tolist() == sizes
+    r = rows if with_rows else None
+    ctx.expert_fwd(Xp, off, te, Wgu, Wd, base, M, GU, A, Yp, r)
+    ctx.expert_bwd(dy, T, row_of, gate, tok, off, te, Xp, GU, A, Yp, Wgu, Wd, base, M, None, dYp, dGU, dx, dgate, None,
+                   None, B.BWD_SKIP_WGRAD, r)
+    torch.cuda.synchronize()
+    ctx.check_status()
+    ctx.close()
+    off = off.tolist()
+    used = off[-1]
+    pad = tok[:used] < 0
+    for t in (GU, A, Yp, dGU):
+        assert not t[:used][pad].any()                            # zeros (and no NaN) on pad rows
+
+    def close(got, want):
+        assert (got.float() - want.float()).abs().max() <= 1e-2 * want.float().abs().max()
+
+    for e, n in enumerate(sizes):
+        if n == 0:
+            continue
+        s = slice(off[e], off[e] + n)
+        X, Wg, Wu, W2 = (t.float() for t in (Xp[s], Wgu[base + e, :f], Wgu[base + e, f:], Wd[base + e]))
+        G, U = X @ Wg.T, X @ Wu.T
+        close(GU[s, :f], G)
+        close(GU[s, f:], U)
+        close(A[s], torch.nn.functional.silu(G) * U)
+        close(Yp[s], A[s].float() @ W2.T)
+        dA = dYp[s].float() @ W2
+        G, U = GU[s, :f].float(), GU[s, f:].float()
+        sig = torch.sigmoid(G)
+        close(dGU[s, :f], dA * U * sig * (1 + G * (1 - sig)))
+        close(dGU[s, f:], dA * G * sig)
+        close(dx[tok[s].long()], dGU[s].float() @ Wgu[base + e].float())
