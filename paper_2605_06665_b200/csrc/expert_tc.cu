@@ -54,6 +54,7 @@ struct GemmParams {
   int Mdim, Ndim, Kdim;         // wgrad: dW is [Mdim, Ndim]; row tiles: output columns, contraction
   int f;                        // expert width (fwd1 / dgrad1 addressing)
   int overwrite;                // 1 = the output is written, 0 = it is added to (wgrad, dgrad2)
+  const int32_t* rows;          // weight gradient on CTA pairs: [n_layers][n_experts] group sizes, or NULL
   int uniform_rows;             // wgrad without offsets: group e = rows [e*Kdim, (e+1)*Kdim) of this many
   int32_t* status;
 };
@@ -639,13 +640,34 @@ constexpr uint32_t kPairHalfBytes = 128 * BK * 2;            // 128 (M or N) x 6
 constexpr uint32_t kPairStageBytes = 2 * kPairHalfBytes;
 static_assert(kPairStages * kPairStageBytes + kEpiWarps * 8192 == kBarOffset, "shared-memory budget");
 
-__device__ __forceinline__ int wgrad_kblocks(const GemmParams& p, int e) {
-  int kb = 0;
-  for (int l = 0; l < p.n_layers; ++l) {
-    const int32_t* off = p.offsets + (int64_t)l * (p.n_experts + 1);
-    kb += (off[e + 1] - off[e]) / BK;
+// Group sizes against padded groups: 12 layers of 1501 tokens over 96 experts (31 rows in groups of 128) 962 ->
+// 642 us; at 341 rows per group, where 64-row k-blocks drop a twelfth of the steps, 3.11 -> 3.07 ms (zeros cost
+// little under the power cap).
+// Rows of expert e in layer l that the contraction runs over: its tokens if the caller gave their number (what
+// follows up to the next group start is zero), else the padded group.
+__device__ __forceinline__ int wgrad_rows(const GemmParams& p, int l, int e) {
+  const int32_t* off = p.offsets + (int64_t)l * (p.n_experts + 1) + e;
+  const int padded = off[1] - off[0];
+  return p.rows ? min(max(p.rows[(int64_t)l * p.n_experts + e], 0), padded) : padded;
+}
+// The rows of one expert in up to 32 layers, one layer per lane: what a role needs for a tile, loaded while the
+// tile before it runs (three dependent loads per layer in the issuing thread had cost 5 % of the kernel).
+struct LaneRows {
+  int first, end, rows;                                    // raw: group start, next group start, group size
+  __device__ __forceinline__ void load(const GemmParams& p, int l0, int e, int lane) {
+    const int l = min(l0 + lane, p.n_layers - 1);
+    const int32_t* off = p.offsets + (int64_t)l * (p.n_experts + 1) + e;
+    first = off[0];
+    end = off[1];
+    rows = p.rows ? p.rows[(int64_t)l * p.n_experts + e] : 0x7fffffff;
   }
-  return kb;
+  __device__ __forceinline__ int count() const { return min(max(rows, 0), end - first); }
+};
+// 16-row steps of an expert over all layers: the length of its tiles
+__device__ __forceinline__ int wgrad_steps(const GemmParams& p, int e) {
+  int steps = 0;
+  for (int l = 0; l < p.n_layers; ++l) steps += (wgrad_rows(p, l, e) + 15) / 16;
+  return steps;
 }
 
 // Tile of `pair` in `round` when a sorted tile list is dealt out forwards and backwards alternately.
@@ -696,88 +718,131 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   // experts are taken in order of decreasing length (ties by index) and dealt to the CTA pairs
   // boustrophedon-wise (first deal: pair 0 .. P-1, second deal: pair P-1 .. 0, ...), so that every deal holds
   // tiles of similar size, the long ones come first, and no pair collects the longest tile of every deal.
-  uint16_t* order = reinterpret_cast<uint16_t*>(smem + kBarOffset + 512);   // [n_experts] i-th longest expert
-  int* kb_of = reinterpret_cast<int*>(smem + kPairStages * kPairStageBytes);  // scratch in the (still idle) staging tiles
-  for (int e = threadIdx.x; e < p.n_experts; e += blockDim.x) kb_of[e] = wgrad_kblocks(p, e);
+  uint16_t* order = reinterpret_cast<uint16_t*>(smem + kBarOffset + 512);   // [n_experts] i-th longest expert, [1] how many have rows
+  int* steps_of = reinterpret_cast<int*>(smem + kPairStages * kPairStageBytes);  // scratch in the (still idle) staging tiles
+  for (int e = threadIdx.x; e < p.n_experts; e += blockDim.x) steps_of[e] = wgrad_steps(p, e);
   __syncthreads();
   for (int e = threadIdx.x; e < p.n_experts; e += blockDim.x) {
-    const int mine = kb_of[e];
-    int rank_e = 0;
+    const int mine = steps_of[e];
+    int rank_e = 0, with_rows = 0;
     for (int o = 0; o < p.n_experts; ++o) {
-      const int other = kb_of[o];
+      const int other = steps_of[o];
       rank_e += (other > mine || (other == mine && o < e)) ? 1 : 0;
+      with_rows += other > 0 ? 1 : 0;
     }
     order[rank_e] = (uint16_t)e;
+    if (e == 0) order[p.n_experts] = (uint16_t)with_rows;                    // experts without rows come last
   }
-  __syncthreads();                                                           // kb_of is dead from here on
+  __syncthreads();                                                           // steps_of is dead from here on
+  const int live = (int)order[p.n_experts] * per_e;                          // tiles that have a contraction
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (one in each CTA)
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int round = 0; round * n_pairs < total && ok; ++round) {
-        const int tile = snake_tile(round, pair, n_pairs);
-        if (tile >= total) continue;
-        const int e = order[tile / per_e], rem = tile % per_e, mt = rem / n_nt, nt = rem % n_nt;
-        const int kblocks = wgrad_kblocks(p, e);
-        int layer = 0, r = p.offsets[e], r_end = p.offsets[e + 1];
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!tc::mbar_wait(&empty_bar[stage], phase ^ 1u, abort)) { report_timeout(p, abort, 21); ok = false; break; }
-          while (r >= r_end) {                          // next layer that has rows for this expert
-            ++layer;
-            const int32_t* off = p.offsets + (int64_t)layer * (p.n_experts + 1);
-            r = off[e];
-            r_end = off[e + 1];
+    // (the whole warp walks the rows, lane 0 issues)
+    int stage = 0;
+    uint32_t phase = 0;
+    bool ok = true;
+    LaneRows next{};
+    if (pair < live) next.load(p, 0, order[pair / per_e], lane);
+    for (int round = 0; ok; ++round) {
+      const int tile = snake_tile(round, pair, n_pairs);
+      if (tile >= live) break;                            // the deals are in order: nothing but empty tiles from here
+      const int e = order[tile / per_e], rem = tile % per_e, mt = rem / n_nt, nt = rem % n_nt;
+      for (int l0 = 0; l0 < p.n_layers && ok; l0 += 32) {
+        LaneRows cur = next;
+        if (l0 > 0) cur.load(p, l0, e, lane);
+        if (l0 + 32 >= p.n_layers) {                      // the next tile's rows
+          const int nx = snake_tile(round + 1, pair, n_pairs);
+          if (nx < live) next.load(p, 0, order[nx / per_e], lane);
+        }
+        const int count = cur.count();
+        for (int l = 0; l < min(32, p.n_layers - l0) && ok; ++l) {
+          const int n = __shfl_sync(0xffffffffu, count, l);
+          const int row0 = (l0 + l) * p.layer_stride_rows + __shfl_sync(0xffffffffu, cur.first, l);
+          for (int done = 0; done < n; done += BK) {
+            if (!tc::mbar_wait(&empty_bar[stage], phase ^ 1u, abort)) {
+              if (lane == 0) report_timeout(p, abort, 21);
+              ok = false;
+              break;
+            }
+            if (lane == 0) {
+              uint8_t* sA = smem + stage * kPairStageBytes;
+              uint8_t* sB = sA + kPairHalfBytes;
+              if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], 2 * kPairStageBytes);   // both CTAs' bytes
+              // this CTA's two 64-column blocks of each operand, one box each
+              tc::tma_load_3d_pair(sA, &tmA, &full_bar[stage], 0, row0 + done, mt * 4 + rank * 2);
+              tc::tma_load_3d_pair(sB, &tmB, &full_bar[stage], 0, row0 + done, nt * 4 + rank * 2);
+            }
+            __syncwarp();
+            if (++stage == kPairStages) { stage = 0; phase ^= 1u; }
           }
-          const int grow = layer * p.layer_stride_rows + r;
-          uint8_t* sA = smem + stage * kPairStageBytes;
-          uint8_t* sB = sA + kPairHalfBytes;
-          if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], 2 * kPairStageBytes);   // both CTAs' bytes
-          // this CTA's two 64-column blocks of each operand, one box each
-          tc::tma_load_3d_pair(sA, &tmA, &full_bar[stage], 0, grow, mt * 4 + rank * 2);
-          tc::tma_load_3d_pair(sB, &tmB, &full_bar[stage], 0, grow, nt * 4 + rank * 2);
-          r += BK;
-          if (++stage == kPairStages) { stage = 0; phase ^= 1u; }
+          ok = __all_sync(0xffffffffu, ok);
         }
       }
-      if (!ok)
-        for (int i = 0; i < 200; ++i) __nanosleep(1000);
     }
+    if (!ok)
+      for (int i = 0; i < 200; ++i) __nanosleep(1000);
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (leader CTA only)
-    if (lane == 0 && rank == 0) {
+    // (the whole warp walks the rows, lane 0 issues)
+    if (rank == 0) {
       constexpr uint32_t idesc = tc::instr_desc_bf16(256, true, true, 256);
       constexpr uint32_t kstep = (16 * 128) >> 4;             // descriptor units per K = 16 (MN-major)
       int stage = 0;
       uint32_t phase = 0;
-      int local = 0;
       bool ok = true;
-      for (int round = 0; round * n_pairs < total && ok; ++round) {
+      LaneRows next{};
+      if (pair < live) next.load(p, 0, order[pair / per_e], lane);
+      for (int round = 0; ok; ++round) {
         const int tile = snake_tile(round, pair, n_pairs);
-        if (tile >= total) continue;
-        const int kblocks = wgrad_kblocks(p, order[tile / per_e]);
-        if (kblocks == 0) continue;
-        const int acc = local & 1;
-        const uint32_t acc_phase = (local >> 1) & 1;
-        ++local;
-        if (!tc::mbar_wait(&tmem_empty[acc], acc_phase ^ 1u, abort)) { report_timeout(p, abort, 22); break; }
+        if (tile >= live) break;
+        const int acc = round & 1;
+        if (!tc::mbar_wait(&tmem_empty[acc], ((round >> 1) & 1) ^ 1u, abort)) {
+          if (lane == 0) report_timeout(p, abort, 22);
+          break;
+        }
         tc::tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * 256;
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!tc::mbar_wait(&full_bar[stage], phase, abort)) { report_timeout(p, abort, 23); ok = false; break; }
-          tc::tc_fence_after_sync();
-          const uint32_t aaddr = tc::smem_u32(smem + stage * kPairStageBytes);
-          const uint64_t adesc = tc::smem_desc_sw128(aaddr, kMnBlockBytes, 1024);
-          const uint64_t bdesc = tc::smem_desc_sw128(aaddr + kPairHalfBytes, kMnBlockBytes, 1024);
+        uint32_t accumulate = 0;
+        for (int l0 = 0; l0 < p.n_layers && ok; l0 += 32) {
+          LaneRows cur = next;
+          if (l0 > 0) cur.load(p, l0, order[tile / per_e], lane);
+          const int count = cur.count();
+          if (l0 + 32 >= p.n_layers) {
+            const int nx = snake_tile(round + 1, pair, n_pairs);
+            if (nx < live) next.load(p, 0, order[nx / per_e], lane);
+          }
+          for (int l = 0; l < min(32, p.n_layers - l0) && ok; ++l) {
+            const int n = __shfl_sync(0xffffffffu, count, l);
+            for (int done = 0; done < n; done += BK) {
+              if (!tc::mbar_wait(&full_bar[stage], phase, abort)) {
+                if (lane == 0) report_timeout(p, abort, 23);
+                ok = false;
+                break;
+              }
+              tc::tc_fence_after_sync();
+              if (lane == 0) {
+                const uint32_t aaddr = tc::smem_u32(smem + stage * kPairStageBytes);
+                const uint64_t adesc = tc::smem_desc_sw128(aaddr, kMnBlockBytes, 1024);
+                const uint64_t bdesc = tc::smem_desc_sw128(aaddr + kPairHalfBytes, kMnBlockBytes, 1024);
+                if (n - done > 48) {
 #pragma unroll
-          for (int j = 0; j < BK / 16; ++j)
-            tc::umma_bf16_pair(d_tmem, adesc + j * kstep, bdesc + j * kstep, idesc, (kb | j) != 0 ? 1u : 0u);
-          tc::umma_commit_pair(&empty_bar[stage], 3);           // frees the stage in both CTAs
-          if (++stage == kPairStages) { stage = 0; phase ^= 1u; }
+                  for (int j = 0; j < BK / 16; ++j)
+                    tc::umma_bf16_pair(d_tmem, adesc + j * kstep, bdesc + j * kstep, idesc, j > 0 ? 1u : accumulate);
+                } else {                                        // only zeros behind row n
+                  for (int j = 0; 16 * j < n - done; ++j)
+                    tc::umma_bf16_pair(d_tmem, adesc + j * kstep, bdesc + j * kstep, idesc, j > 0 ? 1u : accumulate);
+                }
+                tc::umma_commit_pair(&empty_bar[stage], 3);     // frees the stage in both CTAs
+              }
+              accumulate = 1;
+              __syncwarp();
+              if (++stage == kPairStages) { stage = 0; phase ^= 1u; }
+            }
+            ok = __all_sync(0xffffffffu, ok);
+          }
         }
-        if (ok) tc::umma_commit_pair(&tmem_full[acc], 3);       // accumulator complete, both CTAs
+        if (ok && lane == 0) tc::umma_commit_pair(&tmem_full[acc], 3);       // accumulator complete, both CTAs
       }
     }
   } else {
@@ -791,7 +856,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       const int e = order[tile / per_e], rem = tile % per_e, mt = rem / n_nt, nt = rem % n_nt;
       const int m0 = mt * 256 + rank * 128 + quarter * 32;
       const int grow = (p.expert_base + e) * p.Mdim + m0;
-      if (wgrad_kblocks(p, e) == 0) {
+      if (tile >= live) {
         if (p.overwrite && m0 < p.Mdim) {               // no rows anywhere: the gradient of this tile is zero
           if (lane == 0) tc::bulk_wait_read<0>();
           __syncwarp();
@@ -1376,6 +1441,7 @@ int wgrad_pair(unipool_ctx* ctx, const PoolWgradArgs& a, cudaStream_t s) {
   const uint64_t rows = (uint64_t)(a.n_layers > 1 ? (int64_t)a.n_layers * a.layer_stride_rows : ctx->row_capacity);
   GemmParams p{};
   p.offsets = a.offsets;
+  p.rows = a.rows;
   p.n_experts = a.n_experts;
   p.expert_base = a.expert_base;
   p.n_layers = a.n_layers;

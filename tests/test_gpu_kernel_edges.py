@@ -142,3 +142,51 @@ def test_expert_ffn_at_the_edges_of_its_units(sizes, d, f, with_rows):
         close(dGU[s, :f], dA * U * sig * (1 + G * (1 - sig)))
         close(dGU[s, f:], dA * G * sig)
         close(dx[tok[s].long()], dGU[s].float() @ Wgu[base + e].float())
+
+
+@pytest.mark.parametrize("overwrite", [True, False])
+@pytest.mark.parametrize("sizes", [
+    [[0, 0, 0, 0], [0, 0, 0, 0]],
+    [[1, 15, 16, 17], [63, 64, 65, 0], [0, 127, 128, 129], [33, 0, 48, 1000]],
+    [[5, 0, 7, 200]],
+])
+def test_weight_gradient_leaves_the_padding_out(sizes, overwrite):
+    """With the group sizes the contraction stops at the last 16 rows that hold a token; what is left out are zeros,
+    so the sums are those of the padded contraction up to the sign of zero: equal, bit for bit."""
+    import torch
+    from paper_2605_06665_b200 import binding as B
+    L, M, d, f = len(sizes), 4, 192, 320
+    T = max(sum(s) for s in sizes)
+    ctx = B.Context(B.make_config(d, f, M, 1, L, max(T, 1), B.BF16, 1e-6, 2.0))
+    cap = ctx.row_capacity
+    g = torch.Generator(device="cuda").manual_seed(2)
+    off = np.zeros((L, M + 1), dtype=np.int32)
+    for l, s in enumerate(sizes):
+        off[l, 1:] = np.cumsum([(n + 127) // 128 * 128 for n in s])
+    ops = [torch.zeros(L, cap, w, dtype=torch.bfloat16, device="cuda") for w in (d, f, d, 2 * f)]
+    for l, s in enumerate(sizes):
+        for e, n in enumerate(s):
+            for t in ops:
+                t[l, off[l, e]:off[l, e] + n].normal_(generator=g)
+    rows = torch.tensor(sizes, dtype=torch.int32, device="cuda")
+    offs = torch.from_numpy(off).cuda()
+    got = []
+    for r in (None, rows):
+        dgu, dd = torch.full((M, 2 * f, d), 3.0, device="cuda"), torch.full((M, d, f), -2.0, device="cuda")
+        ctx.pool_wgrad(L, cap, offs, *ops, 0, M, dgu, dd, B.WGRAD_OVERWRITE if overwrite else 0, r)
+        torch.cuda.synchronize()
+        got.append((dgu, dd))
+    ctx.check_status()
+    ctx.close()
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    Xp, A, dYp, dGU = (t.float() for t in ops)
+    for e in range(M):
+        want = torch.zeros(2 * f, d, device="cuda") if overwrite else torch.full((2 * f, d), 3.0, device="cuda")
+        down = torch.zeros(d, f, device="cuda") if overwrite else torch.full((d, f), -2.0, device="cuda")
+        for l in range(L):
+            s = slice(off[l, e], off[l, e + 1])
+            want += dGU[l, s].T @ Xp[l, s]
+            down += dYp[l, s].T @ A[l, s]
+        # exact products, fp32 sums of at most some 1200 terms: 1e-5 of the largest value
+        assert (got[1][0][e] - want).abs().max() <= 1e-5 * max(want.abs().max().item(), 1.0)
+        assert (got[1][1][e] - down).abs().max() <= 1e-5 * max(down.abs().max().item(), 1.0)
