@@ -1,192 +1,255 @@
-// Grouped SwiGLU expert FFN on CUDA cores with exact fp32 accumulation.
-// This is the arithmetic path of the fp32 mode (parity bound 1e-5, which TF32
-// tensor-core products cannot meet); it also accepts bf16 storage.
+// Grouped SwiGLU expert FFN on CUDA cores with exact fp32 accumulation: the arithmetic path of the fp32 mode
+// (parity bound 1e-5, which TF32 tensor-core products cannot meet).
 #include "common.cuh"
 #include "simt_gemm.cuh"
 
 namespace unipool {
 
-// C[rows, N] = A[rows, K] * B_e(k, n) for every 64-row tile of the permuted row
-// space; the tile's expert selects B.  Rows at and beyond offsets[n_experts] are
-// skipped (tile_expert < 0).
-template <typename TE>
-__global__ void __launch_bounds__(kSimtThreads)
-grouped_rows_gemm_kernel(const TE* __restrict__ A, int64_t lda, const TE* __restrict__ B,
-                         int64_t b_expert_stride, int64_t b_sk, int64_t b_sn,
-                         const int32_t* __restrict__ tile_expert, int expert_base,
-                         TE* __restrict__ C, int64_t ldc, int N, int K, int n_row_tiles) {
-  const int n0 = blockIdx.x * kSimtTile;
-  for (int rt = blockIdx.y; rt < n_row_tiles; rt += gridDim.y) {
-    const int m0 = rt * kSimtTile;
-    const int e = tile_expert[m0 / UNIPOOL_ROW_ALIGN];
-    if (e < 0) continue;                     // uniform over the block
-    float acc[4][4] = {};
-    SimtOperands<TE, TE> op{A, lda, 1, B + (int64_t)(expert_base + e) * b_expert_stride, b_sk, b_sn};
-    simt_tile_mainloop(op, m0, n0, m0 + kSimtTile, N, 0, K, acc);
-    const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+namespace {
+
+constexpr int kRowTile = 64;     // rows of a tile; groups start at multiples of UNIPOOL_ROW_ALIGN = 128
+
+struct RowGemm {
+  const float* A; int64_t lda;                      // [rows, K]
+  const float* B; int64_t b_expert, ldb;            // expert's weights: along K [N, K], across K [K, N]
+  const int32_t* tile_expert; const int32_t* offsets; const int32_t* rows;   // rows: true group sizes or NULL
+  int expert_base;
+  float *C, *C2;
+  const float* GU;
+  int N, K, f, n_row_tiles;
+  bool vec;                                         // every pointer is 16-byte aligned (row lengths are multiples of 64)
+};
+
+enum RowEpilogue {
+  kStore,      // C [rows, N]
+  kSwiglu,     // the tile is TN/2 gate and the same TN/2 up columns: GU -> C [rows, 2f], A = silu(G) U -> C2 [rows, f]
+  kSwigluBwd,  // the tile is dA: dG = dA U silu'(G), dU = dA silu(G) -> C [rows, 2f], G and U from GU
+};
+
+// C = A B_e for every 64-row tile of the permuted row space; the tile's expert selects B.  Tiles at and beyond
+// offsets[n_experts] are skipped (tile_expert < 0); tiles behind a group's last token hold zeros and get zeros.
+template <int TN, int KG, Major BM, RowEpilogue EPI>
+__global__ void __launch_bounds__(SimtTile<kRowTile, TN, KG>::kThreads)
+grouped_rows_gemm_kernel(const RowGemm p) {
+  using T = SimtTile<kRowTile, TN, KG>;
+  __shared__ typename T::Smem sm;
+  const int n0 = blockIdx.x * (EPI == kSwiglu ? TN / 2 : TN);
+  for (int rt = blockIdx.y; rt < p.n_row_tiles; rt += gridDim.y) {
+    const int m0 = rt * kRowTile;
+    const int e = p.tile_expert[m0 / UNIPOOL_ROW_ALIGN];
+    if (e < 0) continue;                            // uniform over the block
+    const bool empty = p.rows != nullptr && m0 - p.offsets[e] >= p.rows[e];
+    const float* B = p.B + (int64_t)(p.expert_base + e) * p.b_expert;
+    T t;
+    t.template run<kAlongK, BM>(
+        sm, empty ? 0 : p.K / kSimtKC,
+        [&](int c, int i, int k) { return ld4(p.A + (int64_t)(m0 + i) * p.lda + c * kSimtKC + k, p.vec); },
+        [&](int c, int i, int k) {
+          if (EPI == kSwiglu) i = i < TN / 2 ? n0 + i : p.f + n0 + i - TN / 2;
+          else i += n0;
+          const int kk = c * kSimtKC + k;
+          return ld4(BM == kAlongK ? B + (int64_t)i * p.ldb + kk : B + (int64_t)kk * p.ldb + i, p.vec);
+        });
+    if (threadIdx.x < kSimtGroup) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < T::MR; ++i) {
+        const int64_t r = m0 + T::row(i);
+        if constexpr (EPI == kStore) {
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        int n = n0 + tx * 4 + j;
-        if (n < N) C[(int64_t)(m0 + ty * 4 + i) * ldc + n] = from_f32<TE>(acc[i][j]);
+          for (int j = 0; j < T::NR; j += 4)
+            st4(p.C + r * p.N + n0 + T::col(j),
+                make_float4(t.value(i, j), t.value(i, j + 1), t.value(i, j + 2), t.value(i, j + 3)), p.vec);
+        } else if constexpr (EPI == kSwiglu) {
+          float g[4], u[4], a[4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j) { g[j] = t.value(i, j); u[j] = t.value(i, j + 4); a[j] = silu_f(g[j]) * u[j]; }
+          const int n = n0 + T::col(0);
+          st4(p.C + r * 2 * p.f + n, make_float4(g[0], g[1], g[2], g[3]), p.vec);
+          st4(p.C + r * 2 * p.f + p.f + n, make_float4(u[0], u[1], u[2], u[3]), p.vec);
+          st4(p.C2 + r * p.f + n, make_float4(a[0], a[1], a[2], a[3]), p.vec);
+        } else {
+#pragma unroll
+          for (int j = 0; j < T::NR; j += 4) {
+            const int n = n0 + T::col(j);
+            const float4 g4 = ld4(p.GU + r * 2 * p.f + n, p.vec);
+            const float4 u4 = ld4(p.GU + r * 2 * p.f + p.f + n, p.vec);
+            const float g[4] = {g4.x, g4.y, g4.z, g4.w}, u[4] = {u4.x, u4.y, u4.z, u4.w};
+            float dg[4], du[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const float dA = t.value(i, j + q);
+              dg[q] = dA * u[q] * silu_grad_f(g[q]);
+              du[q] = dA * silu_f(g[q]);
+            }
+            st4(p.C + r * 2 * p.f + n, make_float4(dg[0], dg[1], dg[2], dg[3]), p.vec);
+            st4(p.C + r * 2 * p.f + p.f + n, make_float4(du[0], du[1], du[2], du[3]), p.vec);
+          }
+        }
       }
+    }
+    if (gridDim.y < p.n_row_tiles) __syncthreads();  // the next tile reuses the buffers
   }
 }
 
-// dW[e][m, n] += sum over the rows r of group e (of every listed layer) of P[r, m] * Q[r, n].
-template <typename TE>
-__global__ void __launch_bounds__(kSimtThreads)
-grouped_k_gemm_kernel(const TE* __restrict__ P, int64_t ldp, const TE* __restrict__ Q, int64_t ldq,
-                      const int32_t* __restrict__ offsets, int n_experts, int expert_base,
-                      int n_layers, int64_t layer_stride_rows, float* __restrict__ dW,
-                      int64_t w_expert_stride, int Mdim, int Ndim, bool overwrite) {
-  const int m0 = blockIdx.x * kSimtTile, n0 = blockIdx.y * kSimtTile;
-  const int e = blockIdx.z;
-  float acc[4][4] = {};
-  for (int l = 0; l < n_layers; ++l) {
-    const int32_t* off = offsets + (int64_t)l * (n_experts + 1);
-    const int r0 = off[e], r1 = off[e + 1];
-    if (r1 <= r0) continue;
-    const TE* Pl = P + l * layer_stride_rows * ldp;
-    const TE* Ql = Q + l * layer_stride_rows * ldq;
-    SimtOperands<TE, TE> op{Pl, 1, ldp, Ql, ldq, 1};
-    simt_tile_mainloop(op, m0, n0, Mdim, Ndim, r0, r1, acc);
-  }
-  float* out = dW + (int64_t)(expert_base + e) * w_expert_stride;
-  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+// dW[e][m, n] (+)= sum over the rows r of group e (of every listed layer) of P[r, m] * Q[r, n].
+struct PoolGemm {
+  const float* P; int ldp; const float* Q; int ldq;
+  const int32_t* offsets; const int32_t* rows;      // rows [n_layers, n_experts] or NULL
+  int n_experts, expert_base, n_layers; int64_t layer_stride_rows;
+  float* dW; int Mdim, Ndim; bool overwrite, vec;
+};
+
+__global__ void __launch_bounds__(kSimtGroup)
+grouped_k_gemm_kernel(const PoolGemm p) {
+  using T = SimtTile<64, 64, 1>;
+  __shared__ typename T::Smem sm;
+  const int m0 = blockIdx.x * 64, n0 = blockIdx.y * 64, e = blockIdx.z;
+  auto rows_of = [&](int l) {
+    const int32_t* off = p.offsets + (int64_t)l * (p.n_experts + 1) + e;
+    return p.rows ? min(p.rows[(int64_t)l * p.n_experts + e], off[1] - off[0]) : off[1] - off[0];
+  };
+  int n_chunks = 0;
+  for (int l = 0; l < p.n_layers; ++l) n_chunks += (rows_of(l) + kSimtKC - 1) / kSimtKC;
+  // the chunk being fetched: rows [row0, row0 + left) of its layer are still to come (chunks are asked for in order)
+  int layer = -1, at = -1, left = 0;
+  int64_t row0 = 0;
+  auto seek = [&](int c) {
+    if (c == at) return;
+    at = c;
+    row0 += kSimtKC;
+    left -= kSimtKC;
+    while (left <= 0) {
+      ++layer;
+      left = rows_of(layer);
+      row0 = layer * p.layer_stride_rows + p.offsets[(int64_t)layer * (p.n_experts + 1) + e];
+    }
+  };
+  T t;
+  t.template run<kAcrossK, kAcrossK>(
+      sm, n_chunks,
+      [&](int c, int i, int k) {
+        seek(c);
+        return k < left ? ld4(p.P + (row0 + k) * p.ldp + m0 + i, p.vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+      },
+      [&](int c, int i, int k) {
+        return k < left ? ld4(p.Q + (row0 + k) * p.ldq + n0 + i, p.vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+      });
+  float* out = p.dW + (int64_t)(p.expert_base + e) * p.Mdim * p.Ndim;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int m = m0 + ty * 4 + i;
-    if (m >= Mdim) continue;
+  for (int i = 0; i < T::MR; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int n = n0 + tx * 4 + j;
-      if (n < Ndim) out[(int64_t)m * Ndim + n] = overwrite ? acc[i][j] : out[(int64_t)m * Ndim + n] + acc[i][j];
+    for (int j = 0; j < T::NR; j += 4) {
+      float* o = out + (int64_t)(m0 + T::row(i)) * p.Ndim + n0 + T::col(j);
+      float4 v = make_float4(t.value(i, j), t.value(i, j + 1), t.value(i, j + 2), t.value(i, j + 3));
+      if (!p.overwrite) {
+        v = make_float4(v.x + o[0], v.y + o[1], v.z + o[2], v.w + o[3]);
+      }
+      st4(o, v, p.vec);
+    }
+}
+
+template <Major BM, RowEpilogue EPI>
+int rows_gemm(unipool_ctx* ctx, RowGemm p, int n_experts, cudaStream_t s) {
+  p.vec = aligned16(p.A, p.B, p.C, p.C2, p.GU);
+  const int gy = p.n_row_tiles < 4096 ? p.n_row_tiles : 4096;
+  if constexpr (EPI != kSwiglu) {
+    // Tiles a full batch gives (a group ends on half a tile): below two blocks per SM narrower tiles, two groups of
+    // threads on each.
+    const int64_t tiles = ((int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k / kRowTile + n_experts / 2) * (p.N / 64);
+    if (tiles < 2 * ctx->sm_count) {
+      grouped_rows_gemm_kernel<32, 2, BM, EPI><<<dim3(p.N / 32, gy), 2 * kSimtGroup, 0, s>>>(p);
+      UP_LAUNCH_CHECK();
+      return UNIPOOL_OK;
     }
   }
-}
-
-// A[r, j] = silu(G[r, j]) * U[r, j] over rows < offsets_end.
-template <typename TE>
-__global__ void swiglu_kernel(const TE* __restrict__ GU, TE* __restrict__ A,
-                              const int32_t* __restrict__ offsets_end, int f) {
-  const int64_t total = (int64_t)(*offsets_end) * f;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t r = i / f;
-    int j = (int)(i % f);
-    float g = to_f32(GU[r * 2 * f + j]), u = to_f32(GU[r * 2 * f + f + j]);
-    A[i] = from_f32<TE>(silu_f(g) * u);
-  }
-}
-
-// In place on dGU, whose U half holds dA on entry:
-//   dG = dA * U * silu'(G) -> dGU[:, :f];   dU = dA * silu(G) -> dGU[:, f:].
-template <typename TE>
-__global__ void swiglu_bwd_kernel(const TE* __restrict__ GU, TE* __restrict__ dGU,
-                                  const int32_t* __restrict__ offsets_end, int f) {
-  const int64_t total = (int64_t)(*offsets_end) * f;
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t r = i / f;
-    int j = (int)(i % f);
-    float g = to_f32(GU[r * 2 * f + j]), u = to_f32(GU[r * 2 * f + f + j]);
-    float dA = to_f32(dGU[r * 2 * f + f + j]);
-    dGU[r * 2 * f + j] = from_f32<TE>(dA * u * silu_grad_f(g));
-    dGU[r * 2 * f + f + j] = from_f32<TE>(dA * silu_f(g));
-  }
-}
-
-template <typename TE>
-static int fwd_impl(unipool_ctx* ctx, const ExpertFwdArgs& a, cudaStream_t s) {
-  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff;
-  const int n_row_tiles = (int)(ctx->row_capacity / kSimtTile);
-  const int gy = n_row_tiles < 4096 ? n_row_tiles : 4096;
-  const TE* Xp = static_cast<const TE*>(a.Xp);
-  const TE* Wgu = static_cast<const TE*>(a.W_gu);
-  const TE* Wd = static_cast<const TE*>(a.W_down);
-  TE* GU = static_cast<TE*>(a.GU);
-  TE* A = static_cast<TE*>(a.A);
-  TE* Yp = static_cast<TE*>(a.Yp);
-  // GU = Xp W_gu[e]^T : B(k, n) = W_gu[e][n, k]
-  {
-  PhaseTimer pt(ctx, UNIPOOL_PH_EXPERT_FWD_GU, 2, s);
-  grouped_rows_gemm_kernel<TE><<<dim3(2 * f / kSimtTile, gy), kSimtThreads, 0, s>>>(
-      Xp, d, Wgu, (int64_t)2 * f * d, 1, d, a.tile_expert, a.expert_base, GU, 2 * f, 2 * f, d, n_row_tiles);
-  UP_LAUNCH_CHECK();
-  swiglu_kernel<TE><<<ctx->sm_count * 8, 256, 0, s>>>(GU, A, a.offsets + a.n_experts, f);
-  UP_LAUNCH_CHECK();
-  }
-  PhaseTimer pt(ctx, UNIPOOL_PH_EXPERT_FWD_DOWN, 1, s);
-  // Yp = A W_down[e]^T : B(k, n) = W_down[e][n, k]
-  grouped_rows_gemm_kernel<TE><<<dim3(d / kSimtTile, gy), kSimtThreads, 0, s>>>(
-      A, f, Wd, (int64_t)d * f, 1, f, a.tile_expert, a.expert_base, Yp, d, d, f, n_row_tiles);
+  grouped_rows_gemm_kernel<64, 1, BM, EPI><<<dim3(p.N / (EPI == kSwiglu ? 32 : 64), gy), kSimtGroup, 0, s>>>(p);
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;
 }
 
-template <typename TE>
-static int wgrad_impl(unipool_ctx* ctx, const PoolWgradArgs& a, cudaStream_t s) {
-  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff;
-  // dW_down[e][d, f] += dYp_e^T A_e
-  if (a.dW_down != nullptr) {
-  PhaseTimer pt(ctx, UNIPOOL_PH_WGRAD_DOWN, 1, s);
-  grouped_k_gemm_kernel<TE><<<dim3(d / kSimtTile, f / kSimtTile, a.n_experts), kSimtThreads, 0, s>>>(
-      static_cast<const TE*>(a.dYp), d, static_cast<const TE*>(a.A), f, a.offsets, a.n_experts,
-      a.expert_base, a.n_layers, a.layer_stride_rows, a.dW_down, (int64_t)d * f, d, f, a.overwrite);
-  UP_LAUNCH_CHECK();
-  }
-  if (a.dW_gu == nullptr) return UNIPOOL_OK;
-  PhaseTimer pt(ctx, UNIPOOL_PH_WGRAD_GU, 1, s);
-  // dW_gu[e][2f, d] += dGU_e^T Xp_e
-  grouped_k_gemm_kernel<TE><<<dim3(2 * f / kSimtTile, d / kSimtTile, a.n_experts), kSimtThreads, 0, s>>>(
-      static_cast<const TE*>(a.dGU), 2 * f, static_cast<const TE*>(a.Xp), d, a.offsets, a.n_experts,
-      a.expert_base, a.n_layers, a.layer_stride_rows, a.dW_gu, (int64_t)2 * f * d, 2 * f, d, a.overwrite);
-  UP_LAUNCH_CHECK();
-  return UNIPOOL_OK;
+template <typename Args>
+RowGemm row_gemm(const unipool_ctx* ctx, const Args& a) {
+  RowGemm p{};
+  p.tile_expert = a.tile_expert;
+  p.offsets = a.offsets;
+  p.rows = a.rows;
+  p.expert_base = a.expert_base;
+  p.f = ctx->cfg.d_ff;
+  p.b_expert = (int64_t)ctx->cfg.d_model * ctx->cfg.d_ff;
+  p.n_row_tiles = (int)(ctx->row_capacity / kRowTile);
+  return p;
 }
 
-template <typename TE>
-static int bwd_impl(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
-  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff;
-  const int n_row_tiles = (int)(ctx->row_capacity / kSimtTile);
-  const int gy = n_row_tiles < 4096 ? n_row_tiles : 4096;
-  const TE* dYp = static_cast<const TE*>(a.dYp);
-  TE* dGU = static_cast<TE*>(a.dGU);
-  // dA = dYp W_down[e] : B(k, n) = W_down[e][k, n]; lands in the U half of dGU
-  {
-  PhaseTimer pt(ctx, UNIPOOL_PH_DGRAD_DOWN, 2, s);
-  grouped_rows_gemm_kernel<TE><<<dim3(f / kSimtTile, gy), kSimtThreads, 0, s>>>(
-      dYp, d, static_cast<const TE*>(a.W_down), (int64_t)d * f, f, 1, a.tile_expert, a.expert_base,
-      dGU + f, 2 * f, f, d, n_row_tiles);
-  UP_LAUNCH_CHECK();
-  swiglu_bwd_kernel<TE><<<ctx->sm_count * 8, 256, 0, s>>>(static_cast<const TE*>(a.GU), dGU,
-                                                          a.offsets + a.n_experts, f);
-  UP_LAUNCH_CHECK();
-  }
-  // dXp = dGU W_gu[e] : B(k, n) = W_gu[e][k, n]
-  {
-  PhaseTimer pt(ctx, UNIPOOL_PH_DGRAD_GU, 1, s);
-  grouped_rows_gemm_kernel<TE><<<dim3(d / kSimtTile, gy), kSimtThreads, 0, s>>>(
-      dGU, 2 * f, static_cast<const TE*>(a.W_gu), (int64_t)2 * f * d, d, 1, a.tile_expert,
-      a.expert_base, static_cast<TE*>(a.dXp), d, d, 2 * f, n_row_tiles);
-  UP_LAUNCH_CHECK();
-  }
-  if (a.wgrad) {
-    PoolWgradArgs w{1, 0, a.offsets, a.Xp, a.A, a.dYp, a.dGU, a.expert_base, a.n_experts, a.dW_gu, a.dW_down,
-                    a.overwrite, a.rows};
-    return wgrad_impl<TE>(ctx, w, s);
-  }
-  return UNIPOOL_OK;
-}
+}  // namespace
 
 int expert_fwd_simt(unipool_ctx* ctx, const ExpertFwdArgs& a, cudaStream_t s) {
-  return ctx->cfg.dtype == UNIPOOL_BF16 ? fwd_impl<__nv_bfloat16>(ctx, a, s) : fwd_impl<float>(ctx, a, s);
+  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff;
+  {
+    PhaseTimer pt(ctx, UNIPOOL_PH_EXPERT_FWD_GU, 1, s);
+    RowGemm p = row_gemm(ctx, a);                    // GU = Xp W_gu[e]^T, A = silu(G) U
+    p.A = static_cast<const float*>(a.Xp); p.lda = d; p.K = d;
+    p.B = static_cast<const float*>(a.W_gu); p.b_expert *= 2; p.ldb = d; p.N = f;
+    p.C = static_cast<float*>(a.GU); p.C2 = static_cast<float*>(a.A);
+    const int rc = rows_gemm<kAlongK, kSwiglu>(ctx, p, a.n_experts, s);
+    if (rc != UNIPOOL_OK) return rc;
+  }
+  PhaseTimer pt(ctx, UNIPOOL_PH_EXPERT_FWD_DOWN, 1, s);
+  RowGemm p = row_gemm(ctx, a);                      // Yp = A W_down[e]^T
+  p.A = static_cast<const float*>(a.A); p.lda = f; p.K = f;
+  p.B = static_cast<const float*>(a.W_down); p.ldb = f; p.N = d;
+  p.C = static_cast<float*>(a.Yp);
+  return rows_gemm<kAlongK, kStore>(ctx, p, a.n_experts, s);
 }
-int expert_bwd_simt(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
-  return ctx->cfg.dtype == UNIPOOL_BF16 ? bwd_impl<__nv_bfloat16>(ctx, a, s) : bwd_impl<float>(ctx, a, s);
-}
+
 int pool_wgrad_simt(unipool_ctx* ctx, const PoolWgradArgs& a, cudaStream_t s) {
-  return ctx->cfg.dtype == UNIPOOL_BF16 ? wgrad_impl<__nv_bfloat16>(ctx, a, s) : wgrad_impl<float>(ctx, a, s);
+  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff;
+  PoolGemm p{};
+  p.offsets = a.offsets; p.rows = a.rows;
+  p.n_experts = a.n_experts; p.expert_base = a.expert_base;
+  p.n_layers = a.n_layers; p.layer_stride_rows = a.layer_stride_rows;
+  p.overwrite = a.overwrite;
+  if (a.dW_down != nullptr) {                        // dW_down[e] [d, f] (+)= dYp_e^T A_e
+    PhaseTimer pt(ctx, UNIPOOL_PH_WGRAD_DOWN, 1, s);
+    p.P = static_cast<const float*>(a.dYp); p.ldp = d;
+    p.Q = static_cast<const float*>(a.A); p.ldq = f;
+    p.dW = a.dW_down; p.Mdim = d; p.Ndim = f; p.vec = aligned16(p.P, p.Q, p.dW);
+    grouped_k_gemm_kernel<<<dim3(d / 64, f / 64, a.n_experts), kSimtGroup, 0, s>>>(p);
+    UP_LAUNCH_CHECK();
+  }
+  if (a.dW_gu == nullptr) return UNIPOOL_OK;
+  PhaseTimer pt(ctx, UNIPOOL_PH_WGRAD_GU, 1, s);     // dW_gu[e] [2f, d] (+)= dGU_e^T Xp_e
+  p.P = static_cast<const float*>(a.dGU); p.ldp = 2 * f;
+  p.Q = static_cast<const float*>(a.Xp); p.ldq = d;
+  p.dW = a.dW_gu; p.Mdim = 2 * f; p.Ndim = d; p.vec = aligned16(p.P, p.Q, p.dW);
+  grouped_k_gemm_kernel<<<dim3(2 * f / 64, d / 64, a.n_experts), kSimtGroup, 0, s>>>(p);
+  UP_LAUNCH_CHECK();
+  return UNIPOOL_OK;
+}
+
+int expert_bwd_simt(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
+  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff;
+  {
+    PhaseTimer pt(ctx, UNIPOOL_PH_DGRAD_DOWN, 1, s);
+    RowGemm p = row_gemm(ctx, a);                    // dA = dYp W_down[e], then dG, dU
+    p.A = static_cast<const float*>(a.dYp); p.lda = d; p.K = d;
+    p.B = static_cast<const float*>(a.W_down); p.ldb = f; p.N = f;
+    p.C = static_cast<float*>(a.dGU); p.GU = static_cast<const float*>(a.GU);
+    const int rc = rows_gemm<kAcrossK, kSwigluBwd>(ctx, p, a.n_experts, s);
+    if (rc != UNIPOOL_OK) return rc;
+  }
+  {
+    PhaseTimer pt(ctx, UNIPOOL_PH_DGRAD_GU, 1, s);
+    RowGemm p = row_gemm(ctx, a);                    // dXp = dGU W_gu[e]
+    p.A = static_cast<const float*>(a.dGU); p.lda = 2 * f; p.K = 2 * f;
+    p.B = static_cast<const float*>(a.W_gu); p.b_expert *= 2; p.ldb = d; p.N = d;
+    p.C = static_cast<float*>(a.dXp);
+    const int rc = rows_gemm<kAcrossK, kStore>(ctx, p, a.n_experts, s);
+    if (rc != UNIPOOL_OK) return rc;
+  }
+  if (!a.wgrad) return UNIPOOL_OK;
+  PoolWgradArgs w{1, 0, a.offsets, a.Xp, a.A, a.dYp, a.dGU, a.expert_base, a.n_experts, a.dW_gu, a.dW_down,
+                  a.overwrite, a.rows};
+  return pool_wgrad_simt(ctx, w, s);
 }
 
 }  // namespace unipool

@@ -7,23 +7,28 @@
 namespace unipool {
 
 // ---------------------------------------------------------------- logits  z = x W_r^T (+ bias)
-template <typename TX>
-__global__ void __launch_bounds__(kSimtThreads)
-router_logits_kernel(const TX* __restrict__ x, const float* __restrict__ W_r,
-                     const float* __restrict__ bias, float* __restrict__ z, int T, int M, int d) {
-  const int m0 = blockIdx.x * kSimtTile, n0 = blockIdx.y * kSimtTile;
-  float acc[4][4] = {};
-  SimtOperands<TX, float> op{x, d, 1, W_r, 1, d};
-  simt_tile_mainloop(op, m0, n0, T, M, 0, d, acc);
-  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+// Few tiles (one per 32 tokens and 32 experts), so four groups of threads share a tile's contraction.
+using RouterTile = SimtTile<32, 32, 4>;
+
+__global__ void __launch_bounds__(RouterTile::kThreads)
+router_logits_kernel(const float* __restrict__ x, const float* __restrict__ W_r,
+                     const float* __restrict__ bias, float* __restrict__ z, int T, int M, int d, bool vec) {
+  __shared__ RouterTile::Smem sm;
+  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+  RouterTile t;
+  t.run<kAlongK, kAlongK>(
+      sm, d / kSimtKC,
+      [&](int c, int i, int k) { return ld4(x + (int64_t)(m0 + i) * d + c * kSimtKC + k, vec, m0 + i < T ? 4 : 0); },
+      [&](int c, int i, int k) { return ld4(W_r + (int64_t)(n0 + i) * d + c * kSimtKC + k, vec, n0 + i < M ? 4 : 0); });
+  if (threadIdx.x >= kSimtGroup) return;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int t = m0 + ty * 4 + i;
-    if (t >= T) continue;
+  for (int i = 0; i < RouterTile::MR; ++i) {
+    const int tok = m0 + t.row(i);
+    if (tok >= T) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int e = n0 + tx * 4 + j;
-      if (e < M) z[(int64_t)t * M + e] = acc[i][j] + (bias ? bias[e] : 0.f);
+    for (int j = 0; j < RouterTile::NR; ++j) {
+      const int e = n0 + t.col(j);
+      if (e < M) z[(int64_t)tok * M + e] = t.value(i, j) + (bias ? bias[e] : 0.f);
     }
   }
 }
@@ -164,16 +169,11 @@ int route_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float
   }
   if (ctx->cfg.dtype == UNIPOOL_BF16)
     return route_tc_launch(ctx, x, T, W_r, sigma, bias, M, idx, gate, counts, score_sum, znorm, z_saved, s);
-  dim3 g1((T + kSimtTile - 1) / kSimtTile, (M + kSimtTile - 1) / kSimtTile);
   {
-  PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_LOGITS, 1, s);
-  if (ctx->cfg.dtype == UNIPOOL_BF16)
-    router_logits_kernel<__nv_bfloat16><<<g1, kSimtThreads, 0, s>>>(
-        static_cast<const __nv_bfloat16*>(x), W_r, bias, z_saved, T, M, d);
-  else
-    router_logits_kernel<float><<<g1, kSimtThreads, 0, s>>>(static_cast<const float*>(x), W_r, bias,
-                                                            z_saved, T, M, d);
-  UP_LAUNCH_CHECK();
+    PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_LOGITS, 1, s);
+    router_logits_kernel<<<dim3((T + 31) / 32, (M + 31) / 32), RouterTile::kThreads, 0, s>>>(
+        static_cast<const float*>(x), W_r, bias, z_saved, T, M, d, aligned16(x, W_r));
+    UP_LAUNCH_CHECK();
   }
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_SELECT, 1, s);
   const int per_block = kRouteWarps * kRouteTokensPerWarp;
@@ -259,50 +259,64 @@ router_dz_kernel(const float* __restrict__ z, const float* __restrict__ znorm,
 }
 
 // dx[t,:] += dz[t,:] W_r     (K = M)
-template <typename TX>
-__global__ void __launch_bounds__(kSimtThreads)
-router_dx_kernel(const float* __restrict__ dz, const float* __restrict__ W_r, TX* __restrict__ dx,
-                 int T, int M, int d) {
-  const int m0 = blockIdx.x * kSimtTile, n0 = blockIdx.y * kSimtTile;
-  float acc[4][4] = {};
-  SimtOperands<float, float> op{dz, M, 1, W_r, d, 1};
-  simt_tile_mainloop(op, m0, n0, T, d, 0, M, acc);
-  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+using RouterDxTile = SimtTile<32, 32, 1>;
+
+__global__ void __launch_bounds__(RouterDxTile::kThreads)
+router_dx_kernel(const float* __restrict__ dz, const float* __restrict__ W_r, float* __restrict__ dx,
+                 int T, int M, int d, bool vec) {
+  __shared__ RouterDxTile::Smem sm;
+  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+  const bool vec_z = (M & 3) == 0;                   // dz is a workspace array of rows of M
+  RouterDxTile t;
+  t.run<kAlongK, kAcrossK>(
+      sm, (M + kSimtKC - 1) / kSimtKC,
+      [&](int c, int i, int k) {
+        const int kk = c * kSimtKC + k;
+        return ld4(dz + (int64_t)(m0 + i) * M + kk, vec_z, m0 + i < T ? M - kk : 0);
+      },
+      [&](int c, int i, int k) {
+        const int kk = c * kSimtKC + k;
+        return ld4(W_r + (int64_t)kk * d + n0 + i, vec, kk < M ? 4 : 0);
+      });
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int t = m0 + ty * 4 + i;
-    if (t >= T) continue;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int q = n0 + tx * 4 + j;
-      if (q < d) {
-        int64_t o = (int64_t)t * d + q;
-        dx[o] = from_f32<TX>(to_f32(dx[o]) + acc[i][j]);
-      }
-    }
+  for (int i = 0; i < RouterDxTile::MR; ++i) {
+    const int tok = m0 + t.row(i);
+    if (tok >= T) continue;
+    float* o = dx + (int64_t)tok * d + n0 + t.col(0);
+    st4(o, make_float4(o[0] + t.value(i, 0), o[1] + t.value(i, 1), o[2] + t.value(i, 2), o[3] + t.value(i, 3)), vec);
   }
 }
 
-// dW_r[m,:] += sum_t dz[t,m] x[t,:]   (K = T, split over blockIdx.z, fp32 atomics)
-template <typename TX>
-__global__ void __launch_bounds__(kSimtThreads)
-router_dw_kernel(const float* __restrict__ dz, const TX* __restrict__ x, float* __restrict__ dW_r,
-                 int T, int M, int d, int k_len) {
-  const int m0 = blockIdx.x * kSimtTile, n0 = blockIdx.y * kSimtTile;
-  const int k_begin = blockIdx.z * k_len;
-  const int k_end = min(T, k_begin + k_len);
-  float acc[4][4] = {};
-  SimtOperands<float, TX> op{dz, 1, M, x, d, 1};
-  simt_tile_mainloop(op, m0, n0, M, d, k_begin, k_end, acc);
-  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;
+// dW_r[m,:] += sum_t dz[t,m] x[t,:]   (K = T, cut into runs of k_len tokens over blockIdx.z: one run adds in
+// place, several by atomics)
+__global__ void __launch_bounds__(RouterTile::kThreads)
+router_dw_kernel(const float* __restrict__ dz, const float* __restrict__ x, float* __restrict__ dW_r,
+                 int T, int M, int d, int k_len, bool vec) {
+  __shared__ RouterTile::Smem sm;
+  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+  const int k_begin = blockIdx.z * k_len, k_end = min(T, k_begin + k_len);
+  const bool vec_z = (M & 3) == 0;
+  RouterTile t;
+  t.run<kAcrossK, kAcrossK>(
+      sm, (k_end - k_begin + kSimtKC - 1) / kSimtKC,
+      [&](int c, int i, int k) {
+        const int tok = k_begin + c * kSimtKC + k;
+        return ld4(dz + (int64_t)tok * M + m0 + i, vec_z, tok < k_end ? M - m0 - i : 0);
+      },
+      [&](int c, int i, int k) {
+        const int tok = k_begin + c * kSimtKC + k;
+        return ld4(x + (int64_t)tok * d + n0 + i, vec, tok < k_end ? 4 : 0);
+      });
+  if (threadIdx.x >= kSimtGroup) return;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    int m = m0 + ty * 4 + i;
+  for (int i = 0; i < RouterTile::MR; ++i) {
+    const int m = m0 + t.row(i);
     if (m >= M) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      int q = n0 + tx * 4 + j;
-      if (q < d) atomicAdd(&dW_r[(int64_t)m * d + q], acc[i][j]);
+    for (int j = 0; j < RouterTile::NR; ++j) {
+      float* o = dW_r + (int64_t)m * d + n0 + t.col(j);
+      if (gridDim.z == 1) *o += t.value(i, j);
+      else atomicAdd(o, t.value(i, j));
     }
   }
 }
@@ -323,23 +337,16 @@ int route_bwd_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, f
                                    ctx->cfg.eps, dz, dsigma, ctx->ws.dsigma_acc, ctx->ws.tickets + 1);
   UP_LAUNCH_CHECK();
   }
-  dim3 g2((T + kSimtTile - 1) / kSimtTile, d / kSimtTile);
-  const int k_len = 1024;
-  dim3 g3((M + kSimtTile - 1) / kSimtTile, d / kSimtTile, (T + k_len - 1) / k_len);
-  const bool bf16 = ctx->cfg.dtype == UNIPOOL_BF16;
   {
     PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_BWD_DX, 1, s);
-    if (bf16)
-      router_dx_kernel<__nv_bfloat16><<<g2, kSimtThreads, 0, s>>>(dz, W_r, static_cast<__nv_bfloat16*>(dx), T, M, d);
-    else
-      router_dx_kernel<float><<<g2, kSimtThreads, 0, s>>>(dz, W_r, static_cast<float*>(dx), T, M, d);
+    router_dx_kernel<<<dim3((T + 31) / 32, d / 32), RouterDxTile::kThreads, 0, s>>>(
+        dz, W_r, static_cast<float*>(dx), T, M, d, aligned16(W_r, dx));
     UP_LAUNCH_CHECK();
   }
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_BWD_DW, 1, s);
-  if (bf16)
-    router_dw_kernel<__nv_bfloat16><<<g3, kSimtThreads, 0, s>>>(dz, static_cast<const __nv_bfloat16*>(x), dW_r, T, M, d, k_len);
-  else
-    router_dw_kernel<float><<<g3, kSimtThreads, 0, s>>>(dz, static_cast<const float*>(x), dW_r, T, M, d, k_len);
+  const int k_len = 1024;
+  router_dw_kernel<<<dim3((M + 31) / 32, d / 32, (T + k_len - 1) / k_len), RouterTile::kThreads, 0, s>>>(
+      dz, static_cast<const float*>(x), dW_r, T, M, d, k_len, aligned16(x));
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;
 }

@@ -190,3 +190,95 @@ def test_weight_gradient_leaves_the_padding_out(sizes, overwrite):
         # exact products, fp32 sums of at most some 1200 terms: 1e-5 of the largest value
         assert (got[1][0][e] - want).abs().max() <= 1e-5 * max(want.abs().max().item(), 1.0)
         assert (got[1][1][e] - down).abs().max() <= 1e-5 * max(down.abs().max().item(), 1.0)
+
+
+@pytest.mark.parametrize("sizes,d,f", [
+    ([0, 1, 15, 16, 17, 63, 64, 65, 127, 128, 129], 64, 64),      # narrow tiles, two groups of threads per tile
+    ([500, 0, 700, 1, 2000, 64], 256, 512),                       # wide tiles
+])
+@pytest.mark.parametrize("shift", [0, 1])                         # 1: pointers that are not 16-byte aligned
+def test_fp32_expert_ffn_at_the_edges_of_its_tiles(sizes, d, f, shift):
+    """fp32 mode against float64.  Sums of at most 2000 products: |error| <= 2000 * 2^-24 of the terms' magnitudes,
+    which random signs keep far below 1e-5 of the largest value."""
+    import torch
+    from paper_2605_06665_b200 import binding as B
+    M, T = len(sizes), sum(sizes)
+    ctx = B.Context(B.make_config(d, f, M, 1, 1, T, B.FP32, 1e-6, 2.0))
+    cap = ctx.row_capacity
+    g = torch.Generator(device="cuda").manual_seed(5)
+
+    def new(*s, std=None):
+        n = int(np.prod(s))
+        t = torch.full((n + 4,), float("nan"), device="cuda")[shift:shift + n].view(s)
+        return t if std is None else t.normal_(0, std, generator=g)
+
+    i32 = dict(dtype=torch.int32, device="cuda")
+    x, dy = torch.randn(T, d, device="cuda", generator=g), torch.randn(T, d, device="cuda", generator=g)
+    Wgu, Wd = new(M, 2 * f, d, std=0.05), new(M, d, f, std=0.05)
+    idx = torch.repeat_interleave(torch.arange(M), torch.tensor(sizes))[torch.randperm(T)].to(torch.int32).cuda()[:, None].contiguous()
+    off, row_of, tok, te, rows = (torch.empty(s, **i32) for s in ((M + 1,), (T, 1), (cap,), (cap // 128,), (M,)))
+    rowbuf = lambda w: torch.full((cap, w), float("nan"), device="cuda")
+    Xp, Yp, dYp, dx = rowbuf(d), rowbuf(d), rowbuf(d), torch.empty(T, d, device="cuda")
+    GU, A, dGU = new(cap, 2 * f), new(cap, f), new(cap, 2 * f)
+    dWgu, dWd = new(M, 2 * f, d), new(M, d, f)
+    gate, dgate = torch.rand(T, 1, device="cuda", generator=g) + 0.5, torch.empty(T, 1, device="cuda")
+    ctx.dispatch(x, T, idx, M, off, row_of, tok, te, Xp, rows)
+    ctx.expert_fwd(Xp, off, te, Wgu, Wd, 0, M, GU, A, Yp, rows)
+    ctx.expert_bwd(dy, T, row_of, gate, tok, off, te, Xp, GU, A, Yp, Wgu, Wd, 0, M, None, dYp, dGU, dx, dgate, dWgu, dWd,
+                   B.WGRAD_OVERWRITE, rows)
+    torch.cuda.synchronize()
+    ctx.check_status()
+    ctx.close()
+    used = int(off[-1])
+    pad = tok[:used] < 0
+    for t in (GU, A, Yp, dGU):
+        assert not t[:used][pad].any()
+
+    def close(got, want):
+        assert (got.double() - want).abs().max() <= 1e-5 * max(want.abs().max().item(), 1e-3)
+
+    for e, n in enumerate(sizes):
+        s = slice(int(off[e]), int(off[e]) + n)
+        X, Wg, Wu, W2, dY = (t.double() for t in (Xp[s], Wgu[e, :f], Wgu[e, f:], Wd[e], dYp[s]))
+        if n:
+            G, U = X @ Wg.T, X @ Wu.T
+            close(GU[s], torch.cat([G, U], 1))
+            close(A[s], torch.nn.functional.silu(G) * U)
+            close(Yp[s], A[s].double() @ W2.T)
+            G, U, dA = GU[s, :f].double(), GU[s, f:].double(), dY @ W2
+            sig = torch.sigmoid(G)
+            close(dGU[s], torch.cat([dA * U * sig * (1 + G * (1 - sig)), dA * G * sig], 1))
+            close(dx[tok[s].long()], dGU[s].double() @ Wgu[e].double())
+        close(dWd[e], dY.T @ A[s].double())
+        close(dWgu[e], dGU[s].double().T @ X)
+
+
+@pytest.mark.parametrize("T,M,d", [(1, 1, 64), (33, 13, 128), (512, 16, 256), (1100, 33, 64), (2100, 36, 192)])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_fp32_router_products_at_the_edges_of_their_tiles(T, M, d, shift):
+    """Logits, dx and dW_r of the fp32 router: M with and without 16-byte rows of dz, tokens beyond one run of 1024,
+    router weights that are not 16-byte aligned; against the oracle in float64 (1e-5, as in the parity tests)."""
+    import torch
+    from oracle import unipool_oracle as O
+    from paper_2605_06665_b200 import binding as B
+    k, c, eps = 1, 2.0, 1e-6
+    ctx = B.Context(B.make_config(d, 64, M, k, 1, T, B.FP32, eps, c))
+    g = torch.Generator(device="cuda").manual_seed(T)
+    W = torch.empty(M * d + 4, device="cuda")[shift:shift + M * d].view(M, d).normal_(0, 0.02, generator=g)
+    x, dgate = torch.randn(T, d, device="cuda", generator=g), torch.randn(T, k, device="cuda", generator=g)
+    idx = torch.empty(T, k, dtype=torch.int32, device="cuda")
+    gate, counts = torch.empty(T, k, device="cuda"), torch.empty(M, dtype=torch.int32, device="cuda")
+    S, n, z = torch.empty(M, device="cuda"), torch.empty(T, device="cuda"), torch.empty(T, M, device="cuda")
+    coef = torch.rand(M, device="cuda", generator=g)
+    dx, dW, dsig = torch.ones(T, d, device="cuda"), torch.full((M, d), 2.0, device="cuda"), torch.zeros(1, device="cuda")
+    ctx.route(x, T, W, 1.0, None, M, idx, gate, counts, S, n, z)
+    ctx.route_bwd(x, T, W, 1.0, M, n, z, idx, dgate, coef, dx, dW, dsig)
+    torch.cuda.synchronize()
+    ctx.check_status()
+    ctx.close()
+    f8 = lambda t: t.double().cpu().numpy()
+    ref = O.route(f8(x), f8(W), 1.0, c, eps, k, None, forced_idx=idx.cpu().numpy())
+    rb = O.route_backward(f8(x), f8(W), 1.0, c, eps, ref["z"], ref["n"], idx.cpu().numpy(), f8(dgate), f8(coef))
+    for got, want in ((z, ref["z"]), (dx - 1, rb["dx"]), (dW - 2, rb["dW_r"])):
+        scale = max(np.abs(want).max(), 1.0 if want is not ref["z"] else 0.0)       # dx and dW were added to 1 and 2
+        assert np.abs(f8(got) - want).max() <= 1e-5 * scale
