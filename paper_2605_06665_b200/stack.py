@@ -40,7 +40,7 @@ class UniPoolStack:
         self.c, self.eps = c, eps
         # recompute: keep only x_l and the routing state of a layer; its permuted activations are
         # rebuilt in backward (MoE-layer activation recompute, App. D), so the weight gradient is
-        # taken layer by layer
+        # taken for the few layers whose operands are held at a time (see _wgrad_layers)
         self.recompute = recompute
         self.deferred_wgrad = deferred_wgrad and self.Lg > 1 and not recompute
         self.device = torch.device(device)
@@ -81,11 +81,12 @@ class UniPoolStack:
         self.token_of = e(L, cap, dtype=i32)
         self.tile_expert = e(L, cap // B.ROW_ALIGN, dtype=i32)
         ns = 1 if recompute else L                         # layers whose permuted activations are kept
-        self.Xp = e(ns, cap, d)
+        self.nw = self._wgrad_layers() if recompute else 1
+        self.Xp = e(max(ns, self.nw), cap, d)
         self.GU = e(ns, cap, 2 * f)
-        self.A = e(ns, cap, f)
+        self.A = e(max(ns, self.nw), cap, f)
         self.Yp = e(ns, cap, d)
-        nb = L if self.deferred_wgrad else 1
+        nb = L if self.deferred_wgrad else self.nw
         self.dYp = e(nb, cap, d)
         self.dGU = e(nb, cap, 2 * f)
         self.dx = e(2, T, d)                               # ping-pong dx_{l+1} -> dx_l
@@ -97,6 +98,18 @@ class UniPoolStack:
         self.fbar = e(n_aux, self.m, dtype=f32)
         self.fbar_lag = None                               # f-bar of the previous micro-batch (App. G)
         self._copy_stream = None                           # host <-> device copies beside the compute
+
+    def _wgrad_layers(self):
+        """Layers whose weight gradients are contracted together when activations are recomputed.  Each
+        contraction reads and writes the whole fp32 pool gradient (2.2 + 4.4 ms per layer at 192 experts
+        of 1536 x 4096, 65536 rows, against 1.8 + 3.5 ms of its own), so the operands (Xp, A, dYp, dGU) of
+        as many layers are held as fit into half the pool gradient's own size beside the one that is needed
+        anyway: few rows and a large pool - where the read-modify-write weighs most - allow the most layers."""
+        bytes_per_layer = self.cap * (2 * self.d + 3 * self.f) * torch.empty(0, dtype=self.tdtype).element_size()
+        pool_gradient = self.M * 3 * self.d * self.f * 4
+        most = 1 + pool_gradient // 2 // bytes_per_layer
+        passes = -(-self.Lg // min(self.Lg, most))
+        return -(-self.Lg // passes)
 
     # ------------------------------------------------------------------ parameters
     def load(self, pool, routers):
@@ -137,14 +150,15 @@ class UniPoolStack:
         self.permute_and_experts(l, T)
         c.combine(self.Yp[self.slot(l)], self.row_of[l], self.gate[l], T, self.x[l], self.x[l + 1])
 
-    def permute_and_experts(self, l, T):
+    def permute_and_experts(self, l, T, w=None):
         """dispatch + expert forward of layer l from x_l and its routing decision (also the
-        recompute step of backward)."""
+        recompute step of backward, which keeps Xp and A in slot ``w``)."""
         c, s = self.ctx, self.slot(l)
+        w = s if w is None else w
         c.dispatch(self.x[l], T, self.idx[l], self.m, self.offsets[l], self.row_of[l], self.token_of[l],
-                   self.tile_expert[l], self.Xp[s], self.rows[l])
-        c.expert_fwd(self.Xp[s], self.offsets[l], self.tile_expert[l], self.W_gu, self.W_down,
-                     self.base(l), self.m, self.GU[s], self.A[s], self.Yp[s], self.rows[l])
+                   self.tile_expert[l], self.Xp[w], self.rows[l])
+        c.expert_fwd(self.Xp[w], self.offsets[l], self.tile_expert[l], self.W_gu, self.W_down,
+                     self.base(l), self.m, self.GU[s], self.A[w], self.Yp[s], self.rows[l])
 
     def forward(self, x0=None, T=None):
         T = self.T if T is None else T
@@ -171,18 +185,22 @@ class UniPoolStack:
         return self.loss
 
     # ------------------------------------------------------------------ backward
-    def backward_layer(self, l, dx_next, dx_out, T=None, with_aux=True, overwrite=False):
+    def backward_layer(self, l, dx_next, dx_out, T=None, with_aux=True, overwrite=False, hold=None):
         """``overwrite``: this layer's weight gradient replaces what the pool-gradient
-        slices of its view hold (the first contribution of a step) instead of adding to it."""
+        slices of its view hold (the first contribution of a step) instead of adding to it.
+        ``hold`` (recompute): the operands of the weight gradient stay in this slot for a
+        contraction of several layers by the caller."""
         T = self.T if T is None else T
         c = self.ctx
-        s = l if self.deferred_wgrad else 0
         a = self.slot(l)
+        w = a if hold is None else hold                    # Xp, A
+        s = l if self.deferred_wgrad else hold or 0        # dYp, dGU
         if self.recompute:
-            self.permute_and_experts(l, T)
-        flags = B.BWD_SKIP_WGRAD if self.deferred_wgrad else (B.WGRAD_OVERWRITE if overwrite else 0)
+            self.permute_and_experts(l, T, w)
+        later = self.deferred_wgrad or hold is not None
+        flags = B.BWD_SKIP_WGRAD if later else (B.WGRAD_OVERWRITE if overwrite else 0)
         c.expert_bwd(dx_next, T, self.row_of[l], self.gate[l], self.token_of[l], self.offsets[l],
-                     self.tile_expert[l], self.Xp[a], self.GU[a], self.A[a], self.Yp[a], self.W_gu,
+                     self.tile_expert[l], self.Xp[w], self.GU[a], self.A[w], self.Yp[a], self.W_gu,
                      self.W_down, self.base(l), self.m, dx_next, self.dYp[s], self.dGU[s], dx_out,
                      self.dgate, self.dW_gu, self.dW_down, flags, self.rows[l])
         coef = None
@@ -202,8 +220,15 @@ class UniPoolStack:
         if upstream is not None:
             self.dx[cur, :T].copy_(upstream, non_blocking=True)
         for l in reversed(range(self.L)):
-            first = (not accumulate) and l % self.Lg == self.Lg - 1     # first contribution to its group's experts
-            self.backward_layer(l, self.dx[cur], self.dx[1 - cur], T, with_aux, overwrite=first)
+            i = l % self.Lg                                             # layer inside its sharing group
+            hold = i % self.nw if self.nw > 1 else None
+            # first contribution to its group's experts: the top layer, or the run of layers it belongs to
+            first = (not accumulate) and i >= (self.Lg - 1) // self.nw * self.nw
+            self.backward_layer(l, self.dx[cur], self.dx[1 - cur], T, with_aux, overwrite=first, hold=hold)
+            if hold == 0:                                               # the lowest layer of a run
+                self.ctx.pool_wgrad(min(self.nw, self.Lg - i), self.cap, self.offsets[l:], self.Xp, self.A, self.dYp,
+                                    self.dGU, self.base(l), self.m, self.dW_gu, self.dW_down,
+                                    B.WGRAD_OVERWRITE if first else 0, self.rows[l:])
             cur = 1 - cur
         if self.deferred_wgrad:
             for g in range(self.G):                        # one pass per sharing group over its layers

@@ -282,3 +282,38 @@ def test_fp32_router_products_at_the_edges_of_their_tiles(T, M, d, shift):
     for got, want in ((z, ref["z"]), (dx - 1, rb["dx"]), (dW - 2, rb["dW_r"])):
         scale = max(np.abs(want).max(), 1.0 if want is not ref["z"] else 0.0)       # dx and dW were added to 1 and 2
         assert np.abs(f8(got) - want).max() <= 1e-5 * scale
+
+
+@pytest.mark.parametrize("kw,L,T", [
+    (dict(M=48, k=1), 5, 40),                       # runs of two, two and one layer
+    (dict(M=32, k=2), 4, 70),
+    (dict(M=64, k=2, groups=2), 6, 50),             # two sharing groups of three layers, runs of two and one
+])
+@pytest.mark.parametrize("accumulate", [False, True])
+def test_recomputed_layers_contract_in_runs(kw, L, T, accumulate):
+    """With recompute the weight gradients of a run of layers are contracted together: same sums as layer by layer up
+    to the order of fp32 additions (1e-5, as for the one-pass contraction)."""
+    import torch
+    from paper_2605_06665_b200 import synth
+    from paper_2605_06665_b200.stack import UniPoolStack
+    from parity_utils import rel_max, to_np
+    cfg = dict(L=L, d=256, f=384, T=T, dtype="bf16", private=0, zipf_beta=0.0, **kw)
+    inputs = synth.make_inputs(cfg, seed=4, T=T)
+    x0, up = (torch.from_numpy(inputs[n]).cuda().bfloat16() for n in ("x0", "upstream"))
+    out = []
+    for recompute in (False, True):
+        st = UniPoolStack(L, 256, 384, kw["M"], kw["k"], T, "bf16", 0, c=2.5, recompute=recompute, groups=kw.get("groups"))
+        st.load(inputs["pool"], inputs["routers"])
+        if recompute:
+            assert 1 < st.nw <= st.Lg and st.GU.shape[0] == st.Yp.shape[0] == 1
+        if accumulate:
+            st.zero_grad()
+        else:
+            st.dW_gu.fill_(11.0); st.dW_down.fill_(-2.0)
+        dx = st.step(x0, up, accumulate=accumulate).clone()
+        torch.cuda.synchronize()
+        st.ctx.check_status()
+        out.append((dx, st.dW_gu.clone(), st.dW_down.clone()))
+        st.close()
+    assert torch.equal(out[0][0], out[1][0]) and out[0][1].abs().max() > 0
+    assert rel_max(to_np(out[1][1]), to_np(out[0][1])) < 1e-5 and rel_max(to_np(out[1][2]), to_np(out[0][2])) < 1e-5
