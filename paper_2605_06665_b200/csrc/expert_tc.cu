@@ -675,14 +675,20 @@ __device__ __forceinline__ int snake_tile(int round, int pair, int n_pairs) {
   return round * n_pairs + ((round & 1) ? n_pairs - 1 - pair : pair);
 }
 
+// KR = rows of a k-block: 64 in six stages, 48 in eight or 32 in twelve.  Where a layer gives an expert fewer rows
+// than a k-block holds, the loop is bound by the latency of the k-blocks in flight (some 3500 clocks; without its
+// stores the 1501-token case takes 95 % of the time, with half the bytes 98 %), so more and smaller ones.
+template <int KR>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const __grid_constant__ CUtensorMap tmC0, const GemmParams p) {
+  constexpr int kStages = kPairStages * BK / KR;
+  constexpr uint32_t kHalf = kPairHalfBytes * KR / BK, kStage = 2 * kHalf, kBlock = 128 * KR;   // kBlock: 64 columns
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + kBarOffset);
-  uint64_t* empty_bar = full_bar + kPairStages;
-  uint64_t* tmem_full = empty_bar + kPairStages;
+  uint64_t* empty_bar = full_bar + kStages;
+  uint64_t* tmem_full = empty_bar + kStages;
   uint64_t* tmem_empty = tmem_full + 2;
   uint32_t* tmem_ptr = reinterpret_cast<uint32_t*>(tmem_empty + 2);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_ptr + 1);
@@ -692,7 +698,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kPairStages; ++s) { tc::mbar_init(&full_bar[s], 1); tc::mbar_init(&empty_bar[s], 1); }
+    for (int s = 0; s < kStages; ++s) { tc::mbar_init(&full_bar[s], 1); tc::mbar_init(&empty_bar[s], 1); }
     for (int a = 0; a < 2; ++a) { tc::mbar_init(&tmem_full[a], 1); tc::mbar_init(&tmem_empty[a], 2 * kEpiWarps); }
     *abort = 0;
     tc::fence_barrier_init();
@@ -759,22 +765,22 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         for (int l = 0; l < min(32, p.n_layers - l0) && ok; ++l) {
           const int n = __shfl_sync(0xffffffffu, count, l);
           const int row0 = (l0 + l) * p.layer_stride_rows + __shfl_sync(0xffffffffu, cur.first, l);
-          for (int done = 0; done < n; done += BK) {
+          for (int done = 0; done < n; done += KR) {
             if (!tc::mbar_wait(&empty_bar[stage], phase ^ 1u, abort)) {
               if (lane == 0) report_timeout(p, abort, 21);
               ok = false;
               break;
             }
             if (lane == 0) {
-              uint8_t* sA = smem + stage * kPairStageBytes;
-              uint8_t* sB = sA + kPairHalfBytes;
-              if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], 2 * kPairStageBytes);   // both CTAs' bytes
+              uint8_t* sA = smem + stage * kStage;
+              uint8_t* sB = sA + kHalf;
+              if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], 2 * kStage);   // both CTAs' bytes
               // this CTA's two 64-column blocks of each operand, one box each
               tc::tma_load_3d_pair(sA, &tmA, &full_bar[stage], 0, row0 + done, mt * 4 + rank * 2);
               tc::tma_load_3d_pair(sB, &tmB, &full_bar[stage], 0, row0 + done, nt * 4 + rank * 2);
             }
             __syncwarp();
-            if (++stage == kPairStages) { stage = 0; phase ^= 1u; }
+            if (++stage == kStages) { stage = 0; phase ^= 1u; }
           }
           ok = __all_sync(0xffffffffu, ok);
         }
@@ -814,7 +820,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           }
           for (int l = 0; l < min(32, p.n_layers - l0) && ok; ++l) {
             const int n = __shfl_sync(0xffffffffu, count, l);
-            for (int done = 0; done < n; done += BK) {
+            for (int done = 0; done < n; done += KR) {
               if (!tc::mbar_wait(&full_bar[stage], phase, abort)) {
                 if (lane == 0) report_timeout(p, abort, 23);
                 ok = false;
@@ -822,12 +828,12 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
               }
               tc::tc_fence_after_sync();
               if (lane == 0) {
-                const uint32_t aaddr = tc::smem_u32(smem + stage * kPairStageBytes);
-                const uint64_t adesc = tc::smem_desc_sw128(aaddr, kMnBlockBytes, 1024);
-                const uint64_t bdesc = tc::smem_desc_sw128(aaddr + kPairHalfBytes, kMnBlockBytes, 1024);
-                if (n - done > 48) {
+                const uint32_t aaddr = tc::smem_u32(smem + stage * kStage);
+                const uint64_t adesc = tc::smem_desc_sw128(aaddr, kBlock, 1024);
+                const uint64_t bdesc = tc::smem_desc_sw128(aaddr + kHalf, kBlock, 1024);
+                if (n - done > KR - 16) {
 #pragma unroll
-                  for (int j = 0; j < BK / 16; ++j)
+                  for (int j = 0; j < KR / 16; ++j)
                     tc::umma_bf16_pair(d_tmem, adesc + j * kstep, bdesc + j * kstep, idesc, j > 0 ? 1u : accumulate);
                 } else {                                        // only zeros behind row n
                   for (int j = 0; 16 * j < n - done; ++j)
@@ -837,7 +843,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
               }
               accumulate = 1;
               __syncwarp();
-              if (++stage == kPairStages) { stage = 0; phase ^= 1u; }
+              if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
             ok = __all_sync(0xffffffffu, ok);
           }
@@ -970,12 +976,12 @@ int map_2d(const unipool_ctx* ctx, CUtensorMap* out, const void* base, uint64_t 
 }
 
 // MMA operand read along the contiguous dimension of a row-major matrix [k_rows, n_cols] ("MN-major"):
-// the matrix seen as [n_cols / 64][k_rows][64], a box = `blocks` column blocks x 64 k-rows, laid out
-// block after block (8 KiB each) - one copy instead of one per block.
+// the matrix seen as [n_cols / 64][k_rows][64], a box = `blocks` column blocks x k_box k-rows, laid out
+// block after block (128 k_box bytes each) - one copy instead of one per block.
 int map_mn(const unipool_ctx* ctx, CUtensorMap* out, const void* base, uint64_t n_cols, uint64_t k_rows,
-           uint32_t blocks) {
+           uint32_t blocks, uint32_t k_box) {
   const uint64_t dims[3] = {64, k_rows, n_cols / 64}, strides[2] = {n_cols, 64};
-  const uint32_t box[3] = {64, 64, blocks};
+  const uint32_t box[3] = {64, k_box, blocks};
   return make_tmap(ctx, out, kMapOperand, base, 3, dims, strides, box);
 }
 
@@ -1388,7 +1394,8 @@ bool rows_on_pairs(const unipool_ctx* ctx, int n_experts) {
 //   dgrad down        91/93    110/104   138/120   201/193    262/246     *1073/971   1013/952    164/164
 //   dgrad gate/up    117/124   132/132   154/142   240/212    308/308     *1494/1474  1413/1392   185/191
 // Below ~128 rows every launch is bound by streaming the weights and the token-major kernels keep more bytes in
-// flight; large groups waste nothing in 256-row pair-tiles.  Down and dgrad gate/up gain while a group is one or
+// flight (dgrad down alone gains again up to 48 rows, where it saves reading G and U of the padding: 4 rows 86/78,
+// 31 rows 89/83, 48 rows 90/86, of 1536 x 4096 31 rows 176/167); large groups waste nothing in 256-row pair-tiles.  Down and dgrad gate/up gain while a group is one or
 // two chunks (and need a contraction long enough to hide the epilogue of a wide unit: 384 experts of 768 x 512 lost
 // 10 % on the down projection, 4 % on dgrad gate/up); dgrad down gains longest, its G and U traffic being the
 // same on fewer padded rows; gate/up gains beyond 450 rows only where its contraction is long.
@@ -1399,7 +1406,7 @@ bool weights_on_m(const unipool_ctx* ctx, int mode, int n_experts) {
   switch (mode) {
     case kFwd1: return rows > 150 && rows <= (d >= 1024 ? 1024 : 450);
     case kFwd2: return rows > 150 && rows <= 450 && f > 1024;
-    case kDgrad1: return rows > 100 && rows <= 1200;
+    case kDgrad1: return rows <= 48 || (rows > 100 && rows <= 1200);
     default: return rows > 150 && rows <= 450 && 2 * f > 1024;
   }
 }
@@ -1427,11 +1434,12 @@ int launch_rows(unipool_ctx* ctx, int phase, bool pairs, const CUtensorMap& tmA,
 
 // The pool weight gradient runs on CTA pairs.
 int launch_wgrad(unipool_ctx* ctx, int phase, const CUtensorMap& tmP, const CUtensorMap& tmQ, const CUtensorMap& tmW,
-                 const GemmParams& p, cudaStream_t s) {
+                 const GemmParams& p, int k_rows, cudaStream_t s) {
   UP_REQUIRE(ctx->sm_count >= 2, UNIPOOL_ERR_UNSUPPORTED, "the weight gradient needs a device with CTA pairs");
   PhaseTimer pt(ctx, phase, 1, s);
-  UP_CUDA(cudaFuncSetAttribute(wgrad_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemTotal));
-  wgrad_pair_kernel<<<ctx->sm_count / 2 * 2, kThreads, kPairSmemTotal, s>>>(tmP, tmQ, tmW, p);
+  auto kern = k_rows == 32 ? wgrad_pair_kernel<32> : k_rows == 48 ? wgrad_pair_kernel<48> : wgrad_pair_kernel<64>;
+  UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemTotal));
+  kern<<<ctx->sm_count / 2 * 2, kThreads, kPairSmemTotal, s>>>(tmP, tmQ, tmW, p);
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;
 }
@@ -1448,22 +1456,27 @@ int wgrad_pair(unipool_ctx* ctx, const PoolWgradArgs& a, cudaStream_t s) {
   p.layer_stride_rows = (int)a.layer_stride_rows;
   p.overwrite = a.overwrite ? 1 : 0;
   p.status = ctx->ws.status;
+  // Rows per k-block by the rows the average expert gets in one layer of a full batch.  Both products of 12 layers,
+  // 96 experts of 768 x 2048, k-blocks of 64 / 48 / 32 rows in us: 16 rows 614 / 563 / 480, 26 rows 646 / 616 / 552,
+  // 31 rows 650 / 604 / 633, 41 rows 668 / 644 / 790, 48 rows 678 / 734 / 828; 341 rows 3121 / - / 4248.
+  const int64_t rows_per_expert = (int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k / a.n_experts;
+  const int k_rows = a.rows == nullptr || rows_per_expert > 40 ? 64 : rows_per_expert > 28 ? 48 : 32;
   CUtensorMap tmP, tmQ, tmW;
   int rc;
   if (a.dW_down != nullptr) {                     // dW_down[e] [d, f] (+)= dYp_e^T A_e
-    if ((rc = map_mn(ctx, &tmP, a.dYp, d, rows, 2)) != UNIPOOL_OK) return rc;
-    if ((rc = map_mn(ctx, &tmQ, a.A, f, rows, 2)) != UNIPOOL_OK) return rc;
+    if ((rc = map_mn(ctx, &tmP, a.dYp, d, rows, 2, k_rows)) != UNIPOOL_OK) return rc;
+    if ((rc = map_mn(ctx, &tmQ, a.A, f, rows, 2, k_rows)) != UNIPOOL_OK) return rc;
     if ((rc = map_chunk(ctx, &tmW, a.dW_down, f, (uint64_t)M * d, kMapF32Chunk)) != UNIPOOL_OK) return rc;
     p.Mdim = d; p.Ndim = f;
-    if ((rc = launch_wgrad(ctx, UNIPOOL_PH_WGRAD_DOWN, tmP, tmQ, tmW, p, s)) != UNIPOOL_OK) return rc;
+    if ((rc = launch_wgrad(ctx, UNIPOOL_PH_WGRAD_DOWN, tmP, tmQ, tmW, p, k_rows, s)) != UNIPOOL_OK) return rc;
   }
   if (a.dW_gu == nullptr) return UNIPOOL_OK;
   // dW_gu[e] [2f, d] (+)= dGU_e^T Xp_e
-  if ((rc = map_mn(ctx, &tmP, a.dGU, 2 * f, rows, 2)) != UNIPOOL_OK) return rc;
-  if ((rc = map_mn(ctx, &tmQ, a.Xp, d, rows, 2)) != UNIPOOL_OK) return rc;
+  if ((rc = map_mn(ctx, &tmP, a.dGU, 2 * f, rows, 2, k_rows)) != UNIPOOL_OK) return rc;
+  if ((rc = map_mn(ctx, &tmQ, a.Xp, d, rows, 2, k_rows)) != UNIPOOL_OK) return rc;
   if ((rc = map_chunk(ctx, &tmW, a.dW_gu, d, (uint64_t)M * 2 * f, kMapF32Chunk)) != UNIPOOL_OK) return rc;
   p.Mdim = 2 * f; p.Ndim = d;
-  return launch_wgrad(ctx, UNIPOOL_PH_WGRAD_GU, tmP, tmQ, tmW, p, s);
+  return launch_wgrad(ctx, UNIPOOL_PH_WGRAD_GU, tmP, tmQ, tmW, p, k_rows, s);
 }
 
 }  // namespace

@@ -23,6 +23,6 @@ int make_tmap(const unipool_ctx* ctx, CUtensorMap* out, MapKind kind, const void
 int map_2d(const unipool_ctx* ctx, CUtensorMap* out, const void* base, uint64_t cols, uint64_t rows,
            uint32_t box_cols, uint32_t box_rows, MapKind kind = kMapOperand);
 int map_mn(const unipool_ctx* ctx, CUtensorMap* out, const void* base, uint64_t n_cols, uint64_t k_rows,
-           uint32_t blocks);
+           uint32_t blocks, uint32_t k_box = 64);
 
 }  // namespace unipool

@@ -86,6 +86,7 @@ def test_dispatch_maps_at_the_edges_of_its_chunking(T, k, M, static):
     ([768, 769, 1000, 1, 1152, 1153, 900], 1024, 64),            # gate/up beyond 450 rows, one k-block of K = 64
     ([200] * 40 + [0, 97, 1300], 64, 1216),
     ([110, 120, 130, 140], 256, 320),                            # dgrad down only
+    ([48, 1, 0, 33, 64, 65, 17], 128, 576),                      # dgrad down only, few rows
 ])
 @pytest.mark.parametrize("with_rows", [True, False])
 def test_expert_ffn_at_the_edges_of_its_units(sizes, d, f, with_rows):
@@ -149,6 +150,8 @@ def test_expert_ffn_at_the_edges_of_its_units(sizes, d, f, with_rows):
     [[0, 0, 0, 0], [0, 0, 0, 0]],
     [[1, 15, 16, 17], [63, 64, 65, 0], [0, 127, 128, 129], [33, 0, 48, 1000]],
     [[5, 0, 7, 200]],
+    [[1, 31, 32, 33], [0, 47, 48, 10]],                # 26 rows per expert: k-blocks of 32
+    [[33, 47, 48, 17], [49, 1, 95, 0], [0, 0, 0, 7]],  # 36: k-blocks of 48
 ])
 def test_weight_gradient_leaves_the_padding_out(sizes, overwrite):
     """With the group sizes the contraction stops at the last 16 rows that hold a token; what is left out are zeros,
