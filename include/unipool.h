@@ -304,6 +304,45 @@ int unipool_route_bwd(unipool_ctx* ctx, const void* x, int32_t T, const float* W
                       const int32_t* idx, const float* dgate, const float* dscore_coef,
                       void* dx, float* dW_r, float* dsigma, unipool_stream stream);
 
+/* A whole residual stack x_{l+1} = x_l + MoE_l(x_l) per call: the calls above for every layer, in order, with
+ * the same results.  All arrays are the caller's and stacked over the layers ([n_layers, ...], leading
+ * dimensions as documented above with max_tokens of the context for T).  The struct is read during the call
+ * only.  Layers l with the same l / layers_per_group share the pool experts
+ * [l / layers_per_group * n_experts, + n_experts) and one balance loss. */
+typedef struct {
+  int32_t n_layers, layers_per_group, n_experts;
+  int32_t recompute;      /* 0: Xp, GU, A, Yp hold every layer; 1: one slot (Xp, A: wgrad_layers slots), rebuilt */
+                          /* in backward from x and the routing                                             */
+  int32_t wgrad_layers;   /* layers whose weight gradients are contracted together: 1 = each on its own       */
+                          /* (dYp, dGU: one slot); with recompute runs of so many layers of a group (so many  */
+                          /* slots); else any larger value = all layers of a group (dYp, dGU: every layer)    */
+  const void *W_gu, *W_down;                 /* the pool                                                     */
+  const float *W_r, *sigma, *bias;           /* [L,n_experts,d]; HOST [L]; [L,n_experts] or NULL             */
+  void* x;                                   /* [L+1,T,d]; x[0] is the input                                 */
+  int32_t* idx; float* gate; int32_t* counts; float *score_sum, *znorm, *z;            /* unipool_route       */
+  int32_t *offsets, *rows, *row_of, *token_of, *tile_expert;                           /* unipool_dispatch_rows */
+  void *Xp, *GU, *A, *Yp;
+  float *loss, *coef, *fbar;                 /* per group: [1], [n_experts], [n_experts]                      */
+  void *dYp, *dGU, *dx;                      /* dx [2,T,d]: dx[0] holds the upstream gradient on entry of     */
+                                             /* backward, dx[n_layers % 2] the gradient of x[0] on return     */
+  float *dgate, *dW_gu, *dW_down, *dW_r, *dsigma;
+} unipool_stack;
+
+#define UNIPOOL_STACK_NO_AUX       4   /* unipool_stack_backward without the balance loss's gradient      */
+#define UNIPOOL_STACK_LEAVE_WGRAD  8   /* stacked weight-gradient operands: leave unipool_pool_wgrad_rows */
+                                       /* to the caller                                                   */
+
+/* unipool_router_prepare, then route, dispatch, expert_fwd and combine of every layer. */
+int unipool_stack_forward(unipool_ctx* ctx, const unipool_stack* stack, int32_t T, unipool_stream stream);
+/* unipool_pool_aux_loss of every group; fbar_prev [groups,n_experts] or NULL; T may count several replicas. */
+int unipool_stack_aux_loss(unipool_ctx* ctx, const unipool_stack* stack, int32_t T, float alpha,
+                           const float* fbar_prev, unipool_stream stream);
+/* expert_bwd and route_bwd of every layer from the last to the first, and the weight gradients.  flags:
+ * UNIPOOL_WGRAD_OVERWRITE (the pass's pool gradient replaces what the buffers hold; router gradients always
+ * add), UNIPOOL_STACK_NO_AUX, UNIPOOL_STACK_LEAVE_WGRAD. */
+int unipool_stack_backward(unipool_ctx* ctx, const unipool_stack* stack, int32_t T, int32_t flags,
+                           unipool_stream stream);
+
 /* Distinct-expert accounting (App. E): U(x) = |{ e_l(x) : l = 1..L }|, the number of different pool
  * experts a token selects over all layers (the paper states it for top-1; with top-k every selected
  * expert of every layer counts).  With the shared pool 1 <= U <= min(M, L k); with private experts

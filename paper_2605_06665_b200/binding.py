@@ -18,6 +18,8 @@ ROUTER_NORM, ROUTER_SOFTMAX = 0, 1
 ROW_ALIGN = 128
 BWD_SKIP_WGRAD = 1
 WGRAD_OVERWRITE = 2
+STACK_NO_AUX = 4
+STACK_LEAVE_WGRAD = 8
 
 EXPORTS = (
     "unipool_row_capacity", "unipool_workspace_bytes", "unipool_create", "unipool_destroy",
@@ -26,6 +28,7 @@ EXPORTS = (
     "unipool_pool_aux_loss", "unipool_route_bwd", "unipool_calibrate_c",
     "unipool_profile_enable", "unipool_profile_read", "unipool_dispatch_static",
     "unipool_unique_experts", "unipool_router_prepare", "unipool_selftest_wait",
+    "unipool_stack_forward", "unipool_stack_aux_loss", "unipool_stack_backward",
     "unipool_dispatch_rows", "unipool_expert_fwd_rows", "unipool_expert_bwd_rows", "unipool_pool_wgrad_rows",
 )
 
@@ -43,6 +46,15 @@ class Config(ctypes.Structure):
         ("dtype", ctypes.c_int32), ("eps", ctypes.c_float), ("c", ctypes.c_float),
         ("router_mode", ctypes.c_int32),
     ]
+
+
+class Stack(ctypes.Structure):
+    """unipool_stack: the arrays of a whole residual stack."""
+    POINTERS = ("W_gu", "W_down", "W_r", "sigma", "bias", "x", "idx", "gate", "counts", "score_sum", "znorm", "z",
+                "offsets", "rows", "row_of", "token_of", "tile_expert", "Xp", "GU", "A", "Yp", "loss", "coef", "fbar",
+                "dYp", "dGU", "dx", "dgate", "dW_gu", "dW_down", "dW_r", "dsigma")
+    _fields_ = ([(n, ctypes.c_int32) for n in ("n_layers", "layers_per_group", "n_experts", "recompute", "wgrad_layers")]
+                + [(n, ctypes.c_void_p) for n in POINTERS])
 
 
 class UniPoolError(RuntimeError):
@@ -108,6 +120,13 @@ def lib():
     L.unipool_pool_aux_loss.argtypes = [vp, vp, vp, i32, i32, i32, f32, vp, vp, vp, vp, vp]
     L.unipool_route_bwd.restype = ctypes.c_int
     L.unipool_route_bwd.argtypes = [vp, vp, i32, vp, f32, i32, vp, vp, vp, vp, vp, vp, vp, vp, vp]
+    stackp = ctypes.POINTER(Stack)
+    L.unipool_stack_forward.restype = ctypes.c_int
+    L.unipool_stack_forward.argtypes = [vp, stackp, i32, vp]
+    L.unipool_stack_aux_loss.restype = ctypes.c_int
+    L.unipool_stack_aux_loss.argtypes = [vp, stackp, i32, f32, vp, vp]
+    L.unipool_stack_backward.restype = ctypes.c_int
+    L.unipool_stack_backward.argtypes = [vp, stackp, i32, i32, vp]
     L.unipool_unique_experts.restype = ctypes.c_int
     L.unipool_unique_experts.argtypes = [vp, vp, vp, i32, i32, vp, vp, vp]
     L.unipool_calibrate_c.restype = ctypes.c_int
@@ -235,6 +254,15 @@ class Context:
         _check(lib().unipool_route_bwd(self.handle, _p(x), T, _p(W_r), sigma, n_experts, _p(znorm),
                                        _p(z_saved), _p(idx), _p(dgate), _p(dscore_coef), _p(dx), _p(dW_r),
                                        _p(dsigma), _stream()))
+
+    def stack_forward(self, stack, T):
+        _check(lib().unipool_stack_forward(self.handle, ctypes.byref(stack), T, _stream()))
+
+    def stack_aux_loss(self, stack, T, alpha, fbar_prev=None):
+        _check(lib().unipool_stack_aux_loss(self.handle, ctypes.byref(stack), T, alpha, _p(fbar_prev), _stream()))
+
+    def stack_backward(self, stack, T, flags=0):
+        _check(lib().unipool_stack_backward(self.handle, ctypes.byref(stack), T, flags, _stream()))
 
     def unique_experts(self, idx, expert_base, L, T, unique, total):
         _check(lib().unipool_unique_experts(self.handle, _p(idx), _p(expert_base), L, T, _p(unique), _p(total),

@@ -3,6 +3,8 @@
 ``UniPoolStack`` owns the device buffers (PyTorch tensors) and issues, per layer,
 the library calls route -> dispatch -> expert_fwd -> combine (forward), then
 pool_aux_loss, then expert_bwd -> route_bwd per layer in reverse (backward).
+(``forward``, ``aux_loss`` and ``backward`` issue these calls for all layers from one native call
+each, ``forward_layer`` and ``backward_layer`` one layer's from Python.)
 It contains no arithmetic of its own: every tensor it returns was written by a
 CUDA kernel of the library.
 
@@ -18,6 +20,8 @@ replaces the NormRouter of Eq. 7 by the conventional softmax router of the paper
 baselines (Sec. 5.1) in every layer.
 """
 from __future__ import annotations
+
+import ctypes
 
 import numpy as np
 import torch
@@ -140,6 +144,19 @@ class UniPoolStack:
     def zero_router_grad(self):
         self.dW_r.zero_(); self.dsigma.zero_()
 
+    def _arrays(self):
+        """This stack's arrays as they are now, for the calls that run all layers."""
+        wgrad = self.Lg if self.deferred_wgrad else self.nw
+        sigma = (ctypes.c_float * self.L)(*self.sigma)
+        s = B.Stack(self.L, self.Lg, self.m, int(self.recompute), wgrad)
+        for n in B.Stack.POINTERS:
+            if n != "sigma":
+                t = getattr(self, n)
+                setattr(s, n, None if t is None else t.data_ptr())
+        s.sigma = ctypes.addressof(sigma)
+        s.keep = sigma                                     # lives as long as the struct
+        return s
+
     # ------------------------------------------------------------------ forward
     def forward_layer(self, l, T=None):
         T = self.T if T is None else T
@@ -150,57 +167,45 @@ class UniPoolStack:
         self.permute_and_experts(l, T)
         c.combine(self.Yp[self.slot(l)], self.row_of[l], self.gate[l], T, self.x[l], self.x[l + 1])
 
-    def permute_and_experts(self, l, T, w=None):
+    def permute_and_experts(self, l, T):
         """dispatch + expert forward of layer l from x_l and its routing decision (also the
-        recompute step of backward, which keeps Xp and A in slot ``w``)."""
+        recompute step of backward)."""
         c, s = self.ctx, self.slot(l)
-        w = s if w is None else w
         c.dispatch(self.x[l], T, self.idx[l], self.m, self.offsets[l], self.row_of[l], self.token_of[l],
-                   self.tile_expert[l], self.Xp[w], self.rows[l])
-        c.expert_fwd(self.Xp[w], self.offsets[l], self.tile_expert[l], self.W_gu, self.W_down,
-                     self.base(l), self.m, self.GU[s], self.A[w], self.Yp[s], self.rows[l])
+                   self.tile_expert[l], self.Xp[s], self.rows[l])
+        c.expert_fwd(self.Xp[s], self.offsets[l], self.tile_expert[l], self.W_gu, self.W_down,
+                     self.base(l), self.m, self.GU[s], self.A[s], self.Yp[s], self.rows[l])
 
     def forward(self, x0=None, T=None):
         T = self.T if T is None else T
         if x0 is not None:
             self.x[0, :T].copy_(x0, non_blocking=True)
-        # the routers' weights may have changed since the last pass: one kernel re-forms the bf16 terms
-        # of all layers (used by this forward pass and by the backward pass that follows it)
-        self.ctx.router_prepare(self.W_r, self.L, self.m)
-        for l in range(self.L):
-            self.forward_layer(l, T)
+        # (the routers' weights may have changed since the last pass: their bf16 terms are formed anew, used by
+        # this forward pass and by the backward pass that follows it)
+        self.ctx.stack_forward(self._arrays(), T)
         return self.x[self.L]
 
     def aux_loss(self, T=None, fbar_prev=None, replicas=1):
         """``replicas``: the statistics were summed over this many data-parallel replicas of T tokens."""
         T = (self.T if T is None else T) * replicas
-        c = self.ctx
-        if fbar_prev is not None and fbar_prev.dim() == 1:
-            fbar_prev = fbar_prev.reshape(1, -1)
-        for g in range(self.G):
-            l0 = g * self.Lg
-            c.pool_aux_loss(self.counts[l0:l0 + self.Lg], self.score_sum[l0:l0 + self.Lg], self.Lg, self.m, T,
-                            self.alpha, None if fbar_prev is None else fbar_prev[g],
-                            self.loss[g:g + 1], self.coef[g], self.fbar[g])
+        if fbar_prev is not None:
+            fbar_prev = fbar_prev.contiguous()             # [groups, m]
+        self.ctx.stack_aux_loss(self._arrays(), T, self.alpha, fbar_prev)
         return self.loss
 
     # ------------------------------------------------------------------ backward
-    def backward_layer(self, l, dx_next, dx_out, T=None, with_aux=True, overwrite=False, hold=None):
+    def backward_layer(self, l, dx_next, dx_out, T=None, with_aux=True, overwrite=False):
         """``overwrite``: this layer's weight gradient replaces what the pool-gradient
-        slices of its view hold (the first contribution of a step) instead of adding to it.
-        ``hold`` (recompute): the operands of the weight gradient stay in this slot for a
-        contraction of several layers by the caller."""
+        slices of its view hold (the first contribution of a step) instead of adding to it."""
         T = self.T if T is None else T
         c = self.ctx
+        s = l if self.deferred_wgrad else 0
         a = self.slot(l)
-        w = a if hold is None else hold                    # Xp, A
-        s = l if self.deferred_wgrad else hold or 0        # dYp, dGU
         if self.recompute:
-            self.permute_and_experts(l, T, w)
-        later = self.deferred_wgrad or hold is not None
-        flags = B.BWD_SKIP_WGRAD if later else (B.WGRAD_OVERWRITE if overwrite else 0)
+            self.permute_and_experts(l, T)
+        flags = B.BWD_SKIP_WGRAD if self.deferred_wgrad else (B.WGRAD_OVERWRITE if overwrite else 0)
         c.expert_bwd(dx_next, T, self.row_of[l], self.gate[l], self.token_of[l], self.offsets[l],
-                     self.tile_expert[l], self.Xp[w], self.GU[a], self.A[w], self.Yp[a], self.W_gu,
+                     self.tile_expert[l], self.Xp[a], self.GU[a], self.A[a], self.Yp[a], self.W_gu,
                      self.W_down, self.base(l), self.m, dx_next, self.dYp[s], self.dGU[s], dx_out,
                      self.dgate, self.dW_gu, self.dW_down, flags, self.rows[l])
         coef = None
@@ -216,40 +221,29 @@ class UniPoolStack:
         ``dp.GradientExchange``): the gradients are summed over the data-parallel replicas, each
         buffer as soon as it is complete (dW_down while dW_gu is still being computed)."""
         T = self.T if T is None else T
-        cur = 0
         if upstream is not None:
-            self.dx[cur, :T].copy_(upstream, non_blocking=True)
-        for l in reversed(range(self.L)):
-            i = l % self.Lg                                             # layer inside its sharing group
-            hold = i % self.nw if self.nw > 1 else None
-            # first contribution to its group's experts: the top layer, or the run of layers it belongs to
-            first = (not accumulate) and i >= (self.Lg - 1) // self.nw * self.nw
-            self.backward_layer(l, self.dx[cur], self.dx[1 - cur], T, with_aux, overwrite=first, hold=hold)
-            if hold == 0:                                               # the lowest layer of a run
-                self.ctx.pool_wgrad(min(self.nw, self.Lg - i), self.cap, self.offsets[l:], self.Xp, self.A, self.dYp,
-                                    self.dGU, self.base(l), self.m, self.dW_gu, self.dW_down,
-                                    B.WGRAD_OVERWRITE if first else 0, self.rows[l:])
-            cur = 1 - cur
-        if self.deferred_wgrad:
+            self.dx[0, :T].copy_(upstream, non_blocking=True)
+        flags = (0 if accumulate else B.WGRAD_OVERWRITE) | (0 if with_aux else B.STACK_NO_AUX)
+        if exchange is not None:
+            flags |= B.STACK_LEAVE_WGRAD
+        self.ctx.stack_backward(self._arrays(), T, flags)
+        if self.deferred_wgrad and exchange is not None:
             for g in range(self.G):                        # one pass per sharing group over its layers
                 l0 = g * self.Lg
                 flags = 0 if accumulate else B.WGRAD_OVERWRITE
                 args = (self.Lg, self.cap, self.offsets[l0:], self.Xp[l0:], self.A[l0:], self.dYp[l0:],
                         self.dGU[l0:], g * self.m, self.m)
-                if exchange is None:
-                    self.ctx.pool_wgrad(*args, self.dW_gu, self.dW_down, flags, self.rows[l0:])
-                else:
-                    e0, e1 = g * self.m, (g + 1) * self.m
-                    self.ctx.pool_wgrad(*args, None, self.dW_down, flags, self.rows[l0:])
-                    exchange.launch([self.dW_down[e0:e1]])
-                    self.ctx.pool_wgrad(*args, self.dW_gu, None, flags, self.rows[l0:])
-                    exchange.launch([self.dW_gu[e0:e1]])
+                e0, e1 = g * self.m, (g + 1) * self.m
+                self.ctx.pool_wgrad(*args, None, self.dW_down, flags, self.rows[l0:])
+                exchange.launch([self.dW_down[e0:e1]])
+                self.ctx.pool_wgrad(*args, self.dW_gu, None, flags, self.rows[l0:])
+                exchange.launch([self.dW_gu[e0:e1]])
         if exchange is not None:
             if not self.deferred_wgrad:
                 exchange.launch([self.dW_down, self.dW_gu])
             exchange.launch([self.dW_r, self.dsigma])
             exchange.finish()
-        return self.dx[cur]
+        return self.dx[self.L % 2]
 
     def step(self, x0=None, upstream=None, T=None, accumulate=True, exchange=None, out=None):
         """One pass of the whole hot path: forward, balance loss, backward.  With ``exchange`` the
