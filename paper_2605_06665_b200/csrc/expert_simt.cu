@@ -7,8 +7,6 @@ namespace unipool {
 
 namespace {
 
-constexpr int kRowTile = 64;     // rows of a tile; groups start at multiples of UNIPOOL_ROW_ALIGN = 128
-
 struct RowGemm {
   const float* A; int64_t lda;                      // [rows, K]
   const float* B; int64_t b_expert, ldb;            // expert's weights: along K [N, K], across K [K, N]
@@ -26,16 +24,18 @@ enum RowEpilogue {
   kSwigluBwd,  // the tile is dA: dG = dA U silu'(G), dU = dA silu(G) -> C [rows, 2f], G and U from GU
 };
 
-// C = A B_e for every 64-row tile of the permuted row space; the tile's expert selects B.  Tiles at and beyond
+// C = A B_e for every TM-row tile of the permuted row space; the tile's expert selects B.  Tiles at and beyond
 // offsets[n_experts] are skipped (tile_expert < 0); tiles behind a group's last token hold zeros and get zeros.
-template <int TN, int KG, Major BM, RowEpilogue EPI>
-__global__ void __launch_bounds__(SimtTile<kRowTile, TN, KG>::kThreads)
+template <int TM, int KG, Major BM, RowEpilogue EPI>
+__global__ void __launch_bounds__(SimtTile<TM, KG>::kThreads)
 grouped_rows_gemm_kernel(const RowGemm p) {
-  using T = SimtTile<kRowTile, TN, KG>;
-  __shared__ typename T::Smem sm;
+  using T = SimtTile<TM, KG>;
+  constexpr int TN = kSimtN;
+  extern __shared__ float4 smem_raw[];
+  typename T::Smem& sm = *reinterpret_cast<typename T::Smem*>(smem_raw);
   const int n0 = blockIdx.x * (EPI == kSwiglu ? TN / 2 : TN);
   for (int rt = blockIdx.y; rt < p.n_row_tiles; rt += gridDim.y) {
-    const int m0 = rt * kRowTile;
+    const int m0 = rt * TM;
     const int e = p.tile_expert[m0 / UNIPOOL_ROW_ALIGN];
     if (e < 0) continue;                            // uniform over the block
     const bool empty = p.rows != nullptr && m0 - p.offsets[e] >= p.rows[e];
@@ -99,9 +99,9 @@ struct PoolGemm {
   float* dW; int Mdim, Ndim; bool overwrite, vec;
 };
 
-__global__ void __launch_bounds__(kSimtGroup)
+__global__ void __launch_bounds__(SimtTile<64, 2>::kThreads)
 grouped_k_gemm_kernel(const PoolGemm p) {
-  using T = SimtTile<64, 64, 1>;
+  using T = SimtTile<64, 2>;
   __shared__ typename T::Smem sm;
   const int m0 = blockIdx.x * 64, n0 = blockIdx.y * 64, e = blockIdx.z;
   auto rows_of = [&](int l) {
@@ -110,18 +110,18 @@ grouped_k_gemm_kernel(const PoolGemm p) {
   };
   int n_chunks = 0;
   for (int l = 0; l < p.n_layers; ++l) n_chunks += (rows_of(l) + kSimtKC - 1) / kSimtKC;
-  // the chunk being fetched: rows [row0, row0 + left) of its layer are still to come (chunks are asked for in order)
+  // the chunk being fetched: rows [row0, row0 + left) of its layer are still to come (a group asks for its chunks in order)
   int layer = -1, at = -1, left = 0;
   int64_t row0 = 0;
   auto seek = [&](int c) {
-    if (c == at) return;
-    at = c;
-    row0 += kSimtKC;
-    left -= kSimtKC;
-    while (left <= 0) {
-      ++layer;
-      left = rows_of(layer);
-      row0 = layer * p.layer_stride_rows + p.offsets[(int64_t)layer * (p.n_experts + 1) + e];
+    for (; at < c; ++at) {
+      row0 += kSimtKC;
+      left -= kSimtKC;
+      while (left <= 0) {
+        ++layer;
+        left = rows_of(layer);
+        row0 = layer * p.layer_stride_rows + p.offsets[(int64_t)layer * (p.n_experts + 1) + e];
+      }
     }
   };
   T t;
@@ -134,6 +134,7 @@ grouped_k_gemm_kernel(const PoolGemm p) {
       [&](int c, int i, int k) {
         return k < left ? ld4(p.Q + (row0 + k) * p.ldq + n0 + i, p.vec) : make_float4(0.f, 0.f, 0.f, 0.f);
       });
+  if (threadIdx.x >= kSimtGroup) return;
   float* out = p.dW + (int64_t)(p.expert_base + e) * p.Mdim * p.Ndim;
 #pragma unroll
   for (int i = 0; i < T::MR; ++i)
@@ -148,23 +149,33 @@ grouped_k_gemm_kernel(const PoolGemm p) {
     }
 }
 
-template <Major BM, RowEpilogue EPI>
-int rows_gemm(unipool_ctx* ctx, RowGemm p, int n_experts, cudaStream_t s) {
-  p.vec = aligned16(p.A, p.B, p.C, p.C2, p.GU);
-  const int gy = p.n_row_tiles < 4096 ? p.n_row_tiles : 4096;
-  if constexpr (EPI != kSwiglu) {
-    // Tiles a full batch gives (a group ends on half a tile): below two blocks per SM narrower tiles, two groups of
-    // threads on each.
-    const int64_t tiles = ((int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k / kRowTile + n_experts / 2) * (p.N / 64);
-    if (tiles < 2 * ctx->sm_count) {
-      grouped_rows_gemm_kernel<32, 2, BM, EPI><<<dim3(p.N / 32, gy), 2 * kSimtGroup, 0, s>>>(p);
-      UP_LAUNCH_CHECK();
-      return UNIPOOL_OK;
-    }
-  }
-  grouped_rows_gemm_kernel<64, 1, BM, EPI><<<dim3(p.N / (EPI == kSwiglu ? 32 : 64), gy), kSimtGroup, 0, s>>>(p);
+template <int TM, int KG, Major BM, RowEpilogue EPI>
+int rows_gemm_as(const unipool_ctx* ctx, RowGemm p, cudaStream_t s) {
+  auto kern = grouped_rows_gemm_kernel<TM, KG, BM, EPI>;
+  constexpr int smem = (int)sizeof(typename SimtTile<TM, KG>::Smem);
+  if (smem > 48 * 1024) UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  p.n_row_tiles = (int)(ctx->row_capacity / TM);
+  const int gy = p.n_row_tiles < 8192 ? p.n_row_tiles : 8192;
+  kern<<<dim3(p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN), gy), SimtTile<TM, KG>::kThreads, smem, s>>>(p);
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;
+}
+
+template <Major BM, RowEpilogue EPI>
+int rows_gemm(unipool_ctx* ctx, RowGemm p, int n_experts, cudaStream_t s) {
+  p.vec = aligned16(p.A, p.B);
+  // 64 x 64 tiles of a full batch (a group ends on half a tile).  Many: whole tiles, one group of threads on each, two
+  // on a long contraction; fewer: two groups, and half tiles where the weights are read across K; few: half tiles,
+  // two or four groups.  In us, TM = 64 with 1 / 2 / 4 groups, 32 with 1 / 2 / 4 (16 experts of 256 x 512, 64 rows each):
+  // gate/up (384 tiles) 46/41/57, 45/41/44; down (96) 44/29/27, 35/30/27; dgrad down (192) 48/45/63, 39/36/42; dgrad
+  // gate/up (96) 82/48/40, 63/49/44; 24 experts of 384 x 768, 250 rows: 2544 tiles 208/210/345, 252/255/279; 636 tiles
+  // 137/119/167, 156/155/141; 1272 tiles 145/157/303, 153/154/201.
+  const int64_t tiles = ((int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k / 64 + n_experts / 2) *
+                        (p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN));
+  if (tiles >= 600)
+    return p.K >= 768 ? rows_gemm_as<64, 2, BM, EPI>(ctx, p, s) : rows_gemm_as<64, 1, BM, EPI>(ctx, p, s);
+  if (tiles >= 350 && BM == kAlongK) return rows_gemm_as<64, 2, BM, EPI>(ctx, p, s);
+  return p.K >= 512 ? rows_gemm_as<32, 4, BM, EPI>(ctx, p, s) : rows_gemm_as<32, 2, BM, EPI>(ctx, p, s);
 }
 
 template <typename Args>
@@ -176,7 +187,6 @@ RowGemm row_gemm(const unipool_ctx* ctx, const Args& a) {
   p.expert_base = a.expert_base;
   p.f = ctx->cfg.d_ff;
   p.b_expert = (int64_t)ctx->cfg.d_model * ctx->cfg.d_ff;
-  p.n_row_tiles = (int)(ctx->row_capacity / kRowTile);
   return p;
 }
 
@@ -213,7 +223,7 @@ int pool_wgrad_simt(unipool_ctx* ctx, const PoolWgradArgs& a, cudaStream_t s) {
     p.P = static_cast<const float*>(a.dYp); p.ldp = d;
     p.Q = static_cast<const float*>(a.A); p.ldq = f;
     p.dW = a.dW_down; p.Mdim = d; p.Ndim = f; p.vec = aligned16(p.P, p.Q, p.dW);
-    grouped_k_gemm_kernel<<<dim3(d / 64, f / 64, a.n_experts), kSimtGroup, 0, s>>>(p);
+    grouped_k_gemm_kernel<<<dim3(d / 64, f / 64, a.n_experts), SimtTile<64, 2>::kThreads, 0, s>>>(p);
     UP_LAUNCH_CHECK();
   }
   if (a.dW_gu == nullptr) return UNIPOOL_OK;
@@ -221,7 +231,7 @@ int pool_wgrad_simt(unipool_ctx* ctx, const PoolWgradArgs& a, cudaStream_t s) {
   p.P = static_cast<const float*>(a.dGU); p.ldp = 2 * f;
   p.Q = static_cast<const float*>(a.Xp); p.ldq = d;
   p.dW = a.dW_gu; p.Mdim = 2 * f; p.Ndim = d; p.vec = aligned16(p.P, p.Q, p.dW);
-  grouped_k_gemm_kernel<<<dim3(2 * f / 64, d / 64, a.n_experts), kSimtGroup, 0, s>>>(p);
+  grouped_k_gemm_kernel<<<dim3(2 * f / 64, d / 64, a.n_experts), SimtTile<64, 2>::kThreads, 0, s>>>(p);
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;
 }

@@ -7,14 +7,15 @@
 namespace unipool {
 
 // ---------------------------------------------------------------- logits  z = x W_r^T (+ bias)
-// Few tiles (one per 32 tokens and 32 experts), so four groups of threads share a tile's contraction.
-using RouterTile = SimtTile<32, 32, 4>;
+// Few tiles (one per 32 tokens and 64 experts), so four groups of threads share a tile's contraction.
+using RouterTile = SimtTile<32, 4>;
 
 __global__ void __launch_bounds__(RouterTile::kThreads)
 router_logits_kernel(const float* __restrict__ x, const float* __restrict__ W_r,
                      const float* __restrict__ bias, float* __restrict__ z, int T, int M, int d, bool vec) {
-  __shared__ RouterTile::Smem sm;
-  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+  extern __shared__ float4 smem_raw[];
+  RouterTile::Smem& sm = *reinterpret_cast<RouterTile::Smem*>(smem_raw);
+  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * kSimtN;
   RouterTile t;
   t.run<kAlongK, kAlongK>(
       sm, d / kSimtKC,
@@ -171,7 +172,8 @@ int route_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float
     return route_tc_launch(ctx, x, T, W_r, sigma, bias, M, idx, gate, counts, score_sum, znorm, z_saved, s);
   {
     PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_LOGITS, 1, s);
-    router_logits_kernel<<<dim3((T + 31) / 32, (M + 31) / 32), RouterTile::kThreads, 0, s>>>(
+    UP_CUDA(cudaFuncSetAttribute(router_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RouterTile::Smem)));
+    router_logits_kernel<<<dim3((T + 31) / 32, (M + 63) / 64), RouterTile::kThreads, sizeof(RouterTile::Smem), s>>>(
         static_cast<const float*>(x), W_r, bias, z_saved, T, M, d, aligned16(x, W_r));
     UP_LAUNCH_CHECK();
   }
@@ -259,13 +261,13 @@ router_dz_kernel(const float* __restrict__ z, const float* __restrict__ znorm,
 }
 
 // dx[t,:] += dz[t,:] W_r     (K = M)
-using RouterDxTile = SimtTile<32, 32, 1>;
+using RouterDxTile = SimtTile<32, 1>;
 
 __global__ void __launch_bounds__(RouterDxTile::kThreads)
 router_dx_kernel(const float* __restrict__ dz, const float* __restrict__ W_r, float* __restrict__ dx,
                  int T, int M, int d, bool vec) {
   __shared__ RouterDxTile::Smem sm;
-  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * kSimtN;
   const bool vec_z = (M & 3) == 0;                   // dz is a workspace array of rows of M
   RouterDxTile t;
   t.run<kAlongK, kAcrossK>(
@@ -282,8 +284,8 @@ router_dx_kernel(const float* __restrict__ dz, const float* __restrict__ W_r, fl
   for (int i = 0; i < RouterDxTile::MR; ++i) {
     const int tok = m0 + t.row(i);
     if (tok >= T) continue;
-    float* o = dx + (int64_t)tok * d + n0 + t.col(0);
-    st4(o, make_float4(o[0] + t.value(i, 0), o[1] + t.value(i, 1), o[2] + t.value(i, 2), o[3] + t.value(i, 3)), vec);
+#pragma unroll
+    for (int j = 0; j < RouterDxTile::NR; ++j) dx[(int64_t)tok * d + n0 + t.col(j)] += t.value(i, j);
   }
 }
 
@@ -292,8 +294,9 @@ router_dx_kernel(const float* __restrict__ dz, const float* __restrict__ W_r, fl
 __global__ void __launch_bounds__(RouterTile::kThreads)
 router_dw_kernel(const float* __restrict__ dz, const float* __restrict__ x, float* __restrict__ dW_r,
                  int T, int M, int d, int k_len, bool vec) {
-  __shared__ RouterTile::Smem sm;
-  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * 32;
+  extern __shared__ float4 smem_raw[];
+  RouterTile::Smem& sm = *reinterpret_cast<RouterTile::Smem*>(smem_raw);
+  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * kSimtN;
   const int k_begin = blockIdx.z * k_len, k_end = min(T, k_begin + k_len);
   const bool vec_z = (M & 3) == 0;
   RouterTile t;
@@ -339,13 +342,14 @@ int route_bwd_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, f
   }
   {
     PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_BWD_DX, 1, s);
-    router_dx_kernel<<<dim3((T + 31) / 32, d / 32), RouterDxTile::kThreads, 0, s>>>(
+    router_dx_kernel<<<dim3((T + 31) / 32, d / 64), RouterDxTile::kThreads, 0, s>>>(
         dz, W_r, static_cast<float*>(dx), T, M, d, aligned16(W_r, dx));
     UP_LAUNCH_CHECK();
   }
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_BWD_DW, 1, s);
   const int k_len = 1024;
-  router_dw_kernel<<<dim3((M + 31) / 32, d / 32, (T + k_len - 1) / k_len), RouterTile::kThreads, 0, s>>>(
+  UP_CUDA(cudaFuncSetAttribute(router_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RouterTile::Smem)));
+  router_dw_kernel<<<dim3((M + 31) / 32, d / 64, (T + k_len - 1) / k_len), RouterTile::kThreads, sizeof(RouterTile::Smem), s>>>(
       dz, static_cast<const float*>(x), dW_r, T, M, d, k_len, aligned16(x));
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;

@@ -1,15 +1,15 @@
 // CUDA-core tiled GEMM building block with fp32 accumulation, for the fp32 mode of the library (its 1e-5
 // parity bound rules out TF32).
 //
-// Bound by the FMA pipe (72 TFLOP/s at 1.9 GHz) where there are enough tiles, by latency below that.  A group of
-// 128 threads owns a TM x TN tile, (TM / 16) x (TN / 8) results per thread, multiplied with packed
-// fma.rn.f32x2 (each half an IEEE fp32 fma: half the instructions for the same sums); chunks of 16 of the
-// contraction go through double-buffered shared memory, fetched into registers one chunk ahead with 16-byte
-// loads.  KG such groups in a block share a tile by taking every KG-th chunk and add up at the end: a long
-// contraction over few tiles then still fills the chip.
-// Sixteen 64-token experts of 256 x 512, against one 4 x 4 result tile per thread fed by scalar loads and separate
-// SwiGLU kernels: gate/up 69 -> 48 us, down 37 -> 32, dgrad down 39 -> 33, dgrad gate/up 72 -> 53, weight gradients of
-// four layers 350 -> 124; router logits of 512 tokens 29 -> 11, router weight gradient 55 -> 15.
+// Bound by the FMA pipe (72 TFLOP/s at 1.9 GHz) and the register side of shared memory where there are many tiles
+// (40 TFLOP/s in the weight gradient of 24 experts of 384 x 768), by latency and synchronisation below that.  A group
+// of 64 threads owns a TM x 64 tile, TM / 8 x 8 results per thread, multiplied with packed fma.rn.f32x2 (each half an
+// IEEE fp32 fma: half the instructions for the same sums); chunks of 16 of the contraction go through
+// double-buffered shared memory, fetched into registers one chunk ahead with 16-byte loads, and the operands of
+// step k + 1 are read while step k is multiplied.  KG such groups in a block share a tile by taking every KG-th
+// chunk and add up at the end: a long contraction over few tiles then still fills the chip.  (Both operands along K
+// in shared memory, pairs along K, saves the duplication of a: no faster, and slower by a third where a weight is
+// read across K.)
 #pragma once
 
 #include "common.cuh"
@@ -17,7 +17,8 @@
 namespace unipool {
 
 constexpr int kSimtKC = 16;        // k-chunk staged in shared memory
-constexpr int kSimtGroup = 128;    // threads of a k-group: 16 x 8
+constexpr int kSimtGroup = 64;     // threads of a k-group: 8 x 8
+constexpr int kSimtN = 64;         // columns of a tile
 
 // How an operand lies in memory: kAlongK element (i, k) = p[i * ld + k], kAcrossK element (i, k) = p[k * ld + i].
 enum Major { kAlongK, kAcrossK };
@@ -37,11 +38,11 @@ __device__ __forceinline__ float4 ld4(const float* p, bool vec, int n) {
 }
 template <typename... P> inline bool aligned16(P... p) { return ((... | reinterpret_cast<uintptr_t>(p)) & 15) == 0; }
 
-template <int TM, int TN, int KG>
+template <int TM, int KG>
 struct SimtTile {
-  static constexpr int MR = TM / 16, NR = TN / 8, kThreads = KG * kSimtGroup;
+  static constexpr int TN = kSimtN, MR = TM / 8, NR = 8, kThreads = KG * kSimtGroup;
   static constexpr int kA4 = TM * kSimtKC / 4 / kSimtGroup, kB4 = TN * kSimtKC / 4 / kSimtGroup;   // float4 per thread
-  static_assert((MR == 4 || MR == 2) && (NR == 8 || NR == 4), "result tile of a thread");
+  static_assert(MR == 8 || MR == 4, "result tile of a thread");
   struct Smem {
     float a[KG][2][kSimtKC][TM + 4];
     float b[KG][2][kSimtKC][TN + 4];
@@ -51,7 +52,7 @@ struct SimtTile {
   // results of this thread: row(i), column(j) inside the tile
   __device__ static int ty() { return (threadIdx.x % kSimtGroup) / 8; }
   __device__ static int tx() { return threadIdx.x % 8; }
-  __device__ static int row(int i) { return ty() * MR + i; }
+  __device__ static int row(int i) { return i < 4 ? ty() * 4 + i : TM / 2 + ty() * 4 + i - 4; }
   __device__ static int col(int j) { return j < 4 ? tx() * 4 + j : TN / 2 + tx() * 4 + j - 4; }
   __device__ float value(int i, int j) const {
     const unsigned long long v = acc[i][j / 2];
@@ -79,6 +80,19 @@ struct SimtTile {
       } else {
         *reinterpret_cast<float4*>(&s[p / (T / 4)][p % (T / 4) * 4]) = r[q];
       }
+    }
+  }
+  struct Frag { float a[MR]; unsigned long long b[NR / 2]; };
+  __device__ static void read(Frag& f, const float (*sa)[TM + 4], const float (*sb)[TN + 4], int k) {
+#pragma unroll
+    for (int h = 0; h < MR / 4; ++h) {
+      const float4 v = *reinterpret_cast<const float4*>(&sa[k][h * (TM / 2) + ty() * 4]);
+      f.a[4 * h] = v.x; f.a[4 * h + 1] = v.y; f.a[4 * h + 2] = v.z; f.a[4 * h + 3] = v.w;
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&sb[k][h * (TN / 2) + tx() * 4]);
+      f.b[2 * h] = v.x; f.b[2 * h + 1] = v.y;
     }
   }
 
@@ -114,28 +128,18 @@ struct SimtTile {
       stash<BM, TN>(sb, rb);
       __syncthreads();                             // also: everyone is done with the buffer the next chunk goes to
       if (it + 1 < n_it) load(it + 1);
+      Frag f[2];
+      read(f[0], sa, sb, 0);
 #pragma unroll
       for (int k = 0; k < kSimtKC; ++k) {
-        float a[MR];
-        unsigned long long b[NR / 2];
-        if constexpr (MR == 4) {
-          const float4 v = *reinterpret_cast<const float4*>(&sa[k][ty() * 4]);
-          a[0] = v.x; a[1] = v.y; a[2] = v.z; a[3] = v.w;
-        } else {
-          const float2 v = *reinterpret_cast<const float2*>(&sa[k][ty() * 2]);
-          a[0] = v.x; a[1] = v.y;
-        }
-#pragma unroll
-        for (int h = 0; h < NR / 4; ++h) {
-          const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&sb[k][h * (TN / 2) + tx() * 4]);
-          b[2 * h] = v.x; b[2 * h + 1] = v.y;
-        }
+        if (k + 1 < kSimtKC) read(f[(k + 1) & 1], sa, sb, k + 1);
+        const Frag& c = f[k & 1];
 #pragma unroll
         for (int i = 0; i < MR; ++i) {
           unsigned long long aa;
-          asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(a[i]));
+          asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(c.a[i]));
 #pragma unroll
-          for (int j = 0; j < NR / 2; ++j) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(aa), "l"(b[j]));
+          for (int j = 0; j < NR / 2; ++j) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(aa), "l"(c.b[j]));
         }
       }
     }
