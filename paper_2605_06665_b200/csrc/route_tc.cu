@@ -19,7 +19,8 @@ namespace {
 
 constexpr int kTile = 128;             // tokens per CTA tile = TMEM lanes
 constexpr int kBK = 64;                // k-block: 64 bf16 = one 128-byte swizzle row
-constexpr int kMaxStages = 8;
+constexpr int kMaxStages = 12;
+constexpr uint32_t kTailBars = 384;      // barriers and flags behind the z tiles
 constexpr uint32_t kXBytes = kTile * kBK * 2;
 constexpr int kEpiWarps = 8;           // two per TMEM lane quarter: they take alternate 32-expert chunks
 constexpr int kThreads = 64 + 32 * kEpiWarps;   // warp 0 TMA producer, warp 1 MMA issuer, warps 2-9 epilogue
@@ -34,9 +35,8 @@ struct RouteParams {
   int32_t* acc_counts; long long* acc_sums; uint32_t* ticket;   // [M] accumulators of all CTAs (start at zero,
                                                                 // left at zero), [0] CTAs done, [1] non-finite sum
   const int32_t* split_any;            // [3] does split s hold a non-zero anywhere
-  int stages;                          // operand stages that fit into shared memory
+  uint32_t op_bytes;                   // shared memory for operand stages
   int n1, n2;                          // MMA N of the first (<= 256) and second instruction; n1 + n2 = ceil16(M)
-  uint32_t stage_bytes;
   int32_t* status;
 };
 
@@ -130,7 +130,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int M = p.M;
-  uint8_t* zstage = smem + (size_t)p.stages * p.stage_bytes;      // [8 warps] 32 x 32 fp32 tiles of z
+  uint8_t* zstage = smem + p.op_bytes;                              // [8 warps] 32 x 32 fp32 tiles of z
   uint8_t* tail = zstage + kEpiWarps * kZStage;
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(tail);
   uint64_t* empty_bar = full_bar + kMaxStages;
@@ -140,7 +140,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   uint32_t* tmem_ptr = reinterpret_cast<uint32_t*>(xbar + 8);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_ptr + 1);
   int* last_flag = const_cast<int*>(abort) + 1;
-  float* xnorm = reinterpret_cast<float*>(tail + 256);              // [2 halves][128 tokens][2] partial norm terms
+  float* xnorm = reinterpret_cast<float*>(tail + kTailBars);              // [2 halves][128 tokens][2] partial norm terms
   float* xtopv = xnorm + 2 * kTile * 2;                             // [128 tokens][KMAX] keys of the second warp
   int* xtopi = reinterpret_cast<int*>(xtopv + kTile * UNIPOOL_MAX_TOPK);
   int* hist = xtopi + kTile * UNIPOOL_MAX_TOPK;                     // [M]
@@ -155,8 +155,11 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const int n_tp = (p.T + 2 * kTile - 1) / (2 * kTile);             // tile pairs
   const bool two_acc = n_cols <= 256;
 
+  // Which of the weights' three bf16 terms hold anything (term 0 always counts).  A stage takes a k-block of x and of
+  // every such term, as long as three stages fit: x is then read once, not once per term.
+  const int any1 = p.split_any[1], any2 = p.split_any[2];
   if (threadIdx.x == 0) {
-    for (int s = 0; s < p.stages; ++s) { tc::mbar_init(&full_bar[s], 1); tc::mbar_init(&empty_bar[s], 1); }
+    for (int s = 0; s < kMaxStages; ++s) { tc::mbar_init(&full_bar[s], 1); tc::mbar_init(&empty_bar[s], 1); }
     for (int a = 0; a < 2; ++a) { tc::mbar_init(&tmem_full[a], 1); tc::mbar_init(&tmem_empty[a], 2 * kEpiWarps); }
     for (int i = 0; i < 8; ++i) tc::mbar_init(&xbar[i], 2);
     *abort = 0;
@@ -177,6 +180,12 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   tc::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_ptr;
   const uint32_t w1_bytes = (uint32_t)(p.n1 / 2) * (kBK * 2), w2_bytes = (uint32_t)(p.n2 / 2) * (kBK * 2);
+  const uint32_t w_bytes = w1_bytes + w2_bytes;
+  const int n_terms = 1 + (any1 != 0) + (any2 != 0);
+  const int second = any1 != 0 ? 1 : 2;                             // term numbers: 0, second, 2
+  const int tps = p.op_bytes / (kXBytes + n_terms * w_bytes) >= 3 ? n_terms : 1;   // terms per stage
+  const uint32_t stage_bytes = kXBytes + tps * w_bytes;
+  const int stages = min(kMaxStages, (int)(p.op_bytes / stage_bytes));
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (one in each CTA)
@@ -186,18 +195,20 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       bool ok = true;
       for (int tp = pair; tp < n_tp && ok; tp += n_pairs) {
         const int t0 = tp * 2 * kTile + rank * kTile;
-        for (int s = 0; s < 3 && ok; ++s) {
-          if (s > 0 && p.split_any[s] == 0) continue;
+        for (int first = 0; first < n_terms && ok; first += tps) {
           for (int kb = 0; kb < kblocks; ++kb) {
             if (!tc::mbar_wait(&empty_bar[stage], phase ^ 1u, abort)) { route_timeout(p, abort, 11); ok = false; break; }
-            uint8_t* sX = smem + (size_t)stage * p.stage_bytes;
-            uint8_t* sW = sX + kXBytes;
-            if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], 2 * (kXBytes + w1_bytes + w2_bytes));
+            uint8_t* sX = smem + (size_t)stage * stage_bytes;
+            if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], 2 * stage_bytes);
             tc::tma_load_2d_pair(sX, &tmX, &full_bar[stage], kb * kBK, t0);
-            tc::tma_load_2d_pair(sW, &tmW1, &full_bar[stage], kb * kBK, s * M + rank * (p.n1 / 2));
-            if (p.n2 > 0)
-              tc::tma_load_2d_pair(sW + w1_bytes, &tmW2, &full_bar[stage], kb * kBK, s * M + p.n1 + rank * (p.n2 / 2));
-            if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+            for (int i = 0; i < tps; ++i) {
+              const int term = first + i == 0 ? 0 : first + i == 1 ? second : 2;
+              uint8_t* sW = sX + kXBytes + i * w_bytes;
+              tc::tma_load_2d_pair(sW, &tmW1, &full_bar[stage], kb * kBK, term * M + rank * (p.n1 / 2));
+              if (p.n2 > 0)
+                tc::tma_load_2d_pair(sW + w1_bytes, &tmW2, &full_bar[stage], kb * kBK, term * M + p.n1 + rank * (p.n2 / 2));
+            }
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
         }
       }
@@ -206,9 +217,14 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (leader CTA only)
+    // The MMAs of a router are narrow and the thread that issues them is what bounds the main loop: straight-line
+    // groups of four, nothing decided in between.  128 tokens per CTA, 96 experts, d = 768, time to the complete
+    // accumulator: one term 12.4 -> 9.9 us, three terms 23.6 -> 14.1 us (with x read once; with x read three times and
+    // a branch per MMA both were as slow, loads were never the limit).
     if (lane == 0 && rank == 0) {
       const uint32_t idesc1 = tc::instr_desc_bf16(p.n1, false, false, 256);
       const uint32_t idesc2 = tc::instr_desc_bf16(p.n2 > 0 ? p.n2 : 16, false, false, 256);
+      const bool two_mma = p.n2 > 0;
       int stage = 0;
       uint32_t phase = 0;
       bool ok = true;
@@ -220,24 +236,28 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (!tc::mbar_wait(&tmem_empty[acc], acc_phase ^ 1u, abort)) { route_timeout(p, abort, 14); break; }
         tc::tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * 256;
-        uint32_t accumulate = 0;
-        for (int s = 0; s < 3 && ok; ++s) {
-          if (s > 0 && p.split_any[s] == 0) continue;
+        for (int first = 0; first < n_terms && ok; first += tps) {
           for (int kb = 0; kb < kblocks; ++kb) {
             if (!tc::mbar_wait(&full_bar[stage], phase, abort)) { route_timeout(p, abort, 12); ok = false; break; }
             tc::tc_fence_after_sync();
-            const uint32_t xaddr = tc::smem_u32(smem + (size_t)stage * p.stage_bytes);
+            const uint32_t xaddr = tc::smem_u32(smem + (size_t)stage * stage_bytes);
             const uint64_t xdesc = tc::smem_desc_sw128(xaddr, 16, 1024);
-            const uint64_t wdesc = tc::smem_desc_sw128(xaddr + kXBytes, 16, 1024);
-            const uint64_t wdesc2 = tc::smem_desc_sw128(xaddr + kXBytes + w1_bytes, 16, 1024);
+            uint32_t waddr = xaddr + kXBytes;
+            for (int i = 0; i < tps; ++i, waddr += w_bytes) {
+              const uint64_t wdesc = tc::smem_desc_sw128(waddr, 16, 1024);
+              const uint32_t more = (first | kb | i) != 0 ? 1u : 0u;
 #pragma unroll
-            for (int j = 0; j < kBK / 16; ++j) {
-              tc::umma_bf16_pair(d_tmem, xdesc + 2 * j, wdesc + 2 * j, idesc1, accumulate);
-              if (p.n2 > 0) tc::umma_bf16_pair(d_tmem + 256, xdesc + 2 * j, wdesc2 + 2 * j, idesc2, accumulate);
-              accumulate = 1;
+              for (int j = 0; j < kBK / 16; ++j)
+                tc::umma_bf16_pair(d_tmem, xdesc + 2 * j, wdesc + 2 * j, idesc1, j > 0 ? 1u : more);
+              if (two_mma) {
+                const uint64_t wdesc2 = tc::smem_desc_sw128(waddr + w1_bytes, 16, 1024);
+#pragma unroll
+                for (int j = 0; j < kBK / 16; ++j)
+                  tc::umma_bf16_pair(d_tmem + 256, xdesc + 2 * j, wdesc2 + 2 * j, idesc2, j > 0 ? 1u : more);
+              }
             }
             tc::umma_commit_pair(&empty_bar[stage], 3);
-            if (++stage == p.stages) { stage = 0; phase ^= 1u; }
+            if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
         }
         if (ok) tc::umma_commit_pair(&tmem_full[acc], 3);
@@ -299,45 +319,38 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           ss = ss * expf(mx - cm) + part;                 // the first chunk rescales an empty sum
           mx = cm;
         }
+        auto key_of = [&](float zv, int e) {
+          const float u = SOFTMAX ? zv : fmaxf(zv, 0.f);
+          return e >= M ? -INFINITY : u == u ? u : -FLT_MAX;   // NaN logits sort last but stay selectable
+        };
+        // a later equal key stays behind (experts are visited in ascending order)
+        unsigned cand = 0;                                // KMAX > 2: keys that beat the list as it stands
+        if (KMAX <= 2) {                                  // two selects per entry, no branch
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int e = c0 + i;
-          const float u = SOFTMAX ? z[i] : fmaxf(z[i], 0.f);
-          float key = u == u ? u : -FLT_MAX;              // NaN logits sort last but stay selectable
-          if (e >= M) key = -INFINITY;                    // never selected
-          // a later equal key stays behind (experts are visited in ascending order)
-          if (KMAX <= 2) {                                // two selects per entry, no branch
+          for (int i = 0; i < 32; ++i) {
+            const int e = c0 + i;
+            const float key = key_of(z[i], e);
             const bool g0 = key > tv[0], g1 = key > tv[KMAX - 1];
             tv[KMAX - 1] = g0 ? tv[0] : (g1 ? key : tv[KMAX - 1]);
             ti[KMAX - 1] = g0 ? ti[0] : (g1 ? e : ti[KMAX - 1]);
             tv[0] = g0 ? key : tv[0];
             ti[0] = g0 ? e : ti[0];
-          } else if (key > tv[KMAX - 1]) {                // most keys do not enter: test the last entry first
-            float cv = key;
-            int ci = e;
-            bool moved = false;
-#pragma unroll
-            for (int j = 0; j < KMAX; ++j) {
-              const bool sw = moved || cv > tv[j];
-              const float fv = tv[j];
-              const int fi = ti[j];
-              tv[j] = sw ? cv : fv;
-              ti[j] = sw ? ci : fi;
-              cv = sw ? fv : cv;
-              ci = sw ? fi : ci;
-              moved = sw;
-            }
           }
+        } else {
+#pragma unroll
+          for (int i = 0; i < 32; ++i) cand |= key_of(z[i], c0 + i) > tv[KMAX - 1] ? 1u << i : 0u;
         }
-        if (vec) {
-          // the 32 x 32 chunk is staged in shared memory (128-byte swizzle, conflict-free) and leaves by a
-          // TMA store, which clips it at M columns and T rows
+        if (vec || KMAX > 2) {
+          // the 32 x 32 chunk is staged in shared memory (128-byte swizzle, conflict-free); it leaves by a TMA store,
+          // which clips it at M columns and T rows, where rows of z are 16-byte aligned
           if (lane == 0) tc::bulk_wait_read<0>();         // the previous chunk's store has drained the tile
           __syncwarp();
 #pragma unroll
           for (int q = 0; q < 8; ++q)
             *reinterpret_cast<float4*>(my_stage + lane * 128 + ((q ^ (lane & 7)) << 4)) =
                 make_float4(z[4 * q], z[4 * q + 1], z[4 * q + 2], z[4 * q + 3]);
+        }
+        if (vec) {
           tc::fence_proxy_async();
           __syncwarp();
           const int zrow0 = tp * 2 * kTile + rank * kTile + quarter * 32;
@@ -349,6 +362,34 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 #pragma unroll
           for (int i = 0; i < 32; ++i)
             if (c0 + i < M) zrow[c0 + i] = z[i];
+        }
+        if (KMAX > 2) {
+          // Every lane inserts its own next candidate, read back from the staged row: the warp goes round as often as
+          // the busiest lane has candidates, not once per expert that any lane selects (384 experts, top-8: 57
+          // rounds against 192).
+          while (__any_sync(0xffffffffu, cand != 0)) {
+            if (cand != 0) {
+              const int i = __ffs(cand) - 1;
+              cand &= cand - 1;
+              float cv = key_of(*reinterpret_cast<const float*>(my_stage + lane * 128 + (((i >> 2) ^ (lane & 7)) << 4) + (i & 3) * 4), c0 + i);
+              int ci = c0 + i;
+              if (cv > tv[KMAX - 1]) {
+                bool moved = false;
+#pragma unroll
+                for (int j = 0; j < KMAX; ++j) {
+                  const bool sw = moved || cv > tv[j];
+                  const float fv = tv[j];
+                  const int fi = ti[j];
+                  tv[j] = sw ? cv : fv;
+                  ti[j] = sw ? ci : fi;
+                  cv = sw ? fv : cv;
+                  ci = sw ? fi : ci;
+                  moved = sw;
+                }
+              }
+            }
+          }
+          __syncwarp();
         }
       }
       // the two warps of the quarter exchange their partial norms
@@ -658,13 +699,16 @@ int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, fl
   const int n_cols = (M + 15) / 16 * 16;
   p.n1 = n_cols < 256 ? n_cols : 256;
   p.n2 = n_cols - p.n1;
-  p.stage_bytes = kXBytes + (uint32_t)(n_cols / 2) * (kBK * 2);
-  const uint32_t tail_bytes = 256 + 2 * kTile * 2 * 4 + 2 * kTile * UNIPOOL_MAX_TOPK * 4 + UNIPOOL_MAX_EXPERTS * 4 +
+  const uint32_t stage_bytes = kXBytes + (uint32_t)(n_cols / 2) * (kBK * 2);      // with one term
+  const uint32_t tail_bytes = kTailBars + 2 * kTile * 2 * 4 + 2 * kTile * UNIPOOL_MAX_TOPK * 4 + UNIPOOL_MAX_EXPERTS * 4 +
                               kEpiWarps * M * 4 + (M + 31) / 32 * 32 * 4;
   const uint32_t budget = 227 * 1024 - 1024 - tail_bytes - kEpiWarps * kZStage;
-  p.stages = (int)(budget / p.stage_bytes);
-  if (p.stages > kMaxStages) p.stages = kMaxStages;
-  UP_REQUIRE(p.stages >= 2 && ctx->sm_count >= 2, UNIPOOL_ERR_UNSUPPORTED,
+  const int kblocks = d / kBK;
+  // no more than the k-blocks of one tile with all three terms, between three and kMaxStages of them
+  const int most_stages = kblocks < 3 ? 3 : kblocks < kMaxStages ? kblocks : kMaxStages;
+  const uint32_t most = (uint32_t)most_stages * (kXBytes + 3u * (stage_bytes - kXBytes));
+  p.op_bytes = (budget < most ? budget : most) / 1024 * 1024;
+  UP_REQUIRE(p.op_bytes >= 2 * stage_bytes && ctx->sm_count >= 2, UNIPOOL_ERR_UNSUPPORTED,
              "router of %d experts does not fit the logits kernel", M);
   CUtensorMap tmX, tmW1, tmW2, tmZ;
   if ((M & 3) == 0) {
@@ -680,7 +724,7 @@ int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, fl
     tmW2 = tmW1;
   }
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_SELECT, 1, s);
-  const size_t smem = (size_t)p.stages * p.stage_bytes + kEpiWarps * kZStage + tail_bytes + 1024;
+  const size_t smem = (size_t)p.op_bytes + kEpiWarps * kZStage + tail_bytes + 1024;
   const int n_tp = (T + 2 * kTile - 1) / (2 * kTile);
   const int max_pairs = ctx->sm_count / 2;
   const int grid = 2 * (n_tp < max_pairs ? n_tp : max_pairs);

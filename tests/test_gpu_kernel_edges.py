@@ -320,3 +320,36 @@ def test_recomputed_layers_contract_in_runs(kw, L, T, accumulate):
         st.close()
     assert torch.equal(out[0][0], out[1][0]) and out[0][1].abs().max() > 0
     assert rel_max(to_np(out[1][1]), to_np(out[0][1])) < 1e-5 and rel_max(to_np(out[1][2]), to_np(out[0][2])) < 1e-5
+
+
+@pytest.mark.parametrize("T,M,d,k", [
+    (1, 8, 64, 8), (257, 10, 64, 3), (130, 256, 128, 8), (300, 257, 128, 5), (520, 512, 64, 8), (300, 384, 832, 8), (33, 96, 768, 2),
+])
+@pytest.mark.parametrize("bits", ["bf16", "fp32"])                # one or three bf16 terms of the router weights
+def test_bf16_router_at_the_edges_of_its_stages(T, M, d, k, bits):
+    """Selection with many candidates per lane, one and two MMAs per k-block, one or three weight terms per stage, fewer
+    k-blocks than stages; against the oracle in float64 as in the parity tests."""
+    import torch
+    from oracle import unipool_oracle as O
+    from paper_2605_06665_b200 import binding as B
+    from parity_utils import check_routing, rel_max, to_np
+    eps, c = 1e-6, 2.0
+    ctx = B.Context(B.make_config(d, 64, M, k, 1, T, B.BF16, eps, c))
+    g = torch.Generator(device="cuda").manual_seed(T)
+    W = torch.empty(M, d, device="cuda").normal_(0, 0.02, generator=g)
+    if bits == "bf16":
+        W = W.bfloat16().float()
+    x = torch.randn(T, d, device="cuda", generator=g).bfloat16()
+    idx, gate = torch.empty(T, k, dtype=torch.int32, device="cuda"), torch.empty(T, k, device="cuda")
+    counts, S = torch.empty(M, dtype=torch.int32, device="cuda"), torch.empty(M, device="cuda")
+    n, z = torch.empty(T, device="cuda"), torch.empty(T, M, device="cuda")
+    ctx.route(x, T, W, 1.0, None, M, idx, gate, counts, S, n, z)
+    torch.cuda.synchronize()
+    ctx.check_status()
+    ctx.close()
+    f8 = lambda t: t.double().cpu().numpy()
+    ref = O.route(f8(x), f8(W), 1.0, c, eps, k, None)
+    check_routing(to_np(idx), ref["z"], ref["idx"], k)
+    ref = O.route(f8(x), f8(W), 1.0, c, eps, k, None, forced_idx=to_np(idx))
+    assert rel_max(to_np(z), ref["z"]) < 1e-5 and rel_max(to_np(gate), ref["g"]) < 1e-5
+    assert (to_np(counts) == ref["counts"]).all() and rel_max(to_np(S), ref["S"]) < 1e-5
