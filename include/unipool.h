@@ -29,7 +29,8 @@
  *   A layer's T*k (token, slot) assignments are sorted by expert, token-major
  *   inside an expert.  Group e starts at offsets[e], a multiple of
  *   UNIPOOL_ROW_ALIGN rows; rows between the end of a group and the next start
- *   are pad rows and hold zeros in every permuted buffer.  Buffers in this
+ *   are pad rows and hold zeros in every permuted buffer (except that
+ *   unipool_expert_bwd_rows may leave those of dYp and dGU unwritten).  Buffers in this
  *   space have unipool_row_capacity() rows; rows >= offsets[n_experts] are
  *   never touched.
  */
@@ -207,8 +208,10 @@ int unipool_expert_fwd(unipool_ctx* ctx, const void* Xp, const int32_t* offsets,
  * writes rows [n_experts] int32, the tokens of each group (group e = rows offsets[e] .. offsets[e] + rows[e]
  * - 1; the rest up to offsets[e+1] is padding).  Given to the other three ([n_layers, n_experts] for
  * unipool_pool_wgrad_rows), the tensor-core kernels leave the padding out of their products instead of
- * multiplying its zeros; results and contents of the buffers are those of the calls without `rows`, which
- * they are when it is NULL.  `rows` must be what the dispatch of the same layer wrote. */
+ * multiplying its zeros, and the pad rows of dYp and dGU are written no further than the next multiple of 16
+ * rows of a group (with zeros; what the others hold is unspecified).  Results are those of the calls without
+ * `rows`, which these are when it is NULL: the backward and the pool_wgrad call of a layer are given `rows` both
+ * or neither.  `rows` must be what the dispatch of the same layer wrote. */
 int unipool_dispatch_rows(unipool_ctx* ctx, const void* x, int32_t T, const int32_t* idx,
                           int32_t n_experts, int32_t* offsets, int32_t* row_of, int32_t* token_of,
                           int32_t* tile_expert, int32_t* rows, void* Xp, unipool_stream stream);

@@ -315,7 +315,7 @@ int unipool_expert_bwd_rows(unipool_ctx* ctx, const void* dy, int32_t T, const i
   const bool wgrad = !(flags & UNIPOOL_BWD_SKIP_WGRAD);
   if (wgrad) { CHECK_PTR(dW_gu); CHECK_PTR(dW_down); }
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  int rc = combine_bwd_launch(ctx, dy, T, row_of, gate, token_of, offsets, n_experts, Yp, dYp, dgate, s);
+  int rc = combine_bwd_launch(ctx, dy, T, row_of, gate, token_of, offsets, rows, n_experts, Yp, dYp, dgate, s);
   if (rc != UNIPOOL_OK) return rc;
   ExpertBwdArgs a{offsets, tile_expert, Xp, GU, A, W_gu, W_down, expert_base, n_experts,
                   dYp, dGU, ctx->ws.dXp, dW_gu, dW_down, wgrad, (flags & UNIPOOL_WGRAD_OVERWRITE) != 0, rows};

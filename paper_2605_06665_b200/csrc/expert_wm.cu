@@ -593,7 +593,8 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
           }
         }
       }
-      if (live && half == 0 && q.pad_lo < q.pad_hi) {              // pad rows behind the group's last unit
+      const bool pads = MODE != kDgrad1 || p.rows == nullptr;
+      if (pads && live && half == 0 && q.pad_lo < q.pad_hi) {              // pad rows behind the group's last unit
         if constexpr (MODE == kFwd1) {
           zero_rows(p.out0, 2 * p.f, feat, q.pad_lo, q.pad_hi, lane);
           zero_rows(p.out0, 2 * p.f, p.f + feat, q.pad_lo, q.pad_hi, lane);

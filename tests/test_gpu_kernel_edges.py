@@ -121,8 +121,13 @@ def test_expert_ffn_at_the_edges_of_its_units(sizes, d, f, with_rows):
     off = off.tolist()
     used = off[-1]
     pad = tok[:used] < 0
-    for t in (GU, A, Yp, dGU):
+    for t in (Xp, GU, A, Yp):
         assert not t[:used][pad].any()                            # zeros (and no NaN) on pad rows
+    if with_rows:                                                 # of dYp, dGU those up to the next multiple of 16 rows
+        for e, n in enumerate(sizes):
+            pad[off[e] + (n + 15) // 16 * 16:off[e + 1]] = False
+    for t in (dYp, dGU):
+        assert not t[:used][pad].any()
 
     def close(got, want):
         assert (got.float() - want.float()).abs().max() <= 1e-2 * want.float().abs().max()
@@ -154,8 +159,8 @@ def test_expert_ffn_at_the_edges_of_its_units(sizes, d, f, with_rows):
     [[33, 47, 48, 17], [49, 1, 95, 0], [0, 0, 0, 7]],  # 36: k-blocks of 48
 ])
 def test_weight_gradient_leaves_the_padding_out(sizes, overwrite):
-    """With the group sizes the contraction stops at the last 16 rows that hold a token; what is left out are zeros,
-    so the sums are those of the padded contraction up to the sign of zero: equal, bit for bit."""
+    """With the group sizes the contraction stops at the last 16 rows that hold a token, whatever the rest of the padding
+    holds; what is left out of the padded contraction are zeros, so the sums are equal, bit for bit."""
     import torch
     from paper_2605_06665_b200 import binding as B
     L, M, d, f = len(sizes), 4, 192, 320
@@ -175,6 +180,11 @@ def test_weight_gradient_leaves_the_padding_out(sizes, overwrite):
     offs = torch.from_numpy(off).cuda()
     got = []
     for r in (None, rows):
+        if r is not None:
+            for l, s in enumerate(sizes):
+                for e, n in enumerate(s):
+                    for t in ops:
+                        t[l, off[l, e] + (n + 15) // 16 * 16:off[l, e + 1]] = float("nan")
         dgu, dd = torch.full((M, 2 * f, d), 3.0, device="cuda"), torch.full((M, d, f), -2.0, device="cuda")
         ctx.pool_wgrad(L, cap, offs, *ops, 0, M, dgu, dd, B.WGRAD_OVERWRITE if overwrite else 0, r)
         torch.cuda.synchronize()
@@ -187,7 +197,7 @@ def test_weight_gradient_leaves_the_padding_out(sizes, overwrite):
         want = torch.zeros(2 * f, d, device="cuda") if overwrite else torch.full((2 * f, d), 3.0, device="cuda")
         down = torch.zeros(d, f, device="cuda") if overwrite else torch.full((d, f), -2.0, device="cuda")
         for l in range(L):
-            s = slice(off[l, e], off[l, e + 1])
+            s = slice(off[l, e], off[l, e] + sizes[l][e])
             want += dGU[l, s].T @ Xp[l, s]
             down += dYp[l, s].T @ A[l, s]
         # exact products, fp32 sums of at most some 1200 terms: 1e-5 of the largest value
