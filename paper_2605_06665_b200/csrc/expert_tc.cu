@@ -1388,26 +1388,27 @@ bool rows_on_pairs(const unipool_ctx* ctx, int n_experts) {
 // Weights or tokens on the M side, by the rows the average expert gets from a full batch (the group sizes
 // themselves are on the device).  Measured per GEMM, interleaved, tokens / weights on M in us (768 x 2048; the
 // figures of 1536 x 4096 are marked *):
-//   rows                85        125       170       341        500         682         1024*       1365
-//   gate/up          126/130   143/145   180/171   271/266    363/363     *1678/1602  1589/1590   213/223
-//   down              70/75     78/82     90/86    132/123    169/169     *760/763    728/724     101/107
-//   dgrad down        91/93    110/104   138/120   201/193    262/246     *1073/971   1013/952    164/164
-//   dgrad gate/up    117/124   132/132   154/142   240/212    308/308     *1494/1474  1413/1392   185/191
-// Below ~128 rows every launch is bound by streaming the weights and the token-major kernels keep more bytes in
-// flight (dgrad down alone gains again up to 48 rows, where it saves reading G and U of the padding: 4 rows 86/78,
-// 31 rows 89/83, 48 rows 90/86, of 1536 x 4096 31 rows 176/167); large groups waste nothing in 256-row pair-tiles.  Down and dgrad gate/up gain while a group is one or
-// two chunks (and need a contraction long enough to hide the epilogue of a wide unit: 384 experts of 768 x 512 lost
-// 10 % on the down projection, 4 % on dgrad gate/up); dgrad down gains longest, its G and U traffic being the
-// same on fewer padded rows; gate/up gains beyond 450 rows only where its contraction is long.
+//   rows                31         66        125       170       229       341       546      819      *128      *1024
+//   gate/up          125/127   126/129   141/146   180/171   199/211   268/263   244/240  228/227  708/626  1589/1479
+//   down              69/68     69/69     78/77     91/81    102/90    131/124   118/122  113/116  334/334   728/724
+//   dgrad down        87/70     89/80    108/100   138/112   150/133   199/192   183/172  174/166  465/400  1014/951
+//   dgrad gate/up    116/109   117/113   130/125   154/134   178/151   235/209   205/212  199/204  596/581  1401/1384
+// Few rows: every launch streams the weights, and what is left to gain are the rows of the padding that the token-major
+// kernels read (gate/up reads few of them, and both forms write its pad rows).  Large groups waste nothing in 256-row
+// pair-tiles: down and dgrad gate/up gain while a group is one or two chunks, and need a contraction long enough to
+// hide the epilogue of a unit (384 experts of 768 x 512, 341 rows: down 112/129, dgrad gate/up 185/202); dgrad down
+// gains longest, its G and U traffic being the same on fewer padded rows; gate/up gains further where its contraction
+// is long.  Many narrow experts under skewed routing lose with few rows: the largest group sets the size of a
+// stage (393 experts of 768 x 320, 92 rows: dgrad down 54/58, dgrad gate/up 46/59).
 bool weights_on_m(const unipool_ctx* ctx, int mode, int n_experts) {
   if (ctx->sm_count < 2 || n_experts > kWmMaxExperts) return false;
   const int64_t rows = (int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k / n_experts;
   const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff;
   switch (mode) {
-    case kFwd1: return rows > 150 && rows <= (d >= 1024 ? 1024 : 450);
-    case kFwd2: return rows > 150 && rows <= 450 && f > 1024;
-    case kDgrad1: return rows <= 48 || (rows > 100 && rows <= 1200);
-    default: return rows > 150 && rows <= 450 && 2 * f > 1024;
+    case kFwd1: return rows > (d >= 1024 ? 100 : 150) && rows <= (d >= 1024 ? 1024 : 600);
+    case kFwd2: return rows <= 450 && f > 1024;
+    case kDgrad1: return rows <= 1200 && (rows <= 48 || rows > 100 || f > 1024);
+    default: return rows <= 450 && 2 * f > 1024;
   }
 }
 

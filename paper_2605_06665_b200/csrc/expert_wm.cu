@@ -52,17 +52,23 @@ template <int MODE> struct Wm {
   static constexpr bool kAMn = MODE == kDgrad1 || MODE == kDgrad2;
   static constexpr int kMaxTok = kDual ? 192 : kIo ? 256 : 384; // tokens of a unit
   static constexpr uint32_t kABytes = kDual ? 2 * 16384 : 16384;
-  static constexpr uint32_t kStageBytes = kABytes + kMaxTok / 2 * 128;
-  static constexpr int kStages = kDual ? 4 : 5;
+  // Room for the operands of four or five k-blocks of the largest unit.  A launch whose largest unit is smaller divides
+  // it into more, and the plain GEMMs take two k-blocks a stage where that leaves three stages: with few tokens the
+  // launch streams weights, and waits, barriers and TMA issues per 16 KB were what held it back (31 rows of
+  // 768 x 2048, five stages of one k-block / ten / five of two: down 70 / 66 / 66 us, dgrad gate/up 113 / 113 / 111;
+  // 64 rows of 1536 x 4096: down 337 / 322 / 305, dgrad gate/up 609 / 595 / 535).
+  static constexpr uint32_t kStageRoom = (kDual ? 4 : 5) * (kABytes + kMaxTok / 2 * 128);
+  static constexpr int kMaxStages = kDual ? 5 : kIo ? 8 : 11;
   // gate/up: the epilogue warps keep a unit's last two blocks of both accumulators in registers (see there), so
   // they are two warpgroups of their own that take over the registers of the first (setmaxnreg)
   static constexpr int kEpiBase = kDual ? 4 : 2;                // first epilogue warp
   static constexpr int kThreads = 32 * (kEpiBase + kEpi) + (kIo ? 128 : 0);
-  static constexpr uint32_t kStaging = kStages * kStageBytes;
+  static constexpr uint32_t kStaging = kStageRoom;
   static constexpr int kRing = 4;                               // dgrad1: (G, U) blocks in flight per lane quarter
   static constexpr uint32_t kStagingBytes = kIo ? 4 * kRing * 2 * kTileBytes : kEpi * (kDual ? 3 : 1) * kTileBytes;
   static constexpr uint32_t kBars = kStaging + kStagingBytes;
-  static constexpr uint32_t kTable = kBars + 384;               // one word per expert of the launch
+  static constexpr uint32_t kTable = kBars + (kIo ? 432 : 384);   // one word per expert of the launch
+  static_assert((2 * kMaxStages + 4 + (kIo ? 8 * kRing : 0)) * 8 + 16 <= (kIo ? 432 : 384), "barrier block");
   static_assert(kTable + 4 * kWmMaxExperts + 1024 <= kSmemMax, "shared-memory budget");
 };
 
@@ -112,11 +118,18 @@ __device__ __forceinline__ int group_n16(const WmParams& p, int e) {
   return ((p.rows ? min(max(p.rows[e], 0), padded) : padded) + 15) / 16;
 }
 
-// Fills in unit u.  q.pos, q.cum: list position and units before it, moved on from an earlier unit's.
+// Fills in unit u.  q.pos, q.cum: list position and units before it, moved on from an earlier unit's; `single`: every
+// group is one chunk, the list position follows from u (the walk over the experts of a deal, 25 of them at three
+// weight tiles each, held up all roles: dgrad gate/up 85 -> 68 us at 768 x 256 and 20
+// rows, 146 -> 136 us at 768 x 2048 and 170 rows).
 template <int MODE, bool ROWS = true>
-__device__ __forceinline__ void seek(const WmParams& p, const uint32_t* list, int u, Unit& q) {
+__device__ __forceinline__ void seek(const WmParams& p, const uint32_t* list, bool single, int u, Unit& q) {
   uint32_t word;
   int n16, chunks;
+  if (single) {
+    q.pos = u / p.n_wt;
+    q.cum = q.pos * p.n_wt;
+  }
   for (;;) {
     word = list[q.pos];
     n16 = (int)(word >> 9);
@@ -224,19 +237,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(Wm<MODE>::kThreads, 
 wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ TokenMaps tmB,
           const __grid_constant__ BlockMaps tmC0, const __grid_constant__ BlockMaps tmC1, const WmParams p) {
   using W = Wm<MODE>;
-  constexpr int kStages = W::kStages;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(smem + W::kBars);
-  uint64_t* empty_bar = full_bar + kStages;
-  uint64_t* tmem_full = empty_bar + kStages;                 // [2] by unit parity
+  uint64_t* empty_bar = full_bar + W::kMaxStages;
+  uint64_t* tmem_full = empty_bar + W::kMaxStages;           // [2] by unit parity
   uint64_t* tmem_empty = tmem_full + 2;                      // [2]
   uint64_t* ring_full = tmem_empty + 2;                      // dgrad1: [4][kRing] a block's G and U have landed
   uint64_t* ring_staged = ring_full + (W::kIo ? 4 * W::kRing : 0);   // dgrad1: dG and dU are in their place
   uint32_t* tmem_ptr = reinterpret_cast<uint32_t*>(ring_staged + (W::kIo ? 4 * W::kRing : 0));
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_ptr + 1);
-  static_assert((2 * kStages + 4 + (W::kIo ? 8 * W::kRing : 0)) * 8 + 12 <= 384, "barrier block");
-  int* n_units = reinterpret_cast<int*>(tmem_ptr + 2);
+  int* n_units = reinterpret_cast<int*>(tmem_ptr + 2);       // [0] units, [1] groups with tokens
   uint32_t* list = reinterpret_cast<uint32_t*>(smem + W::kTable);              // [n_experts]
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
@@ -244,7 +255,7 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) { tc::mbar_init(&full_bar[s], 1); tc::mbar_init(&empty_bar[s], 1); }
+    for (int s = 0; s < W::kMaxStages; ++s) { tc::mbar_init(&full_bar[s], 1); tc::mbar_init(&empty_bar[s], 1); }
     for (int a = 0; a < 2; ++a) { tc::mbar_init(&tmem_full[a], 1); tc::mbar_init(&tmem_empty[a], 2 * kEpi); }
     if constexpr (W::kIo)
       for (int i = 0; i < 4 * W::kRing; ++i) { tc::mbar_init(&ring_full[i], 1); tc::mbar_init(&ring_staged[i], 1); }
@@ -259,7 +270,7 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
   // the list of experts: a thread ranks its expert by counting the larger keys (unit size, then lower index first);
   // every CTA computes the same list
   uint32_t* key = reinterpret_cast<uint32_t*>(smem);                           // the stages are idle still
-  if (threadIdx.x == 0) *n_units = 0;
+  if (threadIdx.x == 0) n_units[0] = n_units[1] = 0;
   const int n4 = (p.n_experts + 3) & ~3;
   for (int e = threadIdx.x; e < n4; e += blockDim.x) {
     uint32_t v = 0;                                                            // no tokens: behind all others
@@ -284,21 +295,32 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
       list[before] = (uint32_t)e | (uint32_t)n16 << 9;
       units = group_chunks<MODE>(n16) * p.n_wt;
     }
+    const int groups = __popc(__ballot_sync(0xffffffffu, units > 0));
     units = __reduce_add_sync(0xffffffffu, units);
-    if (lane == 0 && units > 0) atomicAdd(n_units, units);
+    if (lane == 0 && units > 0) { atomicAdd(n_units, units); atomicAdd(n_units + 1, groups); }
   }
   tc::tc_fence_before_sync();
   __syncthreads();
   tc::cluster_sync();                                        // both CTAs' barriers exist before any remote use
   tc::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_ptr;
-  const int total = *n_units;
+  const int total = n_units[0];
+  const bool single = total == n_units[1] * p.n_wt;
   tc::fence_proxy_async();                                   // the scratch above is about to be written by TMA
   const int kblocks = p.Kdim / kBK;
+  // the list begins with the largest units
+  uint32_t stage_bytes = W::kStageRoom;
+  if (total > 0) {
+    const int n16 = (int)(list[0] >> 9), size = chunk_size<MODE>(n16, group_chunks<MODE>(n16));
+    stage_bytes = W::kABytes + (uint32_t)(size / 2 + 15) / 16 * (16 * 128);
+  }
+  const int slots = min(W::kMaxStages, (int)(W::kStageRoom / stage_bytes));
+  const int kpb = !W::kDual && !W::kIo && slots >= 6 ? 2 : 1, n_stages = slots / kpb;   // k-blocks a stage, stages
+  const uint32_t stage_step = (uint32_t)kpb * stage_bytes;
 
   if (warp < W::kEpiBase) {
-  // gate/up: 384 threads are launched with 168 registers: 40 x 128 + 232 x 256 = 168 x 384
-  if constexpr (W::kDual) tc::regs_dec<40>();
+  // gate/up: 384 threads are launched with 168 registers: 48 x 128 + 224 x 256 <= 168 x 384
+  if constexpr (W::kDual) tc::regs_dec<48>();
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (one in each CTA)
     if (lane == 0) {
@@ -306,28 +328,31 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
       uint32_t phase = 0;
       bool ok = true;
       Unit q{}, next{};
-      if (pair < total) seek<MODE>(p, list, pair, next);
+      if (pair < total) seek<MODE>(p, list, single, pair, next);
       for (int round = 0; ok; ++round) {
         if (snake(round, pair, n_pairs) >= total) break;
         q = next;                                            // the next unit is looked up while this one streams
-        if (snake(round + 1, pair, n_pairs) < total) seek<MODE>(p, list, snake(round + 1, pair, n_pairs), next);
+        if (snake(round + 1, pair, n_pairs) < total) seek<MODE>(p, list, single, snake(round + 1, pair, n_pairs), next);
         const int pe = p.expert_base + q.e;
         const int box = (q.h + 15) / 16;
         const CUtensorMap* mapB = &tmB.m[box - 1];
-        const uint32_t tx = 2 * (W::kABytes + (uint32_t)box * (16 * 128));
+        const uint32_t tx1 = 2 * (W::kABytes + (uint32_t)box * (16 * 128));
         const int trow = q.t0 + rank * q.h;
-        for (int kb = 0; kb < kblocks; ++kb) {
+        for (int kb0 = 0; kb0 < kblocks; kb0 += kpb) {
           if (!tc::mbar_wait(&empty_bar[stage], phase ^ 1u, abort)) { wm_timeout(p, abort, 41); ok = false; break; }
-          uint8_t* sA = smem + stage * W::kStageBytes;
-          if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], tx);              // both CTAs' bytes
-          if constexpr (MODE == kFwd1)         // 128 gate and the same 128 up features: W_gu as [2M][f][d]
-            tc::tma_load_3d_pair(sA, &tmA, &full_bar[stage], kb * kBK, q.wt * 256 + rank * 128, 2 * pe);
-          else if constexpr (MODE == kFwd2)    // 128 rows of W_down
-            tc::tma_load_2d_pair(sA, &tmA, &full_bar[stage], kb * kBK, pe * p.Mdim + q.wt * 256 + rank * 128);
-          else                                 // 128 columns of W_down / W_gu: two 64-column blocks
-            tc::tma_load_3d_pair(sA, &tmA, &full_bar[stage], 0, pe * p.Kdim + kb * kBK, q.wt * 4 + rank * 2);
-          tc::tma_load_2d_pair(sA + W::kABytes, mapB, &full_bar[stage], kb * kBK, trow);
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+          const int kb1 = min(kb0 + kpb, kblocks);
+          uint8_t* sA = smem + (uint32_t)stage * stage_step;
+          if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], (uint32_t)(kb1 - kb0) * tx1);     // both CTAs' bytes
+          for (int kb = kb0; kb < kb1; ++kb, sA += stage_bytes) {
+            if constexpr (MODE == kFwd1)         // 128 gate and the same 128 up features: W_gu as [2M][f][d]
+              tc::tma_load_3d_pair(sA, &tmA, &full_bar[stage], kb * kBK, q.wt * 256 + rank * 128, 2 * pe);
+            else if constexpr (MODE == kFwd2)    // 128 rows of W_down
+              tc::tma_load_2d_pair(sA, &tmA, &full_bar[stage], kb * kBK, pe * p.Mdim + q.wt * 256 + rank * 128);
+            else                                 // 128 columns of W_down / W_gu: two 64-column blocks
+              tc::tma_load_3d_pair(sA, &tmA, &full_bar[stage], 0, pe * p.Kdim + kb * kBK, q.wt * 4 + rank * 2);
+            tc::tma_load_2d_pair(sA + W::kABytes, mapB, &full_bar[stage], kb * kBK, trow);
+          }
+          if (++stage == n_stages) { stage = 0; phase ^= 1u; }
         }
       }
       if (!ok)
@@ -335,54 +360,78 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (leader CTA only)
-    if (lane == 0 && rank == 0) {
+    // The plain GEMMs run the loop as a whole warp and one lane issues: eight MMAs of N = 176 take 704 clocks, a lane
+    // alone needs as long to issue them (against that: down 131 -> 126 us, dgrad gate/up 226 -> 213 at 96 experts of
+    // 768 x 2048, 341 rows; 879 -> 832 and 1715 -> 1629 at 1536 x 4096).  Gate/up and dgrad down are bound by their
+    // epilogues' share of shared memory, and did not gain (their registers: 272 -> 274, 194 -> 197 us).
+    constexpr bool kWarp = !W::kDual && !W::kIo;
+    if (rank == 0 && (kWarp || lane == 0)) {
       constexpr uint32_t a_lbo = W::kAMn ? kMnBlock : 16;
       constexpr uint32_t a_step = (W::kAMn ? 16 * 128 : 32) >> 4;          // descriptor units per K = 16
+      const uint32_t issue = lane == 0 ? 1u : 0u;
+      auto uni = [](uint32_t v) { return kWarp ? tc::uniform(v) : v; };
+      auto all = [](bool v) { return kWarp ? __all_sync(0xffffffffu, v) != 0 : v; };
+      auto mma = [&](uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t accumulate) {
+        if constexpr (kWarp) tc::umma_bf16_pair_if(issue, d, ad, bd, idesc, accumulate);
+        else tc::umma_bf16_pair(d, ad, bd, idesc, accumulate);
+      };
+      auto commit = [&](uint64_t* bar) {                                   // arrives in both CTAs
+        if constexpr (kWarp) tc::umma_commit_pair_if(issue, bar, 3);
+        else tc::umma_commit_pair(bar, 3);
+      };
+      const int n_total = (int)uni((uint32_t)total), per = (int)uni((uint32_t)kpb), n_st = (int)uni((uint32_t)n_stages);
+      const uint32_t tmem = uni(tmem_base), smem0 = uni(tc::smem_u32(smem)), bytes = uni(stage_bytes);
       int stage = 0;
       uint32_t phase = 0;
       int local = 0;
       bool ok = true, wide_before = false;
-      Unit q{}, next{};
-      if (pair < total) seek<MODE, false>(p, list, pair, next);
-      for (; ok && snake(local, pair, n_pairs) < total; ++local) {
-        q = next;
-        if (snake(local + 1, pair, n_pairs) < total) seek<MODE, false>(p, list, snake(local + 1, pair, n_pairs), next);
-        const int cols = W::kDual || q.two ? 2 * q.N : q.N;
+      Unit next{};
+      if (pair < n_total) seek<MODE, false>(p, list, single, pair, next);
+      for (; ok && snake(local, pair, n_pairs) < n_total; ++local) {
+        const int N = (int)uni((uint32_t)next.N);
+        const bool two = W::kDual || uni(next.two ? 1u : 0u) != 0;
+        if (snake(local + 1, pair, n_pairs) < n_total) seek<MODE, false>(p, list, single, snake(local + 1, pair, n_pairs), next);
+        const int cols = two ? 2 * N : N;
         const bool wide = cols > 256;
         // the accumulator of two units ago, and the previous one if either reaches into the other's half
-        if (local >= 2 && !tc::mbar_wait(&tmem_empty[local & 1], ((local >> 1) & 1) ^ 1u, abort)) {
-          wm_timeout(p, abort, 42);
-          break;
-        }
-        if (local >= 1 && (wide || wide_before) &&
-            !tc::mbar_wait(&tmem_empty[(local - 1) & 1], ((local - 1) >> 1) & 1, abort)) {
-          wm_timeout(p, abort, 42);
+        ok = local < 2 || tc::mbar_wait(&tmem_empty[local & 1], ((local >> 1) & 1) ^ 1u, abort);
+        if (ok && local >= 1 && (wide || wide_before))
+          ok = tc::mbar_wait(&tmem_empty[(local - 1) & 1], ((local - 1) >> 1) & 1, abort);
+        if (!all(ok)) {
+          if (issue) wm_timeout(p, abort, 42);
           break;
         }
         wide_before = wide;
         tc::tc_fence_after_sync();
-        const uint32_t d0 = tmem_base + (wide ? 0 : (local & 1) * 256), d1 = d0 + (wide ? kSecond : 128);
-        const uint32_t idesc = tc::instr_desc_bf16(q.N, W::kAMn, false, 256);
-        const uint32_t b2 = q.two ? (uint32_t)(q.N / 2 * 128) >> 4 : 0;    // second MMA: the next N / 2 tokens
-        for (int kb = 0; kb < kblocks; ++kb) {
-          if (!tc::mbar_wait(&full_bar[stage], phase, abort)) { wm_timeout(p, abort, 43); ok = false; break; }
-          tc::tc_fence_after_sync();
-          const uint32_t aaddr = tc::smem_u32(smem + stage * W::kStageBytes);
+        const uint32_t d0 = tmem + (wide ? 0 : (local & 1) * 256), d1 = d0 + (wide ? kSecond : 128);
+        const uint32_t idesc = tc::instr_desc_bf16(N, W::kAMn, false, 256);
+        const uint32_t b2 = !W::kDual && two ? (uint32_t)(N / 2 * 128) >> 4 : 0;   // second MMA: the next N / 2 tokens
+        auto block = [&](uint32_t aaddr, uint32_t more) {                  // the MMAs of one k-block
           const uint64_t adesc = tc::smem_desc_sw128(aaddr, a_lbo, 1024);
           const uint64_t bdesc = tc::smem_desc_sw128(aaddr + W::kABytes, 16, 1024);
 #pragma unroll
-          for (int j = 0; j < kBK / 16; ++j)
-            tc::umma_bf16_pair(d0, adesc + j * a_step, bdesc + j * 2, idesc, (kb | j) != 0 ? 1u : 0u);
-          if (W::kDual || q.two) {
+          for (int j = 0; j < kBK / 16; ++j) mma(d0, adesc + j * a_step, bdesc + j * 2, idesc, j > 0 ? 1u : more);
+          if (two) {
             const uint64_t adesc2 = W::kDual ? adesc + (16384 >> 4) : adesc;
 #pragma unroll
             for (int j = 0; j < kBK / 16; ++j)
-              tc::umma_bf16_pair(d1, adesc2 + j * a_step, bdesc + b2 + j * 2, idesc, (kb | j) != 0 ? 1u : 0u);
+              mma(d1, adesc2 + j * a_step, bdesc + b2 + j * 2, idesc, j > 0 ? 1u : more);
           }
-          tc::umma_commit_pair(&empty_bar[stage], 3);             // frees the stage in both CTAs
-          if (++stage == kStages) { stage = 0; phase ^= 1u; }
+        };
+        for (int kb = 0; kb < kblocks; kb += per) {
+          ok = all(tc::mbar_wait(&full_bar[stage], phase, abort));
+          if (!ok) {
+            if (issue) wm_timeout(p, abort, 43);
+            break;
+          }
+          tc::tc_fence_after_sync();
+          const uint32_t aaddr = smem0 + (uint32_t)stage * ((uint32_t)per * bytes);
+          block(aaddr, kb != 0 ? 1u : 0u);
+          if (per > 1 && kb + 1 < kblocks) block(aaddr + bytes, 1u);
+          commit(&empty_bar[stage]);                                       // frees the stage
+          if (++stage == n_st) { stage = 0; phase ^= 1u; }
         }
-        if (ok) tc::umma_commit_pair(&tmem_full[local & 1], 3);   // accumulator complete, both CTAs
+        if (ok) commit(&tmem_full[local & 1]);                             // accumulator complete
       }
     }
   }
@@ -401,7 +450,7 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
         bool ok = true;
         auto feature = [&](const Unit& q) { return q.wt * 256 + rank * 128 + quarter * 32; };
         bool more = pair < total, live = more;                            // blocks left to fetch, to store
-        if (more) { seek<MODE>(p, list, pair, lq); sq = lq; }
+        if (more) { seek<MODE>(p, list, single, pair, lq); sq = lq; }
         while (live && ok) {
           while (fetched < stored + W::kRing - 1 && more) {
             if (feature(lq) < p.f) {
@@ -421,7 +470,7 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
               lb = 0;
               const int u = snake(++lr, pair, n_pairs);
               more = u < total;
-              if (more) seek<MODE>(p, list, u, lq);
+              if (more) seek<MODE>(p, list, single, u, lq);
             }
           }
           if (feature(sq) < p.f) {
@@ -441,7 +490,7 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
             sb = 0;
             const int u = snake(++sr, pair, n_pairs);
             live = u < total;
-            if (live) seek<MODE>(p, list, u, sq);
+            if (live) seek<MODE>(p, list, single, u, sq);
           }
         }
         if (!ok)
@@ -451,7 +500,7 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
     }
   } else {
     // ------------------------------------------------------------ epilogue: this CTA's 128 weight rows
-    if constexpr (W::kDual) tc::regs_inc<232>();
+    if constexpr (W::kDual) tc::regs_inc<224>();
     const int quarter = warp & 3, half = (warp - W::kEpiBase) >> 2;
     const int ew = (warp - W::kEpiBase) & 3;
     uint8_t* stg = smem + W::kStaging + (W::kIo ? ew * (W::kRing * 2 * kTileBytes)
@@ -461,7 +510,7 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
     bool ok = true;
     Unit q{};
     for (; ok && snake(local, pair, n_pairs) < total; ++local) {
-      seek<MODE>(p, list, snake(local, pair, n_pairs), q);
+      seek<MODE>(p, list, single, snake(local, pair, n_pairs), q);
       const int feat = q.wt * 256 + rank * 128 + quarter * 32;     // first of this warp's 32 weight rows
       const bool live = feat < p.Mdim;
       const bool wide = (W::kDual || q.two ? 2 * q.N : q.N) > 256;

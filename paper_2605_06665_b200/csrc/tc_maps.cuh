@@ -15,7 +15,7 @@ enum Mode : int {
   kWgrad = 4,   // dW[e] (+)= P_e^T Q_e                 A MN-major, B MN-major,         ragged K
 };
 
-constexpr int kWmMaxExperts = 416;        // experts of a launch of the weights-on-M kernels (their shared-memory table)
+constexpr int kWmMaxExperts = 400;        // experts of a launch of the weights-on-M kernels (their shared-memory table)
 
 enum MapKind { kMapOperand, kMapBf16Chunk, kMapF32Chunk };
 int make_tmap(const unipool_ctx* ctx, CUtensorMap* out, MapKind kind, const void* base, int rank,

@@ -85,8 +85,10 @@ def test_dispatch_maps_at_the_edges_of_its_chunking(T, k, M, static):
     ([129, 512, 513, 0, 639, 640, 300], 192, 576),               # partial weight tiles
     ([768, 769, 1000, 1, 1152, 1153, 900], 1024, 64),            # gate/up beyond 450 rows, one k-block of K = 64
     ([200] * 40 + [0, 97, 1300], 64, 1216),
-    ([110, 120, 130, 140], 256, 320),                            # dgrad down only
-    ([48, 1, 0, 33, 64, 65, 17], 128, 576),                      # dgrad down only, few rows
+    ([110, 120, 130, 140], 256, 320),                            # both dgrads
+    ([48, 1, 0, 33, 64, 65, 17], 128, 576),                      # both dgrads, few rows: stages of two k-blocks
+    ([20, 1, 0, 33, 16, 5, 17], 192, 1216),                      # odd numbers of k-blocks in such stages
+    ([384, 1, 0, 33, 16, 5, 17] * 3, 64, 1088),                  # one large unit among small ones
 ])
 @pytest.mark.parametrize("with_rows", [True, False])
 def test_expert_ffn_at_the_edges_of_its_units(sizes, d, f, with_rows):
