@@ -155,8 +155,8 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const int n_tp = (p.T + 2 * kTile - 1) / (2 * kTile);             // tile pairs
   const bool two_acc = n_cols <= 256;
 
-  // Which of the weights' three bf16 terms hold anything (term 0 always counts).  A stage takes a k-block of x and of
-  // every such term, as long as three stages fit: x is then read once, not once per term.
+  // Which of the weights' three bf16 terms hold anything (term 0 always counts).  A term's products are added up over all
+  // k-blocks before the next term's: the order of the sums is part of the logits' last bits.
   const int any1 = p.split_any[1], any2 = p.split_any[2];
   if (threadIdx.x == 0) {
     for (int s = 0; s < kMaxStages; ++s) { tc::mbar_init(&full_bar[s], 1); tc::mbar_init(&empty_bar[s], 1); }
@@ -183,8 +183,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const uint32_t w_bytes = w1_bytes + w2_bytes;
   const int n_terms = 1 + (any1 != 0) + (any2 != 0);
   const int second = any1 != 0 ? 1 : 2;                             // term numbers: 0, second, 2
-  const int tps = p.op_bytes / (kXBytes + n_terms * w_bytes) >= 3 ? n_terms : 1;   // terms per stage
-  const uint32_t stage_bytes = kXBytes + tps * w_bytes;
+  const uint32_t stage_bytes = kXBytes + w_bytes;
   const int stages = min(kMaxStages, (int)(p.op_bytes / stage_bytes));
 
   if (warp == 0) {
@@ -195,19 +194,17 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
       bool ok = true;
       for (int tp = pair; tp < n_tp && ok; tp += n_pairs) {
         const int t0 = tp * 2 * kTile + rank * kTile;
-        for (int first = 0; first < n_terms && ok; first += tps) {
+        for (int i = 0; i < n_terms && ok; ++i) {
+          const int term = i == 0 ? 0 : i == 1 ? second : 2;
           for (int kb = 0; kb < kblocks; ++kb) {
             if (!tc::mbar_wait(&empty_bar[stage], phase ^ 1u, abort)) { route_timeout(p, abort, 11); ok = false; break; }
             uint8_t* sX = smem + (size_t)stage * stage_bytes;
             if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], 2 * stage_bytes);
             tc::tma_load_2d_pair(sX, &tmX, &full_bar[stage], kb * kBK, t0);
-            for (int i = 0; i < tps; ++i) {
-              const int term = first + i == 0 ? 0 : first + i == 1 ? second : 2;
-              uint8_t* sW = sX + kXBytes + i * w_bytes;
-              tc::tma_load_2d_pair(sW, &tmW1, &full_bar[stage], kb * kBK, term * M + rank * (p.n1 / 2));
-              if (p.n2 > 0)
-                tc::tma_load_2d_pair(sW + w1_bytes, &tmW2, &full_bar[stage], kb * kBK, term * M + p.n1 + rank * (p.n2 / 2));
-            }
+            uint8_t* sW = sX + kXBytes;
+            tc::tma_load_2d_pair(sW, &tmW1, &full_bar[stage], kb * kBK, term * M + rank * (p.n1 / 2));
+            if (p.n2 > 0)
+              tc::tma_load_2d_pair(sW + w1_bytes, &tmW2, &full_bar[stage], kb * kBK, term * M + p.n1 + rank * (p.n2 / 2));
             if (++stage == stages) { stage = 0; phase ^= 1u; }
           }
         }
@@ -219,8 +216,8 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     // ------------------------------------------------------------ MMA issuer (leader CTA only)
     // The MMAs of a router are narrow and the thread that issues them is what bounds the main loop: straight-line
     // groups of four, nothing decided in between.  128 tokens per CTA, 96 experts, d = 768, time to the complete
-    // accumulator: one term 12.4 -> 9.9 us, three terms 23.6 -> 14.1 us (with x read once; with x read three times and
-    // a branch per MMA both were as slow, loads were never the limit).
+    // accumulator: one term 12.4 -> 9.9 us.  (A stage with a k-block of x and of all three terms reads x once instead
+    // of three times and is no faster: loads are not the limit.)
     if (lane == 0 && rank == 0) {
       const uint32_t idesc1 = tc::instr_desc_bf16(p.n1, false, false, 256);
       const uint32_t idesc2 = tc::instr_desc_bf16(p.n2 > 0 ? p.n2 : 16, false, false, 256);
@@ -236,25 +233,23 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         if (!tc::mbar_wait(&tmem_empty[acc], acc_phase ^ 1u, abort)) { route_timeout(p, abort, 14); break; }
         tc::tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * 256;
-        for (int first = 0; first < n_terms && ok; first += tps) {
+        for (int i = 0; i < n_terms && ok; ++i) {
           for (int kb = 0; kb < kblocks; ++kb) {
             if (!tc::mbar_wait(&full_bar[stage], phase, abort)) { route_timeout(p, abort, 12); ok = false; break; }
             tc::tc_fence_after_sync();
             const uint32_t xaddr = tc::smem_u32(smem + (size_t)stage * stage_bytes);
             const uint64_t xdesc = tc::smem_desc_sw128(xaddr, 16, 1024);
-            uint32_t waddr = xaddr + kXBytes;
-            for (int i = 0; i < tps; ++i, waddr += w_bytes) {
-              const uint64_t wdesc = tc::smem_desc_sw128(waddr, 16, 1024);
-              const uint32_t more = (first | kb | i) != 0 ? 1u : 0u;
+            const uint32_t waddr = xaddr + kXBytes;
+            const uint64_t wdesc = tc::smem_desc_sw128(waddr, 16, 1024);
+            const uint32_t more = (i | kb) != 0 ? 1u : 0u;
+#pragma unroll
+            for (int j = 0; j < kBK / 16; ++j)
+              tc::umma_bf16_pair(d_tmem, xdesc + 2 * j, wdesc + 2 * j, idesc1, j > 0 ? 1u : more);
+            if (two_mma) {
+              const uint64_t wdesc2 = tc::smem_desc_sw128(waddr + w1_bytes, 16, 1024);
 #pragma unroll
               for (int j = 0; j < kBK / 16; ++j)
-                tc::umma_bf16_pair(d_tmem, xdesc + 2 * j, wdesc + 2 * j, idesc1, j > 0 ? 1u : more);
-              if (two_mma) {
-                const uint64_t wdesc2 = tc::smem_desc_sw128(waddr + w1_bytes, 16, 1024);
-#pragma unroll
-                for (int j = 0; j < kBK / 16; ++j)
-                  tc::umma_bf16_pair(d_tmem + 256, xdesc + 2 * j, wdesc2 + 2 * j, idesc2, j > 0 ? 1u : more);
-              }
+                tc::umma_bf16_pair(d_tmem + 256, xdesc + 2 * j, wdesc2 + 2 * j, idesc2, j > 0 ? 1u : more);
             }
             tc::umma_commit_pair(&empty_bar[stage], 3);
             if (++stage == stages) { stage = 0; phase ^= 1u; }
@@ -705,8 +700,7 @@ int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, fl
   const uint32_t budget = 227 * 1024 - 1024 - tail_bytes - kEpiWarps * kZStage;
   const int kblocks = d / kBK;
   // no more than the k-blocks of one tile with all three terms, between three and kMaxStages of them
-  const int most_stages = kblocks < 3 ? 3 : kblocks < kMaxStages ? kblocks : kMaxStages;
-  const uint32_t most = (uint32_t)most_stages * (kXBytes + 3u * (stage_bytes - kXBytes));
+  const uint32_t most = (uint32_t)kMaxStages * stage_bytes;
   p.op_bytes = (budget < most ? budget : most) / 1024 * 1024;
   UP_REQUIRE(p.op_bytes >= 2 * stage_bytes && ctx->sm_count >= 2, UNIPOOL_ERR_UNSUPPORTED,
              "router of %d experts does not fit the logits kernel", M);
