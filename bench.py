@@ -35,15 +35,26 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of a workload's dominant kernel,
-# from the ncu capture summarised in profiles/grouped_gemm_978m_slice_ncu.txt: the 978m_slice case (an
-# eighth of the experts and of the rows of one 978m layer) moved 733.9 + 207.8 MB; a full launch is eight
+# from the ncu capture summarised in profiles/wm_kernels_978m_slice_ncu.txt: the 978m_slice case (an
+# eighth of the experts and of the rows of one 978m layer) moved 637.8 + 201.2 MB; a full launch is eight
 # times that (weights and activations both grow with the units processed).
-NCU_TRAFFIC = {("978m", "expert_fwd_gu"): 8 * (733.89e6 + 207.79e6)}
+NCU_TRAFFIC = {("978m", "expert_fwd_gu"): 8 * (637.8e6 + 201.2e6)}
 
-# kernel behind each grouped-GEMM phase (for the roofline's `kernel` field) and launches of one dispatch-map call
-GEMM_KERNEL = {"expert_fwd_gu": "grouped_gemm_tc_kernel", "expert_fwd_down": "grouped_gemm_tc_kernel",
-               "dgrad_down": "grouped_gemm_tc_kernel", "dgrad_gu": "grouped_gemm_tc_kernel",
-               "wgrad_down": "wgrad_pair_kernel", "wgrad_gu": "wgrad_pair_kernel"}
+
+
+def gemm_kernel(phase, rows, d, f):
+    """Kernel behind a grouped-GEMM phase (for the roofline's `kernel` field): the library's rules on the rows a full
+    batch gives the average expert (weights_on_m and rows_on_pairs in csrc/expert_tc.cu)."""
+    if phase.startswith("wgrad"):
+        return "wgrad_pair_kernel"
+    on_m = {"expert_fwd_gu": (100 if d >= 1024 else 150) < rows <= (1024 if d >= 1024 else 600),
+            "expert_fwd_down": rows <= 450 and f > 1024,
+            "dgrad_down": rows <= 1200 and (rows <= 48 or rows > 100 or f > 1024),
+            "dgrad_gu": rows <= 450 and 2 * f > 1024}[phase]
+    return "wm_kernel" if on_m else "row_pair_kernel" if rows >= 512 else "grouped_gemm_tc_kernel"
+
+
+# launches of one dispatch-map call
 DISPATCH_MAP_LAUNCHES = 1
 
 METRIC = "moe_layer_fwd_bwd_tokens_per_s"
@@ -301,11 +312,7 @@ def measure_workload(name, args, world, rank, dev, full):
     gemm_ms = {n: kernels[n]["ms_per_step"] for n in GEMM_PHASES if n in kernels}
     dominant = max(gemm_ms, key=gemm_ms.get)
     dom = kernels[dominant]
-    # the library runs the row-tile GEMMs on CTA pairs when a full batch gives the average expert of a
-    # layer's view four row tiles of 128 rows
-    kernel_name = GEMM_KERNEL[dominant]
-    if kernel_name == "grouped_gemm_tc_kernel" and T * k >= 4 * 128 * mw:
-        kernel_name = "row_pair_kernel"
+    kernel_name = gemm_kernel(dominant, T * k // mw, d, f)
     # per launch of the dominant kernel: algorithmic bytes / FLOPs over its average CUDA-event duration
     if dom["bound"] == "hbm":
         roofline = dict(kernel=kernel_name + ":" + dominant, bound="hbm", achieved=dom["gbs"],

@@ -216,8 +216,8 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     // ------------------------------------------------------------ MMA issuer (leader CTA only)
     // The MMAs of a router are narrow and the thread that issues them is what bounds the main loop: straight-line
     // groups of four, nothing decided in between.  128 tokens per CTA, 96 experts, d = 768, time to the complete
-    // accumulator: one term 12.4 -> 9.9 us.  (A stage with a k-block of x and of all three terms reads x once instead
-    // of three times and is no faster: loads are not the limit.)
+    // accumulator: one term 12.4 -> 9.9 us.  (All three terms of a k-block in one stage would read x once; it
+    // gains at most 1 % of a forward pass and changes the order of the sums.)
     if (lane == 0 && rank == 0) {
       const uint32_t idesc1 = tc::instr_desc_bf16(p.n1, false, false, 256);
       const uint32_t idesc2 = tc::instr_desc_bf16(p.n2 > 0 ? p.n2 : 16, false, false, 256);
@@ -698,8 +698,6 @@ int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, fl
   const uint32_t tail_bytes = kTailBars + 2 * kTile * 2 * 4 + 2 * kTile * UNIPOOL_MAX_TOPK * 4 + UNIPOOL_MAX_EXPERTS * 4 +
                               kEpiWarps * M * 4 + (M + 31) / 32 * 32 * 4;
   const uint32_t budget = 227 * 1024 - 1024 - tail_bytes - kEpiWarps * kZStage;
-  const int kblocks = d / kBK;
-  // no more than the k-blocks of one tile with all three terms, between three and kMaxStages of them
   const uint32_t most = (uint32_t)kMaxStages * stage_bytes;
   p.op_bytes = (budget < most ? budget : most) / 1024 * 1024;
   UP_REQUIRE(p.op_bytes >= 2 * stage_bytes && ctx->sm_count >= 2, UNIPOOL_ERR_UNSUPPORTED,

@@ -339,7 +339,7 @@ def test_recomputed_layers_contract_in_runs(kw, L, T, accumulate):
 ])
 @pytest.mark.parametrize("bits", ["bf16", "fp32"])                # one or three bf16 terms of the router weights
 def test_bf16_router_at_the_edges_of_its_stages(T, M, d, k, bits):
-    """Selection with many candidates per lane, one and two MMAs per k-block, one or three weight terms per stage, fewer
+    """Selection with many candidates per lane, one and two MMAs per k-block, one or three weight terms, fewer
     k-blocks than stages; against the oracle in float64 as in the parity tests."""
     import torch
     from oracle import unipool_oracle as O
