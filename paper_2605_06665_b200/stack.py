@@ -196,7 +196,9 @@ class UniPoolStack:
     # ------------------------------------------------------------------ backward
     def backward_layer(self, l, dx_next, dx_out, T=None, with_aux=True, overwrite=False):
         """``overwrite``: this layer's weight gradient replaces what the pool-gradient
-        slices of its view hold (the first contribution of a step) instead of adding to it."""
+        slices of its view hold (the first contribution of a step) instead of adding to it.
+        (Without the group sizes: every pad row of ``dYp`` and ``dGU`` is then written with zeros, so that
+        a ``ctx.pool_wgrad`` over the padded groups can follow.)"""
         T = self.T if T is None else T
         c = self.ctx
         s = l if self.deferred_wgrad else 0
@@ -207,7 +209,7 @@ class UniPoolStack:
         c.expert_bwd(dx_next, T, self.row_of[l], self.gate[l], self.token_of[l], self.offsets[l],
                      self.tile_expert[l], self.Xp[a], self.GU[a], self.A[a], self.Yp[a], self.W_gu,
                      self.W_down, self.base(l), self.m, dx_next, self.dYp[s], self.dGU[s], dx_out,
-                     self.dgate, self.dW_gu, self.dW_down, flags, self.rows[l])
+                     self.dgate, self.dW_gu, self.dW_down, flags)
         coef = None
         if with_aux:
             coef = self.coef[l // self.Lg]

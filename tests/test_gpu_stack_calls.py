@@ -1,0 +1,42 @@
+"""The stack's public calls in the forms that its own step does not use: layer by layer, with arrays of the
+caller's, on small batches.  Each against the path that the parity tests compare with the oracle."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+def make(L, d, f, M, k, T, dtype="bf16", private=0, seed=0, **kw):
+    import torch
+    from paper_2605_06665_b200.stack import UniPoolStack
+    st = UniPoolStack(L, d, f, M, k, T, dtype, private, c=2.0, **kw)
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    for w in (st.W_gu, st.W_down, st.W_r):
+        w.normal_(0, 0.05, generator=g)
+    x0, up = (torch.empty(T, d, device="cuda").normal_(generator=g).to(st.tdtype) for _ in range(2))
+    return st, x0, up
+
+
+@pytest.mark.parametrize("f", [64, 1088])                         # dgrad down on the token-major and the weights-on-M kernels
+def test_backward_layer_leaves_operands_for_a_padded_weight_gradient(f):
+    """A weight gradient over the padded groups after backward_layer: what the pad rows of dYp and dGU held before
+    must not count.  Same sums as the step's own pass, which leaves the padding out: equal, bit for bit."""
+    import torch
+    from paper_2605_06665_b200 import binding as B
+    L, M = 3, 8
+    st, x0, up = make(L, 128, f, M, 2, 600, deferred_wgrad=True)
+    st.step(x0, up, accumulate=False)
+    want = [t.clone() for t in (st.dW_gu, st.dW_down, st.dx[L % 2])]
+    for t in (st.dYp, st.dGU):
+        t.fill_(float("nan"))
+    st.zero_router_grad()
+    dx = up
+    for l in reversed(range(L)):
+        out = torch.empty_like(dx)
+        st.backward_layer(l, dx, out)
+        dx = out
+    st.ctx.pool_wgrad(L, st.cap, st.offsets, st.Xp, st.A, st.dYp, st.dGU, 0, M, st.dW_gu, st.dW_down, B.WGRAD_OVERWRITE)
+    torch.cuda.synchronize()
+    st.ctx.check_status()
+    for got, ref in zip((st.dW_gu, st.dW_down, dx), want):
+        assert torch.equal(got, ref)
+    st.close()
