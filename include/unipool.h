@@ -211,7 +211,8 @@ int unipool_expert_fwd(unipool_ctx* ctx, const void* Xp, const int32_t* offsets,
  * multiplying its zeros, and the pad rows of dYp and dGU are written no further than the next multiple of 16
  * rows of a group (with zeros; what the others hold is unspecified).  Results are those of the calls without
  * `rows`, which these are when it is NULL: the backward and the pool_wgrad call of a layer are given `rows` both
- * or neither.  `rows` must be what the dispatch of the same layer wrote. */
+ * or neither.  unipool_expert_fwd_rows must be given what the dispatch of the same layer wrote;
+ * unipool_expert_bwd_rows counts the groups in token_of and writes `rows` again (T > 0), for the pool_wgrad call. */
 int unipool_dispatch_rows(unipool_ctx* ctx, const void* x, int32_t T, const int32_t* idx,
                           int32_t n_experts, int32_t* offsets, int32_t* row_of, int32_t* token_of,
                           int32_t* tile_expert, int32_t* rows, void* Xp, unipool_stream stream);
@@ -221,7 +222,7 @@ int unipool_expert_fwd_rows(unipool_ctx* ctx, const void* Xp, const int32_t* off
                             unipool_stream stream);
 int unipool_expert_bwd_rows(unipool_ctx* ctx, const void* dy, int32_t T, const int32_t* row_of,
                             const float* gate, const int32_t* token_of, const int32_t* offsets,
-                            const int32_t* rows, const int32_t* tile_expert, const void* Xp, const void* GU,
+                            int32_t* rows, const int32_t* tile_expert, const void* Xp, const void* GU,
                             const void* A, const void* Yp, const void* W_gu, const void* W_down,
                             int32_t expert_base, int32_t n_experts, const void* dx_residual, void* dYp,
                             void* dGU, void* dx, float* dgate, float* dW_gu, float* dW_down, int32_t flags,

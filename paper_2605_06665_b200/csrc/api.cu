@@ -300,7 +300,7 @@ int unipool_combine(unipool_ctx* ctx, const void* Yp, const int32_t* row_of, con
 }
 
 int unipool_expert_bwd_rows(unipool_ctx* ctx, const void* dy, int32_t T, const int32_t* row_of,
-                       const float* gate, const int32_t* token_of, const int32_t* offsets, const int32_t* rows,
+                       const float* gate, const int32_t* token_of, const int32_t* offsets, int32_t* rows,
                        const int32_t* tile_expert, const void* Xp, const void* GU, const void* A,
                        const void* Yp, const void* W_gu, const void* W_down, int32_t expert_base,
                        int32_t n_experts, const void* dx_residual, void* dYp, void* dGU, void* dx,

@@ -157,7 +157,7 @@ int combine_launch(unipool_ctx*, const void* Yp, const int32_t* row_of, const fl
 // (1501 tokens over 96 experts of 768 x 2048, 31 rows in 128: scaling dY 14.6 -> 8.8 us, dgrad down 80 -> 71 us).
 constexpr int kRowStep = 16;
 int combine_bwd_launch(unipool_ctx*, const void* dy, int T, const int32_t* row_of,
-                       const float* gate, const int32_t* token_of, const int32_t* offsets, const int32_t* rows,
+                       const float* gate, const int32_t* token_of, const int32_t* offsets, int32_t* rows,
                        int n_experts, const void* Yp, void* dYp, float* dgate, cudaStream_t);
 int unpermute_sum_launch(unipool_ctx*, const void* dXp, const int32_t* row_of, int T,
                          const void* residual, void* dx, cudaStream_t);

@@ -354,8 +354,9 @@ combine_kernel(const uint4* __restrict__ Yp, const int32_t* __restrict__ row_of,
 
 // Backward of the combine, token-major: for token t and slot j with row r = row_of[t,j]
 //   dgate[t,j] = <dy[t], Yp[r]>,   dYp[r] = gate[t,j] * dy[t];
-// afterwards the pad rows (token_of < 0) below offsets[M] are zeroed, given the group sizes only those up to the next
-// multiple of kRowStep rows.  A warp takes KT slots of one
+// the pad rows (token_of < 0) below offsets[M] are zeroed afterwards; with group_rows, by further warps beside the
+// tokens', only those up to the next multiple of pad_step rows, and the group sizes are counted in token_of and
+// written there: what the array holds on entry may belong to another permute.  A warp takes KT slots of one
 // token; with k > KT the token's slots are split over ceil(k / KT) warps (each re-reads dy[t], which
 // keeps the registers per thread low enough for four resident blocks per SM).
 template <typename T, int KT>
@@ -363,12 +364,29 @@ __global__ void __launch_bounds__(256, 4)
 combine_bwd_kernel(const uint4* __restrict__ dy, const uint4* __restrict__ Yp,
                    const int32_t* __restrict__ row_of, const float* __restrict__ gate,
                    const int32_t* __restrict__ token_of, const int32_t* __restrict__ offsets,
-                   const int32_t* __restrict__ group_rows, int M, uint4* __restrict__ dYp, float* __restrict__ dgate, int n_tokens, int k, int row_vecs) {
+                   int32_t* __restrict__ group_rows, int pad_step, int M, uint4* __restrict__ dYp,
+                   float* __restrict__ dgate, int n_tokens, int k, int row_vecs) {
   constexpr int N = Vec16<T>::N;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int groups = (k + KT - 1) / KT;
   const int n_items = n_tokens * groups;                 // < 2^30: T * k is
-  for (int item = blockIdx.x * 8 + warp; item < n_items; item += gridDim.x * 8) {
+  const int n_pads = group_rows != nullptr ? M * pad_step : 0;
+  for (int item = blockIdx.x * 8 + warp; item < n_items + n_pads; item += gridDim.x * 8) {
+    if (item >= n_items) {
+      const int p = item - n_items, e = p / pad_step, i = p % pad_step, end = offsets[e + 1];
+      int n = end - offsets[e];                          // the padding lies in the group's last 128 rows
+      if (n > 0) {
+        const int32_t* tail = token_of + end - UNIPOOL_ROW_ALIGN;
+        n -= UNIPOOL_ROW_ALIGN;
+#pragma unroll
+        for (int q = 0; q < UNIPOOL_ROW_ALIGN / 32; ++q) n += __popc(__ballot_sync(0xffffffffu, tail[32 * q + lane] >= 0));
+      }
+      if (i == 0 && lane == 0) group_rows[e] = n;
+      if (i >= (-n & (pad_step - 1))) continue;
+      uint4* dst = dYp + (int64_t)(offsets[e] + n + i) * row_vecs;
+      for (int v = lane; v < row_vecs; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
+      continue;
+    }
     const int t = groups == 1 ? item : item / groups, j0 = groups == 1 ? 0 : (item % groups) * KT;
     int rows[KT];
     float g[KT], dot[KT];
@@ -416,15 +434,7 @@ combine_bwd_kernel(const uint4* __restrict__ dy, const uint4* __restrict__ Yp,
       if (lane == 0 && j0 + j < k) dgate[(int64_t)t * k + j0 + j] = dot[j];
     }
   }
-  if (group_rows != nullptr) {
-    for (int p = blockIdx.x * 8 + warp; p < M * kRowStep; p += gridDim.x * 8) {
-      const int e = p / kRowStep, n = group_rows[e], i = p % kRowStep;
-      if (i >= (-n & (kRowStep - 1))) continue;
-      uint4* dst = dYp + (int64_t)(offsets[e] + n + i) * row_vecs;
-      for (int v = lane; v < row_vecs; v += 32) dst[v] = make_uint4(0, 0, 0, 0);
-    }
-    return;
-  }
+  if (group_rows != nullptr) return;
   const int used = offsets[M];
   for (int r = blockIdx.x * 8 + warp; r < used; r += gridDim.x * 8) {
     if (token_of[r] >= 0) continue;
@@ -539,27 +549,30 @@ int combine_launch(unipool_ctx* ctx, const void* Yp, const int32_t* row_of, cons
 template <typename T>
 static void combine_bwd_dispatch_k(int grid, cudaStream_t s, int k, const void* dy, const void* Yp,
                                    const int32_t* row_of, const float* gate, const int32_t* token_of,
-                                   const int32_t* offsets, const int32_t* rows, int M, void* dYp, float* dgate,
+                                   const int32_t* offsets, int32_t* rows, int M, void* dYp, float* dgate,
                                    int n_tokens, int row_vecs) {
+  constexpr int step = sizeof(T) == 2 ? kRowStep : UNIPOOL_ROW_ALIGN;       // (the fp32 kernels read whole groups)
   auto D = static_cast<const uint4*>(dy);
   auto Y = static_cast<const uint4*>(Yp);
   auto O = static_cast<uint4*>(dYp);
-  if (k <= 1) combine_bwd_kernel<T, 1><<<grid, 256, 0, s>>>(D, Y, row_of, gate, token_of, offsets, rows, M, O, dgate, n_tokens, k, row_vecs);
-  else combine_bwd_kernel<T, 2><<<grid, 256, 0, s>>>(D, Y, row_of, gate, token_of, offsets, rows, M, O, dgate, n_tokens, k, row_vecs);
+  if (k <= 1) combine_bwd_kernel<T, 1><<<grid, 256, 0, s>>>(D, Y, row_of, gate, token_of, offsets, rows, step, M, O, dgate, n_tokens, k, row_vecs);
+  else combine_bwd_kernel<T, 2><<<grid, 256, 0, s>>>(D, Y, row_of, gate, token_of, offsets, rows, step, M, O, dgate, n_tokens, k, row_vecs);
 }
 
 int combine_bwd_launch(unipool_ctx* ctx, const void* dy, int T, const int32_t* row_of,
-                       const float* gate, const int32_t* token_of, const int32_t* offsets, const int32_t* rows, int M,
+                       const float* gate, const int32_t* token_of, const int32_t* offsets, int32_t* rows, int M,
                        const void* Yp, void* dYp, float* dgate, cudaStream_t s) {
   if (T == 0) return UNIPOOL_OK;
   const int k = ctx->cfg.top_k;
   const int row_vecs = (int)((size_t)ctx->cfg.d_model * ctx->elem_bytes / 16);
-  const int grid = row_mover_grid(ctx, (int64_t)T * ((k + 1) / 2));     // one warp per token and pair of slots
+  // one warp per token and pair of slots, and per pad row that is to be looked at
+  const int64_t pads = rows == nullptr ? 0 : (int64_t)M * (ctx->cfg.dtype == UNIPOOL_BF16 ? kRowStep : UNIPOOL_ROW_ALIGN);
+  const int grid = row_mover_grid(ctx, (int64_t)T * ((k + 1) / 2) + pads);
   PhaseTimer pt(ctx, UNIPOOL_PH_BWD_SCALE_GATHER, 1, s);
   if (ctx->cfg.dtype == UNIPOOL_BF16)
     combine_bwd_dispatch_k<__nv_bfloat16>(grid, s, k, dy, Yp, row_of, gate, token_of, offsets, rows, M, dYp, dgate, T, row_vecs);
   else
-    combine_bwd_dispatch_k<float>(grid, s, k, dy, Yp, row_of, gate, token_of, offsets, nullptr, M, dYp, dgate, T, row_vecs);
+    combine_bwd_dispatch_k<float>(grid, s, k, dy, Yp, row_of, gate, token_of, offsets, rows, M, dYp, dgate, T, row_vecs);
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;
 }

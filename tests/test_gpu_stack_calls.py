@@ -40,3 +40,38 @@ def test_backward_layer_leaves_operands_for_a_padded_weight_gradient(f):
     for got, ref in zip((st.dW_gu, st.dW_down, dx), want):
         assert torch.equal(got, ref)
     st.close()
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+def test_backward_after_a_permute_without_group_sizes(dtype):
+    """A caller re-routes tokens and permutes them through the context, without the stack's array of group sizes: the
+    backward pass counts the groups itself.  Same result, bit for bit, as with the sizes of that permute."""
+    import torch
+    L, M, T, k = 2, 9, 700, 2
+    got = []
+    for with_rows in (True, False):
+        st, x0, up = make(L, 128, 192, M, k, T, dtype, deferred_wgrad=True)
+        st.forward(x0)                                            # leaves other sizes behind
+        idx = torch.randint(0, M, (L, T, 1), generator=torch.Generator().manual_seed(1), dtype=torch.int32)
+        st.idx.copy_(torch.cat([idx, (idx + 1) % M], 2))
+        st.rows.fill_(3) if not with_rows else None
+        for l in range(L):
+            c = st.ctx
+            rows = st.rows[l] if with_rows else None
+            c.dispatch(st.x[l], T, st.idx[l], M, st.offsets[l], st.row_of[l], st.token_of[l], st.tile_expert[l], st.Xp[l], rows)
+            c.expert_fwd(st.Xp[l], st.offsets[l], st.tile_expert[l], st.W_gu, st.W_down, 0, M, st.GU[l], st.A[l], st.Yp[l], rows)
+            c.combine(st.Yp[l], st.row_of[l], st.gate[l], T, st.x[l], st.x[l + 1])
+        st.aux_loss()
+        st.zero_router_grad()
+        dx = st.backward(up, accumulate=False)
+        torch.cuda.synchronize()
+        st.ctx.check_status()
+        assert (st.rows.cpu() == torch.stack([st.idx[l].flatten().bincount(minlength=M) for l in range(L)]).cpu()).all()
+        got.append([t.clone() for t in (dx, st.dW_gu, st.dW_down, st.dW_r)])
+        st.close()
+    for a, b in zip(*got):
+        assert a.isfinite().all()
+        if a.shape == (L, M, 128):                                # dW_r: blocks of tokens add with atomics, in any order
+            assert (a - b).abs().max() <= 1e-5 * b.abs().max()
+        else:
+            assert torch.equal(a, b)
