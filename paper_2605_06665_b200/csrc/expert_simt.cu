@@ -163,7 +163,7 @@ int rows_gemm_as(const unipool_ctx* ctx, RowGemm p, cudaStream_t s) {
 
 template <Major BM, RowEpilogue EPI>
 int rows_gemm(unipool_ctx* ctx, RowGemm p, int n_experts, cudaStream_t s) {
-  p.vec = aligned16(p.A, p.B);
+  p.vec = aligned16(p.A, p.B, p.C, p.C2, p.GU);    // those that the epilogue has not are NULL
   // 64 x 64 tiles of a full batch (a group ends on half a tile).  Many: whole tiles, one group of threads on each, two
   // on a long contraction; fewer: two groups, and half tiles where the weights are read across K; few: half tiles,
   // two or four groups.  In us, TM = 64 with 1 / 2 / 4 groups, 32 with 1 / 2 / 4 (16 experts of 256 x 512, 64 rows each):

@@ -75,3 +75,36 @@ def test_backward_after_a_permute_without_group_sizes(dtype):
             assert (a - b).abs().max() <= 1e-5 * b.abs().max()
         else:
             assert torch.equal(a, b)
+
+
+def test_fp32_expert_ffn_with_unaligned_results_beside_aligned_operands():
+    """fp32 mode: GU, A and dGU that are not 16-byte aligned, with Xp, dYp and weights that are.  Scalar accesses, the
+    same sums: equal to the aligned buffers', bit for bit."""
+    import torch
+    from paper_2605_06665_b200 import binding as B
+    d, f, M, T = 64, 128, 5, 400
+    g = torch.Generator(device="cuda").manual_seed(5)
+    rnd = lambda *s: torch.empty(*s, device="cuda").normal_(0, 0.1, generator=g)
+    x, dy, Wgu, Wd, gate = rnd(T, d), rnd(T, d), rnd(M, 2 * f, d), rnd(M, d, f), rnd(T, 1)
+    idx = torch.randint(0, M, (T, 1), device="cuda", generator=g, dtype=torch.int32)
+    out = []
+    for shift in (0, 1):
+        ctx = B.Context(B.make_config(d, f, M, 1, 1, T, B.FP32, 1e-6, 2.0))
+        cap = ctx.row_capacity
+        new = lambda w: torch.zeros(cap * w + 4, device="cuda")[shift:shift + cap * w].view(cap, w)
+        i32 = dict(dtype=torch.int32, device="cuda")
+        off, row_of, tok, te, rows = (torch.empty(s, **i32) for s in ((M + 1,), (T, 1), (cap,), (cap // 128,), (M,)))
+        Xp, Yp, dYp = (torch.zeros(cap, d, device="cuda") for _ in range(3))
+        GU, A, dGU, dx, dgate = new(2 * f), new(f), new(2 * f), torch.empty(T, d, device="cuda"), torch.empty(T, 1, device="cuda")
+        dWgu, dWd = torch.empty_like(Wgu), torch.empty_like(Wd)
+        ctx.dispatch(x, T, idx, M, off, row_of, tok, te, Xp, rows)
+        ctx.expert_fwd(Xp, off, te, Wgu, Wd, 0, M, GU, A, Yp, rows)
+        ctx.expert_bwd(dy, T, row_of, gate, tok, off, te, Xp, GU, A, Yp, Wgu, Wd, 0, M, None, dYp, dGU, dx, dgate, dWgu, dWd,
+                       B.WGRAD_OVERWRITE, rows)
+        torch.cuda.synchronize()
+        ctx.check_status()
+        ctx.close()
+        assert (GU.data_ptr() % 16 != 0) == bool(shift)
+        out.append((GU, A, Yp, dGU, dx, dWgu, dWd))
+    for a, b in zip(*out):
+        assert a.abs().max() > 0 and torch.equal(a, b)
