@@ -186,10 +186,14 @@ class UniPoolStack:
         return self.x[self.L]
 
     def aux_loss(self, T=None, fbar_prev=None, replicas=1):
-        """``replicas``: the statistics were summed over this many data-parallel replicas of T tokens."""
+        """``replicas``: the statistics were summed over this many data-parallel replicas of T tokens.
+        ``fbar_prev`` [groups, m] ([m] with one group)."""
         T = (self.T if T is None else T) * replicas
         if fbar_prev is not None:
-            fbar_prev = fbar_prev.contiguous()             # [groups, m]
+            fbar_prev = fbar_prev.reshape(1 if fbar_prev.dim() == 1 else len(fbar_prev), -1)[:self.G, :self.m]
+            if fbar_prev.shape != self.fbar.shape:
+                raise IndexError(f"fbar_prev must hold {self.G} groups of {self.m} token fractions")
+            fbar_prev = fbar_prev.to(self.device, torch.float32).contiguous()
         self.ctx.stack_aux_loss(self._arrays(), T, self.alpha, fbar_prev)
         return self.loss
 

@@ -108,3 +108,28 @@ def test_fp32_expert_ffn_with_unaligned_results_beside_aligned_operands():
         out.append((GU, A, Yp, dGU, dx, dWgu, dWd))
     for a, b in zip(*out):
         assert a.abs().max() > 0 and torch.equal(a, b)
+
+
+def test_previous_fractions_are_taken_per_group():
+    """f-bar of the previous micro-batch: one row per sharing group, dense or not; too few are refused."""
+    import torch
+    L, G, M = 4, 2, 16
+    st, x0, _ = make(L, 64, 64, M, 2, 200, groups=G)
+    st.forward(x0)
+    prev = torch.rand(G, M // G, device="cuda", generator=torch.Generator(device="cuda").manual_seed(1))
+    want = []
+    for g in range(G):                                            # the call of one group
+        loss, coef, fbar = torch.empty(1, device="cuda"), torch.empty(M // G, device="cuda"), torch.empty(M // G, device="cuda")
+        l = slice(g * st.Lg, (g + 1) * st.Lg)
+        st.ctx.pool_aux_loss(st.counts[l], st.score_sum[l], st.Lg, st.m, st.T, st.alpha, prev[g].contiguous(), loss, coef, fbar)
+        want.append((loss, coef))
+    wide = torch.cat([prev, prev + 1], 1)
+    for form in (prev, prev.T.contiguous().T, wide[:, :M // G], wide, torch.cat([prev, prev]), prev.double(), prev.cpu()):
+        st.loss.fill_(-1)
+        st.aux_loss(fbar_prev=form)
+        for g, (loss, coef) in enumerate(want):
+            assert torch.equal(st.loss[g:g + 1], loss) and torch.equal(st.coef[g], coef)
+    for bad in (prev[0], prev[:1], prev[:, :4], prev.flatten()):
+        with pytest.raises(IndexError):
+            st.aux_loss(fbar_prev=bad)
+    st.close()
