@@ -4,7 +4,9 @@
 the library calls route -> dispatch -> expert_fwd -> combine (forward), then
 pool_aux_loss, then expert_bwd -> route_bwd per layer in reverse (backward).
 (``forward``, ``aux_loss`` and ``backward`` issue these calls for all layers from one native call
-each, ``forward_layer`` and ``backward_layer`` one layer's from Python.)
+each, ``forward_layer`` and ``backward_layer`` one layer's from Python.  The native calls take arrays
+stacked over the layers as the constructor makes them; with others - a bias expanded over the layers or a
+list of them, gradients that are slices of a larger buffer - the layers are issued one by one.)
 It contains no arithmetic of its own: every tensor it returns was written by a
 CUDA kernel of the library.
 
@@ -102,6 +104,7 @@ class UniPoolStack:
         self.fbar = e(n_aux, self.m, dtype=f32)
         self.fbar_lag = None                               # f-bar of the previous micro-batch (App. G)
         self._copy_stream = None                           # host <-> device copies beside the compute
+        self._stacked = [(n, getattr(self, n).numel()) for n in B.Stack.POINTERS if n not in ("sigma", "bias")]
 
     def _wgrad_layers(self):
         """Layers whose weight gradients are contracted together when activations are recomputed.  Each
@@ -145,24 +148,43 @@ class UniPoolStack:
         self.dW_r.zero_(); self.dsigma.zero_()
 
     def _arrays(self):
-        """This stack's arrays as they are now, for the calls that run all layers."""
+        """This stack's arrays as they are now, for the calls that run all layers; None if one of them is not
+        a dense array over the layers."""
         wgrad = self.Lg if self.deferred_wgrad else self.nw
-        sigma = (ctypes.c_float * self.L)(*self.sigma)
         s = B.Stack(self.L, self.Lg, self.m, int(self.recompute), wgrad)
-        for n in B.Stack.POINTERS:
-            if n != "sigma":
-                t = getattr(self, n)
-                setattr(s, n, None if t is None else t.data_ptr())
-        s.sigma = ctypes.addressof(sigma)
-        s.keep = sigma                                     # lives as long as the struct
+        for n, numel in self._stacked:
+            t = getattr(self, n)
+            if not t.is_contiguous() or t.numel() != numel:
+                return None
+            setattr(s, n, t.data_ptr())
+        b = self.bias
+        if b is not None:
+            if not (isinstance(b, torch.Tensor) and b.is_cuda and b.dtype is torch.float32 and b.is_contiguous()
+                    and b.shape == (self.L, self.m)):
+                return None
+            s.bias = b.data_ptr()
+        s.keep = (ctypes.c_float * self.L)(*[self.sigma[l] for l in range(self.L)])    # lives as long as the struct
+        s.sigma = ctypes.addressof(s.keep)
         return s
+
+    def _router_prepare(self):
+        """The routers' bf16 terms of all layers, or none where the weights are not one array."""
+        shape = (self.L, self.m, self.d)
+        one = isinstance(self.W_r, torch.Tensor) and self.W_r.shape == shape and self.W_r.is_contiguous()
+        self.ctx.router_prepare(self.W_r if one else None, self.L if one else 0, self.m)
+
+    def _bias(self, l):
+        """Layer l's logit bias as the router reads it: m floats in a row on the device."""
+        b = None if self.bias is None else self.bias[l]
+        if b is not None and b.numel() != self.m:
+            raise ValueError(f"layer {l}: a bias of {b.numel()} values for {self.m} experts")
+        return None if b is None else b.to(self.device, torch.float32).contiguous()
 
     # ------------------------------------------------------------------ forward
     def forward_layer(self, l, T=None):
         T = self.T if T is None else T
         c = self.ctx
-        bias = None if self.bias is None else self.bias[l]
-        c.route(self.x[l], T, self.W_r[l], self.sigma[l], bias, self.m, self.idx[l], self.gate[l],
+        c.route(self.x[l], T, self.W_r[l], self.sigma[l], self._bias(l), self.m, self.idx[l], self.gate[l],
                 self.counts[l], self.score_sum[l], self.znorm[l], self.z[l])
         self.permute_and_experts(l, T)
         c.combine(self.Yp[self.slot(l)], self.row_of[l], self.gate[l], T, self.x[l], self.x[l + 1])
@@ -182,7 +204,13 @@ class UniPoolStack:
             self.x[0, :T].copy_(x0, non_blocking=True)
         # (the routers' weights may have changed since the last pass: their bf16 terms are formed anew, used by
         # this forward pass and by the backward pass that follows it)
-        self.ctx.stack_forward(self._arrays(), T)
+        arrays = self._arrays()
+        if arrays is not None:
+            self.ctx.stack_forward(arrays, T)
+        else:
+            self._router_prepare()
+            for l in range(self.L):
+                self.forward_layer(l, T)
         return self.x[self.L]
 
     def aux_loss(self, T=None, fbar_prev=None, replicas=1):
@@ -194,7 +222,15 @@ class UniPoolStack:
             if fbar_prev.shape != self.fbar.shape:
                 raise IndexError(f"fbar_prev must hold {self.G} groups of {self.m} token fractions")
             fbar_prev = fbar_prev.to(self.device, torch.float32).contiguous()
-        self.ctx.stack_aux_loss(self._arrays(), T, self.alpha, fbar_prev)
+        arrays = self._arrays()
+        if arrays is not None:
+            self.ctx.stack_aux_loss(arrays, T, self.alpha, fbar_prev)
+            return self.loss
+        for g in range(self.G):
+            l0 = g * self.Lg
+            self.ctx.pool_aux_loss(self.counts[l0:l0 + self.Lg], self.score_sum[l0:l0 + self.Lg], self.Lg, self.m, T,
+                                   self.alpha, None if fbar_prev is None else fbar_prev[g],
+                                   self.loss[g:g + 1], self.coef[g], self.fbar[g])
         return self.loss
 
     # ------------------------------------------------------------------ backward
@@ -232,17 +268,28 @@ class UniPoolStack:
         flags = (0 if accumulate else B.WGRAD_OVERWRITE) | (0 if with_aux else B.STACK_NO_AUX)
         if exchange is not None:
             flags |= B.STACK_LEAVE_WGRAD
-        self.ctx.stack_backward(self._arrays(), T, flags)
-        if self.deferred_wgrad and exchange is not None:
+        arrays = self._arrays()
+        if arrays is not None:
+            self.ctx.stack_backward(arrays, T, flags)
+        else:
+            for l in reversed(range(self.L)):
+                cur = (self.L - 1 - l) % 2
+                first = (not accumulate) and l % self.Lg == self.Lg - 1     # first contribution to its group's experts
+                self.backward_layer(l, self.dx[cur], self.dx[1 - cur], T, with_aux, overwrite=first)
+        if self.deferred_wgrad and (exchange is not None or arrays is None):
             for g in range(self.G):                        # one pass per sharing group over its layers
                 l0 = g * self.Lg
                 flags = 0 if accumulate else B.WGRAD_OVERWRITE
                 args = (self.Lg, self.cap, self.offsets[l0:], self.Xp[l0:], self.A[l0:], self.dYp[l0:],
                         self.dGU[l0:], g * self.m, self.m)
+                rows = None if arrays is None else self.rows[l0:]           # as the layers' backward had them
+                if exchange is None:
+                    self.ctx.pool_wgrad(*args, self.dW_gu, self.dW_down, flags, rows)
+                    continue
                 e0, e1 = g * self.m, (g + 1) * self.m
-                self.ctx.pool_wgrad(*args, None, self.dW_down, flags, self.rows[l0:])
+                self.ctx.pool_wgrad(*args, None, self.dW_down, flags, rows)
                 exchange.launch([self.dW_down[e0:e1]])
-                self.ctx.pool_wgrad(*args, self.dW_gu, None, flags, self.rows[l0:])
+                self.ctx.pool_wgrad(*args, self.dW_gu, None, flags, rows)
                 exchange.launch([self.dW_gu[e0:e1]])
         if exchange is not None:
             if not self.deferred_wgrad:

@@ -133,3 +133,68 @@ def test_previous_fractions_are_taken_per_group():
         with pytest.raises(IndexError):
             st.aux_loss(fbar_prev=bad)
     st.close()
+
+
+NAMES = ("x", "dx", "loss", "idx", "gate", "z", "dW_gu", "dW_down", "dW_r", "dsigma")
+
+
+def same(got, want, other_order=("dW_r",)):
+    """Equal bit for bit, but for sums that are taken in another order: dW_r always (its blocks add with atomics), fp32
+    sums of some hundred terms, random signs: 1e-5 of the largest value."""
+    import torch
+    for n, a, w in zip(NAMES, got, want):
+        if n in other_order:
+            assert (a.double() - w.double()).abs().max() <= 1e-5 * w.double().abs().max(), n
+        else:
+            assert torch.equal(a, w), n
+
+
+def stack_results(st, x0, up):
+    import torch
+    dx = st.step(x0, up, accumulate=False)
+    torch.cuda.synchronize()
+    st.ctx.check_status()
+    return [t.clone() for t in (st.x[st.L], dx, st.loss, st.idx, st.gate, st.z, st.dW_gu, st.dW_down, st.dW_r, st.dsigma)]
+
+
+BIAS_FORMS = dict(
+    expanded=lambda b: b[0].expand(*b.shape), list=list, tuple_with_none=lambda b: (None,) + tuple(b[1:]),
+    transposed=lambda b: b.T.contiguous().T, slice_of_a_wider=lambda b: b.repeat(1, 2)[:, :b.shape[1]],
+    double=lambda b: b.double(), host=lambda b: b.cpu())
+
+
+@pytest.mark.parametrize("form", sorted(BIAS_FORMS))
+@pytest.mark.parametrize("kw", [dict(deferred_wgrad=True), dict(recompute=True), dict(dtype="fp32")])
+def test_bias_in_other_forms_than_one_dense_array(form, kw):
+    """A bias whose layers are not the rows of one dense float array gives what the dense array of the same values gives."""
+    import torch
+    L, M = 3, 10
+    st, x0, up = make(L, 64, 128, M, 2, 150, **kw)
+    b = torch.empty(L, M, device="cuda").normal_(generator=torch.Generator(device="cuda").manual_seed(1))
+    given = BIAS_FORMS[form](b)
+    st.bias = torch.stack([torch.zeros(M, device="cuda") if v is None else v.cuda().float() for v in given])
+    want = stack_results(st, x0, up)
+    st.bias = given
+    got = stack_results(st, x0, up)
+    # recompute: layer by layer instead of in runs of layers; fp32: whole groups instead of their tokens
+    same(got, want, ("dW_r", "dW_gu", "dW_down") if "recompute" in kw or "dtype" in kw else ("dW_r",))
+    st.bias = [b[0, :4]] * L
+    with pytest.raises(ValueError):
+        st.forward(x0)
+    st.close()
+
+
+def test_arrays_of_the_caller_that_are_slices_of_larger_ones():
+    """Activations, logits and gradients that the caller keeps in padded arrays of its own; too few scales are refused."""
+    import torch
+    L, M, d, T = 3, 8, 64, 150
+    st, x0, up = make(L, d, 128, M, 2, T, deferred_wgrad=True)
+    want = stack_results(st, x0, up)
+    st.dW_r = torch.zeros(L, M + 2, d, device="cuda")[:, :M]
+    st.z = torch.zeros(L, T + 1, M, device="cuda")[:, :T]
+    st.x = torch.zeros(L + 1, T + 8, d, dtype=st.tdtype, device="cuda")[:, :T]
+    same(stack_results(st, x0, up), want)
+    st.sigma = st.sigma[:2]
+    with pytest.raises(IndexError):
+        st.forward(x0)
+    st.close()
