@@ -33,7 +33,8 @@ from . import binding as B
 
 class UniPoolStack:
     def __init__(self, L, d, f, M, k, T, dtype="bf16", private=0, c=1.0, eps=1e-6, alpha=1e-2,
-                 device="cuda", deferred_wgrad=False, recompute=False, groups=None, router="norm"):
+                 device="cuda", deferred_wgrad=False, recompute=False, groups=None, router="norm",
+                 wgrad_layers=None):
         self.L, self.d, self.f, self.M, self.k, self.T = L, d, f, M, k, T
         if groups is None:
             groups = L if private else 1
@@ -46,8 +47,11 @@ class UniPoolStack:
         self.c, self.eps = c, eps
         # recompute: keep only x_l and the routing state of a layer; its permuted activations are
         # rebuilt in backward (MoE-layer activation recompute, App. D), so the weight gradient is
-        # taken for the few layers whose operands are held at a time (see _wgrad_layers)
+        # taken for the few layers whose operands are held at a time: ``wgrad_layers`` of them (1: one
+        # shared slot, the least memory), by default as _wgrad_layers says or one if those do not fit
         self.recompute = recompute
+        if wgrad_layers is not None and not (recompute and 1 <= wgrad_layers <= self.Lg):
+            raise ValueError("wgrad_layers: 1 to the layers of a sharing group, with recompute")
         self.deferred_wgrad = deferred_wgrad and self.Lg > 1 and not recompute
         self.device = torch.device(device)
         self.tdtype = torch.bfloat16 if dtype == "bf16" else torch.float32
@@ -87,14 +91,8 @@ class UniPoolStack:
         self.token_of = e(L, cap, dtype=i32)
         self.tile_expert = e(L, cap // B.ROW_ALIGN, dtype=i32)
         ns = 1 if recompute else L                         # layers whose permuted activations are kept
-        self.nw = self._wgrad_layers() if recompute else 1
-        self.Xp = e(max(ns, self.nw), cap, d)
         self.GU = e(ns, cap, 2 * f)
-        self.A = e(max(ns, self.nw), cap, f)
         self.Yp = e(ns, cap, d)
-        nb = L if self.deferred_wgrad else self.nw
-        self.dYp = e(nb, cap, d)
-        self.dGU = e(nb, cap, 2 * f)
         self.dx = e(2, T, d)                               # ping-pong dx_{l+1} -> dx_l
         self.dgate = e(T, k, dtype=f32)
         # balance loss
@@ -104,14 +102,32 @@ class UniPoolStack:
         self.fbar = e(n_aux, self.m, dtype=f32)
         self.fbar_lag = None                               # f-bar of the previous micro-batch (App. G)
         self._copy_stream = None                           # host <-> device copies beside the compute
+        # operands of the weight gradient
+        self.nw = 1 if not recompute else wgrad_layers or self._wgrad_layers()
+        try:
+            self._make_operands(e)
+        except torch.OutOfMemoryError:
+            if wgrad_layers or self.nw == 1:
+                raise
+            self.nw = 1
+            self._make_operands(e)
         self._stacked = [(n, getattr(self, n).numel()) for n in B.Stack.POINTERS if n not in ("sigma", "bias")]
+
+    def _make_operands(self, e):
+        self.Xp = self.A = self.dYp = self.dGU = None
+        ns = self.nw if self.recompute else self.L
+        nb = self.L if self.deferred_wgrad else self.nw
+        self.Xp, self.A = e(ns, self.cap, self.d), e(ns, self.cap, self.f)
+        self.dYp, self.dGU = e(nb, self.cap, self.d), e(nb, self.cap, 2 * self.f)
 
     def _wgrad_layers(self):
         """Layers whose weight gradients are contracted together when activations are recomputed.  Each
         contraction reads and writes the whole fp32 pool gradient (2.2 + 4.4 ms per layer at 192 experts
         of 1536 x 4096, 65536 rows, against 1.8 + 3.5 ms of its own), so the operands (Xp, A, dYp, dGU) of
         as many layers are held as fit into half the pool gradient's own size beside the one that is needed
-        anyway: few rows and a large pool - where the read-modify-write weighs most - allow the most layers."""
+        anyway: few rows and a large pool - where the read-modify-write weighs most - allow the most layers.
+        (Permuted activations and operands, one layer -> so many: 24 layers of 32768 tokens over those 192 experts
+        4.5 -> 10.0 GB, three layers; 12 of 1501 tokens over 96 of 768 x 2048 0.38 -> 1.08 GB, four.)"""
         bytes_per_layer = self.cap * (2 * self.d + 3 * self.f) * torch.empty(0, dtype=self.tdtype).element_size()
         pool_gradient = self.M * 3 * self.d * self.f * 4
         most = 1 + pool_gradient // 2 // bytes_per_layer

@@ -198,3 +198,46 @@ def test_arrays_of_the_caller_that_are_slices_of_larger_ones():
     with pytest.raises(IndexError):
         st.forward(x0)
     st.close()
+
+
+def test_recompute_holds_as_few_layers_as_asked_or_as_fit():
+    """wgrad_layers=1 is one shared slot for every permuted array; the default holds more layers, and one where more do
+    not fit the device."""
+    import torch
+    shape = (8, 512, 1024, 128, 1, 128)
+
+    def build(**kw):
+        torch.cuda.empty_cache()
+        return make(*shape, recompute=True, **kw)
+
+    def slots(st):
+        return [getattr(st, n).shape[0] for n in ("Xp", "A", "dYp", "dGU", "GU", "Yp")]
+
+    torch.cuda.empty_cache()
+    before = torch.cuda.memory_reserved()
+    st, x0, up = build(wgrad_layers=1)
+    need = torch.cuda.memory_reserved() - before
+    assert slots(st) == [1] * 6
+    want = stack_results(st, x0, up)
+    st.close()
+    del st
+    st, x0, up = build()
+    assert slots(st) == [4, 4, 4, 4, 1, 1]
+    same(stack_results(st, x0, up), want, ("dW_r", "dW_gu", "dW_down"))
+    st.close()
+    del st
+    torch.cuda.empty_cache()
+    limit = torch.cuda.memory_reserved() + need + 200e6                          # four layers need 400 MB more than one
+    torch.cuda.set_per_process_memory_fraction(limit / torch.cuda.get_device_properties(0).total_memory)
+    try:
+        with pytest.raises(torch.OutOfMemoryError):
+            build(wgrad_layers=4)
+        st, x0, up = build()
+    finally:
+        torch.cuda.set_per_process_memory_fraction(1.0)
+    assert slots(st) == [1] * 6
+    same(stack_results(st, x0, up), want, ("dW_r", "dW_gu", "dW_down"))
+    st.close()
+    for kw in (dict(recompute=True, wgrad_layers=0), dict(recompute=True, wgrad_layers=9), dict(wgrad_layers=2)):
+        with pytest.raises(ValueError):
+            make(*shape, **kw)
