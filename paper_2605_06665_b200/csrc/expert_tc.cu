@@ -744,7 +744,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (one in each CTA)
-    // (the whole warp walks the rows, lane 0 issues)
+    // (the whole warp walks the layers, lane 0 alone waits and issues)
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
@@ -765,24 +765,19 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         for (int l = 0; l < min(32, p.n_layers - l0) && ok; ++l) {
           const int n = __shfl_sync(0xffffffffu, count, l);
           const int row0 = (l0 + l) * p.layer_stride_rows + __shfl_sync(0xffffffffu, cur.first, l);
-          for (int done = 0; done < n; done += KR) {
-            if (!tc::mbar_wait(&empty_bar[stage], phase ^ 1u, abort)) {
-              if (lane == 0) report_timeout(p, abort, 21);
-              ok = false;
-              break;
-            }
-            if (lane == 0) {
+          ok = tc::lane0(lane, [&] {
+            for (int done = 0; done < n; done += KR) {
+              if (!tc::mbar_wait(&empty_bar[stage], phase ^ 1u, abort)) { report_timeout(p, abort, 21); return false; }
               uint8_t* sA = smem + stage * kStage;
               uint8_t* sB = sA + kHalf;
               if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], 2 * kStage);   // both CTAs' bytes
               // this CTA's two 64-column blocks of each operand, one box each
               tc::tma_load_3d_pair(sA, &tmA, &full_bar[stage], 0, row0 + done, mt * 4 + rank * 2);
               tc::tma_load_3d_pair(sB, &tmB, &full_bar[stage], 0, row0 + done, nt * 4 + rank * 2);
+              if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
-            __syncwarp();
-            if (++stage == kStages) { stage = 0; phase ^= 1u; }
-          }
-          ok = __all_sync(0xffffffffu, ok);
+            return true;
+          });
         }
       }
     }
@@ -790,7 +785,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       for (int i = 0; i < 200; ++i) __nanosleep(1000);
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (leader CTA only)
-    // (the whole warp walks the rows, lane 0 issues)
+    // (the whole warp walks the layers, lane 0 alone waits and issues)
     if (rank == 0) {
       constexpr uint32_t idesc = tc::instr_desc_bf16(256, true, true, 256);
       constexpr uint32_t kstep = (16 * 128) >> 4;             // descriptor units per K = 16 (MN-major)
@@ -803,10 +798,12 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const int tile = snake_tile(round, pair, n_pairs);
         if (tile >= live) break;
         const int acc = round & 1;
-        if (!tc::mbar_wait(&tmem_empty[acc], ((round >> 1) & 1) ^ 1u, abort)) {
-          if (lane == 0) report_timeout(p, abort, 22);
-          break;
-        }
+        ok = tc::lane0(lane, [&] {
+          if (tc::mbar_wait(&tmem_empty[acc], ((round >> 1) & 1) ^ 1u, abort)) return true;
+          report_timeout(p, abort, 22);
+          return false;
+        });
+        if (!ok) break;
         tc::tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * 256;
         uint32_t accumulate = 0;
@@ -820,14 +817,10 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           }
           for (int l = 0; l < min(32, p.n_layers - l0) && ok; ++l) {
             const int n = __shfl_sync(0xffffffffu, count, l);
-            for (int done = 0; done < n; done += KR) {
-              if (!tc::mbar_wait(&full_bar[stage], phase, abort)) {
-                if (lane == 0) report_timeout(p, abort, 23);
-                ok = false;
-                break;
-              }
-              tc::tc_fence_after_sync();
-              if (lane == 0) {
+            ok = tc::lane0(lane, [&] {
+              for (int done = 0; done < n; done += KR) {
+                if (!tc::mbar_wait(&full_bar[stage], phase, abort)) { report_timeout(p, abort, 23); return false; }
+                tc::tc_fence_after_sync();
                 const uint32_t aaddr = tc::smem_u32(smem + stage * kStage);
                 const uint64_t adesc = tc::smem_desc_sw128(aaddr, kBlock, 1024);
                 const uint64_t bdesc = tc::smem_desc_sw128(aaddr + kHalf, kBlock, 1024);
@@ -840,12 +833,11 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
                     tc::umma_bf16_pair(d_tmem, adesc + j * kstep, bdesc + j * kstep, idesc, j > 0 ? 1u : accumulate);
                 }
                 tc::umma_commit_pair(&empty_bar[stage], 3);     // frees the stage in both CTAs
+                accumulate = 1;
+                if (++stage == kStages) { stage = 0; phase ^= 1u; }
               }
-              accumulate = 1;
-              __syncwarp();
-              if (++stage == kStages) { stage = 0; phase ^= 1u; }
-            }
-            ok = __all_sync(0xffffffffu, ok);
+              return true;
+            });
           }
         }
         if (ok && lane == 0) tc::umma_commit_pair(&tmem_full[acc], 3);       // accumulator complete, both CTAs

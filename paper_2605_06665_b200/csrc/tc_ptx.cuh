@@ -56,6 +56,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   }
 }
 
+// Runs f, which waits, in lane 0 alone and gives its answer to the whole warp: lanes that each waited for themselves
+// could disagree where a wait gives up, and part before the next warp-wide instruction.
+template <typename F> __device__ __forceinline__ bool lane0(int lane, F f) {
+  int ok = 1;
+  if (lane == 0) ok = f() ? 1 : 0;
+  return __shfl_sync(0xffffffffu, ok, 0) != 0;
+}
+
 // ---------------------------------------------------------------- TMA (no multicast anywhere)
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, uint64_t* bar, int c0, int c1) {
   asm volatile(
