@@ -694,8 +694,11 @@ int wm_launch(unipool_ctx* ctx, int phase, const CUtensorMap& tmA, const TokenMa
               const BlockMaps& tmC1, const WmParams& p, cudaStream_t s) {
   PhaseTimer pt(ctx, phase, 1, s);
   auto kern = wm_kernel<MODE>;
+  // (the limit belongs to the function, not to the launch: the same for every caller, or a thread with fewer experts
+  // lowers it between another's call and launch)
+  constexpr int most = (int)Wm<MODE>::kTable + 4 * kWmMaxExperts + 1024;
   const int smem = (int)Wm<MODE>::kTable + 4 * p.n_experts + 1024;
-  UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
   kern<<<ctx->sm_count / 2 * 2, Wm<MODE>::kThreads, smem, s>>>(tmA, tmB, tmC0, tmC1, p);
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;

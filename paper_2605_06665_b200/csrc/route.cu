@@ -181,9 +181,8 @@ int route_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float
   const int per_block = kRouteWarps * kRouteTokensPerWarp;
   const int blocks = (T + per_block - 1) / per_block;
   const size_t smem = (size_t)(2 * kRouteWarps * M) * sizeof(float) + (size_t)M * sizeof(int);
+  static_assert((2 * kRouteWarps + 1) * UNIPOOL_MAX_EXPERTS * 4 <= 48 * 1024, "no opt-in to more shared memory");
   auto kern = ctx->cfg.router_mode == UNIPOOL_ROUTER_SOFTMAX ? router_select_kernel<true> : router_select_kernel<false>;
-  if (smem > 48 * 1024)
-    UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   kern<<<blocks, kRouteWarps * 32, smem, s>>>(
       z_saved, T, M, k, sigma * ctx->cfg.c, ctx->cfg.eps, idx, gate, znorm, counts, score_sum,
       ctx->ws.route_counts, ctx->ws.route_sums, ctx->ws.tickets + 0);

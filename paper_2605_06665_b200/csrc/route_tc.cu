@@ -20,6 +20,7 @@ namespace {
 constexpr int kTile = 128;             // tokens per CTA tile = TMEM lanes
 constexpr int kBK = 64;                // k-block: 64 bf16 = one 128-byte swizzle row
 constexpr int kMaxStages = 12;
+constexpr uint32_t kSmemMax = 227 * 1024;
 constexpr uint32_t kTailBars = 384;      // barriers and flags behind the z tiles
 constexpr uint32_t kXBytes = kTile * kBK * 2;
 constexpr int kEpiWarps = 8;           // two per TMEM lane quarter: they take alternate 32-expert chunks
@@ -697,7 +698,7 @@ int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, fl
   const uint32_t stage_bytes = kXBytes + (uint32_t)(n_cols / 2) * (kBK * 2);      // with one term
   const uint32_t tail_bytes = kTailBars + 2 * kTile * 2 * 4 + 2 * kTile * UNIPOOL_MAX_TOPK * 4 + UNIPOOL_MAX_EXPERTS * 4 +
                               kEpiWarps * M * 4 + (M + 31) / 32 * 32 * 4;
-  const uint32_t budget = 227 * 1024 - 1024 - tail_bytes - kEpiWarps * kZStage;
+  const uint32_t budget = kSmemMax - 1024 - tail_bytes - kEpiWarps * kZStage;
   const uint32_t most = (uint32_t)kMaxStages * stage_bytes;
   p.op_bytes = (budget < most ? budget : most) / 1024 * 1024;
   UP_REQUIRE(p.op_bytes >= 2 * stage_bytes && ctx->sm_count >= 2, UNIPOOL_ERR_UNSUPPORTED,
@@ -723,7 +724,8 @@ int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, fl
   const bool softmax = ctx->cfg.router_mode == UNIPOOL_ROUTER_SOFTMAX;
   auto kern = k <= 2 ? (softmax ? route_tc_kernel<2, true> : route_tc_kernel<2, false>)
                      : (softmax ? route_tc_kernel<UNIPOOL_MAX_TOPK, true> : route_tc_kernel<UNIPOOL_MAX_TOPK, false>);
-  UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // (the function's limit, shared by all threads: not lowered to this launch's smem)
+  UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
   kern<<<grid, kThreads, smem, s>>>(tmX, tmW1, tmW2, tmZ, p);
   UP_LAUNCH_CHECK();
   return UNIPOOL_OK;

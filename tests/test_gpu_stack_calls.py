@@ -254,3 +254,36 @@ def test_an_expired_wait_of_one_lane_is_known_to_its_warp():
         ctx.check_status()
     ctx.check_status()
     ctx.close()
+
+
+def test_host_threads_with_contexts_of_different_sizes():
+    """Launches of the same kernels with few and many experts from two threads: neither is refused for the shared memory
+    that the other asked for (before, one thread could lower the function's limit between another's call and launch)."""
+    import threading
+    import torch
+    L, d, f, T = 300, 256, 1600, 64                               # many layers: the threads meet inside the native loop
+    stacks = [make(L, d, f, M, 1, T, recompute=True) for M in (4, 300)]           # the weights-on-M kernels and the router
+    [st.W_down.mul_(1e-3) for st, _, _ in stacks]                 # so that 300 residual layers stay finite
+    want = [st.forward(x0).clone() for st, x0, _ in stacks]
+    torch.cuda.synchronize()
+    errors = []
+
+    def work(i):
+        try:
+            st, x0, _ = stacks[i]
+            with torch.cuda.stream(torch.cuda.Stream()):
+                for _ in range(20):
+                    st.forward(x0)
+                torch.cuda.current_stream().synchronize()
+        except Exception as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(2)]
+    [t.start() for t in threads]
+    [t.join() for t in threads]
+    torch.cuda.synchronize()
+    assert not errors
+    for (st, _, _), w in zip(stacks, want):
+        st.ctx.check_status()
+        assert torch.equal(st.x[L], w)
+        st.close()
