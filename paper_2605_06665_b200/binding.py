@@ -219,14 +219,16 @@ class Context:
     def router_prepare(self, W_r, n_layers, n_experts):
         _check(lib().unipool_router_prepare(self.handle, _p(W_r), n_layers, n_experts, _stream()))
 
-    # (``rows`` [.., n_experts]: the group sizes; NULL makes the _rows calls the plain ones)
+    # (``rows`` [.., n_experts]: the group sizes, for the _rows entry points)
     def dispatch(self, x, T, idx, n_experts, offsets, row_of, token_of, tile_expert, Xp, rows=None):
-        _check(lib().unipool_dispatch_rows(self.handle, _p(x), T, _p(idx), n_experts, _p(offsets), _p(row_of),
-                                           _p(token_of), _p(tile_expert), _p(rows), _p(Xp), _stream()))
+        f, r = (lib().unipool_dispatch, ()) if rows is None else (lib().unipool_dispatch_rows, (_p(rows),))
+        _check(f(self.handle, _p(x), T, _p(idx), n_experts, _p(offsets), _p(row_of), _p(token_of), _p(tile_expert), *r,
+                 _p(Xp), _stream()))
 
     def expert_fwd(self, Xp, offsets, tile_expert, W_gu, W_down, expert_base, n_experts, GU, A, Yp, rows=None):
-        _check(lib().unipool_expert_fwd_rows(self.handle, _p(Xp), _p(offsets), _p(rows), _p(tile_expert), _p(W_gu),
-                                             _p(W_down), expert_base, n_experts, _p(GU), _p(A), _p(Yp), _stream()))
+        f, r = (lib().unipool_expert_fwd, ()) if rows is None else (lib().unipool_expert_fwd_rows, (_p(rows),))
+        _check(f(self.handle, _p(Xp), _p(offsets), *r, _p(tile_expert), _p(W_gu), _p(W_down), expert_base, n_experts,
+                 _p(GU), _p(A), _p(Yp), _stream()))
 
     def combine(self, Yp, row_of, gate, T, residual, y):
         _check(lib().unipool_combine(self.handle, _p(Yp), _p(row_of), _p(gate), T, _p(residual), _p(y),
@@ -234,17 +236,16 @@ class Context:
 
     def expert_bwd(self, dy, T, row_of, gate, token_of, offsets, tile_expert, Xp, GU, A, Yp, W_gu, W_down,
                    expert_base, n_experts, dx_residual, dYp, dGU, dx, dgate, dW_gu, dW_down, flags=0, rows=None):
-        _check(lib().unipool_expert_bwd_rows(self.handle, _p(dy), T, _p(row_of), _p(gate), _p(token_of),
-                                             _p(offsets), _p(rows), _p(tile_expert), _p(Xp), _p(GU), _p(A), _p(Yp),
-                                             _p(W_gu), _p(W_down), expert_base, n_experts, _p(dx_residual),
-                                             _p(dYp), _p(dGU), _p(dx), _p(dgate), _p(dW_gu), _p(dW_down),
-                                             flags, _stream()))
+        f, r = (lib().unipool_expert_bwd, ()) if rows is None else (lib().unipool_expert_bwd_rows, (_p(rows),))
+        _check(f(self.handle, _p(dy), T, _p(row_of), _p(gate), _p(token_of), _p(offsets), *r, _p(tile_expert), _p(Xp),
+                 _p(GU), _p(A), _p(Yp), _p(W_gu), _p(W_down), expert_base, n_experts, _p(dx_residual), _p(dYp), _p(dGU),
+                 _p(dx), _p(dgate), _p(dW_gu), _p(dW_down), flags, _stream()))
 
     def pool_wgrad(self, n_layers, layer_stride_rows, offsets, Xp, A, dYp, dGU, expert_base, n_experts,
                    dW_gu, dW_down, flags=0, rows=None):
-        _check(lib().unipool_pool_wgrad_rows(self.handle, n_layers, layer_stride_rows, _p(offsets), _p(rows), _p(Xp),
-                                             _p(A), _p(dYp), _p(dGU), expert_base, n_experts, _p(dW_gu), _p(dW_down),
-                                             flags, _stream()))
+        f, r = (lib().unipool_pool_wgrad, ()) if rows is None else (lib().unipool_pool_wgrad_rows, (_p(rows),))
+        _check(f(self.handle, n_layers, layer_stride_rows, _p(offsets), *r, _p(Xp), _p(A), _p(dYp), _p(dGU), expert_base,
+                 n_experts, _p(dW_gu), _p(dW_down), flags, _stream()))
 
     def pool_aux_loss(self, counts, score_sum, L, n_experts, T, alpha, fbar_prev, loss, dscore_coef, fbar_out):
         _check(lib().unipool_pool_aux_loss(self.handle, _p(counts), _p(score_sum), L, n_experts, T, alpha,

@@ -287,3 +287,65 @@ def test_host_threads_with_contexts_of_different_sizes():
         st.ctx.check_status()
         assert torch.equal(st.x[L], w)
         st.close()
+
+
+@pytest.mark.parametrize("shape,kw", [
+    ((3, 64, 128, 9, 2, 300), dict(deferred_wgrad=True)),
+    ((3, 64, 128, 9, 2, 300), {}),
+    ((3, 128, 192, 9, 2, 300), dict(dtype="fp32", deferred_wgrad=True)),
+    ((4, 64, 128, 16, 2, 300), dict(groups=2, deferred_wgrad=True)),
+    ((3, 64, 128, 24, 1, 300), dict(private=8, router="softmax")),
+    ((5, 256, 384, 48, 1, 40), dict(recompute=True)),             # runs of two, two and one layer
+    ((5, 256, 384, 48, 1, 40), dict(recompute=True, wgrad_layers=1)),
+    ((2, 768, 2048, 96, 2, 16384), dict(deferred_wgrad=True)),    # the sizes that the oracle checks layer by layer
+    ((2, 768, 2048, 16, 2, 16384), dict(private=8)),
+    ((2, 768, 512, 384, 8, 16384), dict(deferred_wgrad=True)),
+    ((2, 1536, 4096, 192, 2, 32768), dict(recompute=True)),
+])
+def test_native_loops_give_what_the_layers_give_one_by_one(shape, kw):
+    """forward, aux_loss and backward against the same calls layer by layer, which the parity tests compare with the
+    oracle: every array equal, bit for bit, but for sums in another order (weight gradients of recomputed runs of layers;
+    fp32: of whole groups instead of their tokens)."""
+    import torch
+    L = shape[0]
+    st, x0, up = make(*shape, **kw)
+    state = ("x", "idx", "gate", "counts", "score_sum", "znorm", "z", "offsets", "row_of", "token_of", "tile_expert", "loss",
+             "coef", "fbar", "dgate")
+    both = []
+    for native in (True, False):
+        st.zero_grad()
+        if native:
+            dx = st.step(x0, up)
+        else:
+            st.ctx.router_prepare(st.W_r, L, st.m)
+            st.x[0].copy_(x0)
+            for l in range(L):
+                st.forward_layer(l)
+            for g in range(st.G):
+                l = slice(g * st.Lg, (g + 1) * st.Lg)
+                st.ctx.pool_aux_loss(st.counts[l], st.score_sum[l], st.Lg, st.m, st.T, st.alpha, None, st.loss[g:g + 1],
+                                     st.coef[g], st.fbar[g])
+            dx = up
+            for l in reversed(range(L)):
+                out = torch.empty_like(up)
+                st.backward_layer(l, dx, out)
+                dx = out
+            for g in range(st.G if st.deferred_wgrad else 0):
+                l = g * st.Lg
+                st.ctx.pool_wgrad(st.Lg, st.cap, st.offsets[l:], st.Xp[l:], st.A[l:], st.dYp[l:], st.dGU[l:], g * st.m, st.m,
+                                  st.dW_gu, st.dW_down)
+        torch.cuda.synchronize()
+        st.ctx.check_status()
+        both.append({n: getattr(st, n).clone() for n in state + ("dW_r", "dsigma", "dW_gu", "dW_down")} | dict(dx=dx.clone()))
+        for n in state:
+            getattr(st, n).zero_()
+    got, want = both
+    other_order = {"dW_r"} | ({"dW_gu", "dW_down"} if st.nw > 1 or "dtype" in kw else set())
+    for n in want:
+        if n in other_order:
+            assert (got[n] - want[n]).abs().max() <= 1e-5 * want[n].abs().max(), n
+        else:
+            assert torch.equal(got[n], want[n]), n
+    st.close()
+    del st, both, got, want
+    torch.cuda.empty_cache()
