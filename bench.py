@@ -40,20 +40,6 @@ if ROOT not in sys.path:
 # times that (weights and activations both grow with the units processed).
 NCU_TRAFFIC = {("978m", "expert_fwd_gu"): 8 * (637.8e6 + 201.2e6)}
 
-
-
-def gemm_kernel(phase, rows, d, f):
-    """Kernel behind a grouped-GEMM phase (for the roofline's `kernel` field): the library's rules on the rows a full
-    batch gives the average expert (weights_on_m and rows_on_pairs in csrc/expert_tc.cu)."""
-    if phase.startswith("wgrad"):
-        return "wgrad_pair_kernel"
-    on_m = {"expert_fwd_gu": (100 if d >= 1024 else 150) < rows <= (1024 if d >= 1024 else 600),
-            "expert_fwd_down": rows <= 450 and f > 1024,
-            "dgrad_down": rows <= 1200 and (rows <= 48 or rows > 100 or f > 1024),
-            "dgrad_gu": rows <= 450 and 2 * f > 1024}[phase]
-    return "wm_kernel" if on_m else "row_pair_kernel" if rows >= 512 else "grouped_gemm_tc_kernel"
-
-
 # launches of one dispatch-map call
 DISPATCH_MAP_LAUNCHES = 1
 
@@ -312,7 +298,7 @@ def measure_workload(name, args, world, rank, dev, full):
     gemm_ms = {n: kernels[n]["ms_per_step"] for n in GEMM_PHASES if n in kernels}
     dominant = max(gemm_ms, key=gemm_ms.get)
     dom = kernels[dominant]
-    kernel_name = gemm_kernel(dominant, T * k // mw, d, f)
+    kernel_name = st.ctx.gemm_kernel(dominant, mw)
     # per launch of the dominant kernel: algorithmic bytes / FLOPs over its average CUDA-event duration
     if dom["bound"] == "hbm":
         roofline = dict(kernel=kernel_name + ":" + dominant, bound="hbm", achieved=dom["gbs"],

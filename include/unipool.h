@@ -389,6 +389,10 @@ enum {
 int unipool_profile_enable(unipool_ctx* ctx, int32_t on);
 int unipool_profile_read(unipool_ctx* ctx, double* ms, int64_t* launches);
 
+/* Name of the kernel that a grouped-GEMM phase of this context runs for a router of n_experts experts, with
+ * (sizes_known != 0) or without the group sizes; "" for other phases (host function, a measurement aid). */
+const char* unipool_gemm_kernel(const unipool_ctx* ctx, int32_t phase, int32_t n_experts, int32_t sizes_known);
+
 #ifdef __cplusplus
 }
 #endif

@@ -29,7 +29,7 @@ EXPORTS = (
     "unipool_profile_enable", "unipool_profile_read", "unipool_dispatch_static",
     "unipool_unique_experts", "unipool_router_prepare", "unipool_selftest_wait",
     "unipool_stack_forward", "unipool_stack_aux_loss", "unipool_stack_backward",
-    "unipool_dispatch_rows", "unipool_expert_fwd_rows", "unipool_expert_bwd_rows", "unipool_pool_wgrad_rows",
+    "unipool_gemm_kernel", "unipool_dispatch_rows", "unipool_expert_fwd_rows", "unipool_expert_bwd_rows", "unipool_pool_wgrad_rows",
 )
 
 PHASES = (
@@ -127,6 +127,8 @@ def lib():
     L.unipool_stack_aux_loss.argtypes = [vp, stackp, i32, f32, vp, vp]
     L.unipool_stack_backward.restype = ctypes.c_int
     L.unipool_stack_backward.argtypes = [vp, stackp, i32, i32, vp]
+    L.unipool_gemm_kernel.restype = ctypes.c_char_p
+    L.unipool_gemm_kernel.argtypes = [vp, i32, i32, i32]
     L.unipool_unique_experts.restype = ctypes.c_int
     L.unipool_unique_experts.argtypes = [vp, vp, vp, i32, i32, vp, vp, vp]
     L.unipool_calibrate_c.restype = ctypes.c_int
@@ -279,6 +281,10 @@ class Context:
         launches = (ctypes.c_int64 * n)()
         _check(lib().unipool_profile_read(self.handle, ms, launches))
         return {PHASES[i]: (float(ms[i]), int(launches[i])) for i in range(n)}
+
+    def gemm_kernel(self, phase, n_experts, sizes_known=True):
+        """Name of the kernel behind a grouped-GEMM phase (a name of PHASES), "" for the others."""
+        return lib().unipool_gemm_kernel(self.handle, PHASES.index(phase), n_experts, int(sizes_known)).decode()
 
     def calibrate_c(self, n_experts, top_k, n_samples=100_000, seed=0):
         out = ctypes.c_float()

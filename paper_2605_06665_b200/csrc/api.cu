@@ -211,6 +211,16 @@ int unipool_profile_read(unipool_ctx* ctx, double* ms, int64_t* launches) {
   return UNIPOOL_OK;
 }
 
+const char* unipool_gemm_kernel(const unipool_ctx* ctx, int32_t phase, int32_t n_experts, int32_t sizes_known) {
+  if (ctx == nullptr || n_experts < 1 || n_experts > ctx->cfg.pool_size) return "";
+  const bool wgrad = phase == UNIPOOL_PH_WGRAD_DOWN || phase == UNIPOOL_PH_WGRAD_GU;
+  if (!wgrad && phase != UNIPOOL_PH_EXPERT_FWD_GU && phase != UNIPOOL_PH_EXPERT_FWD_DOWN &&
+      phase != UNIPOOL_PH_DGRAD_DOWN && phase != UNIPOOL_PH_DGRAD_GU)
+    return "";
+  if (!use_tensor_cores(ctx)) return wgrad ? "grouped_k_gemm_kernel" : "grouped_rows_gemm_kernel";
+  return wgrad ? "wgrad_pair_kernel" : row_gemm_kernel(ctx, phase, n_experts, sizes_known != 0);
+}
+
 int unipool_check_status(unipool_ctx* ctx, unipool_stream stream) {
   CHECK_CTX(ctx);
   int32_t host[4] = {0, 0, 0, 0};

@@ -207,6 +207,7 @@ int expert_fwd_simt(unipool_ctx*, const ExpertFwdArgs&, cudaStream_t);
 int expert_bwd_simt(unipool_ctx*, const ExpertBwdArgs&, cudaStream_t);
 int pool_wgrad_simt(unipool_ctx*, const PoolWgradArgs&, cudaStream_t);
 int expert_fwd_tc(unipool_ctx*, const ExpertFwdArgs&, cudaStream_t);
+const char* row_gemm_kernel(const unipool_ctx*, int phase, int n_experts, bool sizes_known);
 int expert_bwd_tc(unipool_ctx*, const ExpertBwdArgs&, cudaStream_t);
 int pool_wgrad_tc(unipool_ctx*, const PoolWgradArgs&, cudaStream_t);
 int wm_fwd_gu(unipool_ctx*, const ExpertFwdArgs&, cudaStream_t);

@@ -1378,29 +1378,63 @@ bool rows_on_pairs(const unipool_ctx* ctx, int n_experts) {
 }
 
 // Weights or tokens on the M side, by the rows the average expert gets from a full batch (the group sizes
-// themselves are on the device).  Measured per GEMM, interleaved, tokens / weights on M in us (768 x 2048; the
-// figures of 1536 x 4096 are marked *):
+// themselves are on the device).  Measured per GEMM, interleaved, tokens / weights on M in us (768 x 2048, 96 experts;
+// the figures of 1536 x 4096, 64 to 192 experts, are marked *):
 //   rows                31         66        125       170       229       341       546      819      *128      *1024
 //   gate/up          125/127   126/129   141/146   180/171   199/211   268/263   244/240  228/227  708/626  1589/1479
 //   down              69/68     69/69     78/77     91/81    102/90    131/124   118/122  113/116  334/334   728/724
 //   dgrad down        87/70     89/80    108/100   138/112   150/133   199/192   183/172  174/166  465/400  1014/951
 //   dgrad gate/up    116/109   117/113   130/125   154/134   178/151   235/209   205/212  199/204  596/581  1401/1384
 // Few rows: every launch streams the weights, and what is left to gain are the rows of the padding that the token-major
-// kernels read (gate/up reads few of them, and both forms write its pad rows).  Large groups waste nothing in 256-row
+// kernels read (gate/up reads few of them, and both forms write its pad rows; without the group sizes there are none to
+// leave out: 31 rows padded to 128, down 69/72, dgrads 89/93 and 117/123).  Large groups waste nothing in 256-row
 // pair-tiles: down and dgrad gate/up gain while a group is one or two chunks, and need a contraction long enough to
-// hide the epilogue of a unit (384 experts of 768 x 512, 341 rows: down 112/129, dgrad gate/up 185/202); dgrad down
-// gains longest, its G and U traffic being the same on fewer padded rows; gate/up gains further where its contraction
-// is long.  Many narrow experts under skewed routing lose with few rows: the largest group sets the size of a
-// stage (393 experts of 768 x 320, 92 rows: dgrad down 54/58, dgrad gate/up 46/59).
-bool weights_on_m(const unipool_ctx* ctx, int mode, int n_experts) {
+// hide the epilogue of a unit; dgrad down gains longest, its G and U traffic being the same on fewer padded rows.
+// Where the lines lie beside the rows, from 2000 shapes of 384..1536 x 256..4096 (weights on M against tokens on M,
+// mean of the shapes on the far side of a line; 'deal': the part of the pairs' rounds that the units fill):
+//   width of the last weight tile  gate/up of 320 and 640 columns +20..35 %, down below 0.8 of a tile +5 %, dgrad down
+//                                  below 0.85 on large groups +5 % where the contraction is short
+//   gate/up, chunks filled         195..265 rows are two half-empty chunks: +5..8 %; 120..190 rows one chunk, -7 % from
+//                                  d = 1024 on and 0 below; 270..560 rows -5 % from d = 1024 on, -1 % at 768 .. 1023, 0
+//                                  below (+8 % at f = 512, 0 at 768); 620..870 rows +5 %
+//   down                           f below 1536 +1 %; 49..130 rows +2 % (a few long groups: -4 %); a poor deal +3..14 %
+//   dgrad gate/up                  more than 192 experts +5..17 % under skewed routing (the largest group sets the size of
+//                                  a stage), 0 under even; 91..130 rows in a poor deal +4 %; large groups in a poor one +8 %
+//   dgrad down, beyond 200 rows    d below 640 +5 %, f below 512 +2..20 %; up to 200 rows f below 512 +2..20 % under
+//                                  skewed routing while d is below 1024 (-10..+5 % under even)
+bool weights_on_m(const unipool_ctx* ctx, int mode, int n_experts, bool sizes_known) {
   if (ctx->sm_count < 2 || n_experts > kWmMaxExperts) return false;
   const int64_t rows = (int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k / n_experts;
-  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff;
+  if (rows > 1200 || (!sizes_known && rows <= BM)) return false;
+  const int d = ctx->cfg.d_model, f = ctx->cfg.d_ff, r = rows < 1 ? 1 : (int)rows;
+  const bool plain = mode == kFwd2 || mode == kDgrad2;
+  const int one = (r + 255) / 256, two = (r + 383) / 384;                  // chunks of an average group: see group_chunks
+  const int chunks = mode == kFwd1 ? (r + 191) / 192 : plain && 384 * two <= 256 * one ? two : one;
+  const int columns = plain ? d : f, tiles = (columns + 255) / 256;
+  const float width = (float)columns / (256 * tiles);
+  const int pairs = ctx->sm_count / 2, units = n_experts * tiles * chunks;
+  const float deal = (float)units / ((units + pairs - 1) / pairs * pairs);
   switch (mode) {
-    case kFwd1: return rows > (d >= 1024 ? 100 : 150) && rows <= (d >= 1024 ? 1024 : 600);
-    case kFwd2: return rows <= 450 && f > 1024;
-    case kDgrad1: return rows <= 1200 && (rows <= 48 || rows > 100 || f > 1024);
-    default: return rows <= 450 && 2 * f > 1024;
+    case kFwd1: {
+      if (width < 0.9f || deal < 0.75f) return false;
+      const bool filled = 10 * r >= 7 * 192 * chunks;
+      if (d >= 1024)
+        return chunks == 1 ? r > 120 && r <= 190 && f >= 1024
+                           : filled && (r <= 560 || r > 900) && r <= 1024 && f >= 768;
+      if (d >= 768) return f >= 2048 && r > 150 && r <= 185 || f >= 1024 && r >= 300 && r <= 384;
+      return f >= 3072 && r >= 300 && r <= 384;
+    }
+    case kFwd2:
+      if (f < 1536 || r > 450 || width < 0.8f) return false;
+      if (r > 48 && r <= 130) return n_experts < 48 && deal >= 0.9f;
+      return r <= 200 || deal >= (r <= 390 ? 0.8f : 0.9f);
+    case kDgrad1:
+      if (r <= 200) return (r <= 48 || r > 100 || f > 1024) && (r <= 48 || f >= 512 || d >= 1024);
+      return d >= 640 && f >= 512 && (width >= 0.85f || d >= 1024);
+    default:
+      if (2 * f <= 1024 || r > 450 || n_experts > 192) return false;
+      if (r > 90 && r <= 130) return deal >= 0.9f;
+      return r <= 200 || deal >= 0.7f;
   }
 }
 
@@ -1584,16 +1618,25 @@ static int rows_dgrad_gu(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t 
   return launch_rows<kDgrad2>(ctx, UNIPOOL_PH_DGRAD_GU, plan, tmA, tmA64, tmB, tmB64, tmBp, tmC0, tmC0, p, s);
 }
 
+const char* row_gemm_kernel(const unipool_ctx* ctx, int phase, int n_experts, bool sizes_known) {
+  const int mode = phase == UNIPOOL_PH_EXPERT_FWD_GU ? kFwd1 : phase == UNIPOOL_PH_EXPERT_FWD_DOWN ? kFwd2
+                 : phase == UNIPOOL_PH_DGRAD_DOWN ? kDgrad1 : kDgrad2;
+  return weights_on_m(ctx, mode, n_experts, sizes_known) ? "wm_kernel"
+         : rows_on_pairs(ctx, n_experts) ? "row_pair_kernel" : "grouped_gemm_tc_kernel";
+}
+
 int expert_fwd_tc(unipool_ctx* ctx, const ExpertFwdArgs& a, cudaStream_t s) {
-  const int rc = weights_on_m(ctx, kFwd1, a.n_experts) ? wm_fwd_gu(ctx, a, s) : rows_fwd_gu(ctx, a, s);
+  const bool sizes = a.rows != nullptr;
+  const int rc = weights_on_m(ctx, kFwd1, a.n_experts, sizes) ? wm_fwd_gu(ctx, a, s) : rows_fwd_gu(ctx, a, s);
   if (rc != UNIPOOL_OK) return rc;
-  return weights_on_m(ctx, kFwd2, a.n_experts) ? wm_fwd_down(ctx, a, s) : rows_fwd_down(ctx, a, s);
+  return weights_on_m(ctx, kFwd2, a.n_experts, sizes) ? wm_fwd_down(ctx, a, s) : rows_fwd_down(ctx, a, s);
 }
 
 int expert_bwd_tc(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {
-  int rc = weights_on_m(ctx, kDgrad1, a.n_experts) ? wm_dgrad_down(ctx, a, s) : rows_dgrad_down(ctx, a, s);
+  const bool sizes = a.rows != nullptr;
+  int rc = weights_on_m(ctx, kDgrad1, a.n_experts, sizes) ? wm_dgrad_down(ctx, a, s) : rows_dgrad_down(ctx, a, s);
   if (rc != UNIPOOL_OK) return rc;
-  rc = weights_on_m(ctx, kDgrad2, a.n_experts) ? wm_dgrad_gu(ctx, a, s) : rows_dgrad_gu(ctx, a, s);
+  rc = weights_on_m(ctx, kDgrad2, a.n_experts, sizes) ? wm_dgrad_gu(ctx, a, s) : rows_dgrad_gu(ctx, a, s);
   if (rc != UNIPOOL_OK || !a.wgrad) return rc;
   PoolWgradArgs w{1, 0, a.offsets, a.Xp, a.A, a.dYp, a.dGU, a.expert_base, a.n_experts, a.dW_gu, a.dW_down,
                   a.overwrite, a.rows};
