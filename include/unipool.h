@@ -367,7 +367,7 @@ int unipool_calibrate_c(unipool_ctx* ctx, int32_t n_experts, int32_t top_k, int3
 
 /* Self-test of the bounded device-side waits (a diagnostic; the paper has no counterpart).  Every
  * pipeline of the library waits on its barriers for a bounded time and reports an expired wait through
- * the status word instead of hanging.  This call launches one warp whose first lane waits, for at most
+ * the status word instead of hanging.  This call launches one warp that waits, for at most
  * limit_cycles SM cycles (0 .. 2e9), on a barrier nobody arrives on: the wait gives up, the kernel
  * returns normally, and the next unipool_check_status returns UNIPOOL_ERR_TIMEOUT and clears the word.
  * The context stays usable. */

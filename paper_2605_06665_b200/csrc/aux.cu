@@ -153,10 +153,10 @@ int calibrate_launch(unipool_ctx* ctx, int E, int k, int n_samples, uint64_t see
   return UNIPOOL_OK;
 }
 
-// Exercises the bounded wait every pipeline of the library is built on: the first lane of a warp waits, for at
-// most limit_cycles SM cycles, on an mbarrier that nobody arrives on.  The wait gives up, the whole warp learns of
-// it, the kernel records the time-out in the status word the way the GEMM and router kernels do (detail: the lanes
-// that know), and returns normally.
+// Exercises the bounded wait every pipeline of the library is built on: a warp waits, for at most limit_cycles SM
+// cycles (half of its lanes for a quarter of that), on an mbarrier that nobody arrives on.  The wait gives up, the
+// kernel records the time-out in the status word the way the GEMM and router kernels do (detail: the lanes that know),
+// and returns normally.
 __global__ void wait_selftest_kernel(long long limit_cycles, int32_t* status) {
   __shared__ uint64_t bar;
   __shared__ int abort_flag;
@@ -166,7 +166,7 @@ __global__ void wait_selftest_kernel(long long limit_cycles, int32_t* status) {
     tc::fence_barrier_init();
   }
   __syncwarp();
-  const bool ok = tc::lane0(threadIdx.x, [&] { return tc::mbar_wait(&bar, 0, &abort_flag, limit_cycles); });
+  const bool ok = tc::mbar_wait_warp(&bar, 0, &abort_flag, threadIdx.x < 16 ? limit_cycles : limit_cycles / 4);
   const unsigned know = __ballot_sync(0xffffffffu, !ok);
   if (threadIdx.x == 0 && !ok) {
     abort_flag = 1;

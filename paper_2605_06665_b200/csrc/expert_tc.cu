@@ -643,8 +643,11 @@ static_assert(kPairStages * kPairStageBytes + kEpiWarps * 8192 == kBarOffset, "s
 // Group sizes against padded groups: 12 layers of 1501 tokens over 96 experts (31 rows in groups of 128) 962 ->
 // 642 us; at 341 rows per group, where 64-row k-blocks drop a twelfth of the steps, 3.11 -> 3.07 ms (zeros cost
 // little under the power cap).
-// Rows of expert e in layer l that the contraction runs over: its tokens if the caller gave their number (what
-// follows up to the next group start is zero), else the padded group.
+// Rows of expert e in layer l that the contraction runs over: its tokens if the caller gave their number, else the
+// padded group.  Behind the tokens the operands hold zeros up to the next multiple of kRowStep rows, the K of one MMA;
+// what dYp and dGU hold further on is not written, so whole k-blocks are loaded but no step of them beyond that is
+// multiplied.
+static_assert(kRowStep == 16, "rows of an MMA step of the contraction");
 __device__ __forceinline__ int wgrad_rows(const GemmParams& p, int l, int e) {
   const int32_t* off = p.offsets + (int64_t)l * (p.n_experts + 1) + e;
   const int padded = off[1] - off[0];
@@ -744,7 +747,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (one in each CTA)
-    // (the whole warp walks the layers, lane 0 alone waits and issues)
+    // (the whole warp walks the rows and waits, lane 0 issues)
     int stage = 0;
     uint32_t phase = 0;
     bool ok = true;
@@ -765,19 +768,22 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         for (int l = 0; l < min(32, p.n_layers - l0) && ok; ++l) {
           const int n = __shfl_sync(0xffffffffu, count, l);
           const int row0 = (l0 + l) * p.layer_stride_rows + __shfl_sync(0xffffffffu, cur.first, l);
-          ok = tc::lane0(lane, [&] {
-            for (int done = 0; done < n; done += KR) {
-              if (!tc::mbar_wait(&empty_bar[stage], phase ^ 1u, abort)) { report_timeout(p, abort, 21); return false; }
+          for (int done = 0; done < n; done += KR) {
+            ok = tc::mbar_wait_warp(&empty_bar[stage], phase ^ 1u, abort);
+            if (!ok) {
+              if (lane == 0) report_timeout(p, abort, 21);
+              break;
+            }
+            if (lane == 0) {
               uint8_t* sA = smem + stage * kStage;
               uint8_t* sB = sA + kHalf;
               if (rank == 0) tc::mbar_expect_tx(&full_bar[stage], 2 * kStage);   // both CTAs' bytes
               // this CTA's two 64-column blocks of each operand, one box each
               tc::tma_load_3d_pair(sA, &tmA, &full_bar[stage], 0, row0 + done, mt * 4 + rank * 2);
               tc::tma_load_3d_pair(sB, &tmB, &full_bar[stage], 0, row0 + done, nt * 4 + rank * 2);
-              if (++stage == kStages) { stage = 0; phase ^= 1u; }
             }
-            return true;
-          });
+            if (++stage == kStages) { stage = 0; phase ^= 1u; }
+          }
         }
       }
     }
@@ -785,7 +791,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
       for (int i = 0; i < 200; ++i) __nanosleep(1000);
   } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer (leader CTA only)
-    // (the whole warp walks the layers, lane 0 alone waits and issues)
+    // (the whole warp walks the rows and waits, lane 0 issues)
     if (rank == 0) {
       constexpr uint32_t idesc = tc::instr_desc_bf16(256, true, true, 256);
       constexpr uint32_t kstep = (16 * 128) >> 4;             // descriptor units per K = 16 (MN-major)
@@ -798,12 +804,10 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
         const int tile = snake_tile(round, pair, n_pairs);
         if (tile >= live) break;
         const int acc = round & 1;
-        ok = tc::lane0(lane, [&] {
-          if (tc::mbar_wait(&tmem_empty[acc], ((round >> 1) & 1) ^ 1u, abort)) return true;
-          report_timeout(p, abort, 22);
-          return false;
-        });
-        if (!ok) break;
+        if (!tc::mbar_wait_warp(&tmem_empty[acc], ((round >> 1) & 1) ^ 1u, abort)) {
+          if (lane == 0) report_timeout(p, abort, 22);
+          break;
+        }
         tc::tc_fence_after_sync();
         const uint32_t d_tmem = tmem_base + acc * 256;
         uint32_t accumulate = 0;
@@ -817,27 +821,29 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
           }
           for (int l = 0; l < min(32, p.n_layers - l0) && ok; ++l) {
             const int n = __shfl_sync(0xffffffffu, count, l);
-            ok = tc::lane0(lane, [&] {
-              for (int done = 0; done < n; done += KR) {
-                if (!tc::mbar_wait(&full_bar[stage], phase, abort)) { report_timeout(p, abort, 23); return false; }
-                tc::tc_fence_after_sync();
+            for (int done = 0; done < n; done += KR) {
+              ok = tc::mbar_wait_warp(&full_bar[stage], phase, abort);
+              if (!ok) {
+                if (lane == 0) report_timeout(p, abort, 23);
+                break;
+              }
+              tc::tc_fence_after_sync();
+              if (lane == 0) {
                 const uint32_t aaddr = tc::smem_u32(smem + stage * kStage);
                 const uint64_t adesc = tc::smem_desc_sw128(aaddr, kBlock, 1024);
                 const uint64_t bdesc = tc::smem_desc_sw128(aaddr + kHalf, kBlock, 1024);
-                if (n - done > KR - 16) {
+                // No step behind row n.  Straight-line, under predicates: a branch around the partial k-blocks costs
+                // every k-block, 98.2 + 178.3 -> 102.9 + 185.1 us for eight experts of 4096 rows, 768 x 2048.
+                tc::umma_bf16_pair(d_tmem, adesc, bdesc, idesc, accumulate);
 #pragma unroll
-                  for (int j = 0; j < KR / 16; ++j)
-                    tc::umma_bf16_pair(d_tmem, adesc + j * kstep, bdesc + j * kstep, idesc, j > 0 ? 1u : accumulate);
-                } else {                                        // only zeros behind row n
-                  for (int j = 0; 16 * j < n - done; ++j)
-                    tc::umma_bf16_pair(d_tmem, adesc + j * kstep, bdesc + j * kstep, idesc, j > 0 ? 1u : accumulate);
-                }
+                for (int j = 1; j < KR / kRowStep; ++j)
+                  tc::umma_bf16_pair_if(kRowStep * j < n - done ? 1u : 0u, d_tmem, adesc + j * kstep, bdesc + j * kstep,
+                                        idesc, 1u);
                 tc::umma_commit_pair(&empty_bar[stage], 3);     // frees the stage in both CTAs
-                accumulate = 1;
-                if (++stage == kStages) { stage = 0; phase ^= 1u; }
               }
-              return true;
-            });
+              accumulate = 1;
+              if (++stage == kStages) { stage = 0; phase ^= 1u; }
+            }
           }
         }
         if (ok && lane == 0) tc::umma_commit_pair(&tmem_full[acc], 3);       // accumulator complete, both CTAs

@@ -244,7 +244,7 @@ def test_recompute_holds_as_few_layers_as_asked_or_as_fit():
 
 
 def test_an_expired_wait_of_one_lane_is_known_to_its_warp():
-    """Warps that act as one let their first lane wait: when the wait gives up, all 32 lanes have its answer."""
+    """Warps that act as one wait as one: when a lane's wait gives up, all 32 have its answer."""
     import torch
     from paper_2605_06665_b200 import binding as B
     ctx = B.Context(B.make_config(64, 64, 8, 1, 1, 64, B.BF16, 1e-6, 1.0))
