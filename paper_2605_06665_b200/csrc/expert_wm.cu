@@ -112,7 +112,8 @@ __device__ __forceinline__ int chunk_size(int n16, int chunks) {          // <= 
   return chunks == 1 ? n16 * 16 : ((n16 * 16 + chunks - 1) / chunks + 31) / 32 * 32;
 }
 
-// tokens of group e in steps of 16
+// tokens of group e in steps of kRowStep
+static_assert(kRowStep == 16, "steps of the unit list");
 __device__ __forceinline__ int group_n16(const WmParams& p, int e) {
   const int padded = p.offsets[e + 1] - p.offsets[e];
   return ((p.rows ? min(max(p.rows[e], 0), padded) : padded) + 15) / 16;

@@ -36,7 +36,8 @@ struct RouteParams {
   int32_t* acc_counts; long long* acc_sums; uint32_t* ticket;   // [M] accumulators of all CTAs (start at zero,
                                                                 // left at zero), [0] CTAs done, [1] non-finite sum
   const int32_t* split_any;            // [3] does split s hold a non-zero anywhere
-  uint32_t op_bytes;                   // shared memory for operand stages
+  int stages;                          // operand stages that fit into shared memory
+  uint32_t stage_bytes;
   int n1, n2;                          // MMA N of the first (<= 256) and second instruction; n1 + n2 = ceil16(M)
   int32_t* status;
 };
@@ -131,7 +132,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   const int M = p.M;
-  uint8_t* zstage = smem + p.op_bytes;                              // [8 warps] 32 x 32 fp32 tiles of z
+  uint8_t* zstage = smem + (size_t)p.stages * p.stage_bytes;        // [8 warps] 32 x 32 fp32 tiles of z
   uint8_t* tail = zstage + kEpiWarps * kZStage;
   uint64_t* full_bar = reinterpret_cast<uint64_t*>(tail);
   uint64_t* empty_bar = full_bar + kMaxStages;
@@ -160,7 +161,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   // k-blocks before the next term's: the order of the sums is part of the logits' last bits.
   const int any1 = p.split_any[1], any2 = p.split_any[2];
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kMaxStages; ++s) { tc::mbar_init(&full_bar[s], 1); tc::mbar_init(&empty_bar[s], 1); }
+    for (int s = 0; s < p.stages; ++s) { tc::mbar_init(&full_bar[s], 1); tc::mbar_init(&empty_bar[s], 1); }
     for (int a = 0; a < 2; ++a) { tc::mbar_init(&tmem_full[a], 1); tc::mbar_init(&tmem_empty[a], 2 * kEpiWarps); }
     for (int i = 0; i < 8; ++i) tc::mbar_init(&xbar[i], 2);
     *abort = 0;
@@ -181,11 +182,10 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   tc::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_ptr;
   const uint32_t w1_bytes = (uint32_t)(p.n1 / 2) * (kBK * 2), w2_bytes = (uint32_t)(p.n2 / 2) * (kBK * 2);
-  const uint32_t w_bytes = w1_bytes + w2_bytes;
   const int n_terms = 1 + (any1 != 0) + (any2 != 0);
   const int second = any1 != 0 ? 1 : 2;                             // term numbers: 0, second, 2
-  const uint32_t stage_bytes = kXBytes + w_bytes;
-  const int stages = min(kMaxStages, (int)(p.op_bytes / stage_bytes));
+  const uint32_t stage_bytes = p.stage_bytes;
+  const int stages = p.stages;
 
   if (warp == 0) {
     // ------------------------------------------------------------ TMA producer (one in each CTA)
@@ -695,13 +695,13 @@ int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, fl
   const int n_cols = (M + 15) / 16 * 16;
   p.n1 = n_cols < 256 ? n_cols : 256;
   p.n2 = n_cols - p.n1;
-  const uint32_t stage_bytes = kXBytes + (uint32_t)(n_cols / 2) * (kBK * 2);      // with one term
+  p.stage_bytes = kXBytes + (uint32_t)(n_cols / 2) * (kBK * 2);
   const uint32_t tail_bytes = kTailBars + 2 * kTile * 2 * 4 + 2 * kTile * UNIPOOL_MAX_TOPK * 4 + UNIPOOL_MAX_EXPERTS * 4 +
                               kEpiWarps * M * 4 + (M + 31) / 32 * 32 * 4;
   const uint32_t budget = kSmemMax - 1024 - tail_bytes - kEpiWarps * kZStage;
-  const uint32_t most = (uint32_t)kMaxStages * stage_bytes;
-  p.op_bytes = (budget < most ? budget : most) / 1024 * 1024;
-  UP_REQUIRE(p.op_bytes >= 2 * stage_bytes && ctx->sm_count >= 2, UNIPOOL_ERR_UNSUPPORTED,
+  p.stages = (int)(budget / p.stage_bytes);
+  if (p.stages > kMaxStages) p.stages = kMaxStages;
+  UP_REQUIRE(p.stages >= 2 && ctx->sm_count >= 2, UNIPOOL_ERR_UNSUPPORTED,
              "router of %d experts does not fit the logits kernel", M);
   CUtensorMap tmX, tmW1, tmW2, tmZ;
   if ((M & 3) == 0) {
@@ -717,7 +717,7 @@ int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, fl
     tmW2 = tmW1;
   }
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_SELECT, 1, s);
-  const size_t smem = (size_t)p.op_bytes + kEpiWarps * kZStage + tail_bytes + 1024;
+  const size_t smem = (size_t)p.stages * p.stage_bytes + kEpiWarps * kZStage + tail_bytes + 1024;
   const int n_tp = (T + 2 * kTile - 1) / (2 * kTile);
   const int max_pairs = ctx->sm_count / 2;
   const int grid = 2 * (n_tp < max_pairs ? n_tp : max_pairs);
