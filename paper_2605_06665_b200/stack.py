@@ -165,14 +165,20 @@ class UniPoolStack:
 
     def _arrays(self):
         """This stack's arrays as they are now, for the calls that run all layers; None if one of them is not
-        a dense array over the layers."""
+        a dense array over the layers.  (Arrays that were given up, as an evaluation may those of backward, are NULL:
+        a call that needs them refuses them.)"""
         wgrad = self.Lg if self.deferred_wgrad else self.nw
         s = B.Stack(self.L, self.Lg, self.m, int(self.recompute), wgrad)
-        for n, numel in self._stacked:
-            t = getattr(self, n)
-            if not t.is_contiguous() or t.numel() != numel:
-                return None
-            setattr(s, n, t.data_ptr())
+        try:
+            for n, numel in self._stacked:
+                t = getattr(self, n)
+                if t is None:
+                    continue
+                if not t.is_contiguous() or t.numel() != numel:
+                    return None
+                setattr(s, n, t.data_ptr())
+        except AttributeError:                             # a list of per-layer arrays
+            return None
         b = self.bias
         if b is not None:
             if not (isinstance(b, torch.Tensor) and b.is_cuda and b.dtype is torch.float32 and b.is_contiguous()

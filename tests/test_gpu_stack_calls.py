@@ -194,6 +194,8 @@ def test_arrays_of_the_caller_that_are_slices_of_larger_ones():
     st.z = torch.zeros(L, T + 1, M, device="cuda")[:, :T]
     st.x = torch.zeros(L + 1, T + 8, d, dtype=st.tdtype, device="cuda")[:, :T]
     same(stack_results(st, x0, up), want)
+    st.znorm = list(torch.zeros(L, T, device="cuda"))             # an array per layer
+    same(stack_results(st, x0, up), want)
     st.sigma = st.sigma[:2]
     with pytest.raises(IndexError):
         st.forward(x0)
@@ -349,3 +351,21 @@ def test_native_loops_give_what_the_layers_give_one_by_one(shape, kw):
     st.close()
     del st, both, got, want
     torch.cuda.empty_cache()
+
+
+def test_evaluation_without_the_arrays_of_backward():
+    """A stack that only evaluates may give up what backward needs; a backward call then is refused, not run."""
+    import torch
+    from paper_2605_06665_b200 import binding as B
+    st, x0, up = make(2, 64, 128, 8, 2, 150, deferred_wgrad=True)
+    want = st.forward(x0).clone()
+    loss = st.aux_loss().clone()
+    for n in ("dYp", "dGU", "dx", "dW_gu", "dW_down"):
+        setattr(st, n, None)
+    assert torch.equal(st.forward(x0), want) and torch.equal(st.aux_loss(), loss)
+    st.dx = torch.empty(2, st.T, st.d, dtype=st.tdtype, device="cuda")
+    with pytest.raises(B.UniPoolError):
+        st.backward(up)
+    torch.cuda.synchronize()
+    st.ctx.check_status()
+    st.close()
