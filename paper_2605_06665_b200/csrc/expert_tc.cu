@@ -1396,18 +1396,19 @@ bool rows_on_pairs(const unipool_ctx* ctx, int n_experts) {
 // leave out: 31 rows padded to 128, down 69/72, dgrads 89/93 and 117/123).  Large groups waste nothing in 256-row
 // pair-tiles: down and dgrad gate/up gain while a group is one or two chunks, and need a contraction long enough to
 // hide the epilogue of a unit; dgrad down gains longest, its G and U traffic being the same on fewer padded rows.
-// Where the lines lie beside the rows, from 2000 shapes of 384..1536 x 256..4096 (weights on M against tokens on M,
-// mean of the shapes on the far side of a line; 'deal': the part of the pairs' rounds that the units fill):
-//   width of the last weight tile  gate/up of 320 and 640 columns +20..35 %, down below 0.8 of a tile +5 %, dgrad down
-//                                  below 0.85 on large groups +5 % where the contraction is short
-//   gate/up, chunks filled         195..265 rows are two half-empty chunks: +5..8 %; 120..190 rows one chunk, -7 % from
-//                                  d = 1024 on and 0 below; 270..560 rows -5 % from d = 1024 on, -1 % at 768 .. 1023, 0
-//                                  below (+8 % at f = 512, 0 at 768); 620..870 rows +5 %
-//   down                           f below 1536 +1 %; 49..130 rows +2 % (a few long groups: -4 %); a poor deal +3..14 %
-//   dgrad gate/up                  more than 192 experts +5..17 % under skewed routing (the largest group sets the size of
-//                                  a stage), 0 under even; 91..130 rows in a poor deal +4 %; large groups in a poor one +8 %
-//   dgrad down, beyond 200 rows    d below 640 +5 %, f below 512 +2..20 %; up to 200 rows f below 512 +2..20 % under
-//                                  skewed routing while d is below 1024 (-10..+5 % under even)
+// Where the lines lie beside the rows: 2000 shapes of 384 .. 1536 x 256 .. 4096 in single bursts, and 320 of them held
+// for a second.  Held, a launch of more than some 100 us ends at the power cap, where weights on M is 3 to 4 % better
+// than in a burst (it moves fewer bytes per FLOP); the lines are those of held launches.  Figures: weights on M against
+// tokens on M, held (burst), time of both GEMMs of the direction.  'Deals': rounds of units over the CTA pairs.
+//   gate/up       last weight tile mostly empty: f = 320, 384, 1088 +10 % (+14 %), 640 +2 % (+5 %); chunks of 192 rows
+//                 more than 0.7 full: -4 .. -12 % (-2 .. -8 %), half full (195 .. 265 rows, below 130): -3 .. -5 % (0 ..
+//                 +2 %) in many deals, +2 .. +3 % (+4 .. +8 %) in fewer than 9
+//   down          61 .. 130 rows: +1 .. +5 % (+1 .. +7 %) below f = 3072, -1 % above; d = 576 (last tile a quarter full)
+//                 +2 .. +4 % beyond 48 rows; a poor deal of large groups +5 .. +20 %, of groups below 130 rows +4 .. +7 %
+//   dgrad down    only a short contraction in large groups: d = 512, f = 832 or 1216, 480 rows +4 .. +7 % (+7 %)
+//   dgrad gate/up more than 192 experts of f = 640 +2 .. +4 % (+3 .. +8 %) under skewed routing (the largest group sets
+//                 the size of a stage); 91 .. 130 rows in a poor deal +1 .. +4 %; large groups in one +7 .. +18 %, small
+//                 ones +8 %
 bool weights_on_m(const unipool_ctx* ctx, int mode, int n_experts, bool sizes_known) {
   if (ctx->sm_count < 2 || n_experts > kWmMaxExperts) return false;
   const int64_t rows = (int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k / n_experts;
@@ -1419,28 +1420,21 @@ bool weights_on_m(const unipool_ctx* ctx, int mode, int n_experts, bool sizes_kn
   const int columns = plain ? d : f, tiles = (columns + 255) / 256;
   const float width = (float)columns / (256 * tiles);
   const int pairs = ctx->sm_count / 2, units = n_experts * tiles * chunks;
-  const float deal = (float)units / ((units + pairs - 1) / pairs * pairs);
+  const float deals = (float)units / pairs, deal = (float)units / ((units + pairs - 1) / pairs * pairs);
+  const float full = r > 200 ? 0.7f : r > 130 ? 0.f : 0.6f;
   switch (mode) {
-    case kFwd1: {
-      if (width < 0.9f || deal < 0.75f) return false;
-      const bool filled = 10 * r >= 7 * 192 * chunks;
-      if (d >= 1024)
-        return chunks == 1 ? r > 120 && r <= 190 && f >= 1024
-                           : filled && (r <= 560 || r > 900) && r <= 1024 && f >= 768;
-      if (d >= 768) return f >= 2048 && r > 150 && r <= 185 || f >= 1024 && r >= 300 && r <= 384;
-      return f >= 3072 && r >= 300 && r <= 384;
-    }
+    case kFwd1:
+      if (r <= (d >= 1024 ? 100 : 150) || r > (d >= 1024 ? 1024 : 600) || width < 0.87f) return false;
+      return deals >= (d >= 1024 ? 10.f : 13.f) || (10 * r >= 7 * 192 * chunks && deals >= 4.f);
     case kFwd2:
-      if (f < 1536 || r > 450 || width < 0.8f) return false;
-      if (r > 48 && r <= 130) return n_experts < 48 && deal >= 0.9f;
-      return r <= 200 || deal >= (r <= 390 ? 0.8f : 0.9f);
+      if (f <= 1024 || r > 450 || (r > 48 && width < 0.8f) || (r > 60 && r <= 130 && f < 3072)) return false;
+      return deal >= full;
     case kDgrad1:
-      if (r <= 200) return (r <= 48 || r > 100 || f > 1024) && (r <= 48 || f >= 512 || d >= 1024);
-      return d >= 640 && f >= 512 && (width >= 0.85f || d >= 1024);
+      return (r <= 48 || r > 100 || f > 1024) && (r <= 200 || d >= 640 || f >= 1280);
     default:
-      if (2 * f <= 1024 || r > 450 || n_experts > 192) return false;
-      if (r > 90 && r <= 130) return deal >= 0.9f;
-      return r <= 200 || deal >= 0.7f;
+      if (2 * f <= 1024 || r > 450 || (n_experts > 192 && f < 768)) return false;
+      if (r > 90 && r <= 130) return deal >= 0.9f && width >= 0.8f;
+      return deal >= full;
   }
 }
 

@@ -21,10 +21,10 @@ def on_weights(d, f, experts, k, T, sizes_known=True, pool=None):
 
 @pytest.mark.parametrize("sizes,d,f,forms,forms_padded", [
     # one chunk of <= 192 tokens at gate/up on average, up to three in the largest groups
-    ([0, 1, 15, 16, 17, 31, 33, 191, 192, 193, 255, 256, 257, 383, 384, 385], 1024, 1984, "WWWW", "WWWW"),
-    ([301, 383, 384, 385, 193, 192, 290], 768, 1216, "WTWT", "WTWT"),      # two chunks; a partial weight tile
-    ([383, 384, 385, 401, 512, 450, 397], 1280, 1728, "WWWW", "WWWW"),     # two MMAs, three chunks
-    ([48, 1, 0, 33, 64, 65, 17], 256, 1600, "TWWW", "TTTT"),               # few rows; an odd number of k-blocks
+    ([0, 1, 15, 16, 17, 31, 33, 191, 192, 193, 255, 256, 257, 383, 384, 385], 1024, 4864, "WWWW", "WWWW"),
+    ([301, 383, 384, 385, 193, 192, 290] * 2, 768, 3008, "WTWT", "WTWT"),  # two chunks; a partial weight tile
+    ([383, 384, 385, 401, 512, 450, 397], 1280, 3840, "WWWW", "WWWW"),     # two MMAs, three chunks
+    ([48, 1, 0, 33, 64, 65, 17] * 3, 768, 1600, "TWWW", "TTTT"),           # few rows; an odd number of k-blocks
 ])
 @pytest.mark.parametrize("with_rows", [True, False])
 def test_weights_on_m_where_it_is_chosen(sizes, d, f, forms, forms_padded, with_rows):
@@ -36,9 +36,10 @@ def test_weights_on_m_where_it_is_chosen(sizes, d, f, forms, forms_padded, with_
 @pytest.mark.parametrize("shape,forms", [
     ((768, 2048, 96, 2, 16384), "WWWW"), ((768, 2048, 96, 2, 1501), "TWWW"), ((768, 2048, 96, 2, 33), "TWWW"),
     ((1536, 4096, 192, 2, 32768), "WWWW"),
-    ((768, 512, 384, 8, 16384), "TTWT"),               # narrow experts
-    ((768, 320, 300, 6, 8000), "TTTT"),                # ... and a half-empty last weight tile
-    ((768, 2048, 96, 2, 11000), "TWWW"),               # 229 rows: two half-empty chunks at gate/up
+    ((768, 512, 384, 8, 16384), "WTWT"),               # narrow experts
+    ((768, 320, 300, 6, 8000), "TTWT"),                # ... and a half-empty last weight tile
+    ((768, 2048, 96, 2, 11000), "WWWW"),               # 229 rows: two half-empty chunks at gate/up, in many deals
+    ((768, 2048, 29, 2, 464), "TTWT"),                 # few rows, and units for 1.2 rounds
     ((384, 768, 24, 2, 4000), "TTTT"),
     ((768, 2048, 40, 2, 16384), "TTWT"), ((768, 2048, 8, 2, 16384), "TTTT"),
     ((768, 2048, 480, 2, 8192), "TTTT"),               # more experts than the unit list holds
