@@ -9,6 +9,7 @@ __global__ void __launch_bounds__(512)
 pool_aux_kernel(const int32_t* __restrict__ counts, const float* __restrict__ S, int L, int M, int T,
                 int k, float alpha, const float* __restrict__ fbar_prev, float* __restrict__ loss,
                 float* __restrict__ coef, float* __restrict__ fbar_out) {
+  grid_wait(counts, S, fbar_prev);
   __shared__ double red[512];
   double term = 0.0;
   for (int i = threadIdx.x; i < M; i += blockDim.x) {
@@ -37,9 +38,7 @@ int aux_launch(unipool_ctx* ctx, const int32_t* counts, const float* S, int L, i
                float alpha, const float* fbar_prev, float* loss, float* coef, float* fbar_out,
                cudaStream_t s) {
   PhaseTimer pt(ctx, UNIPOOL_PH_POOL_AUX, 1, s);
-  pool_aux_kernel<<<1, 512, 0, s>>>(counts, S, L, M, T, ctx->cfg.top_k, alpha, fbar_prev, loss, coef,
-                                    fbar_out);
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(pool_aux_kernel, 1, 512, 0, s, counts, S, L, M, T, ctx->cfg.top_k, alpha, fbar_prev, loss, coef, fbar_out);
   return UNIPOOL_OK;
 }
 

@@ -42,6 +42,42 @@ void set_error(const char* fmt, ...);
     }                                                                                  \
   } while (0)
 
+// ---------------------------------------------------------------- launches
+// Every kernel of a pass is launched with programmatic serialization: the launch itself, and what a kernel does before
+// grid_wait(), run while the last blocks of the kernel before it in the stream drain; its memory is touched behind
+// grid_wait() only.  Between two kernels of an eager pass lie 0.2 us instead of 2.0 .. 2.8; a pass of 16 experts of
+// 256 x 512 over 512 tokens in fp32 (55 launches) takes 856 us instead of 959, a forward pass of 33 tokens through
+// twelve layers 1509 instead of 1632, a step of 16384 tokens over private experts 12455 instead of 12772.
+template <typename... P, typename... A>
+inline cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+#define UP_KERNEL(kern, grid, block, smem, s, ...) \
+  UP_CUDA(unipool::launch_kernel(kern, dim3(grid), dim3(block), smem, s, __VA_ARGS__))
+
+#ifdef __CUDACC__
+// Waits until the kernels before this one in the stream are complete and their writes visible.  All threads call it,
+// before they touch global memory.  The pointers that it is given come out of it, so that no load through them (a
+// read-only one has no order of its own) can be moved in front of it.
+template <typename P>
+__device__ __forceinline__ void after_asm(P& p) { asm volatile("" : "+l"(p)); }
+template <typename... P>
+__device__ __forceinline__ void grid_wait(P&... p) {
+  asm volatile("griddepcontrol.wait;" : : : "memory");
+  (after_asm(p), ...);
+}
+#endif
+
 // ---------------------------------------------------------------- workspace
 // Fixed layout of the caller's workspace; every region is 256-byte aligned.
 struct Workspace {

@@ -42,6 +42,7 @@ __device__ __forceinline__ bool routed(int e, int M, int32_t* status) {
 __global__ void __launch_bounds__(kHistWarps * 32)
 dispatch_hist_kernel(const int32_t* __restrict__ idx, int T, int k, int M, int chunk, ChunkCounts cc,
                      int32_t* __restrict__ status) {
+  grid_wait(idx);
   extern __shared__ int hist[];                      // [kHistWarps][M]
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   for (int i = threadIdx.x; i < kHistWarps * M; i += blockDim.x) hist[i] = 0;
@@ -93,6 +94,7 @@ dispatch_place_kernel(const int32_t* __restrict__ idx, int T, int k, int M, int 
                       int row_vecs, int row_capacity, int32_t* __restrict__ offsets,
                       int32_t* __restrict__ row_of, int32_t* __restrict__ token_of,
                       int32_t* __restrict__ tile_expert, int32_t* __restrict__ group_rows, uint4* __restrict__ Xp) {
+  grid_wait(idx, x);
   extern __shared__ int sm[];
   int* hist = sm;                                   // [8][M] per-warp histograms, then per-warp next rows
   int* start = hist + kDispatchWarps * M;           // [M + 1] group starts
@@ -306,6 +308,7 @@ __global__ void __launch_bounds__(256)
 combine_kernel(const uint4* __restrict__ Yp, const int32_t* __restrict__ row_of,
                const float* __restrict__ gate, const uint4* __restrict__ residual,
                uint4* __restrict__ y, int n_tokens, int k, int row_vecs) {
+  grid_wait(Yp, row_of, gate, residual);
   constexpr int N = Vec16<T>::N;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   for (int t = blockIdx.x * 8 + warp; t < n_tokens; t += gridDim.x * 8) {
@@ -366,6 +369,7 @@ combine_bwd_kernel(const uint4* __restrict__ dy, const uint4* __restrict__ Yp,
                    const int32_t* __restrict__ token_of, const int32_t* __restrict__ offsets,
                    int32_t* __restrict__ group_rows, int pad_step, int M, uint4* __restrict__ dYp,
                    float* __restrict__ dgate, int n_tokens, int k, int row_vecs) {
+  grid_wait(dy, Yp, row_of, gate, token_of, offsets);
   constexpr int N = Vec16<T>::N;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int groups = (k + KT - 1) / KT;
@@ -445,6 +449,7 @@ combine_bwd_kernel(const uint4* __restrict__ dy, const uint4* __restrict__ Yp,
 
 __global__ void dispatch_empty_kernel(int32_t* offsets, int32_t* token_of, int32_t* tile_expert, int32_t* group_rows,
                                       int M, int row_capacity) {
+  grid_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (group_rows != nullptr && i < M) group_rows[i] = 0;
   if (i <= M) offsets[i] = 0;
@@ -480,16 +485,13 @@ static int permute_launch(unipool_ctx* prof, const void* x, int T, int k, const 
     cc.n_super = 0;
   } else {
     PhaseTimer pt(prof, UNIPOOL_PH_DISPATCH_MAPS, 1, s);
-    dispatch_hist_kernel<<<cc.n_super, kHistWarps * 32, kHistWarps * M * sizeof(int), s>>>(idx, T, k, M, chunk, cc, status);
-    UP_LAUNCH_CHECK();
+    UP_KERNEL(dispatch_hist_kernel, cc.n_super, kHistWarps * 32, kHistWarps * M * sizeof(int), s, idx, T, k, M, chunk, cc, status);
   }
   PhaseTimer pt(prof, UNIPOOL_PH_DISPATCH_GATHER, 1, s);
   // A small batch has few chunks but as many pad rows as a large one: blocks without a chunk share those.
   const int grid = n_chunks > sm_count ? n_chunks : sm_count;
-  dispatch_place_kernel<<<grid, kDispatchWarps * 32, place_smem_bytes(M, k, chunk), s>>>(
-      idx, T, k, M, chunk, cc, status, static_cast<const uint4*>(x), row_vecs, cap, offsets, row_of, token_of, tile_expert,
+  UP_KERNEL(dispatch_place_kernel, grid, kDispatchWarps * 32, place_smem_bytes(M, k, chunk), s, idx, T, k, M, chunk, cc, status, static_cast<const uint4*>(x), row_vecs, cap, offsets, row_of, token_of, tile_expert,
       rows, static_cast<uint4*>(Xp));
-  UP_LAUNCH_CHECK();
   return UNIPOOL_OK;
 }
 
@@ -505,8 +507,7 @@ int dispatch_launch(unipool_ctx* ctx, const void* x, int T, const int32_t* idx, 
   const int k = ctx->cfg.top_k, d = ctx->cfg.d_model;
   const int cap = (int)ctx->row_capacity;
   if (T == 0) {
-    dispatch_empty_kernel<<<(cap + 255) / 256, 256, 0, s>>>(offsets, token_of, tile_expert, rows, M, cap);
-    UP_LAUNCH_CHECK();
+    UP_KERNEL(dispatch_empty_kernel, (cap + 255) / 256, 256, 0, s, offsets, token_of, tile_expert, rows, M, cap);
     return UNIPOOL_OK;
   }
   return permute_launch(ctx, x, T, k, idx, M, dispatch_chunk_tokens(T, ctx->sm_count), ctx->sm_count, ctx->ws.block_hist,
@@ -515,15 +516,14 @@ int dispatch_launch(unipool_ctx* ctx, const void* x, int T, const int32_t* idx, 
 }
 
 template <typename T>
-static void combine_dispatch_k(int grid, cudaStream_t s, int k, const void* Yp, const int32_t* row_of,
-                               const float* gate, const void* residual, void* y, int n_tokens, int row_vecs) {
+static int combine_dispatch_k(int grid, cudaStream_t s, int k, const void* Yp, const int32_t* row_of,
+                              const float* gate, const void* residual, void* y, int n_tokens, int row_vecs) {
   auto Y = static_cast<const uint4*>(Yp);
   auto R = static_cast<const uint4*>(residual);
   auto O = static_cast<uint4*>(y);
-  if (k <= 1) combine_kernel<T, 1><<<grid, 256, 0, s>>>(Y, row_of, gate, R, O, n_tokens, k, row_vecs);
-  else if (k <= 2) combine_kernel<T, 2><<<grid, 256, 0, s>>>(Y, row_of, gate, R, O, n_tokens, k, row_vecs);
-  else if (k <= 4) combine_kernel<T, 4><<<grid, 256, 0, s>>>(Y, row_of, gate, R, O, n_tokens, k, row_vecs);
-  else combine_kernel<T, 8><<<grid, 256, 0, s>>>(Y, row_of, gate, R, O, n_tokens, k, row_vecs);
+  auto kern = k <= 1 ? combine_kernel<T, 1> : k <= 2 ? combine_kernel<T, 2> : k <= 4 ? combine_kernel<T, 4> : combine_kernel<T, 8>;
+  UP_KERNEL(kern, grid, 256, 0, s, Y, row_of, gate, R, O, n_tokens, k, row_vecs);
+  return UNIPOOL_OK;
 }
 
 static int combine_phase(unipool_ctx* ctx, int phase, const void* Yp, const int32_t* row_of,
@@ -534,11 +534,8 @@ static int combine_phase(unipool_ctx* ctx, int phase, const void* Yp, const int3
   const int row_vecs = (int)((size_t)ctx->cfg.d_model * ctx->elem_bytes / 16);
   const int grid = row_mover_grid(ctx, T);
   if (ctx->cfg.dtype == UNIPOOL_BF16)
-    combine_dispatch_k<__nv_bfloat16>(grid, s, k, Yp, row_of, gate, residual, y, T, row_vecs);
-  else
-    combine_dispatch_k<float>(grid, s, k, Yp, row_of, gate, residual, y, T, row_vecs);
-  UP_LAUNCH_CHECK();
-  return UNIPOOL_OK;
+    return combine_dispatch_k<__nv_bfloat16>(grid, s, k, Yp, row_of, gate, residual, y, T, row_vecs);
+  return combine_dispatch_k<float>(grid, s, k, Yp, row_of, gate, residual, y, T, row_vecs);
 }
 
 int combine_launch(unipool_ctx* ctx, const void* Yp, const int32_t* row_of, const float* gate, int T,
@@ -547,16 +544,17 @@ int combine_launch(unipool_ctx* ctx, const void* Yp, const int32_t* row_of, cons
 }
 
 template <typename T>
-static void combine_bwd_dispatch_k(int grid, cudaStream_t s, int k, const void* dy, const void* Yp,
-                                   const int32_t* row_of, const float* gate, const int32_t* token_of,
-                                   const int32_t* offsets, int32_t* rows, int M, void* dYp, float* dgate,
-                                   int n_tokens, int row_vecs) {
+static int combine_bwd_dispatch_k(int grid, cudaStream_t s, int k, const void* dy, const void* Yp,
+                                  const int32_t* row_of, const float* gate, const int32_t* token_of,
+                                  const int32_t* offsets, int32_t* rows, int M, void* dYp, float* dgate,
+                                  int n_tokens, int row_vecs) {
   constexpr int step = sizeof(T) == 2 ? kRowStep : UNIPOOL_ROW_ALIGN;       // (the fp32 kernels read whole groups)
   auto D = static_cast<const uint4*>(dy);
   auto Y = static_cast<const uint4*>(Yp);
   auto O = static_cast<uint4*>(dYp);
-  if (k <= 1) combine_bwd_kernel<T, 1><<<grid, 256, 0, s>>>(D, Y, row_of, gate, token_of, offsets, rows, step, M, O, dgate, n_tokens, k, row_vecs);
-  else combine_bwd_kernel<T, 2><<<grid, 256, 0, s>>>(D, Y, row_of, gate, token_of, offsets, rows, step, M, O, dgate, n_tokens, k, row_vecs);
+  UP_KERNEL((k <= 1 ? combine_bwd_kernel<T, 1> : combine_bwd_kernel<T, 2>), grid, 256, 0, s, D, Y, row_of, gate, token_of, offsets, rows,
+            step, M, O, dgate, n_tokens, k, row_vecs);
+  return UNIPOOL_OK;
 }
 
 int combine_bwd_launch(unipool_ctx* ctx, const void* dy, int T, const int32_t* row_of,
@@ -570,11 +568,8 @@ int combine_bwd_launch(unipool_ctx* ctx, const void* dy, int T, const int32_t* r
   const int grid = row_mover_grid(ctx, (int64_t)T * ((k + 1) / 2) + pads);
   PhaseTimer pt(ctx, UNIPOOL_PH_BWD_SCALE_GATHER, 1, s);
   if (ctx->cfg.dtype == UNIPOOL_BF16)
-    combine_bwd_dispatch_k<__nv_bfloat16>(grid, s, k, dy, Yp, row_of, gate, token_of, offsets, rows, M, dYp, dgate, T, row_vecs);
-  else
-    combine_bwd_dispatch_k<float>(grid, s, k, dy, Yp, row_of, gate, token_of, offsets, rows, M, dYp, dgate, T, row_vecs);
-  UP_LAUNCH_CHECK();
-  return UNIPOOL_OK;
+    return combine_bwd_dispatch_k<__nv_bfloat16>(grid, s, k, dy, Yp, row_of, gate, token_of, offsets, rows, M, dYp, dgate, T, row_vecs);
+  return combine_bwd_dispatch_k<float>(grid, s, k, dy, Yp, row_of, gate, token_of, offsets, rows, M, dYp, dgate, T, row_vecs);
 }
 
 int unpermute_sum_launch(unipool_ctx* ctx, const void* dXp, const int32_t* row_of, int T,
@@ -647,8 +642,7 @@ extern "C" int unipool_dispatch_static(const void* x, int32_t T, int32_t d_model
   int32_t* counts = info->addr + 64;
   const int cap = (int)row_capacity;
   if (T == 0) {
-    dispatch_empty_kernel<<<(cap + 255) / 256, 256, 0, s>>>(offsets, token_of, tile_expert, nullptr, n_experts, cap);
-    UP_LAUNCH_CHECK();
+    UP_KERNEL(dispatch_empty_kernel, (cap + 255) / 256, 256, 0, s, offsets, token_of, tile_expert, nullptr, n_experts, cap);
     return UNIPOOL_OK;
   }
   // the counts are fully rewritten by the first kernel for the chunks of this call; nothing else in the

@@ -33,6 +33,7 @@ grouped_rows_gemm_kernel(const RowGemm p) {
   constexpr int TN = kSimtN;
   extern __shared__ float4 smem_raw[];
   typename T::Smem& sm = *reinterpret_cast<typename T::Smem*>(smem_raw);
+  grid_wait();
   const int n0 = blockIdx.x * (EPI == kSwiglu ? TN / 2 : TN);
   for (int rt = blockIdx.y; rt < p.n_row_tiles; rt += gridDim.y) {
     const int m0 = rt * TM;
@@ -103,6 +104,7 @@ __global__ void __launch_bounds__(SimtTile<64, 2>::kThreads)
 grouped_k_gemm_kernel(const PoolGemm p) {
   using T = SimtTile<64, 2>;
   __shared__ typename T::Smem sm;
+  grid_wait();
   const int m0 = blockIdx.x * 64, n0 = blockIdx.y * 64, e = blockIdx.z;
   auto rows_of = [&](int l) {
     const int32_t* off = p.offsets + (int64_t)l * (p.n_experts + 1) + e;
@@ -156,8 +158,7 @@ int rows_gemm_as(const unipool_ctx* ctx, RowGemm p, cudaStream_t s) {
   if (smem > 48 * 1024) UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
   p.n_row_tiles = (int)(ctx->row_capacity / TM);
   const int gy = p.n_row_tiles < 8192 ? p.n_row_tiles : 8192;
-  kern<<<dim3(p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN), gy), SimtTile<TM, KG>::kThreads, smem, s>>>(p);
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(kern, dim3(p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN), gy), (SimtTile<TM, KG>::kThreads), smem, s, p);
   return UNIPOOL_OK;
 }
 
@@ -223,16 +224,14 @@ int pool_wgrad_simt(unipool_ctx* ctx, const PoolWgradArgs& a, cudaStream_t s) {
     p.P = static_cast<const float*>(a.dYp); p.ldp = d;
     p.Q = static_cast<const float*>(a.A); p.ldq = f;
     p.dW = a.dW_down; p.Mdim = d; p.Ndim = f; p.vec = aligned16(p.P, p.Q, p.dW);
-    grouped_k_gemm_kernel<<<dim3(d / 64, f / 64, a.n_experts), SimtTile<64, 2>::kThreads, 0, s>>>(p);
-    UP_LAUNCH_CHECK();
+    UP_KERNEL(grouped_k_gemm_kernel, dim3(d / 64, f / 64, a.n_experts), (SimtTile<64, 2>::kThreads), 0, s, p);
   }
   if (a.dW_gu == nullptr) return UNIPOOL_OK;
   PhaseTimer pt(ctx, UNIPOOL_PH_WGRAD_GU, 1, s);     // dW_gu[e] [2f, d] (+)= dGU_e^T Xp_e
   p.P = static_cast<const float*>(a.dGU); p.ldp = 2 * f;
   p.Q = static_cast<const float*>(a.Xp); p.ldq = d;
   p.dW = a.dW_gu; p.Mdim = 2 * f; p.Ndim = d; p.vec = aligned16(p.P, p.Q, p.dW);
-  grouped_k_gemm_kernel<<<dim3(2 * f / 64, d / 64, a.n_experts), SimtTile<64, 2>::kThreads, 0, s>>>(p);
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(grouped_k_gemm_kernel, dim3(2 * f / 64, d / 64, a.n_experts), (SimtTile<64, 2>::kThreads), 0, s, p);
   return UNIPOOL_OK;
 }
 

@@ -335,6 +335,7 @@ grouped_gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_con
   __syncthreads();
   tc::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_ptr;
+  grid_wait();
 
   int n_nt, n_mt;
   const int n_tiles = tiles_total<MODE>(p, n_nt, n_mt);
@@ -718,6 +719,7 @@ wgrad_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant
   tc::cluster_sync();                                        // both CTAs' barriers exist before any remote use
   tc::tc_fence_after_sync();
   const uint32_t tmem_base = *tmem_ptr;
+  grid_wait();
 
   const int n_mt = (p.Mdim + 255) / 256, n_nt = (p.Ndim + 255) / 256;
   const int per_e = n_mt * n_nt;
@@ -1132,6 +1134,7 @@ row_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__
     tc::tmem_alloc_pair(tmem_ptr, 512);
     tc::tmem_relinquish_pair();
   }
+  grid_wait();
   // pair-tiles before each expert: an expert of n row tiles takes ceil(n / 2), the last one a half
   // pair-tile when n is odd
   for (int e = threadIdx.x; e <= p.n_experts; e += blockDim.x) {
@@ -1366,8 +1369,7 @@ int launch(unipool_ctx* ctx, int phase, const CUtensorMap& tmA, const CUtensorMa
   PhaseTimer pt(ctx, phase, 1, s);
   auto kern = grouped_gemm_tc_kernel<MODE>;
   UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTotal));
-  kern<<<ctx->sm_count, Traits<MODE>::kThreads, kSmemTotal, s>>>(tmA, tmB, tmB64, tmC0, tmC1, p);
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(kern, ctx->sm_count, Traits<MODE>::kThreads, kSmemTotal, s, tmA, tmB, tmB64, tmC0, tmC1, p);
   return UNIPOOL_OK;
 }
 
@@ -1449,13 +1451,12 @@ int launch_rows(unipool_ctx* ctx, int phase, bool pairs, const CUtensorMap& tmA,
   if (pairs) {
     auto kern = row_pair_kernel<MODE>;
     UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemTotal));
-    kern<<<ctx->sm_count / 2 * 2, PairTraits<MODE>::kThreads, kPairSmemTotal, s>>>(tmA, tmA64, tmBp, tmC0, tmC1, p);
+    UP_KERNEL(kern, ctx->sm_count / 2 * 2, PairTraits<MODE>::kThreads, kPairSmemTotal, s, tmA, tmA64, tmBp, tmC0, tmC1, p);
   } else {
     auto kern = grouped_gemm_tc_kernel<MODE>;
     UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemTotal));
-    kern<<<ctx->sm_count, Traits<MODE>::kThreads, kSmemTotal, s>>>(tmA, tmB, tmB64, tmC0, tmC1, p);
+    UP_KERNEL(kern, ctx->sm_count, Traits<MODE>::kThreads, kSmemTotal, s, tmA, tmB, tmB64, tmC0, tmC1, p);
   }
-  UP_LAUNCH_CHECK();
   return UNIPOOL_OK;
 }
 
@@ -1466,8 +1467,7 @@ int launch_wgrad(unipool_ctx* ctx, int phase, const CUtensorMap& tmP, const CUte
   PhaseTimer pt(ctx, phase, 1, s);
   auto kern = k_rows == 32 ? wgrad_pair_kernel<32> : k_rows == 48 ? wgrad_pair_kernel<48> : wgrad_pair_kernel<64>;
   UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmemTotal));
-  kern<<<ctx->sm_count / 2 * 2, kThreads, kPairSmemTotal, s>>>(tmP, tmQ, tmW, p);
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(kern, ctx->sm_count / 2 * 2, kThreads, kPairSmemTotal, s, tmP, tmQ, tmW, p);
   return UNIPOOL_OK;
 }
 

@@ -271,6 +271,7 @@ wm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ Token
     tc::tmem_alloc_pair(tmem_ptr, 512);
     tc::tmem_relinquish_pair();
   }
+  grid_wait();
   // the list of experts: a thread ranks its expert by counting the larger keys (unit size, then lower index first);
   // every CTA computes the same list
   uint32_t* key = reinterpret_cast<uint32_t*>(smem);                           // the stages are idle still
@@ -703,8 +704,7 @@ int wm_launch(unipool_ctx* ctx, int phase, const CUtensorMap& tmA, const TokenMa
   constexpr int most = (int)Wm<MODE>::kTable + 4 * kWmMaxExperts + 1024;
   const int smem = (int)Wm<MODE>::kTable + 4 * p.n_experts + 1024;
   UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most));
-  kern<<<ctx->sm_count / 2 * 2, Wm<MODE>::kThreads, smem, s>>>(tmA, tmB, tmC0, tmC1, p);
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(kern, ctx->sm_count / 2 * 2, Wm<MODE>::kThreads, smem, s, tmA, tmB, tmC0, tmC1, p);
   return UNIPOOL_OK;
 }
 

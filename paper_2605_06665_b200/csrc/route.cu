@@ -13,6 +13,7 @@ using RouterTile = SimtTile<32, 4>;
 __global__ void __launch_bounds__(RouterTile::kThreads)
 router_logits_kernel(const float* __restrict__ x, const float* __restrict__ W_r,
                      const float* __restrict__ bias, float* __restrict__ z, int T, int M, int d, bool vec) {
+  grid_wait(x, W_r, bias);
   extern __shared__ float4 smem_raw[];
   RouterTile::Smem& sm = *reinterpret_cast<RouterTile::Smem*>(smem_raw);
   const int m0 = blockIdx.x * 32, n0 = blockIdx.y * kSimtN;
@@ -54,6 +55,7 @@ router_select_kernel(const float* __restrict__ z, int T, int M, int k, float sig
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   for (int i = threadIdx.x; i < M; i += blockDim.x) hist[i] = 0;
   for (int i = lane; i < M; i += 32) wsum[warp * M + i] = 0.f;
+  grid_wait(z);
   __syncthreads();
 
   float* my = sc + warp * M;
@@ -155,6 +157,7 @@ router_select_kernel(const float* __restrict__ z, int T, int M, int k, float sig
 }
 
 __global__ void zero_stats_kernel(int32_t* counts, float* sums, int M) {
+  grid_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < M) { counts[i] = 0; sums[i] = 0.f; }
 }
@@ -164,8 +167,7 @@ int route_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float
                  float* score_sum, float* znorm, float* z_saved, cudaStream_t s) {
   const int d = ctx->cfg.d_model, k = ctx->cfg.top_k;
   if (T == 0) {
-    zero_stats_kernel<<<(M + 127) / 128, 128, 0, s>>>(counts, score_sum, M);
-    UP_LAUNCH_CHECK();
+    UP_KERNEL(zero_stats_kernel, (M + 127) / 128, 128, 0, s, counts, score_sum, M);
     return UNIPOOL_OK;
   }
   if (ctx->cfg.dtype == UNIPOOL_BF16)
@@ -173,9 +175,8 @@ int route_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float
   {
     PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_LOGITS, 1, s);
     UP_CUDA(cudaFuncSetAttribute(router_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RouterTile::Smem)));
-    router_logits_kernel<<<dim3((T + 31) / 32, (M + 63) / 64), RouterTile::kThreads, sizeof(RouterTile::Smem), s>>>(
-        static_cast<const float*>(x), W_r, bias, z_saved, T, M, d, aligned16(x, W_r));
-    UP_LAUNCH_CHECK();
+    UP_KERNEL(router_logits_kernel, dim3((T + 31) / 32, (M + 63) / 64), RouterTile::kThreads, sizeof(RouterTile::Smem), s,
+              static_cast<const float*>(x), W_r, bias, z_saved, T, M, d, aligned16(x, W_r));
   }
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_SELECT, 1, s);
   const int per_block = kRouteWarps * kRouteTokensPerWarp;
@@ -183,10 +184,8 @@ int route_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float
   const size_t smem = (size_t)(2 * kRouteWarps * M) * sizeof(float) + (size_t)M * sizeof(int);
   static_assert((2 * kRouteWarps + 1) * UNIPOOL_MAX_EXPERTS * 4 <= 48 * 1024, "no opt-in to more shared memory");
   auto kern = ctx->cfg.router_mode == UNIPOOL_ROUTER_SOFTMAX ? router_select_kernel<true> : router_select_kernel<false>;
-  kern<<<blocks, kRouteWarps * 32, smem, s>>>(
-      z_saved, T, M, k, sigma * ctx->cfg.c, ctx->cfg.eps, idx, gate, znorm, counts, score_sum,
-      ctx->ws.route_counts, ctx->ws.route_sums, ctx->ws.tickets + 0);
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(kern, blocks, kRouteWarps * 32, smem, s, z_saved, T, M, k, sigma * ctx->cfg.c, ctx->cfg.eps, idx, gate, znorm,
+            counts, score_sum, ctx->ws.route_counts, ctx->ws.route_sums, ctx->ws.tickets + 0);
   return UNIPOOL_OK;
 }
 
@@ -199,6 +198,7 @@ router_dz_kernel(const float* __restrict__ z, const float* __restrict__ znorm,
                  const float* __restrict__ coef, int T, int M, int k, float sigma, float c, float eps,
                  float* __restrict__ dz, float* __restrict__ dsigma, double* __restrict__ acc,
                  uint32_t* __restrict__ ticket) {
+  grid_wait(z, znorm, idx, dgate, coef);
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int t = blockIdx.x * (blockDim.x / 32) + warp;
   float dsig_part = 0.f;
@@ -265,6 +265,7 @@ using RouterDxTile = SimtTile<32, 1>;
 __global__ void __launch_bounds__(RouterDxTile::kThreads)
 router_dx_kernel(const float* __restrict__ dz, const float* __restrict__ W_r, float* __restrict__ dx,
                  int T, int M, int d, bool vec) {
+  grid_wait(dz, W_r);
   __shared__ RouterDxTile::Smem sm;
   const int m0 = blockIdx.x * 32, n0 = blockIdx.y * kSimtN;
   const bool vec_z = (M & 3) == 0;                   // dz is a workspace array of rows of M
@@ -293,6 +294,7 @@ router_dx_kernel(const float* __restrict__ dz, const float* __restrict__ W_r, fl
 __global__ void __launch_bounds__(RouterTile::kThreads)
 router_dw_kernel(const float* __restrict__ dz, const float* __restrict__ x, float* __restrict__ dW_r,
                  int T, int M, int d, int k_len, bool vec) {
+  grid_wait(dz, x);
   extern __shared__ float4 smem_raw[];
   RouterTile::Smem& sm = *reinterpret_cast<RouterTile::Smem*>(smem_raw);
   const int m0 = blockIdx.x * 32, n0 = blockIdx.y * kSimtN;
@@ -335,22 +337,19 @@ int route_bwd_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, f
   {
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_BWD_DZ, 1, s);
   auto kern = ctx->cfg.router_mode == UNIPOOL_ROUTER_SOFTMAX ? router_dz_kernel<true> : router_dz_kernel<false>;
-  kern<<<(T + 7) / 8, 256, 0, s>>>(z_saved, znorm, idx, dgate, coef, T, M, k, sigma, ctx->cfg.c,
-                                   ctx->cfg.eps, dz, dsigma, ctx->ws.dsigma_acc, ctx->ws.tickets + 1);
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(kern, (T + 7) / 8, 256, 0, s, z_saved, znorm, idx, dgate, coef, T, M, k, sigma, ctx->cfg.c,
+            ctx->cfg.eps, dz, dsigma, ctx->ws.dsigma_acc, ctx->ws.tickets + 1);
   }
   {
     PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_BWD_DX, 1, s);
-    router_dx_kernel<<<dim3((T + 31) / 32, d / 64), RouterDxTile::kThreads, 0, s>>>(
-        dz, W_r, static_cast<float*>(dx), T, M, d, aligned16(W_r, dx));
-    UP_LAUNCH_CHECK();
+    UP_KERNEL(router_dx_kernel, dim3((T + 31) / 32, d / 64), RouterDxTile::kThreads, 0, s,
+              dz, W_r, static_cast<float*>(dx), T, M, d, aligned16(W_r, dx));
   }
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_BWD_DW, 1, s);
   const int k_len = 1024;
   UP_CUDA(cudaFuncSetAttribute(router_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RouterTile::Smem)));
-  router_dw_kernel<<<dim3((M + 31) / 32, d / 64, (T + k_len - 1) / k_len), RouterTile::kThreads, sizeof(RouterTile::Smem), s>>>(
-      dz, static_cast<const float*>(x), dW_r, T, M, d, k_len, aligned16(x));
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(router_dw_kernel, dim3((M + 31) / 32, d / 64, (T + k_len - 1) / k_len), RouterTile::kThreads,
+            sizeof(RouterTile::Smem), s, dz, static_cast<const float*>(x), dW_r, T, M, d, k_len, aligned16(x));
   return UNIPOOL_OK;
 }
 

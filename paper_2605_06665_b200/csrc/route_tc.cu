@@ -52,6 +52,7 @@ template <int kSplitVec>
 __global__ void __launch_bounds__(256)
 router_split_kernel(const float* __restrict__ W, int64_t n, int n_layers, __nv_bfloat16* __restrict__ out,
                     int32_t* __restrict__ any) {
+  grid_wait(W);
   for (int64_t l = blockIdx.y; l < n_layers; l += gridDim.y) {
     const float* w_l = W + l * n;
     __nv_bfloat16* o = out + l * 3 * n;
@@ -157,6 +158,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
   const int n_tp = (p.T + 2 * kTile - 1) / (2 * kTile);             // tile pairs
   const bool two_acc = n_cols <= 256;
 
+  grid_wait();
   // Which of the weights' three bf16 terms hold anything (term 0 always counts).  A term's products are added up over all
   // k-blocks before the next term's: the order of the sums is part of the logits' last bits.
   const int any1 = p.split_any[1], any2 = p.split_any[2];
@@ -537,6 +539,7 @@ router_dz16_kernel(const float* __restrict__ z, const float* __restrict__ znorm,
                    const float* __restrict__ dgate, const float* __restrict__ coef, int T, int M, int Mp, int k,
                    float sigma, float c, float eps, __nv_bfloat16* __restrict__ dz16, float* __restrict__ dsigma,
                    double* __restrict__ acc, uint32_t* __restrict__ ticket) {
+  grid_wait(z, znorm, idx, dgate, coef);
   const int gid = blockIdx.x * blockDim.x + threadIdx.x;
   const int sub = gid & 3;
   const bool live = (gid >> 2) < T;
@@ -637,9 +640,7 @@ static int router_split_launch(unipool_ctx* ctx, const float* W_r, int n_layers,
   const bool vec = (reinterpret_cast<uintptr_t>(W_r) & 15) == 0;
   const int64_t blocks = (n + (vec ? 1023 : 255)) / (vec ? 1024 : 256);
   const dim3 grid((unsigned)(blocks < 1184 ? blocks : 1184), (unsigned)(n_layers < 65535 ? n_layers : 65535));
-  if (vec) router_split_kernel<4><<<grid, 256, 0, s>>>(W_r, n, n_layers, out, flags);
-  else router_split_kernel<1><<<grid, 256, 0, s>>>(W_r, n, n_layers, out, flags);
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(vec ? router_split_kernel<4> : router_split_kernel<1>, grid, 256, 0, s, W_r, n, n_layers, out, flags);
   return UNIPOOL_OK;
 }
 
@@ -726,8 +727,7 @@ int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, fl
                      : (softmax ? route_tc_kernel<UNIPOOL_MAX_TOPK, true> : route_tc_kernel<UNIPOOL_MAX_TOPK, false>);
   // (the function's limit, shared by all threads: not lowered to this launch's smem)
   UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-  kern<<<grid, kThreads, smem, s>>>(tmX, tmW1, tmW2, tmZ, p);
-  UP_LAUNCH_CHECK();
+  UP_KERNEL(kern, grid, kThreads, smem, s, tmX, tmW1, tmW2, tmZ, p);
   return UNIPOOL_OK;
 }
 
@@ -747,10 +747,8 @@ int route_bwd_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r
     const bool softmax = ctx->cfg.router_mode == UNIPOOL_ROUTER_SOFTMAX;
     auto kern = k <= 2 ? (softmax ? router_dz16_kernel<true, 2> : router_dz16_kernel<false, 2>)
                        : (softmax ? router_dz16_kernel<true, UNIPOOL_MAX_TOPK> : router_dz16_kernel<false, UNIPOOL_MAX_TOPK>);
-    kern<<<(int)((threads + 255) / 256), 256, 0, s>>>(
-        z_saved, znorm, idx, dgate, coef, T, M, Mp, k, sigma, ctx->cfg.c, ctx->cfg.eps, dz16, dsigma,
-        ctx->ws.dsigma_acc, ctx->ws.tickets + 1);
-    UP_LAUNCH_CHECK();
+    UP_KERNEL(kern, (unsigned)((threads + 255) / 256), 256, 0, s, z_saved, znorm, idx, dgate, coef, T, M, Mp, k, sigma,
+              ctx->cfg.c, ctx->cfg.eps, dz16, dsigma, ctx->ws.dsigma_acc, ctx->ws.tickets + 1);
   }
   return router_bwd_gemms_tc(ctx, dz16, Mp, terms, x, T, M, dx, dW_r, s);
 }
