@@ -230,6 +230,10 @@ struct PoolWgradArgs {
 int route_tc_launch(unipool_ctx*, const void* x, int T, const float* W_r, float sigma, const float* bias,
                     int n_experts, int32_t* idx, float* gate, int32_t* counts, float* score_sum,
                     float* znorm, float* z_saved, cudaStream_t);
+bool route_on_few(const unipool_ctx*, int T, int n_experts);
+int route_few_launch(unipool_ctx*, const void* x, int T, const float* W_r, float sigma, const float* bias,
+                     int n_experts, int32_t* idx, float* gate, int32_t* counts, float* score_sum,
+                     float* znorm, float* z_saved, cudaStream_t);
 int router_prepare_launch(unipool_ctx*, const float* W_r, int n_layers, int n_experts, cudaStream_t);
 int route_bwd_tc_launch(unipool_ctx*, const void* x, int T, const float* W_r, float sigma, int n_experts,
                         const float* znorm, const float* z_saved, const int32_t* idx, const float* dgate,

@@ -1,0 +1,256 @@
+// Router forward for few tokens in bf16 mode: logits on CUDA cores, selection and statistics, one launch.
+//
+// Bound by latency.  On the tensor cores (route_tc.cu) a CTA pair scores 256 tokens whatever their number: 33 tokens
+// are one pair that loads, multiplies and selects one step after the other while 146 SMs idle.  Here a cluster of eight
+// blocks takes kTok tokens.  A block multiplies them, out of shared memory, with an eighth of the experts' weights,
+// read in fp32 as they are: a warp takes four experts and eight tokens, the lanes along the width, and adds up over the
+// lanes by recursive halving.  Every logit is sent to the block of the cluster that owns its token; there a warp selects.
+#include <cooperative_groups.h>
+
+#include <cfloat>
+#include <climits>
+
+#include "common.cuh"
+#include "simt_gemm.cuh"
+
+namespace unipool {
+
+namespace cg = cooperative_groups;
+
+namespace {
+
+constexpr int kFewWarps = 8;
+constexpr int kFewCluster = 8;                 // blocks that share their tokens' experts
+constexpr int kFewExperts = 4, kFewTokens = 8; // experts and tokens a warp multiplies at a time
+constexpr int kFewAhead = 2;                   // 128-wide steps of the weights fetched ahead of their use
+static_assert(kFewExperts * kFewTokens == 32, "a sum per lane");
+
+struct FewParams {
+  const __nv_bfloat16* x; const float* W_r; const float* bias;
+  int T, M, d, k;
+  float sigma_c, eps;
+  int32_t* idx; float* gate; float* znorm; float* z_saved;
+  int32_t* counts_out; float* sum_out;
+  int32_t* acc_counts; long long* acc_sums; uint32_t* ticket;   // as in route_tc.cu: start at zero, left at zero
+  bool vec;                                    // W_r is 16-byte aligned
+};
+
+// Sums v[i] over the lanes; lane l is left with value l in v[0].
+__device__ __forceinline__ void sum_over_lanes(float (&v)[32], int lane) {
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) {
+    const bool upper = (lane & o) != 0;
+#pragma unroll
+    for (int j = 0; j < o; ++j) {
+      const float send = upper ? v[j] : v[j + o], keep = upper ? v[j + o] : v[j];
+      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+}
+
+template <int kTok, bool SOFTMAX>
+__global__ void __cluster_dims__(kFewCluster, 1, 1) __launch_bounds__(kFewWarps * 32, 2)
+route_few_kernel(const FewParams p) {
+  extern __shared__ float4 smem_raw[];
+  constexpr int kOwn = kTok / kFewCluster;                    // tokens that a block selects for
+  const int M = p.M, d = p.d;
+  float* xs = reinterpret_cast<float*>(smem_raw);             // [kTok][d] the cluster's tokens
+  float* zs = xs + kTok * d;                                  // [kOwn][M] logits of the block's own, then scores
+  int* hist = reinterpret_cast<int*>(zs + kOwn * M);          // [M]
+  __shared__ bool last;
+  cg::cluster_group cluster = cg::this_cluster();
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int rank = (int)cluster.block_rank();
+  const int tc0 = (int)(blockIdx.x / kFewCluster) * kTok, t0 = tc0 + rank * kOwn;
+  for (int i = threadIdx.x; i < M; i += blockDim.x) hist[i] = 0;
+  grid_wait();
+  for (int i = 8 * threadIdx.x; i < kTok * d; i += 8 * blockDim.x) {
+    const int t = tc0 + i / d;
+    uint4 w = make_uint4(0, 0, 0, 0);
+    if (t < p.T) w = __ldg(reinterpret_cast<const uint4*>(p.x + (int64_t)t * d + i % d));
+    float4* dst = reinterpret_cast<float4*>(xs + i);
+    dst[0] = make_float4(__uint_as_float(w.x << 16), __uint_as_float(w.x & 0xffff0000u), __uint_as_float(w.y << 16),
+                         __uint_as_float(w.y & 0xffff0000u));
+    dst[1] = make_float4(__uint_as_float(w.z << 16), __uint_as_float(w.z & 0xffff0000u), __uint_as_float(w.w << 16),
+                         __uint_as_float(w.w & 0xffff0000u));
+  }
+  cluster.sync();                                             // the tokens are staged, and all blocks have started
+
+  constexpr int kGroups = kTok / kFewTokens;
+  const int slice = ((M + kFewCluster - 1) / kFewCluster + kFewExperts - 1) / kFewExperts * kFewExperts;
+  const int e_end = min(M, (rank + 1) * slice);
+  for (int item = warp; item < slice / kFewExperts * kGroups; item += kFewWarps) {
+    const int e0 = rank * slice + item / kGroups * kFewExperts, g = item % kGroups;
+    if (e0 >= e_end) continue;
+    float acc[kFewExperts * kFewTokens];
+#pragma unroll
+    for (int i = 0; i < kFewExperts * kFewTokens; ++i) acc[i] = 0.f;
+    const float* w_e[kFewExperts];
+#pragma unroll
+    for (int q = 0; q < kFewExperts; ++q) w_e[q] = p.W_r + (int64_t)min(e0 + q, e_end - 1) * d;
+    float4 next[kFewAhead][kFewExperts];
+    auto load = [&](int c) {
+#pragma unroll
+      for (int a = 0; a < kFewAhead; ++a)
+#pragma unroll
+        for (int q = 0; q < kFewExperts; ++q)
+          next[a][q] = c + 128 * a < d ? ld4(w_e[q] + c + 128 * a, p.vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    load(4 * lane);
+    for (int c0 = 0; c0 < d; c0 += 128 * kFewAhead) {
+      float4 w[kFewAhead][kFewExperts];
+#pragma unroll
+      for (int a = 0; a < kFewAhead; ++a)
+#pragma unroll
+        for (int q = 0; q < kFewExperts; ++q) w[a][q] = next[a][q];
+      load(c0 + 128 * kFewAhead + 4 * lane);
+#pragma unroll
+      for (int a = 0; a < kFewAhead; ++a) {
+        const int c = c0 + 128 * a + 4 * lane;
+        if (c < d) {
+#pragma unroll
+          for (int t = 0; t < kFewTokens; ++t) {
+            const float4 v = *reinterpret_cast<const float4*>(xs + (g * kFewTokens + t) * d + c);
+#pragma unroll
+            for (int q = 0; q < kFewExperts; ++q) {
+              float& s = acc[q * kFewTokens + t];
+              s = fmaf(w[a][q].x, v.x, s);
+              s = fmaf(w[a][q].y, v.y, s);
+              s = fmaf(w[a][q].z, v.z, s);
+              s = fmaf(w[a][q].w, v.w, s);
+            }
+          }
+        }
+      }
+    }
+    sum_over_lanes(acc, lane);                                // lane l holds expert l / 8, token l % 8
+    const int e = e0 + lane / kFewTokens, t = g * kFewTokens + lane % kFewTokens;
+    if (e < e_end) cluster.map_shared_rank(zs, t / kOwn)[t % kOwn * M + e] = acc[0] + (p.bias ? p.bias[e] : 0.f);
+  }
+  cluster.sync();                                             // the logits have arrived
+
+  // a warp per token: norm (softmax: maximum and sum of exponentials), selection, scores
+  if (warp < kOwn && t0 + warp < p.T) {
+    const int t = t0 + warp;
+    float* z = zs + warp * M;
+    float ss = 0.f, mx = -INFINITY;
+    if (SOFTMAX) {
+      for (int i = lane; i < M; i += 32) mx = fmaxf(mx, z[i]);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+    for (int i = lane; i < M; i += 32) {
+      const float v = z[i];
+      p.z_saved[(int64_t)t * M + i] = v;
+      ss = SOFTMAX ? ss + expf(v - mx) : fmaf(v, v, ss);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    const float n = SOFTMAX ? mx + logf(ss) : sqrtf(ss);       // softmax keeps log sum exp(z) here
+    // NormRouter: a zero logit vector scores zero.  Softmax: 1 / sum of exponentials.
+    const float scale = SOFTMAX ? 1.f / ss : (ss > 0.f ? p.sigma_c / (n + p.eps) : 0.f);
+    if (lane == 0) p.znorm[t] = n;
+    // the order of the scores is the order of max(z, 0) (of z for the softmax); equal keys: the lower expert first
+    uint32_t taken = 0;                                        // bit i: expert lane + 32 i
+    for (int j = 0; j < p.k; ++j) {
+      float bv = -INFINITY;
+      int bi = INT_MAX;
+      for (int i = lane, b = 0; i < M; i += 32, ++b) {
+        const float u = SOFTMAX ? z[i] : fmaxf(z[i], 0.f);
+        const float key = u == u ? u : -FLT_MAX;               // NaN logits sort last but stay selectable
+        if (!(taken >> b & 1u) && key > bv) { bv = key; bi = i; }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
+      }
+      if (bi != INT_MAX && bi % 32 == lane) taken |= 1u << (bi / 32);
+      if (lane == 0) {
+        const float g = SOFTMAX ? scale * expf(bv - mx) : scale * bv;
+        p.idx[(int64_t)t * p.k + j] = bi == INT_MAX ? -1 : bi;
+        p.gate[(int64_t)t * p.k + j] = bv == -FLT_MAX ? __int_as_float(0x7fc00000) : g;
+        if (bi != INT_MAX) atomicAdd(&hist[bi], 1);
+      }
+    }
+    for (int i = lane; i < M; i += 32) z[i] = scale * (SOFTMAX ? expf(z[i] - mx) : fmaxf(z[i], 0.f));
+  }
+  __syncthreads();
+  // The block's statistics, as in route_tc.cu: score sums as multiples of 2^-28 in 64-bit integers, so that the totals
+  // do not depend on the order in which the blocks arrive.
+  const int live = min(kOwn, p.T - t0);
+  for (int i = threadIdx.x; i < M; i += blockDim.x) {
+    float sum = 0.f;
+    for (int t = 0; t < live; ++t) sum += zs[t * M + i];
+    if (hist[i] != 0) atomicAdd(&p.acc_counts[i], hist[i]);
+    if (!(fabsf(sum) < 3.0e10f)) atomicOr(p.ticket + 1, 1u);                    // NaN or out of range
+    else if (sum != 0.f)
+      atomicAdd(reinterpret_cast<unsigned long long*>(&p.acc_sums[i]), (unsigned long long)__float2ll_rn(sum * 268435456.f));
+  }
+  __threadfence();
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return;
+  __threadfence();                       // the block that arrives last publishes the totals and clears the accumulators
+  const bool bad = __ldcg(p.ticket + 1) != 0u;
+  for (int i = threadIdx.x; i < M; i += blockDim.x) {
+    p.counts_out[i] = __ldcg(&p.acc_counts[i]);
+    const long long fixed = __ldcg(&p.acc_sums[i]);
+    p.sum_out[i] = bad ? __int_as_float(0x7fc00000) : (float)((double)fixed * (1.0 / 268435456.0));
+    p.acc_counts[i] = 0;
+    p.acc_sums[i] = 0;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) { p.ticket[0] = 0u; p.ticket[1] = 0u; }
+}
+
+constexpr size_t kFewSmemMax = 100 * 1024;     // two blocks to an SM
+
+size_t few_smem(int tok, int M, int d) { return ((size_t)tok * d + tok / kFewCluster * M + M) * sizeof(float); }
+
+template <int kTok>
+int few_launch(const unipool_ctx* ctx, const FewParams& p, cudaStream_t s) {
+  auto kern = ctx->cfg.router_mode == UNIPOOL_ROUTER_SOFTMAX ? route_few_kernel<kTok, true> : route_few_kernel<kTok, false>;
+  UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kFewSmemMax));
+  UP_KERNEL(kern, (p.T + kTok - 1) / kTok * kFewCluster, kFewWarps * 32, few_smem(kTok, p.M, p.d), s, p);
+  return UNIPOOL_OK;
+}
+
+// Tokens to a cluster: the fewest with which all clusters run at a time (an SM takes two blocks, a GPC of 16 to 18 SMs
+// four clusters; 29 of them run beside one another, of 37 some come second), 0 where that needs more than 16.  Cold
+// weights, norm router, us on the tensor cores with bf16 / fp32 weights -> here:
+//   768 x 96     1 .. 33 tokens 16.7 / 24 -> 9.6, 150 16.7 / 24 -> 11.3, 500 16.5 / 24 -> 14.7; 900 (32 to a cluster) 16.6 / 24 -> 19.5
+//   768 x 384    33 tokens - / 42 -> 15, 150 - / 42 -> 17; 900 - / 41 -> 50      1536 x 192   33 - / 38 -> 15, 150 - / 38 -> 17
+//   512 x 64     33 tokens - / 18 -> 8.1, 150 - / 18 -> 8.7                      2048 x 24    33 - / 39 -> 16, 150 - / 39 -> 17
+// and the logits' error against 64 bits is 1.1e-7 instead of 7e-7 / 3.8e-6 (one rounding a product, no truncated sums).
+int few_tokens(const unipool_ctx* ctx, int T, int M) {
+  const int tok = T <= 8 * (ctx->sm_count / 5) ? 8 : T <= 16 * (ctx->sm_count / 5) ? 16 : 0;
+  return few_smem(tok, M, ctx->cfg.d_model) <= kFewSmemMax ? tok : 0;
+}
+
+}  // namespace
+
+bool route_on_few(const unipool_ctx* ctx, int T, int M) { return few_tokens(ctx, T, M) > 0; }
+
+int route_few_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float sigma, const float* bias, int M,
+                     int32_t* idx, float* gate, int32_t* counts, float* score_sum, float* znorm, float* z_saved,
+                     cudaStream_t s) {
+  // what the tensor maps of the other router ask for, whatever the number of tokens
+  UP_REQUIRE(aligned16(x) && ((M & 3) != 0 || aligned16(z_saved)), UNIPOOL_ERR_INVALID_ARG,
+             "tensor base %p is not 16-byte aligned", aligned16(x) ? static_cast<const void*>(z_saved) : x);
+  FewParams p{};
+  p.x = static_cast<const __nv_bfloat16*>(x); p.W_r = W_r; p.bias = bias;
+  p.T = T; p.M = M; p.d = ctx->cfg.d_model; p.k = ctx->cfg.top_k;
+  p.sigma_c = sigma * ctx->cfg.c; p.eps = ctx->cfg.eps;
+  p.idx = idx; p.gate = gate; p.znorm = znorm; p.z_saved = z_saved;
+  p.counts_out = counts; p.sum_out = score_sum;
+  p.acc_counts = ctx->ws.route_counts; p.acc_sums = reinterpret_cast<long long*>(ctx->ws.route_sums);
+  p.ticket = ctx->ws.tickets + 2;
+  p.vec = aligned16(W_r);
+  PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_SELECT, 1, s);
+  return few_tokens(ctx, T, M) == 8 ? few_launch<8>(ctx, p, s) : few_launch<16>(ctx, p, s);
+}
+
+}  // namespace unipool
