@@ -10,8 +10,8 @@ namespace {
 struct RowGemm {
   const float* A; int64_t lda;                      // [rows, K]
   const float* B; int64_t b_expert, ldb;            // expert's weights: along K [N, K], across K [K, N]
-  const int32_t* tile_expert; const int32_t* offsets; const int32_t* rows;   // rows: true group sizes or NULL
-  int expert_base;
+  const int32_t* offsets; const int32_t* rows;      // [n_experts + 1]; [n_experts] true group sizes or NULL
+  int n_experts, expert_base;
   float *C, *C2;
   const float* GU;
   int N, K, f, n_row_tiles;
@@ -24,68 +24,89 @@ enum RowEpilogue {
   kSwigluBwd,  // the tile is dA: dG = dA U silu'(G), dU = dA silu(G) -> C [rows, 2f], G and U from GU
 };
 
-// C = A B_e for every TM-row tile of the permuted row space; the tile's expert selects B.  Tiles at and beyond
-// offsets[n_experts] are skipped (tile_expert < 0); tiles behind a group's last token hold zeros and get zeros.
-template <int TM, int KG, Major BM, RowEpilogue EPI>
-__global__ void __launch_bounds__(SimtTile<TM, KG>::kThreads)
+// The expert and first row of row tile t, and whether it lies behind the group's last token; false: no such tile.  Tiles
+// with tokens are numbered first, so that the blocks that have work, one after the other, fall evenly on the SMs: numbered
+// as they lie in memory, with the tiles of the 128-row padding between them, some SMs had three blocks with work and some
+// none (SMs active for half of the 39 us of dgrad gate/up, 16 experts of 256 x 512, 64 rows each).
+__device__ __forceinline__ bool find_row_tile(const RowGemm& p, int t, int* expert, int* row, bool* empty) {
+  const int lane = threadIdx.x % 32;
+  auto search = [&](bool pads, int base) {            // every warp for itself; returns the tiles counted
+    for (int e0 = 0; e0 < p.n_experts; e0 += 32) {
+      const int e = e0 + lane;
+      int first = 0, n = 0;
+      if (e < p.n_experts) {
+        first = p.offsets[e];
+        const int all = (p.offsets[e + 1] - first) / kSimtM;
+        const int live = p.rows ? min((max(p.rows[e], 0) + kSimtM - 1) / kSimtM, all) : all;
+        n = pads ? all - live : live;
+        if (pads) first += live * kSimtM;
+      }
+      int upto = n;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, upto, o);
+        if (lane >= o) upto += v;
+      }
+      const unsigned hit = __ballot_sync(0xffffffffu, t < base + upto);
+      if (hit != 0) {
+        const int src = __ffs(hit) - 1;
+        *expert = e0 + src;
+        *row = __shfl_sync(0xffffffffu, first + (t - base - (upto - n)) * kSimtM, src);
+        *empty = pads;
+        return -1;
+      }
+      base += __shfl_sync(0xffffffffu, upto, 31);
+    }
+    return base;
+  };
+  const int live = search(false, 0);
+  return live < 0 || search(true, live) < 0;
+}
+
+// C = A B_e for every 32-row tile of the groups; tiles behind a group's last token hold zeros and get zeros.
+template <int KG, Major BM, RowEpilogue EPI>
+__global__ void __launch_bounds__(SimtTile<KG>::kThreads, SimtTile<KG>::kBlocks)
 grouped_rows_gemm_kernel(const RowGemm p) {
-  using T = SimtTile<TM, KG>;
-  constexpr int TN = kSimtN;
+  grid_wait();
+  using T = SimtTile<KG>;
+  constexpr int TN = kSimtN, kHalf = TN / 2;
   extern __shared__ float4 smem_raw[];
   typename T::Smem& sm = *reinterpret_cast<typename T::Smem*>(smem_raw);
-  grid_wait();
-  const int n0 = blockIdx.x * (EPI == kSwiglu ? TN / 2 : TN);
+  const int n0 = blockIdx.x * (EPI == kSwiglu ? kHalf : TN);
   for (int rt = blockIdx.y; rt < p.n_row_tiles; rt += gridDim.y) {
-    const int m0 = rt * TM;
-    const int e = p.tile_expert[m0 / UNIPOOL_ROW_ALIGN];
-    if (e < 0) continue;                            // uniform over the block
-    const bool empty = p.rows != nullptr && m0 - p.offsets[e] >= p.rows[e];
+    int e, m0;
+    bool empty;
+    if (!find_row_tile(p, rt, &e, &m0, &empty)) break;   // uniform over the block
     const float* B = p.B + (int64_t)(p.expert_base + e) * p.b_expert;
-    T t;
-    t.template run<kAlongK, BM>(
-        sm, empty ? 0 : p.K / kSimtKC,
-        [&](int c, int i, int k) { return ld4(p.A + (int64_t)(m0 + i) * p.lda + c * kSimtKC + k, p.vec); },
+    T::template run<kAlongK, BM>(
+        sm, empty ? 0 : p.K / kSimtKC, p.vec, p.vec, p.A, [](int) {},
+        [&](int c, int i, int k) { return p.A + (int64_t)(m0 + i) * p.lda + c * kSimtKC + k; },
         [&](int c, int i, int k) {
-          if (EPI == kSwiglu) i = i < TN / 2 ? n0 + i : p.f + n0 + i - TN / 2;
+          if (EPI == kSwiglu) i = i < kHalf ? n0 + i : p.f + n0 + i - kHalf;
           else i += n0;
           const int kk = c * kSimtKC + k;
-          return ld4(BM == kAlongK ? B + (int64_t)i * p.ldb + kk : B + (int64_t)kk * p.ldb + i, p.vec);
+          return BM == kAlongK ? B + (int64_t)i * p.ldb + kk : B + (int64_t)kk * p.ldb + i;
         });
-    if (threadIdx.x < kSimtGroup) {
+    constexpr int kCols = EPI == kSwiglu ? kHalf : TN;
 #pragma unroll
-      for (int i = 0; i < T::MR; ++i) {
-        const int64_t r = m0 + T::row(i);
-        if constexpr (EPI == kStore) {
-#pragma unroll
-          for (int j = 0; j < T::NR; j += 4)
-            st4(p.C + r * p.N + n0 + T::col(j),
-                make_float4(t.value(i, j), t.value(i, j + 1), t.value(i, j + 2), t.value(i, j + 3)), p.vec);
-        } else if constexpr (EPI == kSwiglu) {
-          float g[4], u[4], a[4];
-#pragma unroll
-          for (int j = 0; j < 4; ++j) { g[j] = t.value(i, j); u[j] = t.value(i, j + 4); a[j] = silu_f(g[j]) * u[j]; }
-          const int n = n0 + T::col(0);
-          st4(p.C + r * 2 * p.f + n, make_float4(g[0], g[1], g[2], g[3]), p.vec);
-          st4(p.C + r * 2 * p.f + p.f + n, make_float4(u[0], u[1], u[2], u[3]), p.vec);
-          st4(p.C2 + r * p.f + n, make_float4(a[0], a[1], a[2], a[3]), p.vec);
-        } else {
-#pragma unroll
-          for (int j = 0; j < T::NR; j += 4) {
-            const int n = n0 + T::col(j);
-            const float4 g4 = ld4(p.GU + r * 2 * p.f + n, p.vec);
-            const float4 u4 = ld4(p.GU + r * 2 * p.f + p.f + n, p.vec);
-            const float g[4] = {g4.x, g4.y, g4.z, g4.w}, u[4] = {u4.x, u4.y, u4.z, u4.w};
-            float dg[4], du[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const float dA = t.value(i, j + q);
-              dg[q] = dA * u[q] * silu_grad_f(g[q]);
-              du[q] = dA * silu_f(g[q]);
-            }
-            st4(p.C + r * 2 * p.f + n, make_float4(dg[0], dg[1], dg[2], dg[3]), p.vec);
-            st4(p.C + r * 2 * p.f + p.f + n, make_float4(du[0], du[1], du[2], du[3]), p.vec);
-          }
-        }
+    for (int u = 0; u < kSimtM * kCols / 4 / T::kThreads; ++u) {
+      const int q = u * T::kThreads + threadIdx.x, i = q / (kCols / 4), j = q % (kCols / 4) * 4, n = n0 + j;
+      const int64_t r = m0 + i;
+      const float4 v = T::value4(sm, i, j);
+      if constexpr (EPI == kStore) {
+        st4(p.C + r * p.N + n, v, p.vec);
+      } else if constexpr (EPI == kSwiglu) {
+        const float4 u = T::value4(sm, i, j + kHalf);
+        st4(p.C + r * 2 * p.f + n, v, p.vec);
+        st4(p.C + r * 2 * p.f + p.f + n, u, p.vec);
+        st4(p.C2 + r * p.f + n, make_float4(silu_f(v.x) * u.x, silu_f(v.y) * u.y, silu_f(v.z) * u.z, silu_f(v.w) * u.w), p.vec);
+      } else {
+        const float4 g = ld4(p.GU + r * 2 * p.f + n, p.vec), u = ld4(p.GU + r * 2 * p.f + p.f + n, p.vec);
+        st4(p.C + r * 2 * p.f + n,
+            make_float4(v.x * u.x * silu_grad_f(g.x), v.y * u.y * silu_grad_f(g.y), v.z * u.z * silu_grad_f(g.z),
+                        v.w * u.w * silu_grad_f(g.w)), p.vec);
+        st4(p.C + r * 2 * p.f + p.f + n,
+            make_float4(v.x * silu_f(g.x), v.y * silu_f(g.y), v.z * silu_f(g.z), v.w * silu_f(g.w)), p.vec);
       }
     }
     if (gridDim.y < p.n_row_tiles) __syncthreads();  // the next tile reuses the buffers
@@ -100,19 +121,24 @@ struct PoolGemm {
   float* dW; int Mdim, Ndim; bool overwrite, vec;
 };
 
-__global__ void __launch_bounds__(SimtTile<64, 2>::kThreads)
+// (us with 1 / 2 / 4 warps to a tile, and with 64 x 64 tiles of four: 16 experts of 256 x 512, 4 layers of 64 rows, dW_down
+// 43/41/38, 45, dW_gu 74/70/71, 71; 30 of 128 x 384, 38 rows 31/23/22, 23 and 41/39/37, 38)
+using WgradTile = SimtTile<2, 2>;
+
+__global__ void __launch_bounds__(WgradTile::kThreads, WgradTile::kBlocks)
 grouped_k_gemm_kernel(const PoolGemm p) {
-  using T = SimtTile<64, 2>;
-  __shared__ typename T::Smem sm;
   grid_wait();
-  const int m0 = blockIdx.x * 64, n0 = blockIdx.y * 64, e = blockIdx.z;
+  using T = WgradTile;
+  extern __shared__ float4 smem_raw[];
+  typename T::Smem& sm = *reinterpret_cast<typename T::Smem*>(smem_raw);
+  const int m0 = blockIdx.x * kSimtM, n0 = blockIdx.y * kSimtN, e = blockIdx.z;
   auto rows_of = [&](int l) {
     const int32_t* off = p.offsets + (int64_t)l * (p.n_experts + 1) + e;
     return p.rows ? min(p.rows[(int64_t)l * p.n_experts + e], off[1] - off[0]) : off[1] - off[0];
   };
   int n_chunks = 0;
   for (int l = 0; l < p.n_layers; ++l) n_chunks += (rows_of(l) + kSimtKC - 1) / kSimtKC;
-  // the chunk being fetched: rows [row0, row0 + left) of its layer are still to come (a group asks for its chunks in order)
+  // the chunk being fetched: rows [row0, row0 + left) of its layer are still to come (a warp asks for its chunks in order)
   int layer = -1, at = -1, left = 0;
   int64_t row0 = 0;
   auto seek = [&](int c) {
@@ -126,65 +152,66 @@ grouped_k_gemm_kernel(const PoolGemm p) {
       }
     }
   };
-  T t;
-  t.template run<kAcrossK, kAcrossK>(
-      sm, n_chunks,
-      [&](int c, int i, int k) {
-        seek(c);
-        return k < left ? ld4(p.P + (row0 + k) * p.ldp + m0 + i, p.vec) : make_float4(0.f, 0.f, 0.f, 0.f);
-      },
-      [&](int c, int i, int k) {
-        return k < left ? ld4(p.Q + (row0 + k) * p.ldq + n0 + i, p.vec) : make_float4(0.f, 0.f, 0.f, 0.f);
-      });
-  if (threadIdx.x >= kSimtGroup) return;
+  T::template run<kAcrossK, kAcrossK>(
+      sm, n_chunks, p.vec, p.vec, p.P, seek,
+      [&](int, int i, int k) { return k < left ? p.P + (row0 + k) * p.ldp + m0 + i : nullptr; },
+      [&](int, int i, int k) { return k < left ? p.Q + (row0 + k) * p.ldq + n0 + i : nullptr; });
   float* out = p.dW + (int64_t)(p.expert_base + e) * p.Mdim * p.Ndim;
-#pragma unroll
-  for (int i = 0; i < T::MR; ++i)
-#pragma unroll
-    for (int j = 0; j < T::NR; j += 4) {
-      float* o = out + (int64_t)(m0 + T::row(i)) * p.Ndim + n0 + T::col(j);
-      float4 v = make_float4(t.value(i, j), t.value(i, j + 1), t.value(i, j + 2), t.value(i, j + 3));
-      if (!p.overwrite) {
-        v = make_float4(v.x + o[0], v.y + o[1], v.z + o[2], v.w + o[3]);
-      }
-      st4(o, v, p.vec);
+  for (int u = 0; u < kSimtM * kSimtN / 4 / T::kThreads; ++u) {
+    const int q = u * T::kThreads + threadIdx.x, i = q / (kSimtN / 4), j = q % (kSimtN / 4) * 4;
+    float* o = out + (int64_t)(m0 + i) * p.Ndim + n0 + j;
+    float4 v = T::value4(sm, i, j);
+    if (!p.overwrite) {
+      const float4 w = p.vec ? *reinterpret_cast<const float4*>(o) : make_float4(o[0], o[1], o[2], o[3]);
+      v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
     }
+    st4(o, v, p.vec);
+  }
 }
 
-template <int TM, int KG, Major BM, RowEpilogue EPI>
+template <int KG, Major BM, RowEpilogue EPI>
 int rows_gemm_as(const unipool_ctx* ctx, RowGemm p, cudaStream_t s) {
-  auto kern = grouped_rows_gemm_kernel<TM, KG, BM, EPI>;
-  constexpr int smem = (int)sizeof(typename SimtTile<TM, KG>::Smem);
-  if (smem > 48 * 1024) UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  p.n_row_tiles = (int)(ctx->row_capacity / TM);
+  auto kern = grouped_rows_gemm_kernel<KG, BM, EPI>;
+  constexpr int smem = (int)sizeof(typename SimtTile<KG>::Smem);
+  UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  p.n_row_tiles = (int)(ctx->row_capacity / kSimtM);
   const int gy = p.n_row_tiles < 8192 ? p.n_row_tiles : 8192;
-  UP_KERNEL(kern, dim3(p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN), gy), (SimtTile<TM, KG>::kThreads), smem, s, p);
+  UP_KERNEL(kern, dim3(p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN), gy), SimtTile<KG>::kThreads, smem, s, p);
   return UNIPOOL_OK;
 }
 
 template <Major BM, RowEpilogue EPI>
 int rows_gemm(unipool_ctx* ctx, RowGemm p, int n_experts, cudaStream_t s) {
   p.vec = aligned16(p.A, p.B, p.C, p.C2, p.GU);    // those that the epilogue has not are NULL
-  // 64 x 64 tiles of a full batch (a group ends on half a tile).  Many: whole tiles, one group of threads on each, two
-  // on a long contraction; fewer: two groups, and half tiles where the weights are read across K; few: half tiles,
-  // two or four groups.  In us, TM = 64 with 1 / 2 / 4 groups, 32 with 1 / 2 / 4 (16 experts of 256 x 512, 64 rows each):
-  // gate/up (384 tiles) 46/41/57, 45/41/44; down (96) 44/29/27, 35/30/27; dgrad down (192) 48/45/63, 39/36/42; dgrad
-  // gate/up (96) 82/48/40, 63/49/44; 24 experts of 384 x 768, 250 rows: 2544 tiles 208/210/345, 252/255/279; 636 tiles
-  // 137/119/167, 156/155/141; 1272 tiles 145/157/303, 153/154/201.
-  const int64_t tiles = ((int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k / 64 + n_experts / 2) *
-                        (p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN));
-  if (tiles >= 600)
-    return p.K >= 768 ? rows_gemm_as<64, 2, BM, EPI>(ctx, p, s) : rows_gemm_as<64, 1, BM, EPI>(ctx, p, s);
-  if (tiles >= 350 && BM == kAlongK) return rows_gemm_as<64, 2, BM, EPI>(ctx, p, s);
-  return p.K >= 512 ? rows_gemm_as<32, 4, BM, EPI>(ctx, p, s) : rows_gemm_as<32, 2, BM, EPI>(ctx, p, s);
+  // Warps to a tile, by the tiles of a full batch (a group ends on half a tile).  us with 1 / 2 / 4 / 8 warps, and with the
+  // 64 x 64 tiles of two warps that were here before:
+  //   16 experts of 256 x 512, 64 rows      gate/up (640 tiles) 39/31/29/38, 35  down (160) 39/23/21/19, 23
+  //                                         dgrad down (320) 44/29/22/25, 32     dgrad gate/up (160) 75/40/36/32, 39
+  //   32 of 256 x 704, 14 rows              (660) 43/41/45/74, 71   (120) 52/30/27/19, 33   (330) 45/38/39/53, 54   (120) 102/54/47/28, 56
+  //   15 of 384 x 512, 91 rows              (800) 56/45/46/53, 56   (300) 40/35/28/28, 31   (400) 52/38/27/32, 41   (300) 76/66/50/48, 53
+  //   24 of 384 x 768, 250 rows             (4776) 219/227/228/276, 207   (1194) 136/120/114/120, 115
+  //                                         (2388) 160/136/127/169, 139   (1194) 280/235/212/223, 216
+  const int64_t rows = (int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k;
+  const int64_t tiles = (rows / kSimtM + n_experts / 2) * (p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN));
+  if (10 * tiles <= 11 * ctx->sm_count && p.K >= (tiles <= ctx->sm_count ? 256 : 512)) return rows_gemm_as<8, BM, EPI>(ctx, p, s);
+  if (BM == kAlongK && tiles >= 1500) return rows_gemm_as<1, BM, EPI>(ctx, p, s);
+  if (tiles >= 600 && (p.K < 256 || (BM == kAlongK && rows < (int64_t)kSimtM * n_experts))) return rows_gemm_as<2, BM, EPI>(ctx, p, s);
+  return rows_gemm_as<4, BM, EPI>(ctx, p, s);
+}
+
+int k_gemm(const PoolGemm& p, cudaStream_t s) {
+  UP_CUDA(cudaFuncSetAttribute(grouped_k_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WgradTile::Smem)));
+  UP_KERNEL(grouped_k_gemm_kernel, dim3(p.Mdim / kSimtM, p.Ndim / kSimtN, p.n_experts), WgradTile::kThreads,
+            sizeof(WgradTile::Smem), s, p);
+  return UNIPOOL_OK;
 }
 
 template <typename Args>
 RowGemm row_gemm(const unipool_ctx* ctx, const Args& a) {
   RowGemm p{};
-  p.tile_expert = a.tile_expert;
   p.offsets = a.offsets;
   p.rows = a.rows;
+  p.n_experts = a.n_experts;
   p.expert_base = a.expert_base;
   p.f = ctx->cfg.d_ff;
   p.b_expert = (int64_t)ctx->cfg.d_model * ctx->cfg.d_ff;
@@ -224,15 +251,15 @@ int pool_wgrad_simt(unipool_ctx* ctx, const PoolWgradArgs& a, cudaStream_t s) {
     p.P = static_cast<const float*>(a.dYp); p.ldp = d;
     p.Q = static_cast<const float*>(a.A); p.ldq = f;
     p.dW = a.dW_down; p.Mdim = d; p.Ndim = f; p.vec = aligned16(p.P, p.Q, p.dW);
-    UP_KERNEL(grouped_k_gemm_kernel, dim3(d / 64, f / 64, a.n_experts), (SimtTile<64, 2>::kThreads), 0, s, p);
+    const int rc = k_gemm(p, s);
+    if (rc != UNIPOOL_OK) return rc;
   }
   if (a.dW_gu == nullptr) return UNIPOOL_OK;
   PhaseTimer pt(ctx, UNIPOOL_PH_WGRAD_GU, 1, s);     // dW_gu[e] [2f, d] (+)= dGU_e^T Xp_e
   p.P = static_cast<const float*>(a.dGU); p.ldp = 2 * f;
   p.Q = static_cast<const float*>(a.Xp); p.ldq = d;
   p.dW = a.dW_gu; p.Mdim = 2 * f; p.Ndim = d; p.vec = aligned16(p.P, p.Q, p.dW);
-  UP_KERNEL(grouped_k_gemm_kernel, dim3(2 * f / 64, d / 64, a.n_experts), (SimtTile<64, 2>::kThreads), 0, s, p);
-  return UNIPOOL_OK;
+  return k_gemm(p, s);
 }
 
 int expert_bwd_simt(unipool_ctx* ctx, const ExpertBwdArgs& a, cudaStream_t s) {

@@ -7,31 +7,23 @@
 namespace unipool {
 
 // ---------------------------------------------------------------- logits  z = x W_r^T (+ bias)
-// Few tiles (one per 32 tokens and 64 experts), so four groups of threads share a tile's contraction.
-using RouterTile = SimtTile<32, 4>;
+// Few tiles (one per 32 tokens and 64 experts), so eight warps share a tile's contraction.
+using RouterTile = SimtTile<8>;
 
-__global__ void __launch_bounds__(RouterTile::kThreads)
+__global__ void __launch_bounds__(RouterTile::kThreads, RouterTile::kBlocks)
 router_logits_kernel(const float* __restrict__ x, const float* __restrict__ W_r,
                      const float* __restrict__ bias, float* __restrict__ z, int T, int M, int d, bool vec) {
   grid_wait(x, W_r, bias);
   extern __shared__ float4 smem_raw[];
   RouterTile::Smem& sm = *reinterpret_cast<RouterTile::Smem*>(smem_raw);
-  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * kSimtN;
-  RouterTile t;
-  t.run<kAlongK, kAlongK>(
-      sm, d / kSimtKC,
-      [&](int c, int i, int k) { return ld4(x + (int64_t)(m0 + i) * d + c * kSimtKC + k, vec, m0 + i < T ? 4 : 0); },
-      [&](int c, int i, int k) { return ld4(W_r + (int64_t)(n0 + i) * d + c * kSimtKC + k, vec, n0 + i < M ? 4 : 0); });
-  if (threadIdx.x >= kSimtGroup) return;
-#pragma unroll
-  for (int i = 0; i < RouterTile::MR; ++i) {
-    const int tok = m0 + t.row(i);
-    if (tok >= T) continue;
-#pragma unroll
-    for (int j = 0; j < RouterTile::NR; ++j) {
-      const int e = n0 + t.col(j);
-      if (e < M) z[(int64_t)tok * M + e] = t.value(i, j) + (bias ? bias[e] : 0.f);
-    }
+  const int m0 = blockIdx.x * kSimtM, n0 = blockIdx.y * kSimtN;
+  RouterTile::run<kAlongK, kAlongK>(
+      sm, d / kSimtKC, vec, vec, x, [](int) {},
+      [&](int c, int i, int k) { return m0 + i < T ? x + (int64_t)(m0 + i) * d + c * kSimtKC + k : nullptr; },
+      [&](int c, int i, int k) { return n0 + i < M ? W_r + (int64_t)(n0 + i) * d + c * kSimtKC + k : nullptr; });
+  for (int q = threadIdx.x; q < kSimtM * kSimtN; q += RouterTile::kThreads) {
+    const int tok = m0 + q / kSimtN, e = n0 + q % kSimtN;
+    if (tok < T && e < M) z[(int64_t)tok * M + e] = RouterTile::value(sm, q / kSimtN, q % kSimtN) + (bias ? bias[e] : 0.f);
   }
 }
 
@@ -261,68 +253,69 @@ router_dz_kernel(const float* __restrict__ z, const float* __restrict__ znorm,
 }
 
 // dx[t,:] += dz[t,:] W_r     (K = M)
-using RouterDxTile = SimtTile<32, 1>;
+using RouterDxTile = SimtTile<4>;
 
-__global__ void __launch_bounds__(RouterDxTile::kThreads)
+__global__ void __launch_bounds__(RouterDxTile::kThreads, RouterDxTile::kBlocks)
 router_dx_kernel(const float* __restrict__ dz, const float* __restrict__ W_r, float* __restrict__ dx,
-                 int T, int M, int d, bool vec) {
+                 int T, int M, int d, bool vec, bool vec_dx) {
   grid_wait(dz, W_r);
-  __shared__ RouterDxTile::Smem sm;
-  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * kSimtN;
-  const bool vec_z = (M & 3) == 0;                   // dz is a workspace array of rows of M
-  RouterDxTile t;
-  t.run<kAlongK, kAcrossK>(
-      sm, (M + kSimtKC - 1) / kSimtKC,
+  extern __shared__ float4 smem_raw[];
+  RouterDxTile::Smem& sm = *reinterpret_cast<RouterDxTile::Smem*>(smem_raw);
+  const int m0 = blockIdx.x * kSimtM, n0 = blockIdx.y * kSimtN;
+  RouterDxTile::run<kAlongK, kAcrossK>(
+      sm, (M + kSimtKC - 1) / kSimtKC, (M & 3) == 0, vec, dz, [](int) {},     // dz is a workspace array of rows of M
       [&](int c, int i, int k) {
         const int kk = c * kSimtKC + k;
-        return ld4(dz + (int64_t)(m0 + i) * M + kk, vec_z, m0 + i < T ? M - kk : 0);
+        return m0 + i < T && kk < M ? dz + (int64_t)(m0 + i) * M + kk : nullptr;
       },
       [&](int c, int i, int k) {
         const int kk = c * kSimtKC + k;
-        return ld4(W_r + (int64_t)kk * d + n0 + i, vec, kk < M ? 4 : 0);
+        return kk < M ? W_r + (int64_t)kk * d + n0 + i : nullptr;
       });
+  constexpr int kMine = kSimtM * kSimtN / 4 / RouterDxTile::kThreads;
+  float4 old[kMine];
 #pragma unroll
-  for (int i = 0; i < RouterDxTile::MR; ++i) {
-    const int tok = m0 + t.row(i);
+  for (int u = 0; u < kMine; ++u) {
+    const int q = u * RouterDxTile::kThreads + threadIdx.x, tok = m0 + q / (kSimtN / 4);
+    const float* o = dx + (int64_t)tok * d + n0 + q % (kSimtN / 4) * 4;
+    if (tok < T) old[u] = vec_dx ? *reinterpret_cast<const float4*>(o) : make_float4(o[0], o[1], o[2], o[3]);
+  }
+#pragma unroll
+  for (int u = 0; u < kMine; ++u) {
+    const int q = u * RouterDxTile::kThreads + threadIdx.x, tok = m0 + q / (kSimtN / 4), j = q % (kSimtN / 4) * 4;
     if (tok >= T) continue;
-#pragma unroll
-    for (int j = 0; j < RouterDxTile::NR; ++j) dx[(int64_t)tok * d + n0 + t.col(j)] += t.value(i, j);
+    const float4 v = RouterDxTile::value4(sm, q / (kSimtN / 4), j);
+    st4(dx + (int64_t)tok * d + n0 + j, make_float4(old[u].x + v.x, old[u].y + v.y, old[u].z + v.z, old[u].w + v.w), vec_dx);
   }
 }
 
 // dW_r[m,:] += sum_t dz[t,m] x[t,:]   (K = T, cut into runs of k_len tokens over blockIdx.z: one run adds in
 // place, several by atomics)
-__global__ void __launch_bounds__(RouterTile::kThreads)
+__global__ void __launch_bounds__(RouterTile::kThreads, RouterTile::kBlocks)
 router_dw_kernel(const float* __restrict__ dz, const float* __restrict__ x, float* __restrict__ dW_r,
                  int T, int M, int d, int k_len, bool vec) {
   grid_wait(dz, x);
   extern __shared__ float4 smem_raw[];
   RouterTile::Smem& sm = *reinterpret_cast<RouterTile::Smem*>(smem_raw);
-  const int m0 = blockIdx.x * 32, n0 = blockIdx.y * kSimtN;
+  const int m0 = blockIdx.x * kSimtM, n0 = blockIdx.y * kSimtN;
   const int k_begin = blockIdx.z * k_len, k_end = min(T, k_begin + k_len);
-  const bool vec_z = (M & 3) == 0;
-  RouterTile t;
-  t.run<kAcrossK, kAcrossK>(
-      sm, (k_end - k_begin + kSimtKC - 1) / kSimtKC,
+  RouterTile::run<kAcrossK, kAcrossK>(
+      sm, (k_end - k_begin + kSimtKC - 1) / kSimtKC, (M & 3) == 0, vec, dz, [](int) {},
       [&](int c, int i, int k) {
         const int tok = k_begin + c * kSimtKC + k;
-        return ld4(dz + (int64_t)tok * M + m0 + i, vec_z, tok < k_end ? M - m0 - i : 0);
+        return tok < k_end && m0 + i < M ? dz + (int64_t)tok * M + m0 + i : nullptr;
       },
       [&](int c, int i, int k) {
         const int tok = k_begin + c * kSimtKC + k;
-        return ld4(x + (int64_t)tok * d + n0 + i, vec, tok < k_end ? 4 : 0);
+        return tok < k_end ? x + (int64_t)tok * d + n0 + i : nullptr;
       });
-  if (threadIdx.x >= kSimtGroup) return;
-#pragma unroll
-  for (int i = 0; i < RouterTile::MR; ++i) {
-    const int m = m0 + t.row(i);
+  for (int q = threadIdx.x; q < kSimtM * kSimtN; q += RouterTile::kThreads) {
+    const int m = m0 + q / kSimtN;
     if (m >= M) continue;
-#pragma unroll
-    for (int j = 0; j < RouterTile::NR; ++j) {
-      float* o = dW_r + (int64_t)m * d + n0 + t.col(j);
-      if (gridDim.z == 1) *o += t.value(i, j);
-      else atomicAdd(o, t.value(i, j));
-    }
+    float* o = dW_r + (int64_t)m * d + n0 + q % kSimtN;
+    const float v = RouterTile::value(sm, q / kSimtN, q % kSimtN);
+    if (gridDim.z == 1) *o += v;
+    else atomicAdd(o, v);
   }
 }
 
@@ -343,8 +336,9 @@ int route_bwd_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, f
   }
   {
     PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_BWD_DX, 1, s);
-    UP_KERNEL(router_dx_kernel, dim3((T + 31) / 32, d / 64), RouterDxTile::kThreads, 0, s,
-              dz, W_r, static_cast<float*>(dx), T, M, d, aligned16(W_r, dx));
+    UP_CUDA(cudaFuncSetAttribute(router_dx_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RouterDxTile::Smem)));
+    UP_KERNEL(router_dx_kernel, dim3((T + 31) / 32, d / 64), RouterDxTile::kThreads, sizeof(RouterDxTile::Smem), s,
+              dz, W_r, static_cast<float*>(dx), T, M, d, aligned16(W_r), aligned16(dx));
   }
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_BWD_DW, 1, s);
   const int k_len = 1024;

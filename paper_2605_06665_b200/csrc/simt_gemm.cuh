@@ -1,24 +1,24 @@
 // CUDA-core tiled GEMM building block with fp32 accumulation, for the fp32 mode of the library (its 1e-5
 // parity bound rules out TF32).
 //
-// Bound by the FMA pipe (72 TFLOP/s at 1.9 GHz) and the register side of shared memory where there are many tiles
-// (40 TFLOP/s in the weight gradient of 24 experts of 384 x 768), by latency and synchronisation below that.  A group
-// of 64 threads owns a TM x 64 tile, TM / 8 x 8 results per thread, multiplied with packed fma.rn.f32x2 (each half an
-// IEEE fp32 fma: half the instructions for the same sums); chunks of 16 of the contraction go through
-// double-buffered shared memory, fetched into registers one chunk ahead with 16-byte loads, and the operands of
-// step k + 1 are read while step k is multiplied.  KG such groups in a block share a tile by taking every KG-th
-// chunk and add up at the end: a long contraction over few tiles then still fills the chip.  (Both operands along K
-// in shared memory, pairs along K, saves the duplication of a: no faster, and slower by a third where a weight is
-// read across K.)
+// A warp owns a 32 x 64 tile, 8 x 8 results per lane, and works on its own: its chunks of 16 positions of the contraction
+// come by cp.async into shared memory of its own, so that nothing in the loop waits for another warp.  An operand lies
+// there as in memory, so that all copies and loads are 16 bytes wide.  KG warps share a tile by taking every KG-th
+// chunk; their sums meet in shared memory, and all of them write.
+// Bound by the FMA pipe and, as high, the register side of shared memory (8 x 8 results: 64 bytes a lane for 64 products,
+// 128 bytes a clock), in fact by how few warps a launch of the fp32 sizes gives a scheduler: one alone issues in 57 % of
+// its clocks, three in 72 %, three quarters of it FMAs.  Four positions unrolled twice: all sixteen miss the instruction
+// cache, and their loads, moved up, take 255 registers.  Plain FMAs: packed ones (fma.rn.f32x2) take two issue slots, and
+// about one register move each.  32 x 128 tiles load less per product, and were no faster for their fewer warps.
 #pragma once
 
 #include "common.cuh"
 
 namespace unipool {
 
-constexpr int kSimtKC = 16;        // k-chunk staged in shared memory
-constexpr int kSimtGroup = 64;     // threads of a k-group: 8 x 8
-constexpr int kSimtN = 64;         // columns of a tile
+constexpr int kSimtKC = 16;                   // positions of a chunk
+constexpr int kSimtM = 32, kSimtN = 64;       // rows and columns of a tile
+constexpr int kSimtLd = kSimtN + 8;           // row stride of the sums in shared memory
 
 // How an operand lies in memory: kAlongK element (i, k) = p[i * ld + k], kAcrossK element (i, k) = p[k * ld + i].
 enum Major { kAlongK, kAcrossK };
@@ -31,136 +31,155 @@ __device__ __forceinline__ void st4(float* p, float4 v, bool vec) {
   if (vec) { *reinterpret_cast<float4*>(p) = v; return; }
   p[0] = v.x; p[1] = v.y; p[2] = v.z; p[3] = v.w;
 }
-// The first n (<= 4, may be negative) floats at p, zeros for the rest.
-__device__ __forceinline__ float4 ld4(const float* p, bool vec, int n) {
-  if (n >= 4) return ld4(p, vec);
-  return make_float4(n > 0 ? __ldg(p) : 0.f, n > 1 ? __ldg(p + 1) : 0.f, n > 2 ? __ldg(p + 2) : 0.f, 0.f);
-}
 template <typename... P> inline bool aligned16(P... p) { return ((... | reinterpret_cast<uintptr_t>(p)) & 15) == 0; }
 
-template <int TM, int KG>
+// kBytes at `src` into shared memory, zeros where src is NULL (`any`: some readable address).
+template <int kBytes>
+__device__ __forceinline__ void copy_async(uint32_t dst, const float* src, const float* any) {
+  const float* from = src ? src : any;
+  const int n = src ? kBytes : 0;
+  if constexpr (kBytes == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" : : "r"(dst), "l"(from), "r"(n) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" : : "r"(dst), "l"(from), "r"(n) : "memory");
+}
+
+// kStages: chunks in shared memory.  Three cover long contractions over L2 better, two leave room for sixteen warps on an SM.
+template <int KG, int kStages = 3>
 struct SimtTile {
-  static constexpr int TN = kSimtN, MR = TM / 8, NR = 8, kThreads = KG * kSimtGroup;
-  static constexpr int kA4 = TM * kSimtKC / 4 / kSimtGroup, kB4 = TN * kSimtKC / 4 / kSimtGroup;   // float4 per thread
-  static_assert(MR == 8 || MR == 4, "result tile of a thread");
-  struct Smem {
-    float a[KG][2][kSimtKC][TM + 4];
-    float b[KG][2][kSimtKC][TN + 4];
-  };
-  unsigned long long acc[MR][NR / 2];
+  static constexpr int kThreads = KG * 32, kBlocks = (kStages == 3 ? 12 : 16) / KG;   // blocks of an SM
+  struct Stage { float a[kSimtM * kSimtKC], b[kSimtN * kSimtKC]; };
+  union Warp { Stage stage[kStages]; float sums[kSimtM * kSimtLd]; };
+  struct Smem { Warp w[KG]; };
 
-  // results of this thread: row(i), column(j) inside the tile
-  __device__ static int ty() { return (threadIdx.x % kSimtGroup) / 8; }
-  __device__ static int tx() { return threadIdx.x % 8; }
-  __device__ static int row(int i) { return i < 4 ? ty() * 4 + i : TM / 2 + ty() * 4 + i - 4; }
-  __device__ static int col(int j) { return j < 4 ? tx() * 4 + j : TN / 2 + tx() * 4 + j - 4; }
-  __device__ float value(int i, int j) const {
-    const unsigned long long v = acc[i][j / 2];
-    return __uint_as_float(j & 1 ? (uint32_t)(v >> 32) : (uint32_t)v);
+  // Byte offset of element (i, k) of an operand of T rows.  Along K: rows of 64 bytes, their 16-byte pieces exchanged so
+  // that eight rows' pieces of one k lie in different banks.
+  template <Major MJ, int T> __device__ static uint32_t at(int i, int k) {
+    return MJ == kAlongK ? (uint32_t)(i * 64 + (((k >> 2) ^ (i >> 1)) & 3) * 16 + (k & 3) * 4) : (uint32_t)(k * T + i) * 4;
+  }
+  // Row (column) j of a lane's eight; u: ty (tx), of kLanes.
+  template <Major MJ, int kLanes> __device__ static int own(int u, int j) {
+    return MJ == kAlongK ? u + kLanes * j : u * 4 + (j & 3) + (j >> 2) * 4 * kLanes;
   }
 
-  // One operand's chunk: registers <- memory (fetch: float4 at (i, k) for this thread's pieces) and shared
-  // memory <- registers.
-  template <Major MJ, int T, int N4, typename F>
-  __device__ static void fetch(float4 (&r)[N4], F at) {
+  // A chunk of one operand of T rows.  src(i, k): the address of its element, NULL outside; with `vec` that of four, along
+  // K or along the rows as memory has them.
+  template <Major MJ, int T, typename F>
+  __device__ static void fetch(uint32_t dst, bool vec, const float* any, F src) {
+    const int lane = threadIdx.x % 32;
+    if (vec) {
 #pragma unroll
-    for (int q = 0; q < N4; ++q) {
-      const int p = threadIdx.x % kSimtGroup + q * kSimtGroup;
-      r[q] = MJ == kAlongK ? at(p / (kSimtKC / 4), p % (kSimtKC / 4) * 4) : at(p % (T / 4) * 4, p / (T / 4));
-    }
-  }
-  template <Major MJ, int T, int N4>
-  __device__ static void stash(float (*s)[T + 4], const float4 (&r)[N4]) {
-#pragma unroll
-    for (int q = 0; q < N4; ++q) {
-      const int p = threadIdx.x % kSimtGroup + q * kSimtGroup;
-      if (MJ == kAlongK) {
-        const int i = p / (kSimtKC / 4), k = p % (kSimtKC / 4) * 4;
-        s[k][i] = r[q].x; s[k + 1][i] = r[q].y; s[k + 2][i] = r[q].z; s[k + 3][i] = r[q].w;
-      } else {
-        *reinterpret_cast<float4*>(&s[p / (T / 4)][p % (T / 4) * 4]) = r[q];
+      for (int q = 0; q < T / 8; ++q) {
+        const int v = q * 32 + lane, i = MJ == kAlongK ? v / 4 : v % (T / 4) * 4, k = MJ == kAlongK ? v % 4 * 4 : v / (T / 4);
+        copy_async<16>(dst + at<MJ, T>(i, k), src(i, k), any);
+      }
+    } else {
+      for (int q = 0; q < T / 2; ++q) {
+        const int v = q * 32 + lane, i = MJ == kAlongK ? v / kSimtKC : v % T, k = MJ == kAlongK ? v % kSimtKC : v / T;
+        copy_async<4>(dst + at<MJ, T>(i, k), src(i, k), any);
       }
     }
   }
-  struct Frag { float a[MR]; unsigned long long b[NR / 2]; };
-  __device__ static void read(Frag& f, const float (*sa)[TM + 4], const float (*sb)[TN + 4], int k) {
-#pragma unroll
-    for (int h = 0; h < MR / 4; ++h) {
-      const float4 v = *reinterpret_cast<const float4*>(&sa[k][h * (TM / 2) + ty() * 4]);
-      f.a[4 * h] = v.x; f.a[4 * h + 1] = v.y; f.a[4 * h + 2] = v.z; f.a[4 * h + 3] = v.w;
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const ulonglong2 v = *reinterpret_cast<const ulonglong2*>(&sb[k][h * (TN / 2) + tx() * 4]);
-      f.b[2 * h] = v.x; f.b[2 * h + 1] = v.y;
-    }
-  }
 
-  // The tile's sums over n_chunks chunks.  a_at / b_at(chunk, i, k): the float4 of the operand that starts at tile
-  // row (column) i and position k of the chunk, zeros outside - four along K or four along i by its Major.
-  // On return group 0 holds the sums of all groups (the others may leave).
-  template <Major AM, Major BM, typename FA, typename FB>
-  __device__ void run(Smem& s, int n_chunks, FA a_at, FB b_at) {
-    const int g = threadIdx.x / kSimtGroup;
+  // The tile's sums over n_chunks chunks.  begin(chunk) is called in front of a chunk's a_at / b_at(chunk, i, k), the
+  // addresses of element i of the tile's rows (columns), position k of the chunk; NULL: zero.
+  // On return (of all threads) value4 gives the sums.
+  template <Major AM, Major BM, typename FB0, typename FA, typename FB>
+  __device__ static void run(Smem& s, int n_chunks, bool vec_a, bool vec_b, const float* any, FB0 begin, FA a_at, FB b_at) {
+    static_assert(AM == kAlongK || BM == kAcrossK, "not used");
+    const int g = threadIdx.x / 32, lane = threadIdx.x % 32, ty = lane / 8, tx = lane % 8;
+    Warp& w = s.w[g];
+    float acc[8][8];
 #pragma unroll
-    for (int i = 0; i < MR; ++i)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-      for (int j = 0; j < NR / 2; ++j) acc[i][j] = 0ull;
-    const int n_it = (n_chunks + KG - 1) / KG;
-    float4 ra[kA4], rb[kB4];
-    auto load = [&](int it) {
-      const int c = it * KG + g;
-      if (c < n_chunks) {
-        fetch<AM, TM>(ra, [&](int i, int k) { return a_at(c, i, k); });
-        fetch<BM, TN>(rb, [&](int i, int k) { return b_at(c, i, k); });
-      } else {
-#pragma unroll
-        for (int q = 0; q < kA4; ++q) ra[q] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int q = 0; q < kB4; ++q) rb[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int j = 0; j < 8; ++j) acc[i][j] = 0.f;
+    const int n = (n_chunks - g + KG - 1) / KG;
+    const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(&w));
+    auto load = [&](int it, int stage) {
+      if (it < n) {
+        const int c = it * KG + g;
+        begin(c);
+        const uint32_t dst = base + (uint32_t)(stage * sizeof(Stage));
+        fetch<AM, kSimtM>(dst, vec_a, any, [&](int i, int k) { return a_at(c, i, k); });
+        fetch<BM, kSimtN>(dst + (uint32_t)sizeof(float) * kSimtM * kSimtKC, vec_b, any, [&](int i, int k) { return b_at(c, i, k); });
       }
+      asm volatile("cp.async.commit_group;" : : : "memory");
     };
-    if (n_it > 0) load(0);
-    for (int it = 0; it < n_it; ++it) {
-      float (*sa)[TM + 4] = s.a[g][it & 1];
-      float (*sb)[TN + 4] = s.b[g][it & 1];
-      stash<AM, TM>(sa, ra);
-      stash<BM, TN>(sb, rb);
-      __syncthreads();                             // also: everyone is done with the buffer the next chunk goes to
-      if (it + 1 < n_it) load(it + 1);
-      Frag f[2];
-      read(f[0], sa, sb, 0);
 #pragma unroll
-      for (int k = 0; k < kSimtKC; ++k) {
-        if (k + 1 < kSimtKC) read(f[(k + 1) & 1], sa, sb, k + 1);
-        const Frag& c = f[k & 1];
+    for (int it = 0; it < kStages - 1; ++it) load(it, it);
+    int stage = 0;
+    for (int it = 0; it < n; ++it) {
+      asm volatile("cp.async.wait_group %0;" : : "n"(kStages - 2) : "memory");
+      __syncwarp();                                // the chunk is there, and all lanes are done with the one before it
+      load(it + kStages - 1, stage == 0 ? kStages - 1 : stage - 1);
+      const char* sa = reinterpret_cast<const char*>(w.stage[stage].a);
+      const char* sb = reinterpret_cast<const char*>(w.stage[stage].b);
+      if (++stage == kStages) stage = 0;
+      auto four = [](const char* p, float (&v)[4]) {
+        const float4 f = *reinterpret_cast<const float4*>(p);
+        v[0] = f.x; v[1] = f.y; v[2] = f.z; v[3] = f.w;
+      };
+#pragma unroll 2
+      for (int k = 0; k < kSimtKC; k += 4) {
+        float a[8][4];                             // along K: [row][position], across K: [2 position + half][row]
+        if (AM == kAlongK) {
 #pragma unroll
-        for (int i = 0; i < MR; ++i) {
-          unsigned long long aa;
-          asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(c.a[i]));
+          for (int i = 0; i < 8; ++i) four(sa + at<AM, kSimtM>(own<AM, 4>(ty, i), k), a[i]);
+        } else {
 #pragma unroll
-          for (int j = 0; j < NR / 2; ++j) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(aa), "l"(c.b[j]));
+          for (int i = 0; i < 8; ++i) four(sa + at<AM, kSimtM>(own<AM, 4>(ty, i % 2 * 4), k + i / 2), a[i]);
+        }
+        if (BM == kAlongK) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            float b[4];
+            four(sb + at<BM, kSimtN>(own<BM, 8>(tx, j), k), b);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+              for (int i = 0; i < 8; ++i) acc[i][j] = fmaf(a[i][q], b[q], acc[i][j]);
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              float b[4];
+              four(sb + at<BM, kSimtN>(own<BM, 8>(tx, 4 * h), k + q), b);
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                  const float av = AM == kAlongK ? a[i][q] : a[2 * q + i / 4][i % 4];
+                  acc[i][4 * h + j] = fmaf(av, b[j], acc[i][4 * h + j]);
+                }
+            }
         }
       }
     }
-    if constexpr (KG > 1) {                        // groups 1 .. KG-1 hand their sums over through shared memory
-      __syncthreads();
-      constexpr int kSums = MR * NR / 2;
-      unsigned long long* x = reinterpret_cast<unsigned long long*>(&s);
-      static_assert(sizeof(Smem) >= (KG - 1) * kSums * kSimtGroup * 8, "room for the groups' sums");
-      const int t = threadIdx.x % kSimtGroup;
-      if (g > 0) {
+    asm volatile("cp.async.wait_group 0;" : : : "memory");
+    __syncwarp();                                  // the stages are free
 #pragma unroll
-        for (int q = 0; q < kSums; ++q) x[((g - 1) * kSums + q) * kSimtGroup + t] = acc[q / (NR / 2)][q % (NR / 2)];
-      }
-      __syncthreads();
-      if (g == 0) {
-        for (int o = 0; o < KG - 1; ++o)
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-          for (int q = 0; q < kSums; ++q)
-            asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[q / (NR / 2)][q % (NR / 2)]) : "l"(x[(o * kSums + q) * kSimtGroup + t]));
-      }
+      for (int j = 0; j < 8; ++j) w.sums[own<AM, 4>(ty, i) * kSimtLd + own<BM, 8>(tx, j)] = acc[i][j];
+    __syncthreads();
+  }
+
+  // Row r, columns c .. c + 3 of the tile (c a multiple of 4): the warps' sums added up, in their order.
+  __device__ static float4 value4(const Smem& s, int r, int c) {
+    float4 v = *reinterpret_cast<const float4*>(&s.w[0].sums[r * kSimtLd + c]);
+#pragma unroll
+    for (int g = 1; g < KG; ++g) {
+      const float4 o = *reinterpret_cast<const float4*>(&s.w[g].sums[r * kSimtLd + c]);
+      v.x += o.x; v.y += o.y; v.z += o.z; v.w += o.w;
     }
+    return v;
+  }
+  __device__ static float value(const Smem& s, int r, int c) {
+    float v = s.w[0].sums[r * kSimtLd + c];
+#pragma unroll
+    for (int g = 1; g < KG; ++g) v += s.w[g].sums[r * kSimtLd + c];
+    return v;
   }
 };
 
