@@ -304,12 +304,15 @@ template <> struct Vec16<__nv_bfloat16> {
 // y[t] = (residual[t]) + sum_j gate[t,j] * Yp[row_of[t,j]]   (gate == NULL: unit weights)
 // KT = compile-time bound of k (registers for the rows in flight).
 template <typename T, int KT>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, KT <= 4 ? 1 : sizeof(T) == 2 ? 4 : 3)
 combine_kernel(const uint4* __restrict__ Yp, const int32_t* __restrict__ row_of,
                const float* __restrict__ gate, const uint4* __restrict__ residual,
                uint4* __restrict__ y, int n_tokens, int k, int row_vecs) {
   grid_wait(Yp, row_of, gate, residual);
   constexpr int N = Vec16<T>::N;
+  // vectors per lane and pass: one where a token has up to eight rows in flight, for four blocks on an SM instead of one
+  // (16384 tokens of 768, top-8: 55 -> 45 us, 251 MB)
+  constexpr int V = KT > 4 ? 1 : kVpl;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   for (int t = blockIdx.x * 8 + warp; t < n_tokens; t += gridDim.x * 8) {
     int rows[KT];
@@ -319,10 +322,10 @@ combine_kernel(const uint4* __restrict__ Yp, const int32_t* __restrict__ row_of,
       rows[j] = j < k ? row_of[(int64_t)t * k + j] : -1;
       g[j] = (j < k && gate) ? gate[(int64_t)t * k + j] : 1.f;
     }
-    for (int v0 = lane; v0 < row_vecs; v0 += 32 * kVpl) {
-      uint4 rv[kVpl], yv[KT][kVpl];
+    for (int v0 = lane; v0 < row_vecs; v0 += 32 * V) {
+      uint4 rv[V], yv[KT][V];
 #pragma unroll
-      for (int i = 0; i < kVpl; ++i) {
+      for (int i = 0; i < V; ++i) {
         const int v = v0 + 32 * i;
         rv[i] = (residual && v < row_vecs) ? __ldg(residual + (int64_t)t * row_vecs + v) : make_uint4(0, 0, 0, 0);
 #pragma unroll
@@ -331,7 +334,7 @@ combine_kernel(const uint4* __restrict__ Yp, const int32_t* __restrict__ row_of,
                                                     : make_uint4(0, 0, 0, 0);
       }
 #pragma unroll
-      for (int i = 0; i < kVpl; ++i) {
+      for (int i = 0; i < V; ++i) {
         const int v = v0 + 32 * i;
         if (v >= row_vecs) continue;
         float acc[N];
