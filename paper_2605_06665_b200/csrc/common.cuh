@@ -75,7 +75,10 @@ inline cudaError_t launch_kernel(void (*kern)(P...), dim3 grid, dim3 block, size
 // before they touch global memory.  The pointers that it is given come out of it, so that no load through them (a
 // read-only one has no order of its own) can be moved in front of it.
 template <typename P>
-__device__ __forceinline__ void after_asm(P& p) { asm volatile("" : "+l"(p)); }
+__device__ __forceinline__ void after_asm(P& p) {
+  asm volatile("" : "+l"(p));
+  __builtin_assume(__isGlobal(p));             // what the compiler knew of a kernel's argument
+}
 template <typename... P>
 __device__ __forceinline__ void grid_wait(P&... p) {
   asm volatile("griddepcontrol.wait;" : : : "memory");
