@@ -146,7 +146,7 @@ dispatch_place_kernel(const int32_t* __restrict__ idx, int T, int k, int M, int 
     for (int i = threadIdx.x; i < 2 * M; i += blockDim.x) total[i] = 0;       // total and before
     __syncthreads();
     for (int64_t a = threadIdx.x; a < n_assign; a += blockDim.x) {
-      const int e = idx[a];
+      const int e = __ldg(idx + a);
       if (!routed(e, M, me == 0 ? status : nullptr)) continue;
       atomicAdd(&total[e], 1);
       if (a < chunk_a0) atomicAdd(&before[e], 1);
@@ -182,7 +182,7 @@ dispatch_place_kernel(const int32_t* __restrict__ idx, int T, int k, int M, int 
   // (c) this chunk's per-warp histograms -> first row of every warp per expert
   if (n_tok > 0) {
     for (int64_t a = a_begin + lane; a < a_end; a += 32) {
-      const int e = idx[a];
+      const int e = __ldg(idx + a);
       if (e >= 0 && e < M) atomicAdd(&hist[warp * M + e], 1);
     }
     __syncthreads();
@@ -201,7 +201,7 @@ dispatch_place_kernel(const int32_t* __restrict__ idx, int T, int k, int M, int 
     for (int64_t a0 = a_begin; a0 < a_end; a0 += 32) {
       const int64_t a = a0 + lane;
       const bool live = a < a_end;
-      int e = live ? idx[a] : -1;
+      int e = live ? __ldg(idx + a) : -1;
       const bool ok = live && e >= 0 && e < M;
       if (!ok) e = -1 - lane;                                  // unique key: matches nobody
       const unsigned peers = __match_any_sync(0xffffffffu, e);
@@ -319,8 +319,8 @@ combine_kernel(const uint4* __restrict__ Yp, const int32_t* __restrict__ row_of,
     float g[KT];
 #pragma unroll
     for (int j = 0; j < KT; ++j) {
-      rows[j] = j < k ? row_of[(int64_t)t * k + j] : -1;
-      g[j] = (j < k && gate) ? gate[(int64_t)t * k + j] : 1.f;
+      rows[j] = j < k ? __ldg(row_of + (int64_t)t * k + j) : -1;
+      g[j] = (j < k && gate) ? __ldg(gate + (int64_t)t * k + j) : 1.f;
     }
     for (int v0 = lane; v0 < row_vecs; v0 += 32 * V) {
       uint4 rv[V], yv[KT][V];
@@ -380,13 +380,13 @@ combine_bwd_kernel(const uint4* __restrict__ dy, const uint4* __restrict__ Yp,
   const int n_pads = group_rows != nullptr ? M * pad_step : 0;
   for (int item = blockIdx.x * 8 + warp; item < n_items + n_pads; item += gridDim.x * 8) {
     if (item >= n_items) {
-      const int p = item - n_items, e = p / pad_step, i = p % pad_step, end = offsets[e + 1];
-      int n = end - offsets[e];                          // the padding lies in the group's last 128 rows
+      const int p = item - n_items, e = p / pad_step, i = p % pad_step, end = __ldg(offsets + e + 1);
+      int n = end - __ldg(offsets + e);                          // the padding lies in the group's last 128 rows
       if (n > 0) {
         const int32_t* tail = token_of + end - UNIPOOL_ROW_ALIGN;
         n -= UNIPOOL_ROW_ALIGN;
 #pragma unroll
-        for (int q = 0; q < UNIPOOL_ROW_ALIGN / 32; ++q) n += __popc(__ballot_sync(0xffffffffu, tail[32 * q + lane] >= 0));
+        for (int q = 0; q < UNIPOOL_ROW_ALIGN / 32; ++q) n += __popc(__ballot_sync(0xffffffffu, __ldg(tail + 32 * q + lane) >= 0));
       }
       if (i == 0 && lane == 0) group_rows[e] = n;
       if (i >= (-n & (pad_step - 1))) continue;
@@ -399,8 +399,8 @@ combine_bwd_kernel(const uint4* __restrict__ dy, const uint4* __restrict__ Yp,
     float g[KT], dot[KT];
 #pragma unroll
     for (int j = 0; j < KT; ++j) {
-      rows[j] = j0 + j < k ? row_of[(int64_t)t * k + j0 + j] : -1;
-      g[j] = j0 + j < k ? gate[(int64_t)t * k + j0 + j] : 0.f;
+      rows[j] = j0 + j < k ? __ldg(row_of + (int64_t)t * k + j0 + j) : -1;
+      g[j] = j0 + j < k ? __ldg(gate + (int64_t)t * k + j0 + j) : 0.f;
       dot[j] = 0.f;
     }
     for (int v0 = lane; v0 < row_vecs; v0 += 32 * kVpl) {

@@ -59,7 +59,7 @@ router_select_kernel(const float* __restrict__ z, int T, int M, int k, int per_w
       // s = exp(z - max) / sum exp(z - max); the log-sum-exp goes where the NormRouter keeps ||z||
       float mx = -INFINITY;
       for (int i = lane; i < M; i += 32) {
-        float v = zr[i];
+        float v = __ldg(zr + i);
         my[i] = v;
         mx = fmaxf(mx, v);
       }
@@ -82,7 +82,7 @@ router_select_kernel(const float* __restrict__ z, int T, int M, int k, int per_w
     } else {
       float ss = 0.f;
       for (int i = lane; i < M; i += 32) {
-        float v = zr[i];
+        float v = __ldg(zr + i);
         my[i] = v;
         ss = fmaf(v, v, ss);
       }
@@ -199,20 +199,20 @@ router_dz_kernel(const float* __restrict__ z, const float* __restrict__ znorm,
     const float* zr = z + (int64_t)t * M;
     int my_idx = -1;
     float my_dg = 0.f;
-    if (lane < k) { my_idx = idx[(int64_t)t * k + lane]; my_dg = dgate[(int64_t)t * k + lane]; }
-    const float n = znorm[t];
+    if (lane < k) { my_idx = __ldg(idx + (int64_t)t * k + lane); my_dg = __ldg(dgate + (int64_t)t * k + lane); }
+    const float n = __ldg(znorm + t);
     const float ne = n + eps;
     float q = 0.f;
     // pass 1: q = sum_i ds_i * max(z_i, 0)
     for (int i0 = 0; i0 < M; i0 += 32) {
       int i = i0 + lane;
-      float ds = (i < M && coef) ? coef[i] : 0.f;
+      float ds = (i < M && coef) ? __ldg(coef + i) : 0.f;
       for (int j = 0; j < k; ++j) {
         int ej = __shfl_sync(0xffffffffu, my_idx, j);
         float dj = __shfl_sync(0xffffffffu, my_dg, j);
         if (ej == i) ds += dj;
       }
-      if (i < M) q = fmaf(ds, SOFTMAX ? expf(zr[i] - n) : fmaxf(zr[i], 0.f), q);
+      if (i < M) q = fmaf(ds, SOFTMAX ? expf(__ldg(zr + i) - n) : fmaxf(__ldg(zr + i), 0.f), q);
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
@@ -220,14 +220,14 @@ router_dz_kernel(const float* __restrict__ z, const float* __restrict__ znorm,
     const float qn = n > 0.f ? q / (n * ne * ne) : 0.f;
     for (int i0 = 0; i0 < M; i0 += 32) {
       int i = i0 + lane;
-      float ds = (i < M && coef) ? coef[i] : 0.f;
+      float ds = (i < M && coef) ? __ldg(coef + i) : 0.f;
       for (int j = 0; j < k; ++j) {
         int ej = __shfl_sync(0xffffffffu, my_idx, j);
         float dj = __shfl_sync(0xffffffffu, my_dg, j);
         if (ej == i) ds += dj;
       }
       if (i < M) {
-        float zi = zr[i];
+        float zi = __ldg(zr + i);
         float v = n > 0.f ? scale * ((zi > 0.f ? ds / ne : 0.f) - zi * qn) : 0.f;
         if (SOFTMAX) v = expf(zi - n) * (ds - q);          // n holds log sum exp(z)
         dz[(int64_t)t * M + i] = v;

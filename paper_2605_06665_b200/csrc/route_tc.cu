@@ -549,8 +549,8 @@ router_dz16_kernel(const float* __restrict__ z, const float* __restrict__ znorm,
   float dg_sel[KT];
 #pragma unroll
   for (int j = 0; j < KT; ++j) {
-    e_sel[j] = j < k ? idx[(int64_t)t * k + j] : -1;
-    dg_sel[j] = j < k ? dgate[(int64_t)t * k + j] : 0.f;
+    e_sel[j] = j < k ? __ldg(idx + (int64_t)t * k + j) : -1;
+    dg_sel[j] = j < k ? __ldg(dgate + (int64_t)t * k + j) : 0.f;
   }
   auto ds_of = [&](int i) {
     float ds = coef ? __ldg(coef + i) : 0.f;
@@ -559,12 +559,12 @@ router_dz16_kernel(const float* __restrict__ z, const float* __restrict__ znorm,
       if (e_sel[j] == i) ds += dg_sel[j];
     return ds;
   };
-  const float n = znorm[t];                       // ||z||; softmax: log sum exp(z)
+  const float n = __ldg(znorm + t);                       // ||z||; softmax: log sum exp(z)
   const bool vec = (M & 3) == 0;
   float q = 0.f;
   if (vec) {
     for (int i = 4 * sub; i < M; i += 16) {
-      const float4 zv = *reinterpret_cast<const float4*>(zr + i);
+      const float4 zv = __ldg(reinterpret_cast<const float4*>(zr + i));
       const float zz[4] = {zv.x, zv.y, zv.z, zv.w};
 #pragma unroll
       for (int u = 0; u < 4; ++u) q = fmaf(ds_of(i + u), SOFTMAX ? expf(zz[u] - n) : fmaxf(zz[u], 0.f), q);
@@ -587,7 +587,7 @@ router_dz16_kernel(const float* __restrict__ z, const float* __restrict__ znorm,
       for (int i = 4 * sub; i < Mp; i += 16) {
         float v[4] = {0.f, 0.f, 0.f, 0.f};
         if (i < M) {
-          const float4 zv = *reinterpret_cast<const float4*>(zr + i);
+          const float4 zv = __ldg(reinterpret_cast<const float4*>(zr + i));
           v[0] = dz_of(i, zv.x); v[1] = dz_of(i + 1, zv.y); v[2] = dz_of(i + 2, zv.z); v[3] = dz_of(i + 3, zv.w);
         }
         const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
