@@ -22,10 +22,12 @@ void set_error(const char* fmt, ...);
     }                                    \
   } while (0)
 
+// (The runtime keeps an error for cudaGetLastError too: taken there, or whoever asks next takes it for its own.)
 #define UP_CUDA(call)                                                                  \
   do {                                                                                 \
     cudaError_t e__ = (call);                                                          \
     if (e__ != cudaSuccess) {                                                          \
+      cudaGetLastError();                                                              \
       unipool::set_error("%s failed: %s (%s:%d)", #call, cudaGetErrorString(e__), __FILE__, \
                          __LINE__);                                                    \
       return UNIPOOL_ERR_CUDA;                                                         \
