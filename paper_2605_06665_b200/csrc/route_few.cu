@@ -11,6 +11,7 @@
 #include <climits>
 
 #include "common.cuh"
+#include "route_stats.cuh"
 #include "simt_gemm.cuh"
 
 namespace unipool {
@@ -30,23 +31,9 @@ struct FewParams {
   int T, M, d, k;
   float sigma_c, eps;
   int32_t* idx; float* gate; float* znorm; float* z_saved;
-  int32_t* counts_out; float* sum_out;
-  int32_t* acc_counts; long long* acc_sums; uint32_t* ticket;   // as in route_tc.cu: start at zero, left at zero
+  RouteTotals totals;
   bool vec;                                    // W_r is 16-byte aligned
 };
-
-// Sums v[i] over the lanes; lane l is left with value l in v[0].
-__device__ __forceinline__ void sum_over_lanes(float (&v)[32], int lane) {
-#pragma unroll
-  for (int o = 16; o >= 1; o >>= 1) {
-    const bool upper = (lane & o) != 0;
-#pragma unroll
-    for (int j = 0; j < o; ++j) {
-      const float send = upper ? v[j] : v[j + o], keep = upper ? v[j + o] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-    }
-  }
-}
 
 template <int kTok, bool SOFTMAX>
 __global__ void __cluster_dims__(kFewCluster, 1, 1) __launch_bounds__(kFewWarps * 32, 2)
@@ -177,33 +164,23 @@ route_few_kernel(const FewParams p) {
     for (int i = lane; i < M; i += 32) z[i] = scale * (SOFTMAX ? expf(z[i] - mx) : fmaxf(z[i], 0.f));
   }
   __syncthreads();
-  // The block's statistics, as in route_tc.cu: score sums as multiples of 2^-28 in 64-bit integers, so that the totals
-  // do not depend on the order in which the blocks arrive.
   const int live = min(kOwn, p.T - t0);
   for (int i = threadIdx.x; i < M; i += blockDim.x) {
     float sum = 0.f;
     for (int t = 0; t < live; ++t) sum += zs[t * M + i];
-    if (hist[i] != 0) atomicAdd(&p.acc_counts[i], hist[i]);
-    if (!(fabsf(sum) < 3.0e10f)) atomicOr(p.ticket + 1, 1u);                    // NaN or out of range
-    else if (sum != 0.f)
-      atomicAdd(reinterpret_cast<unsigned long long*>(&p.acc_sums[i]), (unsigned long long)__float2ll_rn(sum * 268435456.f));
+    add_route_total(p.totals, i, hist[i], sum);
   }
   __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(p.ticket, 1u) == gridDim.x - 1;
+  uint32_t* ticket = p.totals.ticket;
+  if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   __syncthreads();
   if (!last) return;
   __threadfence();                       // the block that arrives last publishes the totals and clears the accumulators
-  const bool bad = __ldcg(p.ticket + 1) != 0u;
-  for (int i = threadIdx.x; i < M; i += blockDim.x) {
-    p.counts_out[i] = __ldcg(&p.acc_counts[i]);
-    const long long fixed = __ldcg(&p.acc_sums[i]);
-    p.sum_out[i] = bad ? __int_as_float(0x7fc00000) : (float)((double)fixed * (1.0 / 268435456.0));
-    p.acc_counts[i] = 0;
-    p.acc_sums[i] = 0;
-  }
+  const bool bad = __ldcg(ticket + 1) != 0u;
+  for (int i = threadIdx.x; i < M; i += blockDim.x) publish_route_total(p.totals, i, bad);
   __syncthreads();
-  if (threadIdx.x == 0) { p.ticket[0] = 0u; p.ticket[1] = 0u; }
+  if (threadIdx.x == 0) { ticket[0] = 0u; ticket[1] = 0u; }
 }
 
 constexpr size_t kFewSmemMax = 100 * 1024;     // two blocks to an SM
@@ -245,9 +222,7 @@ int route_few_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, f
   p.T = T; p.M = M; p.d = ctx->cfg.d_model; p.k = ctx->cfg.top_k;
   p.sigma_c = sigma * ctx->cfg.c; p.eps = ctx->cfg.eps;
   p.idx = idx; p.gate = gate; p.znorm = znorm; p.z_saved = z_saved;
-  p.counts_out = counts; p.sum_out = score_sum;
-  p.acc_counts = ctx->ws.route_counts; p.acc_sums = reinterpret_cast<long long*>(ctx->ws.route_sums);
-  p.ticket = ctx->ws.tickets + 2;
+  p.totals = {counts, score_sum, ctx->ws.route_counts, reinterpret_cast<long long*>(ctx->ws.route_sums), ctx->ws.tickets + 2};
   p.vec = aligned16(W_r);
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_SELECT, 1, s);
   return few_tokens(ctx, T, M) == 8 ? few_launch<8>(ctx, p, s) : few_launch<16>(ctx, p, s);

@@ -11,6 +11,7 @@
 #include <cuda.h>
 
 #include "common.cuh"
+#include "route_stats.cuh"
 #include "tc_ptx.cuh"
 
 namespace unipool {
@@ -32,9 +33,7 @@ struct RouteParams {
   int T, M, d, k;
   float sigma_c, eps;
   int32_t* idx; float* gate; float* znorm; float* z_saved;
-  int32_t* counts_out; float* sum_out;
-  int32_t* acc_counts; long long* acc_sums; uint32_t* ticket;   // [M] accumulators of all CTAs (start at zero,
-                                                                // left at zero), [0] CTAs done, [1] non-finite sum
+  RouteTotals totals;
   const int32_t* split_any;            // [3] does split s hold a non-zero anywhere
   int stages;                          // operand stages that fit into shared memory
   uint32_t stage_bytes;
@@ -430,17 +429,7 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
           const float s = e < M ? scale * (SOFTMAX ? expf(z - mx) : fmaxf(z, 0.f)) : 0.f;
           sv[i] = live ? s : 0.f;
         }
-        // column sums over the warp's 32 tokens: recursive halving, lane l ends with column c0 + l
-#pragma unroll
-        for (int o = 16; o >= 1; o >>= 1) {
-          const bool upper = (lane & o) != 0;
-#pragma unroll
-          for (int j = 0; j < o; ++j) {
-            const float send = upper ? sv[j] : sv[j + o];
-            const float keep = upper ? sv[j + o] : sv[j];
-            sv[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-          }
-        }
+        sum_over_lanes(sv, lane);                         // over the warp's 32 tokens: lane l ends with column c0 + l
         if (c0 + lane < M) my_wsum[c0 + lane] += sv[0];
       }
       // the accumulator has been read twice by this warp: the next tile may overwrite it
@@ -490,35 +479,24 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
     tc::tc_fence_before_sync();
     // the eight epilogue warps publish the CTA's statistics (named barrier 1: 256 threads)
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    // Counts are integers; a CTA's score sums are rounded to multiples of 2^-28 and added as 64-bit
-    // integers too, so the totals do not depend on the order in which the CTAs arrive (|sum| < 2^35).
     const int et = threadIdx.x - 64;
-    constexpr float kFix = 268435456.f;                   // 2^28
+    uint32_t* ticket = p.totals.ticket;
     for (int i = et; i < M; i += 32 * kEpiWarps) {
       float sum = 0.f;
 #pragma unroll
       for (int w = 0; w < kEpiWarps; ++w) sum += wsum[w * M + i];
-      if (hist[i] != 0) atomicAdd(&p.acc_counts[i], hist[i]);
-      if (!(fabsf(sum) < 3.0e10f)) atomicOr(p.ticket + 1, 1u);          // NaN or out of range
-      else if (sum != 0.f)
-        atomicAdd(reinterpret_cast<unsigned long long*>(&p.acc_sums[i]), (unsigned long long)__float2ll_rn(sum * kFix));
+      add_route_total(p.totals, i, hist[i], sum);
     }
     __threadfence();
     asm volatile("bar.sync 1, 256;" ::: "memory");
-    if (et == 0) *last_flag = atomicAdd(p.ticket, 1u) == gridDim.x - 1 ? 1 : 0;
+    if (et == 0) *last_flag = atomicAdd(ticket, 1u) == gridDim.x - 1 ? 1 : 0;
     asm volatile("bar.sync 1, 256;" ::: "memory");
     if (*last_flag) {                     // the CTA that arrives last publishes the totals and clears the accumulators
       __threadfence();
-      const bool bad = __ldcg(p.ticket + 1) != 0u;
-      for (int i = et; i < M; i += 32 * kEpiWarps) {
-        p.counts_out[i] = __ldcg(&p.acc_counts[i]);
-        const long long fixed = __ldcg(&p.acc_sums[i]);
-        p.sum_out[i] = bad ? __int_as_float(0x7fc00000) : (float)((double)fixed * (1.0 / 268435456.0));
-        p.acc_counts[i] = 0;
-        p.acc_sums[i] = 0;
-      }
+      const bool bad = __ldcg(ticket + 1) != 0u;
+      for (int i = et; i < M; i += 32 * kEpiWarps) publish_route_total(p.totals, i, bad);
       asm volatile("bar.sync 1, 256;" ::: "memory");
-      if (et == 0) { p.ticket[0] = 0u; p.ticket[1] = 0u; }
+      if (et == 0) { ticket[0] = 0u; ticket[1] = 0u; }
     }
   }
 
@@ -688,9 +666,7 @@ int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, fl
   p.bias = bias; p.T = T; p.M = M; p.d = d; p.k = k;
   p.sigma_c = sigma * ctx->cfg.c; p.eps = ctx->cfg.eps;
   p.idx = idx; p.gate = gate; p.znorm = znorm; p.z_saved = z_saved;
-  p.counts_out = counts; p.sum_out = score_sum;
-  p.acc_counts = ctx->ws.route_counts; p.acc_sums = reinterpret_cast<long long*>(ctx->ws.route_sums);
-  p.ticket = ctx->ws.tickets + 2;                        // [2] CTAs done, [3] a non-finite score sum was seen
+  p.totals = {counts, score_sum, ctx->ws.route_counts, reinterpret_cast<long long*>(ctx->ws.route_sums), ctx->ws.tickets + 2};
   p.split_any = flags;
   p.status = ctx->ws.status;
   const int n_cols = (M + 15) / 16 * 16;
