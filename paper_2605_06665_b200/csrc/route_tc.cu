@@ -310,10 +310,11 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
 #pragma unroll
           for (int i = 1; i < 32; ++i) cm = fmaxf(cm, z[i]);
           cm = fmaxf(cm, mx);
+          const float ref = cm == -INFINITY ? 0.f : cm;   // experts masked so far: an empty sum (NaN logits: NaN)
           float part = 0.f;
 #pragma unroll
-          for (int i = 0; i < 32; ++i) part += expf(z[i] - cm);
-          ss = ss * expf(mx - cm) + part;                 // the first chunk rescales an empty sum
+          for (int i = 0; i < 32; ++i) part += expf(z[i] - ref);
+          ss = ss * expf(mx - ref) + part;                // the first chunk rescales an empty sum
           mx = cm;
         }
         auto key_of = [&](float zv, int e) {
@@ -402,9 +403,8 @@ route_tc_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant__
         const float oss = xnorm[((half ^ 1) * kTile + tok_in_tile) * 2];
         const float omx = xnorm[((half ^ 1) * kTile + tok_in_tile) * 2 + 1];
         if (SOFTMAX) {
-          const float cm = fmaxf(mx, omx);
-          // a warp without chunks contributes an empty sum at -inf
-          ss = (mx == -INFINITY ? 0.f : ss * expf(mx - cm)) + (omx == -INFINITY ? 0.f : oss * expf(omx - cm));
+          const float cm = fmaxf(mx, omx), ref = cm == -INFINITY ? 0.f : cm;
+          ss = ss * expf(mx - ref) + oss * expf(omx - ref);   // a warp without chunks has an empty sum at -inf
           mx = cm;
         } else {
           ss = half == 0 ? ss + oss : oss + ss;           // the same order in both warps

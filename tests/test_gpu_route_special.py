@@ -1,9 +1,11 @@
-"""Both routers of the bf16 mode on values out of the ordinary: score sums beyond what their accumulators hold."""
+"""Both routers of the bf16 mode on values out of the ordinary: score sums beyond what their accumulators hold, infinite and NaN
+logits, masked experts, ties."""
 import numpy as np
 import pytest
 import torch
 
-from parity_utils import to_np
+from oracle import unipool_oracle as O
+from parity_utils import f64, to_np
 from paper_2605_06665_b200 import binding as B
 
 pytestmark = pytest.mark.gpu
@@ -35,4 +37,50 @@ def test_score_sums_at_the_range_of_their_accumulators(T, sigma, fits):
     assert np.isnan(out["S"]).all() if not fits else abs(out["S"][3] / (T * sigma) - 1) < 1e-5 and out["S"][[0, 7]].tolist() == [0, 0]
     out = route(ctx, x, W, None, 1)
     assert abs(out["S"][3] / T - 1) < 1e-5 and out["counts"].tolist() == [0, 0, 0, T, 0, 0, 0, 0]
+    ctx.close()
+
+
+def special_bias(kind, M):
+    b = np.zeros(M, np.float32)
+    if kind == "negative": b[np.arange(M) != M // 2] = -600.0       # one logit above zero at most
+    if kind == "infinite": b[3], b[M - 2], b[M // 2] = np.inf, -np.inf, -np.inf
+    if kind == "nan": b[5] = np.nan
+    if kind == "masked": b[:M - 9] = -np.inf                          # all experts of the first chunks of 32
+    return b
+
+
+@pytest.mark.parametrize("kind", ["ties", "negative", "infinite", "nan", "masked"])
+@pytest.mark.parametrize("M,k", [(75, 2), (75, 8), (384, 2), (384, 8), (10, 2)])
+@pytest.mark.parametrize("mode", ["norm", "softmax"])
+def test_both_routers_agree_on_special_logits(mode, M, k, kind):
+    """Logits that are whole numbers, the same in both kernels to the bit: selection is equal, everything else up to the rounding of
+    sums (fp32, M terms of one sign: M / 2 ulp at most; score sums to multiples of 2^-28 in each of some 500 blocks).  Some tokens hold a NaN, an infinity, or nothing but zeros."""
+    rng = np.random.default_rng(M + k)
+    T, d = 500, 64
+    ctx = B.Context(B.make_config(d, 64, M, k, 1, T, B.BF16, 1e-6, 1.0, B.ROUTER_SOFTMAX if mode == "softmax" else B.ROUTER_NORM))
+    x = torch.from_numpy(rng.integers(0, 2, (T, d)).astype(np.float32)).cuda().bfloat16()
+    W = torch.from_numpy(rng.integers(-1, 2, (M, d)).astype(np.float32)).cuda()
+    x[7] = 0.0
+    if kind != "masked":
+        x[11, 2] = float("nan")
+        x[13, 1] = float("inf")
+    b = special_bias(kind, M)
+    bias = torch.from_numpy(b).cuda()
+    whole = route(ctx, x, W, bias, k, few=False)
+    parts = [route(ctx, x[:40].contiguous(), W, bias, k, few=True), route(ctx, x[40:].contiguous(), W, bias, k, few=True)]
+    few = {n: sum(p[n] for p in parts) if n in ("counts", "S") else np.concatenate([p[n] for p in parts]) for n in whole}
+    tol = M * 2.0 ** -24 + 1e-6
+    for n in whole:
+        if n in ("idx", "counts", "z"):
+            np.testing.assert_array_equal(few[n], whole[n], err_msg=n)
+        else:
+            np.testing.assert_allclose(few[n], whole[n], rtol=tol, atol=2e-6, err_msg=n)
+    # tokens whose logits are numbers, against the oracle (the first experts of equal score are taken)
+    with np.errstate(all="ignore"):
+        ref = O.route(f64(to_np(x.float())), f64(to_np(W)), 1.0, 1.0, 1e-6, k, f64(b), mode=mode)
+    ok = np.isfinite(ref["z"]).all(1) if kind != "masked" or mode == "norm" else np.ones(T, bool)
+    assert ok.sum() == (0 if kind in ("infinite", "nan") or (kind, mode) == ("masked", "norm") else T - 2 * (kind != "masked"))
+    np.testing.assert_array_equal(whole["idx"][ok], ref["idx"][ok])
+    np.testing.assert_allclose(whole["gate"][ok], ref["g"][ok], rtol=1e-5, atol=1e-6)
+    ctx.check_status()
     ctx.close()
