@@ -66,8 +66,8 @@ __device__ __forceinline__ bool find_row_tile(const RowGemm& p, int t, int* expe
 // C = A B_e for every 32-row tile of the groups; tiles behind a group's last token hold zeros and get zeros.
 template <int KG, Major BM, RowEpilogue EPI>
 __global__ void __launch_bounds__(SimtTile<KG>::kThreads, SimtTile<KG>::kBlocks)
-grouped_rows_gemm_kernel(const RowGemm p) {
-  grid_wait();
+grouped_rows_gemm_kernel(RowGemm p) {
+  grid_wait(p.A, p.B, p.GU);
   using T = SimtTile<KG>;
   constexpr int TN = kSimtN, kHalf = TN / 2;
   extern __shared__ float4 smem_raw[];
@@ -126,8 +126,8 @@ struct PoolGemm {
 using WgradTile = SimtTile<2, 2>;
 
 __global__ void __launch_bounds__(WgradTile::kThreads, WgradTile::kBlocks)
-grouped_k_gemm_kernel(const PoolGemm p) {
-  grid_wait();
+grouped_k_gemm_kernel(PoolGemm p) {
+  grid_wait(p.P, p.Q);
   using T = WgradTile;
   extern __shared__ float4 smem_raw[];
   typename T::Smem& sm = *reinterpret_cast<typename T::Smem*>(smem_raw);

@@ -37,7 +37,7 @@ struct FewParams {
 
 template <int kTok, bool SOFTMAX>
 __global__ void __cluster_dims__(kFewCluster, 1, 1) __launch_bounds__(kFewWarps * 32, 2)
-route_few_kernel(const FewParams p) {
+route_few_kernel(FewParams p) {
   extern __shared__ float4 smem_raw[];
   constexpr int kOwn = kTok / kFewCluster;                    // tokens that a block selects for
   const int M = p.M, d = p.d;
@@ -50,7 +50,7 @@ route_few_kernel(const FewParams p) {
   const int rank = (int)cluster.block_rank();
   const int tc0 = (int)(blockIdx.x / kFewCluster) * kTok, t0 = tc0 + rank * kOwn;
   for (int i = threadIdx.x; i < M; i += blockDim.x) hist[i] = 0;
-  grid_wait();
+  grid_wait(p.x, p.W_r, p.bias);
   for (int i = 8 * threadIdx.x; i < kTok * d; i += 8 * blockDim.x) {
     const int t = tc0 + i / d;
     uint4 w = make_uint4(0, 0, 0, 0);
