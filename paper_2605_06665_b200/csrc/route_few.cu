@@ -196,15 +196,29 @@ int few_launch(const unipool_ctx* ctx, const FewParams& p, cudaStream_t s) {
 }
 
 // Tokens to a cluster: the fewest with which all clusters run at a time (an SM takes two blocks, a GPC of 16 to 18 SMs
-// four clusters; 29 of them run beside one another, of 37 some come second), 0 where that needs more than 16.  Cold
-// weights, norm router, us on the tensor cores with bf16 / fp32 weights -> here:
-//   768 x 96     1 .. 33 tokens 16.7 / 24 -> 9.6, 150 16.7 / 24 -> 11.3, 500 16.5 / 24 -> 14.7; 900 (32 to a cluster) 16.6 / 24 -> 19.5
-//   768 x 384    33 tokens - / 42 -> 15, 150 - / 42 -> 17; 900 - / 41 -> 50      1536 x 192   33 - / 38 -> 15, 150 - / 38 -> 17
-//   512 x 64     33 tokens - / 18 -> 8.1, 150 - / 18 -> 8.7                      2048 x 24    33 - / 39 -> 16, 150 - / 39 -> 17
-// and the logits' error against 64 bits is 1.1e-7 instead of 7e-7 / 3.8e-6 (one rounding a product, no truncated sums).
+// four clusters; 29 of them run beside one another, of 37 some come second), 0 where that needs more than 16, and where 16
+// of them do not pay: their products grow with M d, the other router's chain with d / 64, and with bf16 weights (one term;
+// three otherwise) that is soon the shorter one.  Norm router, weights read from HBM, us, tensor cores with bf16 weights ->
+// here (tensor cores with fp32 weights):
+//   tokens         33                   150              232 / 240       464
+//   64 x 512       12.0 -> 7.7 (17)     12.1 -> 8.2      12.1 -> 8.8     12.1 -> 9.9
+//   96 x 768       15.6 -> 9.5 (23)     15.7 -> 10.9     15.4 -> 12.3    15.4 -> 14.2
+//   384 x 768      30 -> 14.8 (41)      30 -> 16.4       30 -> 21.7      30 -> 25.7
+//   192 x 1536     22.8 -> 14.5 (37)    22.7 -> 16.6     22.7 -> 18.0    22.8 [27.2 with 16 tokens to a cluster]
+//   24 x 2048      18.3 -> 14.3 (38)    18.3 -> 14.7
+// and at 464 tokens, 16 to a cluster, as shares of the other router's time with bf16 weights (with fp32 weights 0.5 .. 0.75):
+//   width       64 experts   96     128    160    192    256    384    512
+//   768         0.90         0.92   0.90   0.97   0.95   0.89   0.87   0.81
+//   896         0.95         0.95   0.93   1.03   1.02   0.94   0.95   0.91
+//   1024        0.95         0.96   0.95   1.05   1.05   0.98   0.98   0.96
+//   1152        1.00         0.99   0.98   1.13   1.12   1.04   1.05   1.02
+//   1472        1.02         1.04   1.05   1.23   1.22   1.18   1.17   1.16
+// (0.02 to 0.03 less since the kernel's pointers come out of its wait; at the line, 128 x 1408 and 160, 192 x 960 measure 1.00.)
+// The logits' error against 64 bits is 1.1e-7 instead of 7e-7 / 3.8e-6 (one rounding a product, no truncated sums).
 int few_tokens(const unipool_ctx* ctx, int T, int M) {
-  const int tok = T <= 8 * (ctx->sm_count / 5) ? 8 : T <= 16 * (ctx->sm_count / 5) ? 16 : 0;
-  return few_smem(tok, M, ctx->cfg.d_model) <= kFewSmemMax ? tok : 0;
+  const int d = ctx->cfg.d_model, clusters = ctx->sm_count / 5;
+  const int tok = T <= 8 * clusters ? 8 : T <= 16 * clusters && d <= (M <= 128 ? 1408 : 960) ? 16 : 0;
+  return few_smem(tok, M, d) <= kFewSmemMax ? tok : 0;
 }
 
 }  // namespace
