@@ -302,17 +302,14 @@ template <> struct Vec16<__nv_bfloat16> {
 };
 
 // y[t] = (residual[t]) + sum_j gate[t,j] * Yp[row_of[t,j]]   (gate == NULL: unit weights)
-// KT = compile-time bound of k (registers for the rows in flight).
-template <typename T, int KT>
-__global__ void __launch_bounds__(256, KT <= 4 ? 1 : sizeof(T) == 2 ? 4 : 3)
+// KT = compile-time bound of k (registers for the rows in flight), V = 16-byte vectors of a row per lane and pass.
+template <typename T, int KT, int V>
+__global__ void __launch_bounds__(256, V > 1 ? 1 : sizeof(T) == 2 ? 4 : 3)
 combine_kernel(const uint4* __restrict__ Yp, const int32_t* __restrict__ row_of,
                const float* __restrict__ gate, const uint4* __restrict__ residual,
                uint4* __restrict__ y, int n_tokens, int k, int row_vecs) {
   grid_wait(Yp, row_of, gate, residual);
   constexpr int N = Vec16<T>::N;
-  // vectors per lane and pass: one where a token has up to eight rows in flight, for four blocks on an SM instead of one
-  // (16384 tokens of 768, top-8: 55 -> 45 us, 251 MB)
-  constexpr int V = KT > 4 ? 1 : kVpl;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   for (int t = blockIdx.x * 8 + warp; t < n_tokens; t += gridDim.x * 8) {
     int rows[KT];
@@ -518,13 +515,26 @@ int dispatch_launch(unipool_ctx* ctx, const void* x, int T, const int32_t* idx, 
                         tile_expert, rows, Xp, s);
 }
 
+// With up to eight rows in flight three vectors a pass leave an SM one block (176 registers), one vector four (in 64
+// registers, 48 bytes of the bf16 form spilled; three in fp32).  A token's passes follow one another, so few tokens want
+// few passes; as soon as a second round of one-block SMs is needed, more blocks are worth more.  us, three vectors / one:
+//   bf16, top-8   200 tokens of 768 3.6 / 5.3, 1184 5.3 / 6.6, 1185 6.9 / 6.5, 1500 8.0 / 6.9, 4096 15.9 / 12.3, 16384 51 / 44
+//                 1184 of 2944 13.8 / 18.4, 1500 22.0 / 21.8, 2000 24.9 / 24.5, 2400 33.9 / 29.1; 2000 of 384 6.5 / 5.7
+//   fp32, top-8   1184 of 256 4.0 / 5.0, 1500 5.7 / 5.2; 1184 of 768 7.4 / 10.9, 1500 10.3 / 11.6, 2000 11.9 / 13.0, 2600 15.8 / 15.3
+// (One vector at k = 3, 4, where three leave two blocks: top-4, 2000 tokens of 2944 11.3 -> 14.3, 16384 of 768 27.1 -> 26.8.)
+static bool combine_in_few_passes(const unipool_ctx* ctx, int n_tokens, int row_vecs) {
+  const int rounds = ctx->cfg.dtype == UNIPOOL_FP32 && row_vecs > 32 * kVpl ? 2 : 1;
+  return n_tokens <= 8 * rounds * ctx->sm_count;
+}
+
 template <typename T>
-static int combine_dispatch_k(int grid, cudaStream_t s, int k, const void* Yp, const int32_t* row_of,
+static int combine_dispatch_k(const unipool_ctx* ctx, int grid, cudaStream_t s, int k, const void* Yp, const int32_t* row_of,
                               const float* gate, const void* residual, void* y, int n_tokens, int row_vecs) {
   auto Y = static_cast<const uint4*>(Yp);
   auto R = static_cast<const uint4*>(residual);
   auto O = static_cast<uint4*>(y);
-  auto kern = k <= 1 ? combine_kernel<T, 1> : k <= 2 ? combine_kernel<T, 2> : k <= 4 ? combine_kernel<T, 4> : combine_kernel<T, 8>;
+  auto kern = k <= 1 ? combine_kernel<T, 1, kVpl> : k <= 2 ? combine_kernel<T, 2, kVpl> : k <= 4 ? combine_kernel<T, 4, kVpl>
+              : combine_in_few_passes(ctx, n_tokens, row_vecs) ? combine_kernel<T, 8, kVpl> : combine_kernel<T, 8, 1>;
   UP_KERNEL(kern, grid, 256, 0, s, Y, row_of, gate, R, O, n_tokens, k, row_vecs);
   return UNIPOOL_OK;
 }
@@ -537,8 +547,8 @@ static int combine_phase(unipool_ctx* ctx, int phase, const void* Yp, const int3
   const int row_vecs = (int)((size_t)ctx->cfg.d_model * ctx->elem_bytes / 16);
   const int grid = row_mover_grid(ctx, T);
   if (ctx->cfg.dtype == UNIPOOL_BF16)
-    return combine_dispatch_k<__nv_bfloat16>(grid, s, k, Yp, row_of, gate, residual, y, T, row_vecs);
-  return combine_dispatch_k<float>(grid, s, k, Yp, row_of, gate, residual, y, T, row_vecs);
+    return combine_dispatch_k<__nv_bfloat16>(ctx, grid, s, k, Yp, row_of, gate, residual, y, T, row_vecs);
+  return combine_dispatch_k<float>(ctx, grid, s, k, Yp, row_of, gate, residual, y, T, row_vecs);
 }
 
 int combine_launch(unipool_ctx* ctx, const void* Yp, const int32_t* row_of, const float* gate, int T,
