@@ -28,6 +28,7 @@ enum RowEpilogue {
 // with tokens are numbered first, so that the blocks that have work, one after the other, fall evenly on the SMs: numbered
 // as they lie in memory, with the tiles of the 128-row padding between them, some SMs had three blocks with work and some
 // none (SMs active for half of the 39 us of dgrad gate/up, 16 experts of 256 x 512, 64 rows each).
+template <int kRows>
 __device__ __forceinline__ bool find_row_tile(const RowGemm& p, int t, int* expert, int* row, bool* empty) {
   const int lane = threadIdx.x % 32;
   auto search = [&](bool pads, int base) {            // every warp for itself; returns the tiles counted
@@ -36,10 +37,10 @@ __device__ __forceinline__ bool find_row_tile(const RowGemm& p, int t, int* expe
       int first = 0, n = 0;
       if (e < p.n_experts) {
         first = p.offsets[e];
-        const int all = (p.offsets[e + 1] - first) / kSimtM;
-        const int live = p.rows ? min((max(p.rows[e], 0) + kSimtM - 1) / kSimtM, all) : all;
+        const int all = (p.offsets[e + 1] - first) / kRows;
+        const int live = p.rows ? min((max(p.rows[e], 0) + kRows - 1) / kRows, all) : all;
         n = pads ? all - live : live;
-        if (pads) first += live * kSimtM;
+        if (pads) first += live * kRows;
       }
       int upto = n;
 #pragma unroll
@@ -51,7 +52,7 @@ __device__ __forceinline__ bool find_row_tile(const RowGemm& p, int t, int* expe
       if (hit != 0) {
         const int src = __ffs(hit) - 1;
         *expert = e0 + src;
-        *row = __shfl_sync(0xffffffffu, first + (t - base - (upto - n)) * kSimtM, src);
+        *row = __shfl_sync(0xffffffffu, first + (t - base - (upto - n)) * kRows, src);
         *empty = pads;
         return -1;
       }
@@ -63,12 +64,11 @@ __device__ __forceinline__ bool find_row_tile(const RowGemm& p, int t, int* expe
   return live < 0 || search(true, live) < 0;
 }
 
-// C = A B_e for every 32-row tile of the groups; tiles behind a group's last token hold zeros and get zeros.
-template <int KG, Major BM, RowEpilogue EPI>
-__global__ void __launch_bounds__(SimtTile<KG>::kThreads, SimtTile<KG>::kBlocks)
+// C = A B_e for every row tile of the groups; tiles behind a group's last token hold zeros and get zeros.
+template <typename T, Major BM, RowEpilogue EPI>
+__global__ void __launch_bounds__(T::kThreads, T::kBlocks)
 grouped_rows_gemm_kernel(RowGemm p) {
   grid_wait(p.A, p.B, p.GU);
-  using T = SimtTile<KG>;
   constexpr int TN = kSimtN, kHalf = TN / 2;
   extern __shared__ float4 smem_raw[];
   typename T::Smem& sm = *reinterpret_cast<typename T::Smem*>(smem_raw);
@@ -76,9 +76,10 @@ grouped_rows_gemm_kernel(RowGemm p) {
   for (int rt = blockIdx.y; rt < p.n_row_tiles; rt += gridDim.y) {
     int e, m0;
     bool empty;
-    if (!find_row_tile(p, rt, &e, &m0, &empty)) break;   // uniform over the block
+    if (!find_row_tile<T::kRows>(p, rt, &e, &m0, &empty)) break;   // uniform over the block
     const float* B = p.B + (int64_t)(p.expert_base + e) * p.b_expert;
-    T::template run<kAlongK, BM>(
+    T t;
+    t.template run<kAlongK, BM>(
         sm, empty ? 0 : p.K / kSimtKC, p.vec, p.vec, p.A, [](int) {},
         [&](int c, int i, int k) { return p.A + (int64_t)(m0 + i) * p.lda + c * kSimtKC + k; },
         [&](int c, int i, int k) {
@@ -87,27 +88,27 @@ grouped_rows_gemm_kernel(RowGemm p) {
           const int kk = c * kSimtKC + k;
           return BM == kAlongK ? B + (int64_t)i * p.ldb + kk : B + (int64_t)kk * p.ldb + i;
         });
-    constexpr int kCols = EPI == kSwiglu ? kHalf : TN;
-#pragma unroll
-    for (int u = 0; u < kSimtM * kCols / 4 / T::kThreads; ++u) {
-      const int q = u * T::kThreads + threadIdx.x, i = q / (kCols / 4), j = q % (kCols / 4) * 4, n = n0 + j;
-      const int64_t r = m0 + i;
-      const float4 v = T::value4(sm, i, j);
-      if constexpr (EPI == kStore) {
-        st4(p.C + r * p.N + n, v, p.vec);
-      } else if constexpr (EPI == kSwiglu) {
-        const float4 u = T::value4(sm, i, j + kHalf);
+    if constexpr (EPI == kStore) {
+      t.each4(sm, [&](int i, int j, float4 v) { st4(p.C + (int64_t)(m0 + i) * p.N + n0 + j, v, p.vec); });
+    } else if constexpr (EPI == kSwiglu) {
+      t.each4_halves(sm, [&](int i, int j, float4 v, float4 u) {
+        const int64_t r = m0 + i;
+        const int n = n0 + j;
         st4(p.C + r * 2 * p.f + n, v, p.vec);
         st4(p.C + r * 2 * p.f + p.f + n, u, p.vec);
         st4(p.C2 + r * p.f + n, make_float4(silu_f(v.x) * u.x, silu_f(v.y) * u.y, silu_f(v.z) * u.z, silu_f(v.w) * u.w), p.vec);
-      } else {
+      });
+    } else {
+      t.each4(sm, [&](int i, int j, float4 v) {
+        const int64_t r = m0 + i;
+        const int n = n0 + j;
         const float4 g = ld4(p.GU + r * 2 * p.f + n, p.vec), u = ld4(p.GU + r * 2 * p.f + p.f + n, p.vec);
         st4(p.C + r * 2 * p.f + n,
             make_float4(v.x * u.x * silu_grad_f(g.x), v.y * u.y * silu_grad_f(g.y), v.z * u.z * silu_grad_f(g.z),
                         v.w * u.w * silu_grad_f(g.w)), p.vec);
         st4(p.C + r * 2 * p.f + p.f + n,
             make_float4(v.x * silu_f(g.x), v.y * silu_f(g.y), v.z * silu_f(g.z), v.w * silu_f(g.w)), p.vec);
-      }
+      });
     }
     if (gridDim.y < p.n_row_tiles) __syncthreads();  // the next tile reuses the buffers
   }
@@ -121,17 +122,19 @@ struct PoolGemm {
   float* dW; int Mdim, Ndim; bool overwrite, vec;
 };
 
-// (us with 1 / 2 / 4 warps to a tile, and with 64 x 64 tiles of four: 16 experts of 256 x 512, 4 layers of 64 rows, dW_down
-// 43/41/38, 45, dW_gu 74/70/71, 71; 30 of 128 x 384, 38 rows 31/23/22, 23 and 41/39/37, 38)
-using WgradTile = SimtTile<2, 2>;
+// Tiles of 64 x 64, two groups to each.  us of dW_down, dW_gu with warp tiles of two warps / block tiles: 16 experts of 256 x
+// 512, 64 rows 19/19, 29/25; 24 of 384 x 768, 250 rows 103/93, 195/174, very uneven groups 178/159, 306/220; 96 of 768 x 2048,
+// 341 rows 2590/2290, 5150/4560; misaligned, 24 of 384 x 768 155/101, 297/192.  (One group: a quarter slower where an expert has
+// many rows and few tiles.)
+using WgradTile = SimtBlockTile<2>;
 
 __global__ void __launch_bounds__(WgradTile::kThreads, WgradTile::kBlocks)
 grouped_k_gemm_kernel(PoolGemm p) {
   grid_wait(p.P, p.Q);
   using T = WgradTile;
   extern __shared__ float4 smem_raw[];
-  typename T::Smem& sm = *reinterpret_cast<typename T::Smem*>(smem_raw);
-  const int m0 = blockIdx.x * kSimtM, n0 = blockIdx.y * kSimtN, e = blockIdx.z;
+  T::Smem& sm = *reinterpret_cast<T::Smem*>(smem_raw);
+  const int m0 = blockIdx.x * T::kRows, n0 = blockIdx.y * kSimtN, e = blockIdx.z;
   auto rows_of = [&](int l) {
     const int32_t* off = p.offsets + (int64_t)l * (p.n_experts + 1) + e;
     return p.rows ? min(p.rows[(int64_t)l * p.n_experts + e], off[1] - off[0]) : off[1] - off[0];
@@ -152,56 +155,72 @@ grouped_k_gemm_kernel(PoolGemm p) {
       }
     }
   };
-  T::template run<kAcrossK, kAcrossK>(
+  T t;
+  t.run<kAcrossK, kAcrossK>(
       sm, n_chunks, p.vec, p.vec, p.P, seek,
-      [&](int, int i, int k) { return k < left ? p.P + (row0 + k) * p.ldp + m0 + i : nullptr; },
-      [&](int, int i, int k) { return k < left ? p.Q + (row0 + k) * p.ldq + n0 + i : nullptr; });
+      [&](int, int i, int k) -> const float* { return k < left ? p.P + (row0 + k) * p.ldp + m0 + i : nullptr; },
+      [&](int, int i, int k) -> const float* { return k < left ? p.Q + (row0 + k) * p.ldq + n0 + i : nullptr; });
   float* out = p.dW + (int64_t)(p.expert_base + e) * p.Mdim * p.Ndim;
-  for (int u = 0; u < kSimtM * kSimtN / 4 / T::kThreads; ++u) {
-    const int q = u * T::kThreads + threadIdx.x, i = q / (kSimtN / 4), j = q % (kSimtN / 4) * 4;
+  t.each4(sm, [&](int i, int j, float4 v) {
     float* o = out + (int64_t)(m0 + i) * p.Ndim + n0 + j;
-    float4 v = T::value4(sm, i, j);
     if (!p.overwrite) {
       const float4 w = p.vec ? *reinterpret_cast<const float4*>(o) : make_float4(o[0], o[1], o[2], o[3]);
       v = make_float4(v.x + w.x, v.y + w.y, v.z + w.z, v.w + w.w);
     }
     st4(o, v, p.vec);
-  }
+  });
 }
 
-template <int KG, Major BM, RowEpilogue EPI>
+template <typename T, Major BM, RowEpilogue EPI>
 int rows_gemm_as(const unipool_ctx* ctx, RowGemm p, cudaStream_t s) {
-  auto kern = grouped_rows_gemm_kernel<KG, BM, EPI>;
-  constexpr int smem = (int)sizeof(typename SimtTile<KG>::Smem);
+  auto kern = grouped_rows_gemm_kernel<T, BM, EPI>;
+  constexpr int smem = (int)sizeof(typename T::Smem);
   UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-  p.n_row_tiles = (int)(ctx->row_capacity / kSimtM);
+  p.n_row_tiles = (int)(ctx->row_capacity / T::kRows);
   const int gy = p.n_row_tiles < 8192 ? p.n_row_tiles : 8192;
-  UP_KERNEL(kern, dim3(p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN), gy), SimtTile<KG>::kThreads, smem, s, p);
+  UP_KERNEL(kern, dim3(p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN), gy), T::kThreads, smem, s, p);
   return UNIPOOL_OK;
 }
 
 template <Major BM, RowEpilogue EPI>
 int rows_gemm(unipool_ctx* ctx, RowGemm p, int n_experts, cudaStream_t s) {
   p.vec = aligned16(p.A, p.B, p.C, p.C2, p.GU);    // those that the epilogue has not are NULL
-  // Warps to a tile, by the tiles of a full batch (a group ends on half a tile).  us with 1 / 2 / 4 / 8 warps, and with the
-  // 64 x 64 tiles of two warps that were here before:
+  const int64_t rows = (int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k;
+  const int64_t tiles = (rows / kSimtM + n_experts / 2) * (p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN));
+  // Block tiles, by the tiles (of 32 rows) of a full batch, where groups average at least three of them: of fewer rows the
+  // 64-row tiles multiply a third more padding.  From a contraction of 768 on (256 where nothing but it is left to share)
+  // two groups share a tile.  Misaligned operands earlier and whatever the rows: they cost 4-byte copies.  us, warp tiles
+  // (by the rule below) / block tiles with one / two groups:
+  //   16 of 512 x 1024, 512 rows    gate/up (8448 tiles) 459/406/428   down (2112) 249/227/227   dgrad down (4224) 264/242/259   dgrad gate/up (2112) 461/441/431
+  //   96 of 768 x 2048, 341 rows    (68608) 5130/4751/5010   (12864) 2520/2370/2460   (34304) 2940/2420/2650   (12864) 5220/4640/4680
+  //   24 of 384 x 768, 250 rows     (4776) 219/194/195   (1194) 113/126/112   (2388) 129/134/148   (1194) 213/246/208
+  //   32 of 192 x 768, 500 rows     (12384) 270/243/263   (1548) 140/132/133   (6192) 196/178/238   (1548) 259/252/248
+  //   96 of 768 x 2048, 85 rows     (19456) 1470/1640/1730   (3648) 707/844/858   (9728) 886/861/957   (3648) 1460/1670/1650
+  //   misaligned, 24 of 384 x 768   (4776) 343/257/250   (1194) 170/142/140   (2388) 166/155/164   (1194) 285/267/239
+  const bool large = tiles >= (EPI == kSwigluBwd ? (p.vec ? 3000 : 2000) : EPI == kSwiglu || p.vec ? 1500 : 700);
+  if (large && (!p.vec || rows >= (int64_t)3 * kSimtM * n_experts))
+    return p.K >= (EPI == kStore ? 256 : 768) ? rows_gemm_as<SimtBlockTile<2>, BM, EPI>(ctx, p, s)
+                                              : rows_gemm_as<SimtBlockTile<1>, BM, EPI>(ctx, p, s);
+  // Warps to a warp tile (a contraction of 768 and more is at least two sums).  us with 1 / 2 / 4 / 8 warps, and with 64 x 64
+  // tiles of two groups:
   //   16 experts of 256 x 512, 64 rows      gate/up (640 tiles) 39/31/29/38, 35  down (160) 39/23/21/19, 23
   //                                         dgrad down (320) 44/29/22/25, 32     dgrad gate/up (160) 75/40/36/32, 39
   //   32 of 256 x 704, 14 rows              (660) 43/41/45/74, 71   (120) 52/30/27/19, 33   (330) 45/38/39/53, 54   (120) 102/54/47/28, 56
   //   15 of 384 x 512, 91 rows              (800) 56/45/46/53, 56   (300) 40/35/28/28, 31   (400) 52/38/27/32, 41   (300) 76/66/50/48, 53
-  //   24 of 384 x 768, 250 rows             (4776) 219/227/228/276, 207   (1194) 136/120/114/120, 115
-  //                                         (2388) 160/136/127/169, 139   (1194) 280/235/212/223, 216
-  const int64_t rows = (int64_t)ctx->cfg.max_tokens * ctx->cfg.top_k;
-  const int64_t tiles = (rows / kSimtM + n_experts / 2) * (p.N / (EPI == kSwiglu ? kSimtN / 2 : kSimtN));
-  if (10 * tiles <= 11 * ctx->sm_count && p.K >= (tiles <= ctx->sm_count ? 256 : 512)) return rows_gemm_as<8, BM, EPI>(ctx, p, s);
-  if (BM == kAlongK && tiles >= 1500) return rows_gemm_as<1, BM, EPI>(ctx, p, s);
-  if (tiles >= 600 && (p.K < 256 || (BM == kAlongK && rows < (int64_t)kSimtM * n_experts))) return rows_gemm_as<2, BM, EPI>(ctx, p, s);
-  return rows_gemm_as<4, BM, EPI>(ctx, p, s);
+  //   64 of 192 x 128, 250 rows             dgrad down (1064) 53/53/47/56, 67
+  if (10 * tiles <= 11 * ctx->sm_count && p.K >= (tiles <= ctx->sm_count ? 256 : 512))
+    return rows_gemm_as<SimtTile<8>, BM, EPI>(ctx, p, s);
+  if constexpr (BM == kAlongK) {
+    if (tiles >= 1500 && p.K < 768) return rows_gemm_as<SimtTile<1>, BM, EPI>(ctx, p, s);
+    if (tiles >= 1500 || (tiles >= 600 && (p.K < 256 || rows < (int64_t)kSimtM * n_experts)))
+      return rows_gemm_as<SimtTile<2>, BM, EPI>(ctx, p, s);
+  }
+  return rows_gemm_as<SimtTile<4>, BM, EPI>(ctx, p, s);
 }
 
 int k_gemm(const PoolGemm& p, cudaStream_t s) {
   UP_CUDA(cudaFuncSetAttribute(grouped_k_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(WgradTile::Smem)));
-  UP_KERNEL(grouped_k_gemm_kernel, dim3(p.Mdim / kSimtM, p.Ndim / kSimtN, p.n_experts), WgradTile::kThreads,
+  UP_KERNEL(grouped_k_gemm_kernel, dim3(p.Mdim / WgradTile::kRows, p.Ndim / kSimtN, p.n_experts), WgradTile::kThreads,
             sizeof(WgradTile::Smem), s, p);
   return UNIPOOL_OK;
 }

@@ -42,10 +42,11 @@ __device__ __forceinline__ void copy_async(uint32_t dst, const float* src, const
   else asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" : : "r"(dst), "l"(from), "r"(n) : "memory");
 }
 
-// kStages: chunks in shared memory.  Three cover long contractions over L2 better, two leave room for sixteen warps on an SM.
-template <int KG, int kStages = 3>
+// Twelve warps on an SM.  (168 registers: the forward GEMMs of one to four warps spill 12 to 28 bytes.)
+template <int KG>
 struct SimtTile {
-  static constexpr int kThreads = KG * 32, kBlocks = (kStages == 3 ? 12 : 16) / KG;   // blocks of an SM
+  static constexpr int kStages = 3;                // chunks in shared memory
+  static constexpr int kRows = kSimtM, kThreads = KG * 32, kBlocks = 12 / KG;
   struct Stage { float a[kSimtM * kSimtKC], b[kSimtN * kSimtKC]; };
   union Warp { Stage stage[kStages]; float sums[kSimtM * kSimtLd]; };
   struct Smem { Warp w[KG]; };
@@ -180,6 +181,157 @@ struct SimtTile {
 #pragma unroll
     for (int g = 1; g < KG; ++g) v += s.w[g].sums[r * kSimtLd + c];
     return v;
+  }
+  // put(r, c, sums of columns c .. c + 3) for the thread's share of the tile; put2(r, c, those, the same 32 columns on).
+  template <typename F> __device__ static void each4(const Smem& s, F put) {
+#pragma unroll
+    for (int u = 0; u < kRows * kSimtN / 4 / kThreads; ++u) {
+      const int q = u * kThreads + threadIdx.x, r = q / (kSimtN / 4), c = q % (kSimtN / 4) * 4;
+      put(r, c, value4(s, r, c));
+    }
+  }
+  template <typename F> __device__ static void each4_halves(const Smem& s, F put2) {
+#pragma unroll
+    for (int u = 0; u < kRows * kSimtN / 8 / kThreads; ++u) {
+      const int q = u * kThreads + threadIdx.x, r = q / (kSimtN / 8), c = q % (kSimtN / 8) * 4;
+      put2(r, c, value4(s, r, c), value4(s, r, c + kSimtN / 2));
+    }
+  }
+};
+
+// The tile of batches that fill the chip several times over: 64 x 64, shared by all threads of a block.  A group of 64
+// threads keeps 8 x 8 results each, packed in pairs (fma.rn.f32x2: each half an IEEE fp32 fma); chunks go through
+// double-buffered shared memory, fetched into registers one chunk ahead with 16-byte loads (four of 4 bytes where an operand
+// misses that alignment: an eighth of the instructions that 4-byte cp.async would take), and the operands of step k + 1
+// are read while step k is multiplied.  KG groups share a tile by taking every KG-th chunk.
+// Per product it moves two thirds of the warp tile's bytes through L2 and shared memory's other side, which is what counts
+// once every scheduler has warps enough: 16 experts of 1024 x 4096, 512 rows each, forward 43 TFLOP/s against 37 to 41
+// (the rule and the figures: expert_simt.cu).  Twelve warps on an SM, 160 to 168 registers.
+template <int KG>
+struct SimtBlockTile {
+  static constexpr int kGroup = 64, kRows = 64, kThreads = KG * kGroup, kBlocks = 6 / KG, MR = 8, NR = 8;
+  static constexpr int kA4 = kRows * kSimtKC / 4 / kGroup, kB4 = kSimtN * kSimtKC / 4 / kGroup;   // float4 per thread
+  struct Smem {
+    float a[KG][2][kSimtKC][kRows + 4];
+    float b[KG][2][kSimtKC][kSimtN + 4];
+  };
+  unsigned long long acc[MR][NR / 2];
+
+  // results of this thread: row(i), column(j) inside the tile
+  __device__ static int row(int i) { return i % 4 + i / 4 * (kRows / 2) + threadIdx.x % kGroup / 8 * 4; }
+  __device__ static int col(int j) { return j % 4 + j / 4 * (kSimtN / 2) + threadIdx.x % 8 * 4; }
+  __device__ float value(int i, int j) const {
+    const unsigned long long v = acc[i][j / 2];
+    return __uint_as_float(j & 1 ? (uint32_t)(v >> 32) : (uint32_t)v);
+  }
+  __device__ float4 value4(int i, int j) const { return make_float4(value(i, j), value(i, j + 1), value(i, j + 2), value(i, j + 3)); }
+
+  // One operand's chunk: registers <- memory and shared memory <- registers.
+  template <Major MJ, int N4, typename F>
+  __device__ static void fetch(float4 (&r)[N4], bool vec, F src) {
+#pragma unroll
+    for (int q = 0; q < N4; ++q) {
+      const int v = threadIdx.x % kGroup + q * kGroup;
+      const float* p = MJ == kAlongK ? src(v / (kSimtKC / 4), v % (kSimtKC / 4) * 4) : src(v % 16 * 4, v / 16);
+      r[q] = p ? ld4(p, vec) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+  template <Major MJ, int N4>
+  __device__ static void stash(float (*s)[kSimtN + 4], const float4 (&r)[N4]) {
+    static_assert(kRows == kSimtN, "both operands have rows of 64");
+#pragma unroll
+    for (int q = 0; q < N4; ++q) {
+      const int v = threadIdx.x % kGroup + q * kGroup;
+      if (MJ == kAlongK) {
+        const int i = v / (kSimtKC / 4), k = v % (kSimtKC / 4) * 4;
+        s[k][i] = r[q].x; s[k + 1][i] = r[q].y; s[k + 2][i] = r[q].z; s[k + 3][i] = r[q].w;
+      } else {
+        *reinterpret_cast<float4*>(&s[v / 16][v % 16 * 4]) = r[q];
+      }
+    }
+  }
+  struct Frag { float a[MR]; unsigned long long b[NR / 2]; };
+  __device__ static void read(Frag& f, const float (*sa)[kRows + 4], const float (*sb)[kSimtN + 4], int k) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float4 v = *reinterpret_cast<const float4*>(&sa[k][row(4 * h)]);
+      f.a[4 * h] = v.x; f.a[4 * h + 1] = v.y; f.a[4 * h + 2] = v.z; f.a[4 * h + 3] = v.w;
+      const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(&sb[k][col(4 * h)]);
+      f.b[2 * h] = w.x; f.b[2 * h + 1] = w.y;
+    }
+  }
+
+  // As SimtTile::run; on return the first group of threads holds the sums.
+  template <Major AM, Major BM, typename FB0, typename FA, typename FB>
+  __device__ void run(Smem& s, int n_chunks, bool vec_a, bool vec_b, const float*, FB0 begin, FA a_at, FB b_at) {
+    const int g = threadIdx.x / kGroup;
+#pragma unroll
+    for (int i = 0; i < MR; ++i)
+#pragma unroll
+      for (int j = 0; j < NR / 2; ++j) acc[i][j] = 0ull;
+    const int n_it = (n_chunks + KG - 1) / KG;
+    float4 ra[kA4], rb[kB4];
+    auto load = [&](int it) {
+      const int c = it * KG + g;
+      const bool some = c < n_chunks;
+      if (some) begin(c);
+      fetch<AM>(ra, vec_a, [&](int i, int k) -> const float* { return some ? a_at(c, i, k) : nullptr; });
+      fetch<BM>(rb, vec_b, [&](int i, int k) -> const float* { return some ? b_at(c, i, k) : nullptr; });
+    };
+    if (n_it > 0) load(0);
+    for (int it = 0; it < n_it; ++it) {
+      float (*sa)[kRows + 4] = s.a[g][it & 1];
+      float (*sb)[kSimtN + 4] = s.b[g][it & 1];
+      stash<AM>(sa, ra);
+      stash<BM>(sb, rb);
+      __syncthreads();                             // also: everyone is done with the buffer the next chunk goes to
+      if (it + 1 < n_it) load(it + 1);
+      Frag f[2];
+      read(f[0], sa, sb, 0);
+#pragma unroll
+      for (int k = 0; k < kSimtKC; ++k) {
+        if (k + 1 < kSimtKC) read(f[(k + 1) & 1], sa, sb, k + 1);
+        const Frag& c = f[k & 1];
+#pragma unroll
+        for (int i = 0; i < MR; ++i) {
+          unsigned long long aa;
+          asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(c.a[i]));
+#pragma unroll
+          for (int j = 0; j < NR / 2; ++j) asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc[i][j]) : "l"(aa), "l"(c.b[j]));
+        }
+      }
+    }
+    if constexpr (KG > 1) {                        // the other groups hand their sums over through shared memory
+      __syncthreads();
+      constexpr int kSums = MR * NR / 2;
+      unsigned long long* x = reinterpret_cast<unsigned long long*>(&s);
+      static_assert(sizeof(Smem) >= (KG - 1) * kSums * kGroup * 8, "room for the groups' sums");
+      const int t = threadIdx.x % kGroup;
+      if (g > 0) {
+#pragma unroll
+        for (int q = 0; q < kSums; ++q) x[((g - 1) * kSums + q) * kGroup + t] = acc[q / (NR / 2)][q % (NR / 2)];
+      }
+      __syncthreads();
+      if (g == 0) {
+        for (int o = 0; o < KG - 1; ++o)
+#pragma unroll
+          for (int q = 0; q < kSums; ++q)
+            asm("add.rn.f32x2 %0, %0, %1;" : "+l"(acc[q / (NR / 2)][q % (NR / 2)]) : "l"(x[(o * kSums + q) * kGroup + t]));
+      }
+    }
+  }
+
+  template <typename F> __device__ void each4(const Smem&, F put) const {
+    if (threadIdx.x >= kGroup) return;
+#pragma unroll
+    for (int i = 0; i < MR; ++i)
+#pragma unroll
+      for (int j = 0; j < NR; j += 4) put(row(i), col(j), value4(i, j));
+  }
+  template <typename F> __device__ void each4_halves(const Smem&, F put2) const {
+    if (threadIdx.x >= kGroup) return;
+#pragma unroll
+    for (int i = 0; i < MR; ++i) put2(row(i), col(0), value4(i, 0), value4(i, 4));
   }
 };
 

@@ -1,5 +1,5 @@
-"""The fp32 row GEMMs with one, two, four and eight warps to a tile, and the search for a row tile among more experts than
-a warp has lanes."""
+"""The fp32 row GEMMs with one, two, four and eight warps to a warp tile and one and two groups to a block tile, and the search
+for a row tile among more experts than a warp has lanes.  (Four warps: the other fp32 tests.)"""
 import pytest
 import torch
 
@@ -13,9 +13,23 @@ pytestmark = pytest.mark.gpu
     ([64, 0, 1, 31, 32, 33, 95, 96, 97, 0, 128] * 3, 256, 1024),       # one; groups that end on tiles of 32
     ([0, 20], 320, 640),                                    # eight, which 20 chunks do not divide among evenly
     ([1] * 65 + [0] * 30 + [2], 192, 256),                  # 96 experts: three rounds of the search
+    # warp tiles, groups of fewer than 96 rows
+    ([64, 31, 95, 33, 1, 96, 100, 60] * 5, 128, 768),       # one warp: gate/up (misaligned: block tiles)
+    ([64, 31, 95, 33, 1, 96, 100, 60] * 5, 1024, 256),      # one warp: down
+    ([64, 31, 95, 33, 1, 96, 100, 60] * 5, 768, 512),       # two warps, a contraction of 768: gate/up
+    ([64, 31, 95, 33, 1, 96, 100, 60] * 5, 1024, 768),      # two warps, a contraction of 768: down, gate/up
+    ([25, 0, 50, 24] * 10, 1024, 64),                       # two warps, a short contraction: down
+    # block tiles; groups that end at and beside tiles of 64
+    ([200, 0, 64, 511, 321, 129, 128, 1, 65, 63, 448, 470], 128, 768),   # one group: gate/up
+    ([362, 0, 896, 65, 300, 400, 449, 460], 1024, 64),      # one group: down, dgrad gate/up
+    ([362, 0, 896, 65, 300, 400, 449, 460], 1024, 256),     # two groups: down, dgrad gate/up
+    ([127, 513, 0, 321], 768, 1536),                        # two groups, a contraction of 768: gate/up
+    ([1000, 577, 1, 1022, 640, 770], 128, 1536),            # one group: dgrad down
+    ([1000, 577, 1, 1022, 640, 770], 768, 1536),            # two groups: dgrad down
+    ([1311] * 400, 64, 64),                                 # more than 8192 row tiles
 ])
 @pytest.mark.parametrize("shift", [0, 1])
-def test_fp32_ffn_by_warps_to_a_tile(sizes, d, f, shift):
+def test_fp32_ffn_by_tiles(sizes, d, f, shift):
     check_ffn(sizes, d, f, shift)
 
 
