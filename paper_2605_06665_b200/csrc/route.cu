@@ -7,17 +7,18 @@
 namespace unipool {
 
 // ---------------------------------------------------------------- logits  z = x W_r^T (+ bias)
-// Few tiles (one per 32 tokens and 64 experts), so eight warps share a tile's contraction.
-using RouterTile = SimtTile<8>;
-
+// Eight warps share a tile of 32 tokens and 64 experts while every tile has an SM to itself; of more tiles, with four warps
+// to each, an SM takes three.  us of the router with eight / four: 512 tokens, 16 experts of 256 11.9 / 12.8; 1024, 384 of 256 (192
+// tiles) 22.8 / 20.5; 8192, 16 of 256 (256) 23.3 / 21.0; 16384, 96 of 768 123 / 108.  (Eight: 255 registers, 44 bytes spilled.)
+template <typename RouterTile>
 __global__ void __launch_bounds__(RouterTile::kThreads, RouterTile::kBlocks)
 router_logits_kernel(const float* __restrict__ x, const float* __restrict__ W_r,
                      const float* __restrict__ bias, float* __restrict__ z, int T, int M, int d, bool vec) {
   grid_wait(x, W_r, bias);
   extern __shared__ float4 smem_raw[];
-  RouterTile::Smem& sm = *reinterpret_cast<RouterTile::Smem*>(smem_raw);
+  typename RouterTile::Smem& sm = *reinterpret_cast<typename RouterTile::Smem*>(smem_raw);
   const int m0 = blockIdx.x * kSimtM, n0 = blockIdx.y * kSimtN;
-  RouterTile::run<kAlongK, kAlongK>(
+  RouterTile::template run<kAlongK, kAlongK>(
       sm, d / kSimtKC, vec, vec, x, [](int) {},
       [&](int c, int i, int k) { return m0 + i < T ? x + (int64_t)(m0 + i) * d + c * kSimtKC + k : nullptr; },
       [&](int c, int i, int k) { return n0 + i < M ? W_r + (int64_t)(n0 + i) * d + c * kSimtKC + k : nullptr; });
@@ -27,14 +28,24 @@ router_logits_kernel(const float* __restrict__ x, const float* __restrict__ W_r,
   }
 }
 
+template <typename RouterTile>
+static int router_logits_as(const float* x, const float* W_r, const float* bias, float* z, int T, int M, int d, cudaStream_t s) {
+  auto kern = router_logits_kernel<RouterTile>;
+  constexpr int smem = (int)sizeof(typename RouterTile::Smem);
+  UP_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+  UP_KERNEL(kern, dim3((T + kSimtM - 1) / kSimtM, (M + kSimtN - 1) / kSimtN), RouterTile::kThreads, smem, s, x, W_r, bias, z, T, M, d,
+            aligned16(x, W_r));
+  return UNIPOOL_OK;
+}
+
 // ---------------------------------------------------------------- scores, top-k, statistics
 // One warp per token.  Lane l holds experts l, l+32, ...  Selection key: score
 // descending, expert index ascending.
 constexpr int kRouteWarps = 8;
 
-template <bool SOFTMAX>
+template <bool SOFTMAX, int kPerWarp>
 __global__ void __launch_bounds__(kRouteWarps * 32)
-router_select_kernel(const float* __restrict__ z, int T, int M, int k, int per_warp, float sigma_c, float eps,
+router_select_kernel(const float* __restrict__ z, int T, int M, int k, float sigma_c, float eps,
                      int32_t* __restrict__ idx, float* __restrict__ gate, float* __restrict__ znorm,
                      int32_t* __restrict__ counts_out, float* __restrict__ sum_out,
                      int32_t* __restrict__ acc_counts, double* __restrict__ acc_sums,
@@ -50,8 +61,8 @@ router_select_kernel(const float* __restrict__ z, int T, int M, int k, int per_w
   __syncthreads();
 
   float* my = sc + warp * M;
-  const int t_begin = (blockIdx.x * kRouteWarps + warp) * per_warp;
-  for (int tt = 0; tt < per_warp; ++tt) {
+  const int t_begin = (blockIdx.x * kRouteWarps + warp) * kPerWarp;
+  for (int tt = 0; tt < kPerWarp; ++tt) {
     const int t = t_begin + tt;
     if (t >= T) break;
     const float* zr = z + (int64_t)t * M;
@@ -166,18 +177,25 @@ int route_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float
                                                                          score_sum, znorm, z_saved, s);
   {
     PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_LOGITS, 1, s);
-    UP_CUDA(cudaFuncSetAttribute(router_logits_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RouterTile::Smem)));
-    UP_KERNEL(router_logits_kernel, dim3((T + 31) / 32, (M + 63) / 64), RouterTile::kThreads, sizeof(RouterTile::Smem), s,
-              static_cast<const float*>(x), W_r, bias, z_saved, T, M, d, aligned16(x, W_r));
+    const int64_t tiles = (int64_t)((T + kSimtM - 1) / kSimtM) * ((M + kSimtN - 1) / kSimtN);
+    const int rc = (tiles <= ctx->sm_count ? router_logits_as<SimtTile<8>> : router_logits_as<SimtTile<4>>)(
+        static_cast<const float*>(x), W_r, bias, z_saved, T, M, d, s);
+    if (rc != UNIPOOL_OK) return rc;
   }
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_SELECT, 1, s);
-  // a token to a warp while that leaves every SM two blocks at most (512 tokens, 16 experts: 8.9 -> 5.1 us)
-  const int per_warp = T <= 2 * kRouteWarps * ctx->sm_count ? 1 : 4, per_block = kRouteWarps * per_warp;
+  // A token to a warp, or four one after the other: more blocks hide more latency, but each adds its totals of all experts by
+  // atomics.  us of the router with one / four (experts of 256): 512 tokens, 16 experts 12.1 / 15.5; 4800, 16 18.1 / 20.2; 8192, 16
+  // 20.4 / 21.2; 4736, 64 17.4 / 17.7; 9000, 64 25.3 / 22.7; 2400, 96 20.7 / 22.0; 3552, 96 23.5 / 22.3; 4736, 96 25.9 / 23.3;
+  // 2400, 384 33.4 / 37.7; 4736, 512 56.3 / 57.1.
+  const int most = M <= 32 ? 8 : M <= 64 ? 4 : 3;              // blocks to an SM
+  const int per_warp = T <= most * kRouteWarps * ctx->sm_count ? 1 : 4, per_block = kRouteWarps * per_warp;
   const int blocks = (T + per_block - 1) / per_block;
   const size_t smem = (size_t)(2 * kRouteWarps * M) * sizeof(float) + (size_t)M * sizeof(int);
   static_assert((2 * kRouteWarps + 1) * UNIPOOL_MAX_EXPERTS * 4 <= 48 * 1024, "no opt-in to more shared memory");
-  auto kern = ctx->cfg.router_mode == UNIPOOL_ROUTER_SOFTMAX ? router_select_kernel<true> : router_select_kernel<false>;
-  UP_KERNEL(kern, blocks, kRouteWarps * 32, smem, s, z_saved, T, M, k, per_warp, sigma * ctx->cfg.c, ctx->cfg.eps, idx, gate, znorm,
+  const bool softmax = ctx->cfg.router_mode == UNIPOOL_ROUTER_SOFTMAX;
+  auto kern = per_warp == 1 ? (softmax ? router_select_kernel<true, 1> : router_select_kernel<false, 1>)
+                            : (softmax ? router_select_kernel<true, 4> : router_select_kernel<false, 4>);
+  UP_KERNEL(kern, blocks, kRouteWarps * 32, smem, s, z_saved, T, M, k, sigma * ctx->cfg.c, ctx->cfg.eps, idx, gate, znorm,
             counts, score_sum, ctx->ws.route_counts, ctx->ws.route_sums, ctx->ws.tickets + 0);
   return UNIPOOL_OK;
 }
@@ -291,15 +309,17 @@ router_dx_kernel(const float* __restrict__ dz, const float* __restrict__ W_r, fl
 
 // dW_r[m,:] += sum_t dz[t,m] x[t,:]   (K = T, cut into runs of k_len tokens over blockIdx.z: one run adds in
 // place, several by atomics)
-__global__ void __launch_bounds__(RouterTile::kThreads, RouterTile::kBlocks)
+using RouterDwTile = SimtTile<8>;
+
+__global__ void __launch_bounds__(RouterDwTile::kThreads, RouterDwTile::kBlocks)
 router_dw_kernel(const float* __restrict__ dz, const float* __restrict__ x, float* __restrict__ dW_r,
                  int T, int M, int d, int k_len, bool vec) {
   grid_wait(dz, x);
   extern __shared__ float4 smem_raw[];
-  RouterTile::Smem& sm = *reinterpret_cast<RouterTile::Smem*>(smem_raw);
+  RouterDwTile::Smem& sm = *reinterpret_cast<RouterDwTile::Smem*>(smem_raw);
   const int m0 = blockIdx.x * kSimtM, n0 = blockIdx.y * kSimtN;
   const int k_begin = blockIdx.z * k_len, k_end = min(T, k_begin + k_len);
-  RouterTile::run<kAcrossK, kAcrossK>(
+  RouterDwTile::run<kAcrossK, kAcrossK>(
       sm, (k_end - k_begin + kSimtKC - 1) / kSimtKC, (M & 3) == 0, vec, dz, [](int) {},
       [&](int c, int i, int k) {
         const int tok = k_begin + c * kSimtKC + k;
@@ -309,11 +329,11 @@ router_dw_kernel(const float* __restrict__ dz, const float* __restrict__ x, floa
         const int tok = k_begin + c * kSimtKC + k;
         return tok < k_end ? x + (int64_t)tok * d + n0 + i : nullptr;
       });
-  for (int q = threadIdx.x; q < kSimtM * kSimtN; q += RouterTile::kThreads) {
+  for (int q = threadIdx.x; q < kSimtM * kSimtN; q += RouterDwTile::kThreads) {
     const int m = m0 + q / kSimtN;
     if (m >= M) continue;
     float* o = dW_r + (int64_t)m * d + n0 + q % kSimtN;
-    const float v = RouterTile::value(sm, q / kSimtN, q % kSimtN);
+    const float v = RouterDwTile::value(sm, q / kSimtN, q % kSimtN);
     if (gridDim.z == 1) *o += v;
     else atomicAdd(o, v);
   }
@@ -342,9 +362,9 @@ int route_bwd_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, f
   }
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_BWD_DW, 1, s);
   const int k_len = 1024;
-  UP_CUDA(cudaFuncSetAttribute(router_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RouterTile::Smem)));
-  UP_KERNEL(router_dw_kernel, dim3((M + 31) / 32, d / 64, (T + k_len - 1) / k_len), RouterTile::kThreads,
-            sizeof(RouterTile::Smem), s, dz, static_cast<const float*>(x), dW_r, T, M, d, k_len, aligned16(x));
+  UP_CUDA(cudaFuncSetAttribute(router_dw_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(RouterDwTile::Smem)));
+  UP_KERNEL(router_dw_kernel, dim3((M + 31) / 32, d / 64, (T + k_len - 1) / k_len), RouterDwTile::kThreads,
+            sizeof(RouterDwTile::Smem), s, dz, static_cast<const float*>(x), dW_r, T, M, d, k_len, aligned16(x));
   return UNIPOOL_OK;
 }
 

@@ -4,6 +4,7 @@ import pytest
 import torch
 
 from test_gpu_kernel_edges import test_fp32_expert_ffn_at_the_edges_of_its_tiles as check_ffn
+from test_gpu_kernel_edges import test_fp32_router_products_at_the_edges_of_their_tiles as check_router
 
 pytestmark = pytest.mark.gpu
 
@@ -55,3 +56,13 @@ def test_fp32_rows_of_padded_groups_are_the_same():
         assert torch.equal(a[:used], b[:used]) and a[used:].isnan().all() and b[used:].isnan().all()
     ctx.check_status()
     ctx.close()
+
+
+@pytest.mark.parametrize("T,M,d", [
+    (148 * 32, 16, 64), (148 * 32 + 1, 64, 64),             # 148 and 149 tiles of logits: eight and four warps to each
+    (3 * 8 * 148, 65, 128), (3 * 8 * 148 + 1, 65, 128), (8 * 8 * 148, 10, 64), (8 * 8 * 148 + 1, 10, 64),   # one, four tokens to a selecting warp
+    (2000, 300, 192), (37, 512, 128),
+])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_fp32_router_by_tiles(T, M, d, shift):
+    check_router(T, M, d, shift)
