@@ -6,13 +6,14 @@ import pytest
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("M,d", [(5, 64), (96, 192)])
+@pytest.mark.parametrize("T,M,d", [(130, 5, 64), (130, 96, 192), (513, 5, 64), (513, 96, 192)])
 @pytest.mark.parametrize("prepared", [False, True])
-def test_router_terms_of_unaligned_fp32_weights(M, d, prepared):
-    """Router weights that are not 16-byte aligned are split by the scalar branch: same logits, bit for bit."""
+def test_router_terms_of_unaligned_fp32_weights(T, M, d, prepared):
+    """Router weights that are not 16-byte aligned: same logits, bit for bit.  513 tokens read their bf16 terms, split by the
+    scalar branch, 130 the weights themselves (the router for few tokens)."""
     import torch
     from paper_2605_06665_b200 import binding as B
-    T, L = 130, 2
+    L = 2
     ctx = B.Context(B.make_config(d, 64, M, 1, L, T, B.BF16, 1e-6, 2.0))
     g = torch.Generator(device="cuda").manual_seed(3)
     W = torch.empty(L * M * d, device="cuda").normal_(0, 0.02, generator=g)
@@ -25,8 +26,10 @@ def test_router_terms_of_unaligned_fp32_weights(M, d, prepared):
         o = dict(idx=torch.empty(T, 1, dtype=torch.int32, device="cuda"), gate=torch.empty(T, 1, device="cuda"),
                  counts=torch.empty(M, dtype=torch.int32, device="cuda"), score_sum=torch.empty(M, device="cuda"),
                  znorm=torch.empty(T, device="cuda"), z=torch.empty(T, M, device="cuda"))
+        ctx.profile_enable(True)
         ctx.route(x, T, w[M * d:], 1.0, None, M, *o.values())
-        torch.cuda.synchronize()
+        assert ctx.profile_read()["route_logits"][1] == (1 if T > 464 and not prepared else 0)      # the split
+        ctx.profile_enable(False)
         out.append(o)
     ctx.check_status()
     ctx.close()
@@ -336,17 +339,20 @@ def test_recomputed_layers_contract_in_runs(kw, L, T, accumulate):
 
 @pytest.mark.parametrize("T,M,d,k", [
     (1, 8, 64, 8), (257, 10, 64, 3), (130, 256, 128, 8), (300, 257, 128, 5), (520, 512, 64, 8), (300, 384, 832, 8), (33, 96, 768, 2),
+    (465, 8, 64, 8), (513, 10, 64, 3), (700, 256, 128, 8), (600, 257, 128, 5), (640, 384, 832, 8), (465, 96, 768, 2), (1025, 9, 192, 1),
 ])
 @pytest.mark.parametrize("bits", ["bf16", "fp32"])                # one or three bf16 terms of the router weights
-def test_bf16_router_at_the_edges_of_its_stages(T, M, d, k, bits):
+@pytest.mark.parametrize("mode", ["norm", "softmax"])
+def test_bf16_router_at_the_edges_of_its_stages(T, M, d, k, bits, mode):
     """Selection with many candidates per lane, one and two MMAs per k-block, one or three weight terms, fewer
-    k-blocks than stages; against the oracle in float64 as in the parity tests."""
+    k-blocks than stages; against the oracle in float64 as in the parity tests.  (From 465 tokens on the tensor cores, below
+    on clusters of CUDA-core blocks.)"""
     import torch
     from oracle import unipool_oracle as O
     from paper_2605_06665_b200 import binding as B
     from parity_utils import check_routing, rel_max, to_np
     eps, c = 1e-6, 2.0
-    ctx = B.Context(B.make_config(d, 64, M, k, 1, T, B.BF16, eps, c))
+    ctx = B.Context(B.make_config(d, 64, M, k, 1, T, B.BF16, eps, c, B.ROUTER_SOFTMAX if mode == "softmax" else B.ROUTER_NORM))
     g = torch.Generator(device="cuda").manual_seed(T)
     W = torch.empty(M, d, device="cuda").normal_(0, 0.02, generator=g)
     if bits == "bf16":
@@ -355,13 +361,14 @@ def test_bf16_router_at_the_edges_of_its_stages(T, M, d, k, bits):
     idx, gate = torch.empty(T, k, dtype=torch.int32, device="cuda"), torch.empty(T, k, device="cuda")
     counts, S = torch.empty(M, dtype=torch.int32, device="cuda"), torch.empty(M, device="cuda")
     n, z = torch.empty(T, device="cuda"), torch.empty(T, M, device="cuda")
+    ctx.profile_enable(True)
     ctx.route(x, T, W, 1.0, None, M, idx, gate, counts, S, n, z)
-    torch.cuda.synchronize()
+    assert ctx.profile_read()["route_logits"][1] == (1 if T > 464 else 0)               # the tensor-core router splits W
     ctx.check_status()
     ctx.close()
     f8 = lambda t: t.double().cpu().numpy()
-    ref = O.route(f8(x), f8(W), 1.0, c, eps, k, None)
-    check_routing(to_np(idx), ref["z"], ref["idx"], k)
-    ref = O.route(f8(x), f8(W), 1.0, c, eps, k, None, forced_idx=to_np(idx))
+    ref = O.route(f8(x), f8(W), 1.0, c, eps, k, None, mode=mode)
+    check_routing(to_np(idx), ref["z"], ref["idx"], k, mode)
+    ref = O.route(f8(x), f8(W), 1.0, c, eps, k, None, forced_idx=to_np(idx), mode=mode)
     assert rel_max(to_np(z), ref["z"]) < 1e-5 and rel_max(to_np(gate), ref["g"]) < 1e-5
     assert (to_np(counts) == ref["counts"]).all() and rel_max(to_np(S), ref["S"]) < 1e-5

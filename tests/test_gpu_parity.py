@@ -170,6 +170,8 @@ def test_small_fp32_shapes(kw, T):
     (dict(dtype="bf16", d=256, f=256, M=12, k=2, private=4, L=3), 520),
     (dict(dtype="bf16", d=128, f=128, M=10, k=3), 333),     # logit rows that are not 16-byte aligned
     (dict(dtype="bf16", d=64, f=64, M=512, k=8), 257),      # the largest pool and top-k, the smallest widths
+    (dict(dtype="bf16", d=128, f=128, M=10, k=3), 533),     # the same on the tensor-core router
+    (dict(dtype="bf16", d=64, f=64, M=512, k=8), 517),
     (dict(dtype="bf16", d=128, f=192, M=16, k=2), 1),       # a single token
     # groups of several row tiles: the four row-tile GEMMs run on CTA pairs
     (dict(dtype="bf16", d=256, f=320, M=4, k=2, zipf_beta=1.0), 2100),   # skewed: odd and even tile counts, f % 128 = 64
@@ -188,6 +190,8 @@ def test_small_bf16_shapes(kw, T):
     (dict(router="softmax", dtype="bf16", d=256, f=256, M=96, k=2), 700),     # tensor-core router
     (dict(router="softmax", dtype="bf16", d=128, f=128, M=10, k=1), 333),     # unaligned logit rows
     (dict(router="softmax", dtype="bf16", d=128, f=128, M=384, k=8, zipf_beta=0.4), 400),
+    (dict(router="softmax", dtype="bf16", d=128, f=128, M=10, k=1), 533),     # the same on the tensor-core router
+    (dict(router="softmax", dtype="bf16", d=128, f=128, M=384, k=8, zipf_beta=0.4), 500),
     (dict(router="softmax", dtype="bf16", d=256, f=256, M=24, k=1, private=8, L=3), 520),
 ])
 def test_softmax_router_mode(kw, T):
