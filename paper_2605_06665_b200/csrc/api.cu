@@ -70,8 +70,12 @@ Workspace carve_workspace(const unipool_config& cfg, void* base) {
     const size_t per_token = cfg.dtype == UNIPOOL_BF16 ? mp * 2 : (size_t)cfg.pool_size * sizeof(float);
     w.dz = reinterpret_cast<float*>(take((size_t)cfg.max_tokens * per_token));
   }
-  w.w_split = cfg.dtype == UNIPOOL_BF16
-                  ? take((size_t)(cfg.n_layers + 1) * 3 * cfg.pool_size * cfg.d_model * 2) : nullptr;
+  if (cfg.dtype == UNIPOOL_BF16) {
+    const size_t router = (size_t)cfg.pool_size * cfg.d_model, terms = (cfg.n_layers + 1) * 3 * router * 2;
+    char* split = take(terms + cfg.n_layers * router * sizeof(float));
+    w.w_split = split;
+    w.w_copy = reinterpret_cast<float*>(split ? split + terms : nullptr);
+  }
   {
     const size_t tiles = 2 * (((size_t)cfg.max_tokens + 255) / 256);   // CTAs of the router: whole pairs
     w.part_counts = reinterpret_cast<int32_t*>(take(tiles * cfg.pool_size * sizeof(int32_t)));

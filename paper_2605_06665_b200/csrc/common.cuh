@@ -103,6 +103,7 @@ struct Workspace {
   int32_t* split_any;     // [n_layers + 1][4] which bf16 terms of a router's split weights are non-zero
   void*    w_split;       // [n_layers + 1][3, pool_size, d] bf16 terms of the router weights (bf16 mode): one slot
                           // per prepared layer, the last one scratch for routers that were not prepared
+  float*   w_copy;        // [n_layers][pool_size, d] the prepared layers' weights as they are (bf16 mode; same region)
   int32_t* part_counts;   // [2 ceil(max_tokens/256), pool_size] per-CTA routing counts (bf16 mode)
   float*   part_sums;     // [2 ceil(max_tokens/256), pool_size] per-CTA score sums
   float*   part_dsigma;   // [ceil(max_tokens/64)] per-block dsigma terms
@@ -247,6 +248,7 @@ int route_few_launch(unipool_ctx*, const void* x, int T, const float* W_r, float
                      int n_experts, int32_t* idx, float* gate, int32_t* counts, float* score_sum,
                      float* znorm, float* z_saved, cudaStream_t);
 int router_prepare_launch(unipool_ctx*, const float* W_r, int n_layers, int n_experts, cudaStream_t);
+int prepared_layer(const unipool_ctx*, const float* W_r, int n_experts);
 int route_bwd_tc_launch(unipool_ctx*, const void* x, int T, const float* W_r, float sigma, int n_experts,
                         const float* znorm, const float* z_saved, const int32_t* idx, const float* dgate,
                         const float* coef, void* dx, float* dW_r, float* dsigma, cudaStream_t);

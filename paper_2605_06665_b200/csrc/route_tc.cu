@@ -42,15 +42,16 @@ struct RouteParams {
 };
 
 // W_r fp32 [n_layers][n] -> three bf16 terms per layer [n_layers][3][n] (n = M*d); any[4 l + s] != 0 iff
-// term s of layer l has a non-zero element.  A grid row per layer, kSplitVec elements per thread and step.
-// Bound by HBM (4 bytes in, 6 out per weight).  The flags are what needs care: weights that use all of
+// term s of layer l has a non-zero element.  copy (may be NULL): the weights themselves too, for the router of few tokens.
+// A grid row per layer, kSplitVec elements per thread and step.
+// Bound by HBM (4 bytes in, 10 out per weight).  The flags are what needs care: weights that use all of
 // fp32 set them everywhere, and one atomicOr per warp on one address per layer took 1.05 ms for the 12
 // routers of 96 x 768 (9.3 ms for 24 of 192 x 1536); one block-wide vote and at most one atomic per
 // block, skipped when the flag is already seen, takes 16 us (51 us).
 template <int kSplitVec>
 __global__ void __launch_bounds__(256)
 router_split_kernel(const float* __restrict__ W, int64_t n, int n_layers, __nv_bfloat16* __restrict__ out,
-                    int32_t* __restrict__ any) {
+                    float* __restrict__ copy, int32_t* __restrict__ any) {
   grid_wait(W);
   for (int64_t l = blockIdx.y; l < n_layers; l += gridDim.y) {
     const float* w_l = W + l * n;
@@ -62,8 +63,10 @@ router_split_kernel(const float* __restrict__ W, int64_t n, int n_layers, __nv_b
       if constexpr (kSplitVec == 4) {
         const float4 v = __ldg(reinterpret_cast<const float4*>(w_l + i));
         w[0] = v.x; w[1] = v.y; w[2] = v.z; w[3] = v.w;
+        if (copy != nullptr) *reinterpret_cast<float4*>(copy + l * n + i) = v;
       } else {
         w[0] = w_l[i];
+        if (copy != nullptr) copy[l * n + i] = w[0];
       }
       alignas(8) __nv_bfloat16 h[3][kSplitVec];
 #pragma unroll
@@ -611,14 +614,14 @@ static __nv_bfloat16* scratch_terms(unipool_ctx* ctx) {
 // Splits the fp32 router weights of n_layers layers ([n_layers][M][d], contiguous) into three bf16 terms
 // per layer; flags[4 l + s] tells whether term s of layer l has a non-zero element.
 static int router_split_launch(unipool_ctx* ctx, const float* W_r, int n_layers, int M, __nv_bfloat16* out,
-                               int32_t* flags, cudaStream_t s) {
+                               float* copy, int32_t* flags, cudaStream_t s) {
   const int64_t n = (int64_t)M * ctx->cfg.d_model;
   UP_CUDA(cudaMemsetAsync(flags, 0, (size_t)n_layers * 4 * sizeof(int32_t), s));
   // n is a multiple of 64 (d is): four weights per thread unless the caller's array is not 16-byte aligned
   const bool vec = (reinterpret_cast<uintptr_t>(W_r) & 15) == 0;
   const int64_t blocks = (n + (vec ? 1023 : 255)) / (vec ? 1024 : 256);
   const dim3 grid((unsigned)(blocks < 1184 ? blocks : 1184), (unsigned)(n_layers < 65535 ? n_layers : 65535));
-  UP_KERNEL(vec ? router_split_kernel<4> : router_split_kernel<1>, grid, 256, 0, s, W_r, n, n_layers, out, flags);
+  UP_KERNEL(vec ? router_split_kernel<4> : router_split_kernel<1>, grid, 256, 0, s, W_r, n, n_layers, out, copy, flags);
   return UNIPOOL_OK;
 }
 
@@ -627,7 +630,7 @@ int router_prepare_launch(unipool_ctx* ctx, const float* W_r, int n_layers, int 
   if (n_layers == 0) return UNIPOOL_OK;
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_LOGITS, 1, s);
   const int rc = router_split_launch(ctx, W_r, n_layers, M, static_cast<__nv_bfloat16*>(ctx->ws.w_split),
-                                     ctx->ws.split_any, s);
+                                     ctx->ws.w_copy, ctx->ws.split_any, s);
   if (rc != UNIPOOL_OK) return rc;
   ctx->prepared_base = W_r;
   ctx->prepared_layers = n_layers;
@@ -635,23 +638,26 @@ int router_prepare_launch(unipool_ctx* ctx, const float* W_r, int n_layers, int 
   return UNIPOOL_OK;
 }
 
-// The bf16 terms of W_r and their flags: the prepared ones if W_r is a layer of the array last given to
-// unipool_router_prepare, otherwise the scratch set, filled now.
+// The layer that W_r is in the array last given to unipool_router_prepare, -1: none of it.
+int prepared_layer(const unipool_ctx* ctx, const float* W_r, int M) {
+  if (ctx->prepared_base == nullptr || M != ctx->prepared_experts || W_r < ctx->prepared_base) return -1;
+  const int64_t n = (int64_t)M * ctx->cfg.d_model, off = W_r - ctx->prepared_base;
+  return off % n == 0 && off / n < ctx->prepared_layers ? (int)(off / n) : -1;
+}
+
+// The bf16 terms of W_r and their flags: the prepared ones if W_r is a prepared layer, otherwise the scratch set, filled now.
 static int router_terms(unipool_ctx* ctx, const float* W_r, int M, int phase, const __nv_bfloat16** terms,
                         const int32_t** flags, cudaStream_t s) {
-  const int64_t n = (int64_t)M * ctx->cfg.d_model;
-  if (ctx->prepared_base != nullptr && M == ctx->prepared_experts && W_r >= ctx->prepared_base) {
-    const int64_t off = W_r - ctx->prepared_base;
-    if (off % n == 0 && off / n < ctx->prepared_layers) {
-      *terms = static_cast<const __nv_bfloat16*>(ctx->ws.w_split) + (off / n) * 3 * n;
-      *flags = ctx->ws.split_any + 4 * (off / n);
-      return UNIPOOL_OK;
-    }
+  const int l = prepared_layer(ctx, W_r, M);
+  if (l >= 0) {
+    *terms = static_cast<const __nv_bfloat16*>(ctx->ws.w_split) + (int64_t)l * 3 * M * ctx->cfg.d_model;
+    *flags = ctx->ws.split_any + 4 * l;
+    return UNIPOOL_OK;
   }
   *terms = scratch_terms(ctx);
   *flags = ctx->ws.split_any + 4 * ctx->cfg.n_layers;
   PhaseTimer pt(ctx, phase, 1, s);
-  return router_split_launch(ctx, W_r, 1, M, scratch_terms(ctx), ctx->ws.split_any + 4 * ctx->cfg.n_layers, s);
+  return router_split_launch(ctx, W_r, 1, M, scratch_terms(ctx), nullptr, ctx->ws.split_any + 4 * ctx->cfg.n_layers, s);
 }
 
 int route_tc_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float sigma, const float* bias,

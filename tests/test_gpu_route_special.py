@@ -84,3 +84,28 @@ def test_both_routers_agree_on_special_logits(mode, M, k, kind):
     np.testing.assert_allclose(whole["gate"][ok], ref["g"][ok], rtol=1e-5, atol=1e-6)
     ctx.check_status()
     ctx.close()
+
+
+@pytest.mark.parametrize("T", [1, 33, 300, 513])
+@pytest.mark.parametrize("shift", [0, 1])
+def test_prepared_weights_are_a_copy(T, shift):
+    """What unipool_router_prepare was given counts until it is called again, whichever router takes the call; weights that
+    were not prepared count as they are."""
+    M, d, L = 40, 192, 3
+    ctx = B.Context(B.make_config(d, 64, M, 2, L, 513, B.BF16, 1e-6, 2.0))
+    g = torch.Generator(device="cuda").manual_seed(T)
+    W = torch.zeros(L * M * d + shift, device="cuda")[shift:].view(L, M, d).normal_(0, 0.02, generator=g)
+    x = torch.randn(T, d, device="cuda", generator=g).bfloat16()
+    first = W.clone()
+    z = lambda w: x.double() @ w.double().T
+    near = lambda out, w: np.abs(out["z"] - to_np(z(w))).max() < 1e-5 * np.abs(out["z"]).max()
+    ctx.router_prepare(W, L, M)
+    W.normal_(0, 0.02, generator=g)
+    for l in range(L):
+        assert near(route(ctx, x, W[l], None, 2), first[l])
+    ctx.router_prepare(W, L, M)
+    assert near(route(ctx, x, W[2], None, 2), W[2])
+    ctx.router_prepare(None, 0, M)
+    W.copy_(first)
+    assert near(route(ctx, x, W[1], None, 2), first[1])
+    ctx.close()
