@@ -45,9 +45,12 @@ void set_error(const char* fmt, ...);
   } while (0)
 
 // ---------------------------------------------------------------- launches
-// Every kernel of a pass is launched with programmatic serialization: the launch itself, and what a kernel does before
-// grid_wait(), run while the last blocks of the kernel before it in the stream drain; its memory is touched behind
-// grid_wait() only.  Between two kernels of an eager pass lie 0.2 us instead of 2.0 .. 2.8; a pass of 16 experts of
+// Every kernel of a pass is launched with programmatic serialization and waits for the one before it in grid_wait(), behind
+// what of its set-up needs no memory of others (the router on the tensor cores reads two flags first and waits in front of its
+// own).  No kernel triggers its successor early, so that a kernel's blocks start when the last block of the kernel before
+// has left: hidden are the launch and the flush of that kernel's writes, not its last blocks.  (An early trigger would put
+// two kernels' blocks on an SM, which their tensor memory, allocated whole, and shared memory do not allow.)
+// Between two kernels of an eager pass lie 0.2 us instead of 2.0 .. 2.8; a pass of 16 experts of
 // 256 x 512 over 512 tokens in fp32 (55 launches) takes 856 us instead of 959, a forward pass of 33 tokens through
 // twelve layers 1509 instead of 1632, a step of 16384 tokens over private experts 12455 instead of 12772.
 // Not while a stream is captured: the kernels of a graph follow one another within 0.3 us as they are, and with programmatic

@@ -8,8 +8,9 @@
 // Bound by the FMA pipe and, as high, the register side of shared memory (8 x 8 results: 64 bytes a lane for 64 products,
 // 128 bytes a clock), in fact by how few warps a launch of the fp32 sizes gives a scheduler: one alone issues in 57 % of
 // its clocks, three in 72 %, three quarters of it FMAs.  Four positions unrolled twice: all sixteen miss the instruction
-// cache, and their loads, moved up, take 255 registers.  Plain FMAs: packed ones (fma.rn.f32x2) take two issue slots, and
-// about one register move each.  32 x 128 tiles load less per product, and were no faster for their fewer warps.
+// cache, and their loads, moved up, take 255 registers.  Plain FMAs: packed ones (fma.rn.f32x2) keep the pipe twice as long
+// and cost about one register move each, which pays only where issue slots run out (the block tile below).  32 x 128 tiles
+// load less per product, and were no faster for their fewer warps.
 #pragma once
 
 #include "common.cuh"
@@ -204,9 +205,10 @@ struct SimtTile {
 // double-buffered shared memory, fetched into registers one chunk ahead with 16-byte loads (four of 4 bytes where an operand
 // misses that alignment: an eighth of the instructions that 4-byte cp.async would take), and the operands of step k + 1
 // are read while step k is multiplied.  KG groups share a tile by taking every KG-th chunk.
-// Per product it moves two thirds of the warp tile's bytes through L2 and shared memory's other side, which is what counts
-// once every scheduler has warps enough: 16 experts of 1024 x 4096, 512 rows each, forward 43 TFLOP/s against 37 to 41
-// (the rule and the figures: expert_simt.cu).  Twelve warps on an SM, 160 to 168 registers.
+// Its packed products take half the issue slots, which is what counts once every scheduler has warps enough: 16 experts of
+// 512 x 1024, 512 rows each, FMA pipe busy 60 to 66 % of the time in 51 to 54 % of the issue slots, against 54 to 61 % in 68 to 81
+// % with warp tiles (gate/up 482 -> 405 us under the profiler; the rule and more figures: expert_simt.cu).  Twelve warps on an SM,
+// 160 to 168 registers.
 template <int KG>
 struct SimtBlockTile {
   static constexpr int kGroup = 64, kRows = 64, kThreads = KG * kGroup, kBlocks = 6 / KG, MR = 8, NR = 8;
