@@ -208,6 +208,8 @@ int rows_gemm(unipool_ctx* ctx, RowGemm p, int n_experts, cudaStream_t s) {
   //   32 of 256 x 704, 14 rows              (660) 43/41/45/74, 71   (120) 52/30/27/19, 33   (330) 45/38/39/53, 54   (120) 102/54/47/28, 56
   //   15 of 384 x 512, 91 rows              (800) 56/45/46/53, 56   (300) 40/35/28/28, 31   (400) 52/38/27/32, 41   (300) 76/66/50/48, 53
   //   64 of 192 x 128, 250 rows             dgrad down (1064) 53/53/47/56, 67
+  // Eight against four over ten more stacks of 8 to 40 experts: 0.59 to 0.99 of the time at 114 to 153 tiles and K from 256, 0.98 to 1.06
+  // from 165 tiles on.  Two against four in gate/up of 820 to 1820 tiles, K < 256: 0.91 to 1.01.
   if (10 * tiles <= 11 * ctx->sm_count && p.K >= (tiles <= ctx->sm_count ? 256 : 512))
     return rows_gemm_as<SimtTile<8>, BM, EPI>(ctx, p, s);
   if constexpr (BM == kAlongK) {
