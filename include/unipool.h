@@ -143,7 +143,8 @@ int unipool_route(unipool_ctx* ctx, const void* x, int32_t T, const float* W_r, 
 /* Optional set-up of the routers of a bf16 context, once per parameter update.  unipool_route and
  * unipool_route_bwd compute the fp32 logits of Eq. 7 on the tensor cores from three bf16 terms of the
  * fp32 router weights (W = W0 + W1 + W2, every product exact in fp32); unipool_route of few tokens (464
- * at most on 148 SMs) multiplies the weights in fp32.  Without this call each of them reads
+ * at most on 148 SMs) multiplies the weights in fp32 (after unipool_stack_forward, which prepares the routers
+ * for itself and its backward pass but keeps no copy, from the terms).  Without this call each of them reads
  * the W_r it is given, and splits it if it needs the terms, on every call.  With it the terms and a copy of
  * all n_layers routers (W_r [n_layers, n_experts, d], contiguous) are formed by one kernel and kept in the workspace: a
  * later route / route_bwd call whose W_r points at one of these layers (W_r + l*n_experts*d) uses

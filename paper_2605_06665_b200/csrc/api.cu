@@ -161,6 +161,7 @@ int unipool_create(unipool_ctx** out, const unipool_config* cfg, void* workspace
   ctx->tmap_cache = nullptr;
   ctx->prepared_base = nullptr;
   ctx->prepared_layers = ctx->prepared_experts = 0;
+  ctx->prepared_copied = ctx->prepared_now = ctx->copy_read = false;
   cudaError_t e = cudaGetDevice(&ctx->device);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device);
   // the self-cleaning accumulators and the status word start at zero
@@ -267,7 +268,7 @@ int unipool_router_prepare(unipool_ctx* ctx, const float* W_r, int32_t n_layers,
              "n_layers = %d outside [0, %d]", n_layers, ctx->cfg.n_layers);
   if (n_layers > 0) { CHECK_PTR(W_r); CHECK_ROUTER_WIDTH(ctx, n_experts); }
   if (!use_tensor_cores(ctx)) return UNIPOOL_OK;            // the fp32 path reads W_r itself
-  return router_prepare_launch(ctx, W_r, n_layers, n_experts, static_cast<cudaStream_t>(stream));
+  return router_prepare_launch(ctx, W_r, n_layers, n_experts, !ctx->prepared_now || ctx->copy_read, static_cast<cudaStream_t>(stream));
 }
 
 int unipool_dispatch_rows(unipool_ctx* ctx, const void* x, int32_t T, const int32_t* idx,

@@ -154,6 +154,9 @@ struct unipool_ctx {
   void* tmap_cache;   // opaque, owned by the tensor-core GEMM module
   const float* prepared_base;   // router weights last given to unipool_router_prepare (NULL: none)
   int prepared_layers, prepared_experts;
+  bool prepared_copied;         // their fp32 weights were kept too (ws.w_copy)
+  bool prepared_now;            // they were prepared by the running call, from the weights as they are
+  bool copy_read;               // some launch reads ws.w_copy, recorded in a graph maybe: every preparation keeps it up to date
 };
 
 namespace unipool {
@@ -246,11 +249,11 @@ struct PoolWgradArgs {
 int route_tc_launch(unipool_ctx*, const void* x, int T, const float* W_r, float sigma, const float* bias,
                     int n_experts, int32_t* idx, float* gate, int32_t* counts, float* score_sum,
                     float* znorm, float* z_saved, cudaStream_t);
-bool route_on_few(const unipool_ctx*, int T, int n_experts);
+bool route_on_few(const unipool_ctx*, const float* W_r, int T, int n_experts);
 int route_few_launch(unipool_ctx*, const void* x, int T, const float* W_r, float sigma, const float* bias,
                      int n_experts, int32_t* idx, float* gate, int32_t* counts, float* score_sum,
                      float* znorm, float* z_saved, cudaStream_t);
-int router_prepare_launch(unipool_ctx*, const float* W_r, int n_layers, int n_experts, cudaStream_t);
+int router_prepare_launch(unipool_ctx*, const float* W_r, int n_layers, int n_experts, bool copy, cudaStream_t);
 int prepared_layer(const unipool_ctx*, const float* W_r, int n_experts);
 int route_bwd_tc_launch(unipool_ctx*, const void* x, int T, const float* W_r, float sigma, int n_experts,
                         const float* znorm, const float* z_saved, const int32_t* idx, const float* dgate,

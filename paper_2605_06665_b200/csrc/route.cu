@@ -173,7 +173,7 @@ int route_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float
     return UNIPOOL_OK;
   }
   if (ctx->cfg.dtype == UNIPOOL_BF16)
-    return (route_on_few(ctx, T, M) ? route_few_launch : route_tc_launch)(ctx, x, T, W_r, sigma, bias, M, idx, gate, counts,
+    return (route_on_few(ctx, W_r, T, M) ? route_few_launch : route_tc_launch)(ctx, x, T, W_r, sigma, bias, M, idx, gate, counts,
                                                                          score_sum, znorm, z_saved, s);
   {
     PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_LOGITS, 1, s);

@@ -223,7 +223,10 @@ int few_tokens(const unipool_ctx* ctx, int T, int M) {
 
 }  // namespace
 
-bool route_on_few(const unipool_ctx* ctx, int T, int M) { return few_tokens(ctx, T, M) > 0; }
+// (prepared weights count as they were: of those without a copy the other router has the terms)
+bool route_on_few(const unipool_ctx* ctx, const float* W_r, int T, int M) {
+  return few_tokens(ctx, T, M) > 0 && (ctx->prepared_now || ctx->prepared_copied || prepared_layer(ctx, W_r, M) < 0);
+}
 
 int route_few_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, float sigma, const float* bias, int M,
                      int32_t* idx, float* gate, int32_t* counts, float* score_sum, float* znorm, float* z_saved,
@@ -231,8 +234,11 @@ int route_few_launch(unipool_ctx* ctx, const void* x, int T, const float* W_r, f
   // what the tensor maps of the other router ask for, whatever the number of tokens
   UP_REQUIRE(aligned16(x) && ((M & 3) != 0 || aligned16(z_saved)), UNIPOOL_ERR_INVALID_ARG,
              "tensor base %p is not 16-byte aligned", aligned16(x) ? static_cast<const void*>(z_saved) : x);
-  const int layer = prepared_layer(ctx, W_r, M);             // then the weights are those of that time
-  if (layer >= 0) W_r = ctx->ws.w_copy + (int64_t)layer * M * ctx->cfg.d_model;
+  const int layer = ctx->prepared_now ? -1 : prepared_layer(ctx, W_r, M);
+  if (layer >= 0) {
+    W_r = ctx->ws.w_copy + (int64_t)layer * M * ctx->cfg.d_model;
+    ctx->copy_read = true;
+  }
   FewParams p{};
   p.x = static_cast<const __nv_bfloat16*>(x); p.W_r = W_r; p.bias = bias;
   p.T = T; p.M = M; p.d = ctx->cfg.d_model; p.k = ctx->cfg.top_k;

@@ -625,16 +625,17 @@ static int router_split_launch(unipool_ctx* ctx, const float* W_r, int n_layers,
   return UNIPOOL_OK;
 }
 
-int router_prepare_launch(unipool_ctx* ctx, const float* W_r, int n_layers, int M, cudaStream_t s) {
+int router_prepare_launch(unipool_ctx* ctx, const float* W_r, int n_layers, int M, bool copy, cudaStream_t s) {
   ctx->prepared_base = nullptr;
   if (n_layers == 0) return UNIPOOL_OK;
   PhaseTimer pt(ctx, UNIPOOL_PH_ROUTE_LOGITS, 1, s);
   const int rc = router_split_launch(ctx, W_r, n_layers, M, static_cast<__nv_bfloat16*>(ctx->ws.w_split),
-                                     ctx->ws.w_copy, ctx->ws.split_any, s);
+                                     copy ? ctx->ws.w_copy : nullptr, ctx->ws.split_any, s);
   if (rc != UNIPOOL_OK) return rc;
   ctx->prepared_base = W_r;
   ctx->prepared_layers = n_layers;
   ctx->prepared_experts = M;
+  ctx->prepared_copied = copy;
   return UNIPOOL_OK;
 }
 

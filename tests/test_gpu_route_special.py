@@ -109,3 +109,29 @@ def test_prepared_weights_are_a_copy(T, shift):
     W.copy_(first)
     assert near(route(ctx, x, W[1], None, 2), first[1])
     ctx.close()
+
+
+def test_weights_of_a_stack_pass_stay_prepared():
+    """After a pass through a stack, calls for its routers work with the weights of that pass (without a copy of them: from their
+    terms), a later pass with the weights as they are then; also when a call that reads the copy came in between."""
+    from paper_2605_06665_b200.stack import UniPoolStack
+    T, M, d = 33, 24, 128
+    st = UniPoolStack(2, d, 64, M, 2, T, "bf16", c=2.0)
+    g = torch.Generator(device="cuda").manual_seed(9)
+    for t in (st.W_gu, st.W_down, st.W_r):
+        t.normal_(0, 0.05, generator=g)
+    x = torch.randn(T, d, device="cuda", generator=g).bfloat16()
+    near = lambda z, w: np.abs(to_np(z) - to_np(x.double() @ w.double().T)).max() < 1e-5 * np.abs(to_np(z)).max()
+    for copied in (False, True, True):
+        if copied:                                             # read the copy once: from then on every pass keeps one
+            st.ctx.router_prepare(st.W_r, 2, M)
+            route(st.ctx, x, st.W_r[0], None, 2)
+        st.forward(x)
+        assert near(st.z[0], st.W_r[0])
+        old = st.W_r.clone()
+        st.W_r.normal_(0, 0.05, generator=g)
+        ctx_z = route(st.ctx, x, st.W_r[0], None, 2)["z"]
+        assert near(torch.from_numpy(ctx_z), old[0])
+        st.forward(x)
+        assert near(st.z[0], st.W_r[0])
+    st.close()
